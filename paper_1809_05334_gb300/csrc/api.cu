@@ -94,7 +94,7 @@ struct vie_ctx {
     std::string err;
     std::shared_ptr<MeshState> mesh = std::make_shared<MeshState>();
     // request (device)
-    DevBuf row, coef, wt, kap, ieps, frow, qs, perm, pol, orders, stab, ztab, rtab, ew;
+    DevBuf row, coef, wt, kap, ieps, frow, qs, perm, pol, orders, stab, ztab, rtab, ew, fcoef, frec;
     double z_extent = 0;
     // solve buffers
     DevBuf Z, b, x, r, u, w, V, h, y, Minv, MinvH, amax, tcpack, tcpack2, status, acc, J, rt, cout, xs;
@@ -215,6 +215,16 @@ int prepare(vie_ctx *ctx, const vie_request *req, HostReq &H) {
     return VIE_OK;
 }
 
+// the spectral polynomials of the far kernels and their coefficients on the device
+int far_poly(vie_ctx *ctx, const vie::EwaldTables &ew, vie::DevReq &q, cudaStream_t st) {
+    std::vector<float> coef;
+    vie::build_far_poly(ew, q.ef, q.fp, coef);
+    if (coef.empty()) coef.assign(1, 0.f);
+    CK(upload(ctx->fcoef, coef, st));
+    q.fcoef = ctx->fcoef.as<float>();
+    return VIE_OK;
+}
+
 // upload the per-request arrays and build the device views
 int upload_request(vie_ctx *ctx, const HostReq &H, vie::DevReq &q, cudaStream_t st) {
     const vie::Topology &T = ctx->mesh->topo;
@@ -273,6 +283,13 @@ int upload_request(vie_ctx *ctx, const HostReq &H, vie::DevReq &q, cudaStream_t 
     q.rtab = ctx->rtab.as<float4>();
     q.ew = ctx->ew.as<vie::EwaldTables>();
     q.ef = vie::make_ewald_f32(H.ew);
+    if (int e = far_poly(ctx, H.ew, q, st)) return e;
+    const size_t nt = (size_t)T.nt;
+    CK(ctx->frec.ensure(sizeof(float4) * vie::far_record_count(nt, (size_t)nf)));
+    q.ptet = ctx->frec.as<float4>();
+    q.etet = q.ptet + 16 * nt;
+    q.pface = q.etet + 9 * nt;
+    q.eface = q.pface + 12 * ((size_t)nf + 1);
     q.k0 = H.k0; q.kx = H.kx; q.ky = H.ky;
     for (int k = 0; k < 9; ++k) {
         const double phs = H.kx * (k / 3 - 1) * ctx->mesh->topo.a + H.ky * (k % 3 - 1) * ctx->mesh->topo.b;
@@ -1576,9 +1593,16 @@ int vie_green(vie_ctx *ctx, const vie_request *req, const double *d, double *out
     CK(dd.ensure(sizeof(double) * 3 * n));
     CK(dout.ensure(sizeof(double) * 2 * n));
     CK(cudaMemcpy(dd.p, d, sizeof(double) * 3 * n, cudaMemcpyHostToDevice));
-    CK(vie::launch_green(dd.as<double>(), dout.as<double>(), n, precision == VIE_FP64, ctx->stab.as<float>(),
-                         ctx->ztab.as<float2>(), ctx->ew.as<vie::EwaldTables>(), vie::make_ewald_f32(H.ew), st,
-                         ctx->rtab.as<float4>()));
+    vie::DevReq q{};   // the far kernels' form where the request has one
+    q.ef = vie::make_ewald_f32(H.ew);
+    q.stab = ctx->stab.as<float>();
+    if (precision != VIE_FP64)
+        if (int pe = far_poly(ctx, H.ew, q, st)) return pe;
+    if (q.fp.mode != vie::FAR_NONE)
+        CK(vie::launch_green_poly(dd.as<double>(), dout.as<double>(), n, q, st));
+    else
+        CK(vie::launch_green(dd.as<double>(), dout.as<double>(), n, precision == VIE_FP64, ctx->stab.as<float>(),
+                             ctx->ztab.as<float2>(), ctx->ew.as<vie::EwaldTables>(), q.ef, st));
     CK(cudaMemcpy(out, dout.p, sizeof(double) * 2 * n, cudaMemcpyDeviceToHost));
     return VIE_OK;
 }
@@ -1626,6 +1650,7 @@ void release_device_memory(vie_ctx *ctx) {
     ctx->mesh = std::make_shared<MeshState>();
     DevBuf *bufs[] = {&ctx->row, &ctx->coef, &ctx->wt, &ctx->kap, &ctx->ieps, &ctx->frow, &ctx->qs,
                       &ctx->perm, &ctx->pol, &ctx->orders, &ctx->stab, &ctx->ztab, &ctx->rtab, &ctx->ew,
+                      &ctx->fcoef, &ctx->frec,
                       &ctx->Z, &ctx->b, &ctx->x, &ctx->r, &ctx->u, &ctx->w, &ctx->V, &ctx->h, &ctx->y,
                       &ctx->Minv, &ctx->MinvH, &ctx->amax, &ctx->tcpack, &ctx->tcpack2, &ctx->status, &ctx->acc,
                       &ctx->J, &ctx->xs, &ctx->Zh, &ctx->dens,

@@ -31,6 +31,16 @@ template <typename T> __device__ __forceinline__ void cfma(cx<T> &acc, T s, cx<T
     acc.im = fma(s, a.im, acc.im);
 }
 
+// Moments of one ordered element pair: sums of g, r_x g, r_y g and (r_x.r_y) g
+// (r relative to the elements' centroids).
+template <typename T> struct Mom {
+    cx<T> S, A[3], B[3], C;
+    __device__ void zero() {
+        S = {0, 0}; C = {0, 0};
+        for (int d = 0; d < 3; ++d) { A[d] = {0, 0}; B[d] = {0, 0}; }
+    }
+};
+
 // ---------------------------------------------------------------------------
 // Faddeeva function w(z) = exp(-z^2) erfc(-j z) for Im z >= 0 by Weideman's
 // rational expansion (SIAM J. Numer. Anal. 31, 1994):

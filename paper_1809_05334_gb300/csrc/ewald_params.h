@@ -66,7 +66,7 @@ struct EwaldF32 {
     int near_img[9];
     int n_img, p0, np, q0, nq, sym;
     float xs_max, xs_inv_h, z_inv_h, e_mb2, Ef, kx, ky, step_x, step_y;
-    float Eih;                            // E * xs_inv_h: table abscissa per unit distance
+    float Eih;                            // E * xs_inv_h: table intervals per unit distance (a power of two)
     int sq_pq;                            // max(P, Q) >= 1 of the short form; 0 where it does not apply
     int sq_off[SQ_MAX + 1][SQ_MAX + 1];   // order (p, q): offset of its real table in rtab (float4 units)
     int sq_im;                            // offset of the (0, 0) order's imaginary table in rtab
@@ -75,6 +75,24 @@ struct EwaldF32 {
     float ob_kx0, ob_ky0;                 // k_par + 2 pi (p0 / a, q0 / b): the rectangle's first order
     int ob_off[OB_MAX][OB_MAX];           // rectangle entry (i, j): offset of its real table in rtab
     int ob_im[OB_MAX][OB_MAX];            // offset of its imaginary table (propagating order), else -1
+};
+// Spectral series of the far kernels as polynomials.  G_pq(|z|) is an even
+// entire function of z, so on |z| <= z_max each order is one polynomial in
+// t = 2 (z / z_max)^2 - 1, evaluated from warp-uniform coefficients (no gather
+// of table entries per lane).  Orders are kept by row: row i has `nq` columns
+// (the columns of the short form's map: q = 0 .. nq - 1 at normal incidence and
+// in the k_y = 0 fold, the rectangle's columns otherwise) and the degree of its
+// widest column, rounded up to even.  Coefficients: per row [deg + 1][nq rounded up to even] floats
+// from the highest power down, at `off`; the imaginary parts (propagating orders) of rows that have
+// any at `im_off`.
+constexpr int FP_ROWS = 8;
+constexpr int FP_MAX_DEG = 31;
+constexpr int FP_MAX_COEF = 2048;   // 16 KB of shared memory as (c, c) pairs
+enum FarMode : int { FAR_NONE = 0, FAR_NORMAL = 1, FAR_FOLD = 2, FAR_FULL = 3 };
+struct FarPoly {
+    int mode, nq, rows, n_coef;
+    int off[FP_ROWS], deg[FP_ROWS], im_off[FP_ROWS], im_deg[FP_ROWS];   // im_deg -1: no imaginary part
+    float t_scale;   // t = t_scale (z Eih)^2 - 1
 };
 // Ewald splitting parameter: sqrt(pi / ab) balances the spatial and spectral
 // series, bounded below by k0/6 (b = k0 / 2E <= 3 keeps exp(b^2) moderate).  The
@@ -124,7 +142,7 @@ inline EwaldF32 make_ewald_f32(const EwaldTables &t) {
     f.n_img = t.n_img; f.p0 = t.p0; f.np = t.np; f.q0 = t.q0; f.nq = t.nq; f.sym = t.sym;
     f.xs_max = t.xs_max; f.xs_inv_h = t.xs_inv_h; f.z_inv_h = t.z_inv_h; f.e_mb2 = t.e_mb2; f.Ef = t.Ef;
     f.kx = t.kx; f.ky = t.ky; f.step_x = t.step_x; f.step_y = t.step_y;
-    f.Eih = t.Ef * t.xs_inv_h;
+    f.Eih = (float)std::exp2(std::round(std::log2((double)t.Ef * t.xs_inv_h)));   // a power of two (ewald_tables.cpp)
     f.sq_pq = 0;
     const int zero = t.n_tab * NZTAB;   // the zero table
     for (int p = 0; p <= SQ_MAX; ++p)

@@ -5,6 +5,7 @@
 // it).
 #include <algorithm>
 #include <cmath>
+#include <complex>
 #include <cstring>
 #include <vector>
 
@@ -84,7 +85,10 @@ int build_ewald_tables(double a, double b, double k0, double kx, double ky, doub
     // tabulated FP32 path: the truncation of the FP32 series
     const double xc32 = FP32_XCUT, zr = std::max(z_extent, 1e-6) * (1.0 + 1e-6);
     E.xs_max = (float)(xc32 + 0.5);
-    E.xs_inv_h = (float)(NSPAT / (xc32 + 0.5));
+    // intervals per unit of x: such that E xs_inv_h, the table intervals per unit of
+    // distance, is a power of two (distances scaled to table units stay exact) and
+    // the cut falls in the table's upper half
+    E.xs_inv_h = (float)(std::exp2(std::floor(std::log2(NSPAT * E.E / (xc32 + 0.5)))) / E.E);
     E.z_max = (float)zr;
     E.z_inv_h = (float)(NZTAB / zr);
     E.e_mb2 = (float)std::exp(-E.bb * E.bb);
@@ -125,6 +129,169 @@ int build_ewald_tables(double a, double b, double k0, double kx, double ky, doub
         }
     E.n_tab = nt;
     return VIE_OK;
+}
+
+// ---------------------------------------------------------------------------
+// Polynomials of the spectral series
+// ---------------------------------------------------------------------------
+namespace {
+
+using cd = std::complex<double>;
+
+// w(j u) = erfcx(u), Re u >= 0, by Weideman's rational expansion with 40 terms
+// (SIAM J. Numer. Anal. 31, 1994), FP64
+cd erfcx_host(cd u) {
+    constexpr int NT = 40;
+    static const std::vector<double> a = [] {
+        std::vector<double> c(NT + 1, 0.0);
+        const double L = std::sqrt(NT / std::sqrt(2.0));
+        const int M = 16 * NT;
+        for (int k = 0; k < M; ++k) {
+            const double th = -M_PI + (k + 0.5) * 2.0 * M_PI / M, t = L * std::tan(0.5 * th);
+            const double F = std::exp(-t * t) * (L * L + t * t);
+            for (int n = 0; n <= NT; ++n) c[n] += F * std::cos(n * th) / M;
+        }
+        return c;
+    }();
+    const double L = std::sqrt(NT / std::sqrt(2.0));
+    const cd inv = 1.0 / (L + u), z = (L - u) * inv;
+    cd p = a[NT];
+    for (int n = NT - 1; n >= 1; --n) p = cd(p.real() * z.real() - p.imag() * z.imag() + a[n], p.real() * z.imag() + p.imag() * z.real());
+    return inv * (2.0 * p * inv + 1.0 / std::sqrt(M_PI));
+}
+
+// G(z) of table tb: [e^{gz} erfc(g/2E + zE) + e^{-gz} erfc(g/2E - zE)] / (4ab g)
+cd spectral_value(const EwaldTables &t, int tb, double z) {
+    const double E = t.E, gr = t.tab_gamma[tb][0], gi = t.tab_gamma[tb][1];
+    if (gi == 0.0) {
+        const double u = gr / (2 * E);
+        return (std::exp(gr * z) * std::erfc(u + z * E) + std::exp(-gr * z) * std::erfc(u - z * E)) * t.tab_ig[tb][0];
+    }
+    const cd e1 = erfcx_host(cd(z * E, gi / (2 * E)));
+    const double pre = t.tab_pre[tb] * std::exp(-(z * E) * (z * E));
+    const cd sum(2.0 * std::cos(gi * z), 2.0 * pre * e1.imag() - 2.0 * std::sin(gi * z));
+    return sum * cd(t.tab_ig[tb][0], t.tab_ig[tb][1]);
+}
+
+}  // namespace
+
+void build_far_poly(const EwaldTables &t, const EwaldF32 &f, FarPoly &fp, std::vector<float> &coef) {
+    fp = FarPoly{};
+    coef.clear();
+    const int Q = (t.nq - 1) / 2;
+    int rows = 0, nq = 0, mode = FAR_NONE;
+    if (t.sym && f.sq_pq > 0) {
+        mode = FAR_NORMAL;
+        rows = (t.np - 1) / 2 + 1;
+        nq = std::max(3, Q + 1);
+    } else if (!t.sym && f.ob_nr > 0) {
+        mode = f.ob_nq1 > 0 ? FAR_FOLD : FAR_FULL;
+        rows = t.np;
+        nq = f.ob_nq1 > 0 ? std::max(3, Q + 1) : (t.nq <= 4 ? 4 : (t.nq == 7 ? 8 : t.nq));
+    }
+    if (mode == FAR_NONE || rows > FP_ROWS) return;
+    // table of entry (i, j) of the map, -1 outside the cut; whether it is propagating
+    auto entry = [&](int i, int j, bool &prop) {
+        prop = false;
+        int off, im = -1;
+        if (mode == FAR_NORMAL) {
+            off = f.sq_off[i][j];
+            prop = i == 0 && j == 0 && f.sq_im != t.n_tab * NZTAB;
+        } else {
+            off = f.ob_off[i][j];
+            im = f.ob_im[i][j];
+            prop = im >= 0;
+        }
+        const int tb = off / NZTAB;
+        return tb == t.n_tab ? -1 : tb;
+    };
+    // Chebyshev coefficients of every table in use, in t on [-1, 1], from M nodes
+    // (the degree grows as 3.5 + 3.8 E z_max; M leaves room for the tail to show)
+    const double zm = t.z_max, Ez = t.E * zm;
+    if (!(Ez < 9.0)) return;
+    const int M = std::min(48, std::max(14, (int)std::ceil(13 + 4.6 * Ez)));
+    std::vector<std::vector<double>> re(t.n_tab), im(t.n_tab);
+    std::vector<double> cs((size_t)M * M);
+    for (int k = 0; k < M; ++k)
+        for (int n = 0; n < M; ++n) cs[(size_t)k * M + n] = std::cos(M_PI * n * (k + 0.5) / M);
+    double gmax = 0;
+    for (int i = 0; i < rows; ++i)
+        for (int j = 0; j < nq; ++j) {
+            bool prop;
+            const int tb = entry(i, j, prop);
+            if (tb < 0 || !re[tb].empty()) continue;
+            std::vector<double> vr(M), vi(M);
+            for (int k = 0; k < M; ++k) {
+                const double tt = cs[(size_t)k * M + 1];
+                const cd g = spectral_value(t, tb, zm * std::sqrt(0.5 * (tt + 1.0)));
+                vr[k] = g.real();
+                vi[k] = g.imag();
+                gmax = std::max(gmax, std::fabs(vr[k]));
+            }
+            re[tb].assign(M, 0.0);
+            im[tb].assign(M, 0.0);
+            for (int n = 0; n < M; ++n) {
+                double sr = 0, si = 0;
+                for (int k = 0; k < M; ++k) {
+                    sr += vr[k] * cs[(size_t)k * M + n];
+                    si += vi[k] * cs[(size_t)k * M + n];
+                }
+                re[tb][n] = (n ? 2.0 : 1.0) / M * sr;
+                im[tb][n] = (n ? 2.0 : 1.0) / M * si;
+            }
+        }
+    if (!(gmax > 0) || !std::isfinite(gmax)) return;
+    // a column keeps its terms until the rest is below 1e-9 of the largest order
+    // (the FP32 rounding of the sum is 6e-8 of it)
+    const double tol = 1e-9 * gmax;
+    auto degree = [&](const std::vector<double> &c) {
+        double rest = 0;
+        int d = M - 1;
+        while (d > 0 && rest + std::fabs(c[d]) <= tol) rest += std::fabs(c[d--]);
+        return d;
+    };
+    // Chebyshev series up to degree d as a polynomial in t
+    auto monomial = [](const std::vector<double> &c, int d) {
+        std::vector<double> out(d + 1, 0.0), a(d + 1, 0.0), b(d + 1, 0.0), n(d + 1);
+        a[0] = 1.0;   // T_0
+        out[0] += c[0];
+        if (d >= 1) { b[1] = 1.0; out[1] += c[1]; }
+        for (int k = 2; k <= d; ++k) {
+            for (int q = 0; q <= d; ++q) n[q] = (q ? 2.0 * b[q - 1] : 0.0) - a[q];
+            for (int q = 0; q <= k; ++q) out[q] += c[k] * n[q];
+            a.swap(b);
+            b.swap(n);
+        }
+        return out;
+    };
+    fp.rows = rows;
+    fp.nq = nq;
+    for (int i = 0; i < rows; ++i)
+        for (int part = 0; part < 2; ++part) {   // real, imaginary
+            int deg = part ? -1 : 0;
+            std::vector<std::vector<double>> col(nq);
+            for (int j = 0; j < nq; ++j) {
+                bool prop;
+                const int tb = entry(i, j, prop);
+                if (tb < 0 || (part && !prop)) continue;
+                const std::vector<double> &c = part ? im[tb] : re[tb];
+                const int d = degree(c);
+                if (d > FP_MAX_DEG - 1) { fp = FarPoly{}; coef.clear(); return; }
+                col[j] = monomial(c, d);
+                deg = std::max(deg, d);
+            }
+            if (deg > 0) deg = (deg + 1) & ~1;   // even: the kernels take two powers per step
+            (part ? fp.im_off : fp.off)[i] = (int)coef.size();
+            (part ? fp.im_deg : fp.deg)[i] = deg;
+            for (int n = deg; n >= 0; --n)
+                for (int j = 0; j < ((nq + 1) & ~1); ++j)
+                    coef.push_back(j < nq && n < (int)col[j].size() ? (float)col[j][n] : 0.f);
+        }
+    if ((int)coef.size() > FP_MAX_COEF) { fp = FarPoly{}; coef.clear(); return; }
+    fp.n_coef = (int)coef.size();
+    const double zs = zm * f.Eih;
+    fp.t_scale = (float)(2.0 / (zs * zs));
+    fp.mode = mode;
 }
 
 }  // namespace vie

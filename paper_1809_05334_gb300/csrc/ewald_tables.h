@@ -12,4 +12,11 @@ int build_ewald_tables(double a, double b, double k0, double kx, double ky, doub
                        EwaldTables &E, std::vector<double> *orders, const char **why,
                        double split_mult = 0.0);
 
+// Polynomials of the spectral series for the far kernels (FarPoly) from the
+// order map of make_ewald_f32: fp.mode = FAR_NONE where no short form applies,
+// or where an order needs a degree above FP_MAX_DEG (a cell several periods
+// thick); then the general tabulated form is used.  coef receives fp.n_coef
+// floats.
+void build_far_poly(const EwaldTables &t, const EwaldF32 &f, FarPoly &fp, std::vector<float> &coef);
+
 }  // namespace vie

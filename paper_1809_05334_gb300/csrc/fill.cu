@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "device_math.cuh"
+#include "far_poly.cuh"
 #include "fill.h"
 
 namespace vie {
@@ -117,7 +118,7 @@ __global__ void k_build_tables(const EwaldTables *__restrict__ ew, float *stab, 
                                float4 *rtab) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < NSPAT) {
-        const double h = double(ew->xs_max) / NSPAT;
+        const double h = 1.0 / double(ew->xs_inv_h);
         double F0, D0, F1, D1, c[4];
         spatial_node(ew, i * h, F0, D0);
         spatial_node(ew, (i + 1) * h, F1, D1);
@@ -212,18 +213,14 @@ template <typename T> constexpr size_t stab_bytes() { return sizeof(T) == 4 ? 4 
 // ---------------------------------------------------------------------------
 // helpers
 // ---------------------------------------------------------------------------
-template <typename T> struct Mom {
-    cx<T> S, A[3], B[3], C;
-    __device__ void zero() {
-        S = {0, 0}; C = {0, 0};
-        for (int d = 0; d < 3; ++d) { A[d] = {0, 0}; B[d] = {0, 0}; }
-    }
-};
-
 template <typename T>
 __device__ __forceinline__ void atomic_add_c(T *Z, size_t idx, cx<T> v) {
-    atomicAdd(Z + 2 * idx, v.re);
-    atomicAdd(Z + 2 * idx + 1, v.im);
+    if constexpr (sizeof(T) == 4) {
+        red_c(Z, idx, v.re, v.im);
+    } else {
+        atomicAdd(Z + 2 * idx, v.re);
+        atomicAdd(Z + 2 * idx + 1, v.im);
+    }
 }
 
 __device__ __forceinline__ cx<double> ld2(const double *p) { return {p[0], p[1]}; }
@@ -232,6 +229,11 @@ __device__ __forceinline__ cx<double> ld2(const double *p) { return {p[0], p[1]}
 template <typename T>
 __device__ void scatter_tt(const DevMesh &m, const DevReq &q, T *Z, size_t N, int t, int s,
                            const Mom<T> &mo) {
+    if constexpr (sizeof(T) == 4) {
+        scatter_rec<false>(Z, N, float(q.k0 * q.k0), load_tet_rec(q.etet, m.nt, t), load_tet_rec(q.etet, m.nt, s), mo,
+                           false);
+        return;
+    }
     const T *ft = m.far<T>(t);
     const T *fs = m.far<T>(s);
     const T k2 = T(q.k0 * q.k0);
@@ -344,537 +346,6 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 8 : 6)
     if (s != t) scatter_tt<T>(m, q, Z, N, s, t, mr);
 }
 
-// Interval min(floor(x), n - 1) of a table of n intervals and the offset v in
-// it (v in [0, 1]; x >= 0 clamped to n first, so x = n gives interval n - 1 at
-// v = 1), without float <-> int conversions (they run on the quarter-rate
-// pipe): x + 2^23 rounded down holds floor(x) in its low mantissa bits.
-// Callers test the unclamped x against the table's range where it can exceed it.
-__device__ __forceinline__ int table_index(float x, int n, float &v) {
-    const float xc = fminf(x, float(n));
-    const float t = __fadd_rd(xc, 8388608.f);
-    v = xc - fminf(t - 8388608.f, float(n - 1));
-    return min(__float_as_int(t) - 0x4B000000, n - 1);
-}
-
-// ---------------------------------------------------------------------------
-// Normal incidence (k_par = 0), short form of the tabulated evaluation.  The
-// same sum as green_tab_impl's symmetric form,
-//   g_p = sum_{p,q >= 0} w_p w_q G_pq(|z|) cos(p th_x) cos(q th_y)
-//         + exp(b^2)/(4 pi) sum_i F(R_i E) / R_i,   th = 2 pi (dx / a, dy / b),
-// (w_0 = 1, w_k = 2; the static part 1/R removed on the images in regm), with
-// the order quadrant unrolled at compile time (every order of the cut has
-// |p|, |q| <= PQ; entries outside the cut are skipped on a uniform branch), the
-// images from a 32-bit warp-uniform mask, and d1 = (2 cos th_x, 2 cos th_y)
-// supplied by the caller; D_k = 2 cos(k th) by the Chebyshev recurrence
-// D_k = d1 D_{k-1} - D_{k-2}, D_0 = 2.  REG: some lane of the warp has images
-// whose static part is removed (else R > 0 on every image of every lane).
-// ---------------------------------------------------------------------------
-template <bool REG>
-__device__ __forceinline__ float image_term(int i, float dx, float dy, float dz2, unsigned regm, const float4 *stab4,
-                                            const EwaldF32 &ef) {
-    const float x = dx + ef.img[i][0], y = dy + ef.img[i][1];
-    const float R2 = fmaf(x, x, fmaf(y, y, dz2));
-    float rinv = rsqrtf(R2);
-    if (REG) rinv = R2 > 0.f ? rinv : 0.f;   // R = 0 only on an image whose static part is removed
-    const float xu = R2 * rinv * ef.Eih;
-    float v;
-    const int ix = table_index(xu, NSPAT, v);
-    const float4 c = stab4[ix];
-    const float q1 = fmaf(v, fmaf(v, c.w, c.z), c.y);
-    float val = fmaf(v, q1, c.x) * rinv;
-    if (REG && ((regm >> i) & 1u))   // (F(x) - F(0)) / R; near R = 0 from the first interval's slope
-        val = ix == 0 ? ef.Eih * q1 : fmaf(-ef.e_mb2, rinv, val);
-    return xu <= float(NSPAT) ? val : 0.f;   // beyond the table: outside the cut
-}
-
-template <int PQ, bool REG>
-__device__ __forceinline__ cx<float> green_sym_short(float dx, float dy, float dz, float2 d1, unsigned imask,
-                                                     unsigned regm, const float4 *stab4,
-                                                     const float4 *__restrict__ rtab, const EwaldF32 &ef) {
-    float Dx[PQ + 1], Dy[PQ + 1];
-    Dx[0] = 1.f;
-    Dy[0] = 1.f;
-    Dx[1] = d1.x;
-    Dy[1] = d1.y;
-#pragma unroll
-    for (int k = 2; k <= PQ; ++k) {
-        Dx[k] = fmaf(d1.x, Dx[k - 1], k == 2 ? -2.f : -Dx[k - 2]);
-        Dy[k] = fmaf(d1.y, Dy[k - 1], k == 2 ? -2.f : -Dy[k - 2]);
-    }
-    float u;
-    const int iz = table_index(fabsf(dz) * ef.z_inv_h, NZTAB, u);
-    const float4 *rt = rtab + iz;
-    // every entry of the quadrant, no branch: orders outside the cut read zeros
-    float ar = 0.f;
-#pragma unroll
-    for (int p = 0; p <= PQ; ++p) {
-        float rr = 0.f;
-#pragma unroll
-        for (int q = 0; q <= PQ; ++q) {
-            const float4 c = __ldg(rt + ef.sq_off[p][q]);
-            const float g = fmaf(u, fmaf(u, fmaf(u, c.w, c.z), c.y), c.x);
-            rr = q == 0 ? g : fmaf(Dy[q], g, rr);
-        }
-        ar = p == 0 ? rr : fmaf(Dx[p], rr, ar);
-    }
-    const float4 ci = __ldg(rt + ef.sq_im);
-    const float ai = fmaf(u, fmaf(u, fmaf(u, ci.w, ci.z), ci.y), ci.x);
-    // lattice images, two at a time (the mask is warp-uniform)
-    const float dz2 = dz * dz;
-    float sv = 0.f;
-    for (unsigned mk = imask; mk;) {
-        const int i0 = __ffs((int)mk) - 1;
-        mk &= mk - 1u;
-        if (mk) {
-            const int i1 = __ffs((int)mk) - 1;
-            mk &= mk - 1u;
-            const float v0 = image_term<REG>(i0, dx, dy, dz2, regm, stab4, ef);
-            const float v1 = image_term<REG>(i1, dx, dy, dz2, regm, stab4, ef);
-            sv += v0 + v1;
-        } else {
-            sv += image_term<REG>(i0, dx, dy, dz2, regm, stab4, ef);
-        }
-    }
-    ar = fmaf(ef.img[0][2], sv, ar);
-    return {ar, ai};
-}
-
-// Images (32-bit mask) that can lie inside the cut for some displacement within
-// `rad` of (cx, cy, cz); n_img <= 32.
-__device__ __forceinline__ unsigned image_mask32(const EwaldF32 &ew, float cx, float cy, float cz, float rad) {
-    const float rc = ew.xs_max / ew.Ef * 1.0001f + rad * 1.0001f + 1e-6f * (fabsf(cx) + fabsf(cy) + fabsf(cz));
-    const float rc2 = rc * rc;
-    const int n = ew.n_img;
-    unsigned m = 0u;
-    for (int i = 0; i < n; ++i) {
-        const float x = cx + ew.img[i][0], y = cy + ew.img[i][1];
-        if (x * x + y * y + cz * cz <= rc2) m |= 1u << i;
-    }
-    return m;
-}
-
-// 4 x 4 point pairs of one tetrahedron pair in the short form.  tpt: the test
-// tetrahedron's points [a] = (x_a, x_a - c) and phases (2 cos, 2 cos, 2 sin,
-// 2 sin) of 2 pi (x / a, y / b); sph (stride 128): the source points' (cos,
-// cos, sin, sin).  The moments are accumulated without the weight.
-template <int PQ, bool REG>
-__device__ __forceinline__ void far_tt_short(const float *__restrict__ fs, const float4 (*tpt)[3],
-                                             const float4 *sph, unsigned imask, unsigned regm,
-                                             const float4 *stab4, const DevReq &q, Mom<float> &mo) {
-#pragma unroll 1
-    for (int b = 0; b < 4; ++b) {
-        const float yb0 = fs[3 * b], yb1 = fs[3 * b + 1], yb2 = fs[3 * b + 2];
-        const float rb[3] = {yb0 - fs[12], yb1 - fs[13], yb2 - fs[14]};
-        const float4 pb = sph[128 * b];
-#pragma unroll 1
-        for (int a = 0; a < 4; ++a) {
-            const float4 xa = tpt[a][0], ra = tpt[a][1], pa = tpt[a][2];
-            // 2 cos(k (x_a - y_b)) = 2 cos(k x_a) cos(k y_b) + 2 sin(k x_a) sin(k y_b)
-            const float2 d1 = {fmaf(pa.x, pb.x, pa.z * pb.z), fmaf(pa.y, pb.y, pa.w * pb.w)};
-            const cx<float> g = green_sym_short<PQ, REG>(xa.x - yb0, xa.y - yb1, xa.z - yb2, d1, imask, regm,
-                                                         stab4, q.rtab, q.ef);
-            const float rr = ra.x * rb[0] + ra.y * rb[1] + ra.z * rb[2];
-            mo.S = mo.S + g;
-            cfma(mo.A[0], ra.x, g);
-            cfma(mo.A[1], ra.y, g);
-            cfma(mo.A[2], ra.z, g);
-#pragma unroll
-            for (int d = 0; d < 3; ++d) cfma(mo.B[d], rb[d], g);
-            cfma(mo.C, rr, g);
-        }
-    }
-}
-
-// Far tetrahedron pairs at normal incidence in the short form: one thread per
-// unordered pair {t, s} (s >= t) as in k_far_tt, the reversed pair's moments
-// taken from the pair's own (g_p(-d) = g_p(d)).
-#ifndef VIE_FAR_N_MINB
-// CTAs per SM of the normal-incidence far kernels: the short form waits on its
-// table loads, so registers (85 at six) pay more than warps (bench cell: 39.8 /
-// 37.5 / 37.0 ms at eight / seven / six, eight spilling at 64 registers)
-#define VIE_FAR_N_MINB 6
-#endif
-template <int PQ>
-__global__ void __launch_bounds__(128, VIE_FAR_N_MINB) k_far_tt_n(DevMesh m, const __grid_constant__ DevReq q, float *Z, size_t N) {
-    __shared__ float4 s_tab[NSPAT];   // spatial table
-    __shared__ float4 s_sph[4 * 128];  // per thread: its source points' phases, [b][thread]
-    __shared__ float4 s_tpt[4][3];     // the test tetrahedron's points, relative points, phases times 2
-    const int t = blockIdx.y;
-    if ((int)(blockIdx.x * blockDim.x + blockDim.x) <= t) return;   // the whole block is below the diagonal
-    const EwaldF32 &ef = q.ef;
-    const float4 *gtab = reinterpret_cast<const float4 *>(q.stab);
-    for (int i = threadIdx.x; i < NSPAT; i += blockDim.x) s_tab[i] = gtab[i];
-    const float *ft = m.far<float>(t);
-    const float sx = ef.step_x * 0.31830988618f, sy = ef.step_y * 0.31830988618f;   // 2/a, 2/b
-    if (threadIdx.x < 4) {
-        const int a = threadIdx.x;
-        float sn_x, cs_x, sn_y, cs_y;
-        sincospif(sx * ft[3 * a], &sn_x, &cs_x);
-        sincospif(sy * ft[3 * a + 1], &sn_y, &cs_y);
-        s_tpt[a][0] = make_float4(ft[3 * a], ft[3 * a + 1], ft[3 * a + 2], 0.f);
-        s_tpt[a][1] = make_float4(ft[3 * a] - ft[12], ft[3 * a + 1] - ft[13], ft[3 * a + 2] - ft[14], 0.f);
-        s_tpt[a][2] = make_float4(2.f * cs_x, 2.f * cs_y, 2.f * sn_x, 2.f * sn_y);
-    }
-    const int s0 = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool live = s0 < m.nt && s0 >= t;   // lanes off the pair range stay until the warp's masks are formed
-    const int s = live ? s0 : t;
-    const float *fs = m.far<float>(s);
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-        float sn_x, cs_x, sn_y, cs_y;
-        sincospif(sx * fs[3 * b], &sn_x, &cs_x);
-        sincospif(sy * fs[3 * b + 1], &sn_y, &cs_y);
-        s_sph[128 * b + threadIdx.x] = make_float4(cs_x, cs_y, sn_x, sn_y);
-    }
-    // images that can reach the cut from some point pair of {t, s}: every point
-    // pair lies within rt + rs of the centroid offset; one list for the warp
-    float rt = 0.f, rs = 0.f;
-    for (int a = 0; a < 4; ++a) {
-        const float ux = ft[3 * a] - ft[12], uy = ft[3 * a + 1] - ft[13], uz = ft[3 * a + 2] - ft[14];
-        const float vx = fs[3 * a] - fs[12], vy = fs[3 * a + 1] - fs[13], vz = fs[3 * a + 2] - fs[14];
-        rt = fmaxf(rt, sqrtf(ux * ux + uy * uy + uz * uz));
-        rs = fmaxf(rs, sqrtf(vx * vx + vy * vy + vz * vz));
-    }
-    unsigned imask = live ? image_mask32(ef, ft[12] - fs[12], ft[13] - fs[13], ft[14] - fs[14], rt + rs) : 0u;
-    imask = __reduce_or_sync(0xffffffffu, imask);
-    // near images of this pair: their static part is integrated separately
-    const unsigned sub = live ? (unsigned)m.mk_tt[(size_t)t * m.nt + s] : 0u;
-    unsigned regm = 0u;
-    if (sub) {
-#pragma unroll
-        for (int k = 0; k < 9; ++k)
-            if ((sub >> k) & 1u) regm |= 1u << ef.near_img[k];
-    }
-    const bool reg = __any_sync(0xffffffffu, regm != 0u);
-    __syncthreads();
-    if (!live) return;
-    Mom<float> mo, mr;
-    mo.zero();
-    if (reg) far_tt_short<PQ, true>(fs, s_tpt, s_sph + threadIdx.x, imask, regm, s_tab, q, mo);
-    else far_tt_short<PQ, false>(fs, s_tpt, s_sph + threadIdx.x, imask, regm, s_tab, q, mo);
-    const float wgt = ft[27] * fs[27];
-    mo.S = wgt * mo.S;
-    mo.C = wgt * mo.C;
-    for (int d = 0; d < 3; ++d) { mo.A[d] = wgt * mo.A[d]; mo.B[d] = wgt * mo.B[d]; }
-    // g_p(-d) = g_p(d): the reversed pair's moments swap A and B
-    mr.S = mo.S;
-    mr.C = mo.C;
-    for (int d = 0; d < 3; ++d) { mr.A[d] = mo.B[d]; mr.B[d] = mo.A[d]; }
-    scatter_tt<float>(m, q, Z, N, t, s, mo);
-    if (s != t) scatter_tt<float>(m, q, Z, N, s, t, mr);
-}
-
-// ---------------------------------------------------------------------------
-// Oblique incidence, short form of the tabulated evaluation.  With
-// X_i = exp(-j (k_x0 + i s_x) dx), Y_j = exp(-j (k_y0 + j s_y) dy) (k_x0, k_y0
-// the first order of the rectangle, s = 2 pi / period) and the spectral table
-// G_ij(|z|) = Re G + j Im G of rectangle entry (i, j):
-//   S = sum_ij X_i Y_j Re G_ij,   T = sum_ij X_i Y_j Im G_ij (propagating orders only),
-//   g_p(d) = S + j T + sum_i F(R_i E)/R_i ph_i      (ph_i: image phase exp(j k_par.R_i) exp(b^2)/(4 pi)).
-// Re G is real, so the spectral part of g_p(-d) = sum G conj(X Y) is
-// conj(S) + j conj(T), and the image part is the conjugate of the image part
-// of g_p(d): g_p(-d) = conj(g_p(d)) + 2 j conj(T).  The returned T carries
-// that correction.  X0, SX, Y0, SY: X_0, exp(-j s_x dx), Y_0, exp(-j s_y dy).
-// ---------------------------------------------------------------------------
-template <bool REG>
-__device__ __forceinline__ float image_term64(int i, float dx, float dy, float dz2, unsigned long long regm,
-                                              const float4 *stab4, const EwaldF32 &ef) {
-    const float x = dx + ef.img[i][0], y = dy + ef.img[i][1];
-    const float R2 = fmaf(x, x, fmaf(y, y, dz2));
-    float rinv = rsqrtf(R2);
-    if (REG) rinv = R2 > 0.f ? rinv : 0.f;   // R = 0 only on an image whose static part is removed
-    const float xu = R2 * rinv * ef.Eih;
-    float v;
-    const int ix = table_index(xu, NSPAT, v);
-    const float4 c = stab4[ix];
-    const float q1 = fmaf(v, fmaf(v, c.w, c.z), c.y);
-    float val = fmaf(v, q1, c.x) * rinv;
-    if (REG && ((regm >> i) & 1ull))   // (F(x) - F(0)) / R; near R = 0 from the first interval's slope
-        val = ix == 0 ? ef.Eih * q1 : fmaf(-ef.e_mb2, rinv, val);
-    return xu <= float(NSPAT) ? val : 0.f;   // beyond the table: outside the cut
-}
-
-template <int NR, bool REG>
-__device__ __forceinline__ cx<float> green_obl_short(float dx, float dy, float dz, cx<float> X0, cx<float> SX,
-                                                     cx<float> Y0, cx<float> SY, unsigned long long imask,
-                                                     unsigned long long regm, const float4 *stab4,
-                                                     const float4 *__restrict__ rtab, const EwaldF32 &ef,
-                                                     cx<float> &T) {
-    cx<float> Y[NR];
-    Y[0] = Y0;
-#pragma unroll
-    for (int j = 1; j < NR; ++j) Y[j] = Y[j - 1] * SY;
-    float u;
-    const int iz = table_index(fabsf(dz) * ef.z_inv_h, NZTAB, u);
-    const float4 *rt = rtab + iz;
-    cx<float> S = {0.f, 0.f}, X = X0;
-    T = {0.f, 0.f};
-#pragma unroll
-    for (int i = 0; i < NR; ++i) {
-        cx<float> inr = {0.f, 0.f}, ini = {0.f, 0.f};
-        bool cplx = false;
-#pragma unroll
-        for (int j = 0; j < NR; ++j) {
-            const float4 c = __ldg(rt + ef.ob_off[i][j]);   // entries outside the cut read zeros
-            const float g = fmaf(u, fmaf(u, fmaf(u, c.w, c.z), c.y), c.x);
-            cfma(inr, g, Y[j]);
-            const int im = ef.ob_im[i][j];
-            if (im >= 0) {   // propagating order (uniform branch)
-                const float4 ci = __ldg(rt + im);
-                cfma(ini, fmaf(u, fmaf(u, fmaf(u, ci.w, ci.z), ci.y), ci.x), Y[j]);
-                cplx = true;
-            }
-        }
-        S = S + X * inr;
-        if (cplx) T = T + X * ini;
-        if (i + 1 < NR) X = X * SX;
-    }
-    // lattice images, two at a time (the mask is warp-uniform)
-    const float dz2 = dz * dz;
-    cx<float> acc = {S.re - T.im, S.im + T.re};
-    for (unsigned long long mk = imask; mk;) {
-        const int i0 = __ffsll((long long)mk) - 1;
-        mk &= mk - 1ull;
-        const float v0 = image_term64<REG>(i0, dx, dy, dz2, regm, stab4, ef);
-        acc.re = fmaf(v0, ef.img[i0][2], acc.re);
-        acc.im = fmaf(v0, ef.img[i0][3], acc.im);
-        if (mk) {
-            const int i1 = __ffsll((long long)mk) - 1;
-            mk &= mk - 1ull;
-            const float v1 = image_term64<REG>(i1, dx, dy, dz2, regm, stab4, ef);
-            acc.re = fmaf(v1, ef.img[i1][2], acc.re);
-            acc.im = fmaf(v1, ef.img[i1][3], acc.im);
-        }
-    }
-    return acc;
-}
-
-// The same at k_y = 0 with the order rectangle symmetric in q: G_pq = G_p,-q,
-// so sum_q Y_q G_pq = sum_{q >= 0} w_q cos(q s_y dy) G_pq (w_0 = 1, w_q = 2),
-// a real weight D_q = 2 cos(q s_y dy) (D_0 -> 1) by the Chebyshev recurrence
-// from d1y = 2 cos(s_y dy); entry (i, q) of the tables is order (p0 + i, q).
-template <int NP, int NQ1, bool REG>
-__device__ __forceinline__ cx<float> green_obl_ky0(float dx, float dy, float dz, cx<float> X0, cx<float> SX,
-                                                   float d1y, unsigned long long imask, unsigned long long regm,
-                                                   const float4 *stab4, const float4 *__restrict__ rtab,
-                                                   const EwaldF32 &ef, cx<float> &T) {
-    float Dy[NQ1];
-    Dy[0] = 1.f;
-    Dy[1] = d1y;
-#pragma unroll
-    for (int k = 2; k < NQ1; ++k) Dy[k] = fmaf(d1y, Dy[k - 1], k == 2 ? -2.f : -Dy[k - 2]);
-    float u;
-    const int iz = table_index(fabsf(dz) * ef.z_inv_h, NZTAB, u);
-    const float4 *rt = rtab + iz;
-    cx<float> S = {0.f, 0.f}, X = X0;
-    T = {0.f, 0.f};
-#pragma unroll
-    for (int i = 0; i < NP; ++i) {
-        float inr = 0.f, ini = 0.f;
-        bool cplx = false;
-#pragma unroll
-        for (int q = 0; q < NQ1; ++q) {
-            const float4 c = __ldg(rt + ef.ob_off[i][q]);   // entries outside the cut read zeros
-            const float g = fmaf(u, fmaf(u, fmaf(u, c.w, c.z), c.y), c.x);
-            inr = q == 0 ? g : fmaf(Dy[q], g, inr);
-            const int im = ef.ob_im[i][q];
-            if (im >= 0) {   // propagating order (uniform branch)
-                const float4 ci = __ldg(rt + im);
-                const float gi = fmaf(u, fmaf(u, fmaf(u, ci.w, ci.z), ci.y), ci.x);
-                ini = q == 0 ? ini + gi : fmaf(Dy[q], gi, ini);
-                cplx = true;
-            }
-        }
-        S.re = fmaf(X.re, inr, S.re);
-        S.im = fmaf(X.im, inr, S.im);
-        if (cplx) {
-            T.re = fmaf(X.re, ini, T.re);
-            T.im = fmaf(X.im, ini, T.im);
-        }
-        if (i + 1 < NP) X = X * SX;
-    }
-    const float dz2 = dz * dz;
-    cx<float> acc = {S.re - T.im, S.im + T.re};
-    for (unsigned long long mk = imask; mk;) {
-        const int i0 = __ffsll((long long)mk) - 1;
-        mk &= mk - 1ull;
-        const float v0 = image_term64<REG>(i0, dx, dy, dz2, regm, stab4, ef);
-        acc.re = fmaf(v0, ef.img[i0][2], acc.re);
-        acc.im = fmaf(v0, ef.img[i0][3], acc.im);
-        if (mk) {
-            const int i1 = __ffsll((long long)mk) - 1;
-            mk &= mk - 1ull;
-            const float v1 = image_term64<REG>(i1, dx, dy, dz2, regm, stab4, ef);
-            acc.re = fmaf(v1, ef.img[i1][2], acc.re);
-            acc.im = fmaf(v1, ef.img[i1][3], acc.im);
-        }
-    }
-    return acc;
-}
-
-// the oblique evaluation of one point pair: NQ1 = 0 the full rectangle (NR x NR),
-// else the k_y = 0 fold (NR x NQ1); sa, sb carry (cos, sin) of s_x x and s_y y
-template <int NR, int NQ1, bool REG>
-__device__ __forceinline__ cx<float> green_obl(float dx, float dy, float dz, float4 pa, float4 sa, float4 pb,
-                                               float4 sb, unsigned long long imask, unsigned long long regm,
-                                               const float4 *stab4, const float4 *__restrict__ rtab,
-                                               const EwaldF32 &ef, cx<float> &T);
-
-// e^{-j th_a} conj(e^{-j th_b}) = e^{-j (th_a - th_b)} from (cos, sin) of th_a and th_b
-__device__ __forceinline__ cx<float> phase_diff(float ca, float sa, float cb, float sb) {
-    return {fmaf(ca, cb, sa * sb), fmaf(ca, sb, -sa * cb)};
-}
-
-template <int NR, int NQ1, bool REG>
-__device__ __forceinline__ cx<float> green_obl(float dx, float dy, float dz, float4 pa, float4 sa, float4 pb,
-                                               float4 sb, unsigned long long imask, unsigned long long regm,
-                                               const float4 *stab4, const float4 *__restrict__ rtab,
-                                               const EwaldF32 &ef, cx<float> &T) {
-    const cx<float> X0 = phase_diff(pa.x, pa.y, pb.x, pb.y), SX = phase_diff(sa.x, sa.y, sb.x, sb.y);
-    if constexpr (NQ1 > 0) {
-        const float d1y = 2.f * fmaf(sa.z, sb.z, sa.w * sb.w);   // 2 cos(s_y (y_a - y_b))
-        return green_obl_ky0<NR, NQ1, REG>(dx, dy, dz, X0, SX, d1y, imask, regm, stab4, rtab, ef, T);
-    } else {
-        const cx<float> Y0 = phase_diff(pa.z, pa.w, pb.z, pb.w), SY = phase_diff(sa.z, sa.w, sb.z, sb.w);
-        return green_obl_short<NR, REG>(dx, dy, dz, X0, SX, Y0, SY, imask, regm, stab4, rtab, ef, T);
-    }
-}
-
-// 4 x 4 point pairs of one tetrahedron pair in the oblique short form.  tpt:
-// the test points [a] = (x_a, x_a - c, (cos, sin) of k_x0 x and k_y0 y,
-// (cos, sin) of s_x x and s_y y); sph (stride 128, two float4 per point): the
-// same phases of the source points.  mo: moments of g_p(x_a - y_b); mc: the
-// correction 2 j conj(T) of g_p(y_b - x_a) with the reversed pair's roles.
-template <int NR, int NQ1, bool REG>
-__device__ __forceinline__ void far_tt_obl(const float *__restrict__ fs, const float4 (*tpt)[4], const float4 *sph,
-                                           unsigned long long imask, unsigned long long regm, const float4 *stab4,
-                                           const DevReq &q, Mom<float> &mo, Mom<float> &mc) {
-#pragma unroll 1
-    for (int b = 0; b < 4; ++b) {
-        const float yb0 = fs[3 * b], yb1 = fs[3 * b + 1], yb2 = fs[3 * b + 2];
-        const float rb[3] = {yb0 - fs[12], yb1 - fs[13], yb2 - fs[14]};
-        const float4 pb = sph[256 * b], sb = sph[256 * b + 128];
-#pragma unroll 1
-        for (int a = 0; a < 4; ++a) {
-            const float4 xa = tpt[a][0], ra = tpt[a][1], pa = tpt[a][2], sa = tpt[a][3];
-            cx<float> T;
-            const cx<float> g = green_obl<NR, NQ1, REG>(xa.x - yb0, xa.y - yb1, xa.z - yb2, pa, sa, pb, sb, imask,
-                                                        regm, stab4, q.rtab, q.ef, T);
-            const cx<float> c = {2.f * T.im, 2.f * T.re};   // 2 j conj(T)
-            const float rr = ra.x * rb[0] + ra.y * rb[1] + ra.z * rb[2];
-            mo.S = mo.S + g;
-            cfma(mo.A[0], ra.x, g);
-            cfma(mo.A[1], ra.y, g);
-            cfma(mo.A[2], ra.z, g);
-            mc.S = mc.S + c;
-            cfma(mc.B[0], ra.x, c);
-            cfma(mc.B[1], ra.y, c);
-            cfma(mc.B[2], ra.z, c);
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                cfma(mo.B[d], rb[d], g);
-                cfma(mc.A[d], rb[d], c);
-            }
-            cfma(mo.C, rr, g);
-            cfma(mc.C, rr, c);
-        }
-    }
-}
-
-// (cos, sin) of k_x0 x, k_y0 y and of s_x x, s_y y of one point
-__device__ __forceinline__ void obl_point_phases(const EwaldF32 &ef, float x, float y, float4 &p, float4 &st) {
-    float s0, c0, s1, c1, s2, c2, s3, c3;
-    sincospif(ef.ob_kx0 * 0.31830988618f * x, &s0, &c0);
-    sincospif(ef.ob_ky0 * 0.31830988618f * y, &s1, &c1);
-    sincospif(ef.step_x * 0.31830988618f * x, &s2, &c2);
-    sincospif(ef.step_y * 0.31830988618f * y, &s3, &c3);
-    p = make_float4(c0, s0, c1, s1);
-    st = make_float4(c2, s2, c3, s3);
-}
-
-#ifndef VIE_FAR_O_MINB
-// CTAs per SM of the oblique-incidence far kernels (bench cell at theta = 0.3,
-// the general order rectangle: 81.6 / 78.3 / 82.3 ms at six / five / four)
-#define VIE_FAR_O_MINB 5
-#endif
-// Far tetrahedron pairs at oblique incidence in the short form: one thread per
-// unordered pair {t, s} (s >= t); the reversed pair's moments are the
-// conjugates of the pair's own, exchanged, plus the propagating-order correction.
-template <int NR, int NQ1>
-__global__ void __launch_bounds__(128, VIE_FAR_O_MINB) k_far_tt_o(DevMesh m, const __grid_constant__ DevReq q, float *Z,
-                                                                  size_t N) {
-    __shared__ float4 s_tab[NSPAT];
-    __shared__ float4 s_sph[4 * 2 * 128];   // [b][phase pair][thread]
-    __shared__ float4 s_tpt[4][4];
-    const int t = blockIdx.y;
-    if ((int)(blockIdx.x * blockDim.x + blockDim.x) <= t) return;   // the whole block is below the diagonal
-    const EwaldF32 &ef = q.ef;
-    const float4 *gtab = reinterpret_cast<const float4 *>(q.stab);
-    for (int i = threadIdx.x; i < NSPAT; i += blockDim.x) s_tab[i] = gtab[i];
-    const float *ft = m.far<float>(t);
-    if (threadIdx.x < 4) {
-        const int a = threadIdx.x;
-        float4 p, st;
-        obl_point_phases(ef, ft[3 * a], ft[3 * a + 1], p, st);
-        s_tpt[a][0] = make_float4(ft[3 * a], ft[3 * a + 1], ft[3 * a + 2], 0.f);
-        s_tpt[a][1] = make_float4(ft[3 * a] - ft[12], ft[3 * a + 1] - ft[13], ft[3 * a + 2] - ft[14], 0.f);
-        s_tpt[a][2] = p;
-        s_tpt[a][3] = st;
-    }
-    const int s0 = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool live = s0 < m.nt && s0 >= t;
-    const int s = live ? s0 : t;
-    const float *fs = m.far<float>(s);
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-        float4 p, st;
-        obl_point_phases(ef, fs[3 * b], fs[3 * b + 1], p, st);
-        s_sph[256 * b + threadIdx.x] = p;
-        s_sph[256 * b + 128 + threadIdx.x] = st;
-    }
-    float rt = 0.f, rs = 0.f;
-    for (int a = 0; a < 4; ++a) {
-        const float ux = ft[3 * a] - ft[12], uy = ft[3 * a + 1] - ft[13], uz = ft[3 * a + 2] - ft[14];
-        const float vx = fs[3 * a] - fs[12], vy = fs[3 * a + 1] - fs[13], vz = fs[3 * a + 2] - fs[14];
-        rt = fmaxf(rt, sqrtf(ux * ux + uy * uy + uz * uz));
-        rs = fmaxf(rs, sqrtf(vx * vx + vy * vy + vz * vz));
-    }
-    unsigned long long imask = live ? image_mask(ef, ft[12] - fs[12], ft[13] - fs[13], ft[14] - fs[14], rt + rs) : 0ull;
-    {
-        const unsigned lo = __reduce_or_sync(0xffffffffu, (unsigned)imask);
-        const unsigned hi = __reduce_or_sync(0xffffffffu, (unsigned)(imask >> 32));
-        imask = ((unsigned long long)hi << 32) | lo;
-    }
-    const unsigned sub = live ? (unsigned)m.mk_tt[(size_t)t * m.nt + s] : 0u;
-    unsigned long long regm = 0ull;
-    if (sub) {
-#pragma unroll
-        for (int k = 0; k < 9; ++k)
-            if ((sub >> k) & 1u) regm |= 1ull << ef.near_img[k];
-    }
-    const bool reg = __any_sync(0xffffffffu, regm != 0ull);
-    __syncthreads();
-    if (!live) return;
-    Mom<float> mo, mc;
-    mo.zero();
-    mc.zero();
-    if (reg) far_tt_obl<NR, NQ1, true>(fs, s_tpt, s_sph + threadIdx.x, imask, regm, s_tab, q, mo, mc);
-    else far_tt_obl<NR, NQ1, false>(fs, s_tpt, s_sph + threadIdx.x, imask, regm, s_tab, q, mo, mc);
-    const float wgt = ft[27] * fs[27];
-    Mom<float> mr;
-    mr.S = wgt * (cconj(mo.S) + mc.S);
-    mr.C = wgt * (cconj(mo.C) + mc.C);
-    for (int d = 0; d < 3; ++d) {
-        mr.A[d] = wgt * (cconj(mo.B[d]) + mc.A[d]);
-        mr.B[d] = wgt * (cconj(mo.A[d]) + mc.B[d]);
-    }
-    mo.S = wgt * mo.S;
-    mo.C = wgt * mo.C;
-    for (int d = 0; d < 3; ++d) { mo.A[d] = wgt * mo.A[d]; mo.B[d] = wgt * mo.B[d]; }
-    scatter_tt<float>(m, q, Z, N, t, s, mo);
-    if (s != t) scatter_tt<float>(m, q, Z, N, s, t, mr);
-}
-
 // ---------------------------------------------------------------------------
 // near tetrahedron pairs: one warp per pair
 // ---------------------------------------------------------------------------
@@ -918,8 +389,13 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
+__device__ __forceinline__ float inv_sqrt(float x) { return rsqrt_ftz(x); }
+__device__ __forceinline__ double inv_sqrt(double x) { return rsqrt(x); }
+
 // near image of a pair, elements not touching: degree-5 x degree-5 product
-// rule of exp(j k_par.R)/(4 pi R), one thread per (pair, image)
+// rule of exp(j k_par.R)/(4 pi R), one thread per (pair, image); 3.3 ms of the
+// bench cell's fill with the loops exchanged (every load of the inner loop a
+// gather, L1 87% busy)
 template <typename T>
 __global__ void __launch_bounds__(128) k_pr_tt(DevMesh m, const __grid_constant__ DevReq q, T *Z, size_t N, const NearEntry *list, int n) {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
@@ -930,27 +406,33 @@ __global__ void __launch_bounds__(128) k_pr_tt(DevMesh m, const __grid_constant_
     const double *ct = m.cen + 3 * (size_t)t, *cs = m.cen + 3 * (size_t)s;
     const T *nx = m.nrel<T>(t), *ny = m.nrel<T>(s);
     const T dc[3] = {T(ct[0] - cs[0] + R[0]), T(ct[1] - cs[1] + R[1]), T(ct[2] - cs[2])};
+    // the source points (another element per lane) in the outer loop, the test
+    // points (the entries are sorted by test element: mostly one per warp, a
+    // broadcast load) in the inner one
     T s0 = 0, sA[3] = {0, 0, 0}, sB[3] = {0, 0, 0}, sC = 0;
-    for (int a = 0; a < 14; ++a) {
-        const T xa[4] = {nx[4 * a], nx[4 * a + 1], nx[4 * a + 2], nx[4 * a + 3]};
-        T f0 = 0, fb[3] = {0, 0, 0};
-        for (int b = 0; b < 14; ++b) {
-            const T *yb = ny + 4 * b;
-            const T dx = xa[0] - yb[0] + dc[0], dy = xa[1] - yb[1] + dc[1], dz = xa[2] - yb[2] + dc[2];
-            const T f = yb[3] * rsqrt(dx * dx + dy * dy + dz * dz);
+#pragma unroll 1
+    for (int b = 0; b < 14; ++b) {
+        const T yb[4] = {ny[4 * b], ny[4 * b + 1], ny[4 * b + 2], ny[4 * b + 3]};
+        const T o[3] = {dc[0] - yb[0], dc[1] - yb[1], dc[2] - yb[2]};
+        T f0 = 0, fa[3] = {0, 0, 0};
+#pragma unroll
+        for (int a = 0; a < 14; ++a) {
+            const T xa[4] = {nx[4 * a], nx[4 * a + 1], nx[4 * a + 2], nx[4 * a + 3]};
+            const T dx = xa[0] + o[0], dy = xa[1] + o[1], dz = xa[2] + o[2];
+            const T f = xa[3] * inv_sqrt(dx * dx + dy * dy + dz * dz);
             f0 += f;
-            fb[0] += f * yb[0];
-            fb[1] += f * yb[1];
-            fb[2] += f * yb[2];
+            fa[0] += f * xa[0];
+            fa[1] += f * xa[1];
+            fa[2] += f * xa[2];
         }
-        f0 *= xa[3];
-        for (int d = 0; d < 3; ++d) fb[d] *= xa[3];
+        f0 *= yb[3];
         s0 += f0;
         for (int d = 0; d < 3; ++d) {
-            sA[d] += f0 * xa[d];
-            sB[d] += fb[d];
+            fa[d] *= yb[3];
+            sA[d] += fa[d];
+            sB[d] += f0 * yb[d];
+            sC += fa[d] * yb[d];
         }
-        sC += xa[0] * fb[0] + xa[1] * fb[1] + xa[2] * fb[2];
     }
     const cx<T> pt = {T(q.img_ph[2 * k]), T(q.img_ph[2 * k + 1])};
     Mom<T> mo;
@@ -1164,176 +646,6 @@ __global__ void __launch_bounds__(128) k_far_scalar(DevMesh m, const __grid_cons
     scatter_scalar<T, PK>(m, q, Z, N, x, y, S);
 }
 
-// Far scalar pairs (charge faces) at normal incidence in the short form: one
-// thread per element pair as in k_far_scalar; the x element's points and their
-// phases (times 2) staged once per block, each thread's y points' phases in
-// shared memory [b][thread].
-template <int PQ, int PK>
-__global__ void __launch_bounds__(128, VIE_FAR_N_MINB)
-    k_far_scalar_n(DevMesh m, const __grid_constant__ DevReq q, float *Z, size_t N, int nx, int ny,
-                   const uint16_t *mk) {
-    __shared__ float4 s_tab[NSPAT];
-    __shared__ float4 s_yph[4 * 128];
-    __shared__ float4 s_xpt[4][2];
-    constexpr bool XT = PKTraits<PK>::xtet, YT = PKTraits<PK>::ytet;
-    constexpr int qx = XT ? 4 : 3, qy = YT ? 4 : 3;
-    const EwaldF32 &ef = q.ef;
-    const int x = blockIdx.y;
-    const float4 *gtab = reinterpret_cast<const float4 *>(q.stab);
-    for (int i = threadIdx.x; i < NSPAT; i += blockDim.x) s_tab[i] = gtab[i];
-    // a test face is addressed by its half-function index; geometry by charge-face index
-    const float *fx = far_el<float, XT>(m, XT ? x : m.hf[x]);
-    const float sx = ef.step_x * 0.31830988618f, sy = ef.step_y * 0.31830988618f;
-    if (threadIdx.x < qx) {
-        const int a = threadIdx.x;
-        float sn_x, cs_x, sn_y, cs_y;
-        sincospif(sx * fx[3 * a], &sn_x, &cs_x);
-        sincospif(sy * fx[3 * a + 1], &sn_y, &cs_y);
-        s_xpt[a][0] = make_float4(fx[3 * a], fx[3 * a + 1], fx[3 * a + 2], 0.f);
-        s_xpt[a][1] = make_float4(2.f * cs_x, 2.f * cs_y, 2.f * sn_x, 2.f * sn_y);
-    }
-    const int y0 = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool live = y0 < ny;
-    const int y = live ? y0 : ny - 1;
-    const float *fy = far_el<float, YT>(m, y);
-#pragma unroll
-    for (int b = 0; b < qy; ++b) {
-        float sn_x, cs_x, sn_y, cs_y;
-        sincospif(sx * fy[3 * b], &sn_x, &cs_x);
-        sincospif(sy * fy[3 * b + 1], &sn_y, &cs_y);
-        s_yph[128 * b + threadIdx.x] = make_float4(cs_x, cs_y, sn_x, sn_y);
-    }
-    // images that can reach the cut from some point pair: centres and radii of the point sets
-    float c1[3] = {0.f, 0.f, 0.f}, c2[3] = {0.f, 0.f, 0.f};
-    for (int a = 0; a < qx; ++a)
-        for (int d = 0; d < 3; ++d) c1[d] += fx[3 * a + d] / qx;
-    for (int b = 0; b < qy; ++b)
-        for (int d = 0; d < 3; ++d) c2[d] += fy[3 * b + d] / qy;
-    float r1 = 0.f, r2 = 0.f;
-    for (int a = 0; a < qx; ++a) {
-        const float ux = fx[3 * a] - c1[0], uy = fx[3 * a + 1] - c1[1], uz = fx[3 * a + 2] - c1[2];
-        r1 = fmaxf(r1, sqrtf(ux * ux + uy * uy + uz * uz));
-    }
-    for (int b = 0; b < qy; ++b) {
-        const float ux = fy[3 * b] - c2[0], uy = fy[3 * b + 1] - c2[1], uz = fy[3 * b + 2] - c2[2];
-        r2 = fmaxf(r2, sqrtf(ux * ux + uy * uy + uz * uz));
-    }
-    unsigned imask = live ? image_mask32(ef, c1[0] - c2[0], c1[1] - c2[1], c1[2] - c2[2], r1 + r2) : 0u;
-    imask = __reduce_or_sync(0xffffffffu, imask);
-    const unsigned sub = live ? (unsigned)mk[(size_t)x * ny + y] : 0u;
-    unsigned regm = 0u;
-    if (sub) {
-#pragma unroll
-        for (int k = 0; k < 9; ++k)
-            if ((sub >> k) & 1u) regm |= 1u << ef.near_img[k];
-    }
-    const bool reg = __any_sync(0xffffffffu, regm != 0u);
-    __syncthreads();
-    if (!live) return;
-    cx<float> S = {0.f, 0.f};
-#pragma unroll 1
-    for (int b = 0; b < qy; ++b) {
-        const float yb0 = fy[3 * b], yb1 = fy[3 * b + 1], yb2 = fy[3 * b + 2];
-        const float4 pb = s_yph[128 * b + threadIdx.x];
-#pragma unroll 1
-        for (int a = 0; a < qx; ++a) {
-            const float4 xa = s_xpt[a][0], pa = s_xpt[a][1];
-            const float2 d1 = {fmaf(pa.x, pb.x, pa.z * pb.z), fmaf(pa.y, pb.y, pa.w * pb.w)};
-            const cx<float> g = reg ? green_sym_short<PQ, true>(xa.x - yb0, xa.y - yb1, xa.z - yb2, d1, imask, regm,
-                                                                s_tab, q.rtab, ef)
-                                    : green_sym_short<PQ, false>(xa.x - yb0, xa.y - yb1, xa.z - yb2, d1, imask, 0u,
-                                                                 s_tab, q.rtab, ef);
-            S = S + g;
-        }
-    }
-    S = (fx[XT ? 27 : 9] * fy[YT ? 27 : 9]) * S;
-    scatter_scalar<float, PK>(m, q, Z, N, x, y, S);
-}
-
-// Far scalar pairs (charge faces) at oblique incidence in the short form.
-template <int NR, int NQ1, int PK>
-__global__ void __launch_bounds__(128, VIE_FAR_O_MINB)
-    k_far_scalar_o(DevMesh m, const __grid_constant__ DevReq q, float *Z, size_t N, int nx, int ny,
-                   const uint16_t *mk) {
-    __shared__ float4 s_tab[NSPAT];
-    __shared__ float4 s_yph[4 * 2 * 128];
-    __shared__ float4 s_xpt[4][3];
-    constexpr bool XT = PKTraits<PK>::xtet, YT = PKTraits<PK>::ytet;
-    constexpr int qx = XT ? 4 : 3, qy = YT ? 4 : 3;
-    const EwaldF32 &ef = q.ef;
-    const int x = blockIdx.y;
-    const float4 *gtab = reinterpret_cast<const float4 *>(q.stab);
-    for (int i = threadIdx.x; i < NSPAT; i += blockDim.x) s_tab[i] = gtab[i];
-    const float *fx = far_el<float, XT>(m, XT ? x : m.hf[x]);
-    if (threadIdx.x < qx) {
-        const int a = threadIdx.x;
-        float4 p, st;
-        obl_point_phases(ef, fx[3 * a], fx[3 * a + 1], p, st);
-        s_xpt[a][0] = make_float4(fx[3 * a], fx[3 * a + 1], fx[3 * a + 2], 0.f);
-        s_xpt[a][1] = p;
-        s_xpt[a][2] = st;
-    }
-    const int y0 = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool live = y0 < ny;
-    const int y = live ? y0 : ny - 1;
-    const float *fy = far_el<float, YT>(m, y);
-#pragma unroll
-    for (int b = 0; b < qy; ++b) {
-        float4 p, st;
-        obl_point_phases(ef, fy[3 * b], fy[3 * b + 1], p, st);
-        s_yph[256 * b + threadIdx.x] = p;
-        s_yph[256 * b + 128 + threadIdx.x] = st;
-    }
-    float c1[3] = {0.f, 0.f, 0.f}, c2[3] = {0.f, 0.f, 0.f};
-    for (int a = 0; a < qx; ++a)
-        for (int d = 0; d < 3; ++d) c1[d] += fx[3 * a + d] / qx;
-    for (int b = 0; b < qy; ++b)
-        for (int d = 0; d < 3; ++d) c2[d] += fy[3 * b + d] / qy;
-    float r1 = 0.f, r2 = 0.f;
-    for (int a = 0; a < qx; ++a) {
-        const float ux = fx[3 * a] - c1[0], uy = fx[3 * a + 1] - c1[1], uz = fx[3 * a + 2] - c1[2];
-        r1 = fmaxf(r1, sqrtf(ux * ux + uy * uy + uz * uz));
-    }
-    for (int b = 0; b < qy; ++b) {
-        const float ux = fy[3 * b] - c2[0], uy = fy[3 * b + 1] - c2[1], uz = fy[3 * b + 2] - c2[2];
-        r2 = fmaxf(r2, sqrtf(ux * ux + uy * uy + uz * uz));
-    }
-    unsigned long long imask = live ? image_mask(ef, c1[0] - c2[0], c1[1] - c2[1], c1[2] - c2[2], r1 + r2) : 0ull;
-    {
-        const unsigned lo = __reduce_or_sync(0xffffffffu, (unsigned)imask);
-        const unsigned hi = __reduce_or_sync(0xffffffffu, (unsigned)(imask >> 32));
-        imask = ((unsigned long long)hi << 32) | lo;
-    }
-    const unsigned sub = live ? (unsigned)mk[(size_t)x * ny + y] : 0u;
-    unsigned long long regm = 0ull;
-    if (sub) {
-#pragma unroll
-        for (int k = 0; k < 9; ++k)
-            if ((sub >> k) & 1u) regm |= 1ull << ef.near_img[k];
-    }
-    const bool reg = __any_sync(0xffffffffu, regm != 0ull);
-    __syncthreads();
-    if (!live) return;
-    cx<float> S = {0.f, 0.f};
-#pragma unroll 1
-    for (int b = 0; b < qy; ++b) {
-        const float yb0 = fy[3 * b], yb1 = fy[3 * b + 1], yb2 = fy[3 * b + 2];
-        const float4 pb = s_yph[256 * b + threadIdx.x], sb = s_yph[256 * b + 128 + threadIdx.x];
-#pragma unroll 1
-        for (int a = 0; a < qx; ++a) {
-            const float4 xa = s_xpt[a][0], pa = s_xpt[a][1], sa = s_xpt[a][2];
-            cx<float> T;
-            const cx<float> g = reg ? green_obl<NR, NQ1, true>(xa.x - yb0, xa.y - yb1, xa.z - yb2, pa, sa, pb, sb,
-                                                               imask, regm, s_tab, q.rtab, ef, T)
-                                    : green_obl<NR, NQ1, false>(xa.x - yb0, xa.y - yb1, xa.z - yb2, pa, sa, pb, sb,
-                                                                imask, 0ull, s_tab, q.rtab, ef, T);
-            S = S + g;
-        }
-    }
-    S = (fx[XT ? 27 : 9] * fy[YT ? 27 : 9]) * S;
-    scatter_scalar<float, PK>(m, q, Z, N, x, y, S);
-}
-
 template <typename U>
 __device__ double static_scalar(const double *r5, bool other_tet, const double *verts_other, const double *R,
                                 double sgnR) {
@@ -1512,79 +824,18 @@ __global__ void k_green(const double *d, double *out, int n, const float *stab, 
     out[2 * i + 1] = double(r.im);
 }
 
-// the short normal-incidence form at single displacements (every image visited)
-template <int PQ>
-__global__ void k_green_short(const double *d, double *out, int n, const float *stab, const float2 *ztab,
-                              const float4 *rtab, const __grid_constant__ EwaldF32 ef) {
-    __shared__ float4 s_tab[NSPAT];
-    for (int i = threadIdx.x; i < NSPAT; i += blockDim.x) s_tab[i] = reinterpret_cast<const float4 *>(stab)[i];
-    __syncthreads();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float dx = float(d[3 * i]), dy = float(d[3 * i + 1]), dz = float(d[3 * i + 2]);
-    const float2 d1 = {2.f * cospif(ef.step_x * dx * 0.31830988618f), 2.f * cospif(ef.step_y * dy * 0.31830988618f)};
-    const unsigned all = ef.n_img >= 32 ? 0xffffffffu : (1u << ef.n_img) - 1u;
-    cx<float> r = green_sym_short<PQ, true>(dx, dy, dz, d1, all, 0u, s_tab, rtab, ef);
-    out[2 * i] = double(r.re);
-    out[2 * i + 1] = double(r.im);
-}
-
-// the oblique short form at single displacements (every image visited)
-template <int NR, int NQ1>
-__global__ void k_green_obl(const double *d, double *out, int n, const float *stab, const float4 *rtab,
-                            const __grid_constant__ EwaldF32 ef) {
-    __shared__ float4 s_tab[NSPAT];
-    for (int i = threadIdx.x; i < NSPAT; i += blockDim.x) s_tab[i] = reinterpret_cast<const float4 *>(stab)[i];
-    __syncthreads();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float dx = float(d[3 * i]), dy = float(d[3 * i + 1]), dz = float(d[3 * i + 2]);
-    float s0, c0, s1, c1, s2, c2, s3, c3;
-    sincospif(ef.ob_kx0 * 0.31830988618f * dx, &s0, &c0);
-    sincospif(ef.ob_ky0 * 0.31830988618f * dy, &s1, &c1);
-    sincospif(ef.step_x * 0.31830988618f * dx, &s2, &c2);
-    sincospif(ef.step_y * 0.31830988618f * dy, &s3, &c3);
-    const unsigned long long all = ef.n_img >= 64 ? ~0ull : (1ull << ef.n_img) - 1ull;
-    cx<float> T;
-    // point a at d, point b at the origin: (cos, sin) of the phases of d
-    const float4 pa = make_float4(c0, s0, c1, s1), sa = make_float4(c2, s2, c3, s3);
-    const float4 pb = make_float4(1.f, 0.f, 1.f, 0.f), sb = make_float4(1.f, 0.f, 1.f, 0.f);
-    cx<float> r = green_obl<NR, NQ1, true>(dx, dy, dz, pa, sa, pb, sb, all, 0ull, s_tab, rtab, ef, T);
-    out[2 * i] = double(r.re);
-    out[2 * i + 1] = double(r.im);
-}
-
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-// template variant of the oblique short form: 0-2 the full rectangle of side
-// 4, 6, 8; 3-5 the k_y = 0 fold (6 x 3, 8 x 3, 8 x 5)
-inline int obl_variant(const EwaldF32 &ef) {
-    if (ef.ob_nq1 == 0) return ef.ob_nr == 4 ? 0 : (ef.ob_nr == 6 ? 1 : 2);
-    return ef.ob_nq1 == 3 ? (ef.ob_nr == 6 ? 3 : 4) : 5;
-}
-
 template <typename T, int PK>
 void far_scalar(bool sym, dim3 grid, size_t sm, cudaStream_t st, const DevMesh &m, const DevReq &q, T *Z, size_t N,
                 int nx, int ny, const uint16_t *mk) {
     if constexpr (sizeof(T) == 4) {
-        if (sym && q.ef.sq_pq > 0) {   // normal incidence, short form
-            switch (q.ef.sq_pq) {
-                case 1: k_far_scalar_n<1, PK><<<grid, 128, 0, st>>>(m, q, Z, N, nx, ny, mk); break;
-                case 2: k_far_scalar_n<2, PK><<<grid, 128, 0, st>>>(m, q, Z, N, nx, ny, mk); break;
-                case 3: k_far_scalar_n<3, PK><<<grid, 128, 0, st>>>(m, q, Z, N, nx, ny, mk); break;
-                default: k_far_scalar_n<4, PK><<<grid, 128, 0, st>>>(m, q, Z, N, nx, ny, mk); break;
-            }
-        } else if (!sym && q.ef.ob_nr > 0) {   // oblique incidence, short form
-            switch (obl_variant(q.ef)) {
-                case 0: k_far_scalar_o<4, 0, PK><<<grid, 128, 0, st>>>(m, q, Z, N, nx, ny, mk); break;
-                case 1: k_far_scalar_o<6, 0, PK><<<grid, 128, 0, st>>>(m, q, Z, N, nx, ny, mk); break;
-                case 2: k_far_scalar_o<8, 0, PK><<<grid, 128, 0, st>>>(m, q, Z, N, nx, ny, mk); break;
-                case 3: k_far_scalar_o<6, 3, PK><<<grid, 128, 0, st>>>(m, q, Z, N, nx, ny, mk); break;
-                case 4: k_far_scalar_o<8, 3, PK><<<grid, 128, 0, st>>>(m, q, Z, N, nx, ny, mk); break;
-                default: k_far_scalar_o<8, 5, PK><<<grid, 128, 0, st>>>(m, q, Z, N, nx, ny, mk); break;
-            }
-        } else if (sym) k_far_scalar<T, PK, true><<<grid, 128, sm, st>>>(m, q, Z, N, nx, ny, mk);
+        if (q.fp.mode != FAR_NONE) {
+            launch_far_scalar(PK, m, q, Z, N, st);
+            return;
+        }
+        if (sym) k_far_scalar<T, PK, true><<<grid, 128, sm, st>>>(m, q, Z, N, nx, ny, mk);
         else k_far_scalar<T, PK, false><<<grid, 128, sm, st>>>(m, q, Z, N, nx, ny, mk);
     } else {
         k_far_scalar<T, PK, false><<<grid, 128, sm, st>>>(m, q, Z, N, nx, ny, mk);
@@ -1602,33 +853,23 @@ cudaError_t launch_fill(const DevMesh &m, const DevReq &q, T *Z, size_t ld, doub
     dim3 blk(128);
     k_gram<T><<<(m.nt + 127) / 128, blk, 0, st>>>(m, q, Z, N); ++g_launches;
     if (b) { k_rhs<<<(m.nt + 127) / 128, blk, 0, st>>>(m, q, b); ++g_launches; }
+    if (sizeof(T) == 4) launch_far_prep(m, q, st);   // element records of the FP32 kernels
     const size_t sm = stab_bytes<T>();
     if (far0) cudaEventRecord(far0, st);
     const bool sym = sizeof(T) == 4 && q.ef.sym;   // normal incidence: the symmetric tabulated path
     if constexpr (sizeof(T) == 4) {
         const dim3 gtt((m.nt + 127) / 128, m.nt);
-        if (sym && q.ef.sq_pq > 0) {   // normal incidence, short form
-            switch (q.ef.sq_pq) {
-                case 1: k_far_tt_n<1><<<gtt, blk, 0, st>>>(m, q, Z, N); break;
-                case 2: k_far_tt_n<2><<<gtt, blk, 0, st>>>(m, q, Z, N); break;
-                case 3: k_far_tt_n<3><<<gtt, blk, 0, st>>>(m, q, Z, N); break;
-                default: k_far_tt_n<4><<<gtt, blk, 0, st>>>(m, q, Z, N); break;
-            }
-        } else if (!sym && q.ef.ob_nr > 0) {   // oblique incidence, short form
-            switch (obl_variant(q.ef)) {
-                case 0: k_far_tt_o<4, 0><<<gtt, blk, 0, st>>>(m, q, Z, N); break;
-                case 1: k_far_tt_o<6, 0><<<gtt, blk, 0, st>>>(m, q, Z, N); break;
-                case 2: k_far_tt_o<8, 0><<<gtt, blk, 0, st>>>(m, q, Z, N); break;
-                case 3: k_far_tt_o<6, 3><<<gtt, blk, 0, st>>>(m, q, Z, N); break;
-                case 4: k_far_tt_o<8, 3><<<gtt, blk, 0, st>>>(m, q, Z, N); break;
-                default: k_far_tt_o<8, 5><<<gtt, blk, 0, st>>>(m, q, Z, N); break;
-            }
-        } else if (sym) k_far_tt<T, true><<<gtt, blk, sm, st>>>(m, q, Z, N);
-        else k_far_tt<T, false><<<gtt, blk, sm, st>>>(m, q, Z, N);
+        if (q.fp.mode != FAR_NONE) {
+            launch_far_tt(m, q, Z, N, st);
+        } else {
+            if (sym) k_far_tt<T, true><<<gtt, blk, sm, st>>>(m, q, Z, N);
+            else k_far_tt<T, false><<<gtt, blk, sm, st>>>(m, q, Z, N);
+            ++g_launches;
+        }
     } else {
         k_far_tt<T, false><<<dim3((m.nt + 127) / 128, m.nt), blk, sm, st>>>(m, q, Z, N);
+        ++g_launches;
     }
-    ++g_launches;
     if (far1) cudaEventRecord(far1, st);
     auto grid1 = [](int n) { return (unsigned)((n + 127) / 128); };
     if (m.npr[0]) { k_pr_tt<T><<<grid1(m.npr[0]), blk, 0, st>>>(m, q, Z, N, m.pr[0], m.npr[0]); ++g_launches; }
@@ -1677,29 +918,8 @@ cudaError_t launch_erfcx(const double *u, double *out, int n, bool fp64, cudaStr
 }
 
 cudaError_t launch_green(const double *d, double *out, int n, bool fp64, const float *stab, const float2 *ztab,
-                         const EwaldTables *ew, const EwaldF32 &ef, cudaStream_t st, const float4 *rtab) {
-    const unsigned gb = (unsigned)((n + 127) / 128);
+                         const EwaldTables *ew, const EwaldF32 &ef, cudaStream_t st) {
     if (fp64) { k_green<double><<<(n + 127) / 128, 128, 0, st>>>(d, out, n, stab, ztab, ew, ef); ++g_launches; }
-    else if (ef.sym && ef.sq_pq > 0 && rtab) {   // the fill's normal-incidence form
-        switch (ef.sq_pq) {
-            case 1: k_green_short<1><<<gb, 128, 0, st>>>(d, out, n, stab, ztab, rtab, ef); break;
-            case 2: k_green_short<2><<<gb, 128, 0, st>>>(d, out, n, stab, ztab, rtab, ef); break;
-            case 3: k_green_short<3><<<gb, 128, 0, st>>>(d, out, n, stab, ztab, rtab, ef); break;
-            default: k_green_short<4><<<gb, 128, 0, st>>>(d, out, n, stab, ztab, rtab, ef); break;
-        }
-        ++g_launches;
-    }
-    else if (!ef.sym && ef.ob_nr > 0 && rtab) {   // the fill's oblique form
-        switch (obl_variant(ef)) {
-            case 0: k_green_obl<4, 0><<<gb, 128, 0, st>>>(d, out, n, stab, rtab, ef); break;
-            case 1: k_green_obl<6, 0><<<gb, 128, 0, st>>>(d, out, n, stab, rtab, ef); break;
-            case 2: k_green_obl<8, 0><<<gb, 128, 0, st>>>(d, out, n, stab, rtab, ef); break;
-            case 3: k_green_obl<6, 3><<<gb, 128, 0, st>>>(d, out, n, stab, rtab, ef); break;
-            case 4: k_green_obl<8, 3><<<gb, 128, 0, st>>>(d, out, n, stab, rtab, ef); break;
-            default: k_green_obl<8, 5><<<gb, 128, 0, st>>>(d, out, n, stab, rtab, ef); break;
-        }
-        ++g_launches;
-    }
     else if (ef.sym) { k_green<float, true><<<(n + 127) / 128, 128, 0, st>>>(d, out, n, stab, ztab, ew, ef); ++g_launches; }
     else { k_green<float><<<(n + 127) / 128, 128, 0, st>>>(d, out, n, stab, ztab, ew, ef); ++g_launches; }
     return cudaGetLastError();

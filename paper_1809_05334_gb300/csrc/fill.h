@@ -53,6 +53,8 @@ struct DevMesh {
     template <typename T> __device__ const T *nrel(int t) const;
     template <typename T> __device__ const T *fnrel(int f) const;
 };
+// float4 of the element records of a mesh (k_far_prep)
+inline size_t far_record_count(size_t nt, size_t nf) { return nt * (4 * 4 + 9) + (nf + 1) * (3 * 4 + 2); }
 template <> __device__ inline const float *DevMesh::far<float>(int t) const { return far32 + 28 * (size_t)t; }
 template <> __device__ inline const double *DevMesh::far<double>(int t) const { return far64 + 28 * (size_t)t; }
 template <> __device__ inline const float *DevMesh::ffar<float>(int f) const { return ffar32 + 12 * (size_t)f; }
@@ -79,6 +81,11 @@ struct DevReq {
     const float4 *rtab;    // real parts of ztab (16 bytes per interval), read for the real tables
     const EwaldTables *ew; // Ewald parameters of the request (device memory)
     EwaldF32 ef;           // FP32 inner-loop parameters (kernel parameter space)
+    FarPoly fp;            // the spectral series as polynomials (fp.mode FAR_NONE: the tabulated form)
+    const float *fcoef;    // their coefficients [fp.n_coef]
+    // element records of the FP32 kernels, built per request (k_far_prep): points
+    // [4 FPT][nt] and [3 FPT][nf], elements [FEL_TET][nt] and [FEL_FACE][nf]
+    float4 *ptet, *pface, *etet, *eface;
 };
 
 // degree-5 rules: barycentric points [14][4] / [7][3] (may be null) and weights
@@ -101,10 +108,18 @@ cudaError_t launch_fill(const DevMesh &m, const DevReq &q, T *Z, size_t ld, doub
 // the request-independent static integrals of the touching near images:
 // touch_half [nto[0]][8] and touch_sc[i] [nto[i]] (i = 1..3)
 cudaError_t launch_static_cache(const DevMesh &m, double *touch_half, double *const touch_sc[4], cudaStream_t st);
+// Builds the element records of a request and runs the far pairs in the
+// polynomial form (q.fp.mode != FAR_NONE): tetrahedron pairs, and pairs with
+// charge faces (pk: 0 tetrahedron-face, 1 half face-tetrahedron, 2 half face-face)
+cudaError_t launch_far_prep(const DevMesh &m, const DevReq &q, cudaStream_t st);
+cudaError_t launch_far_tt(const DevMesh &m, const DevReq &q, float *Z, size_t N, cudaStream_t st);
+cudaError_t launch_far_scalar(int pk, const DevMesh &m, const DevReq &q, float *Z, size_t N, cudaStream_t st);
+// g_p at single displacements in the polynomial form
+cudaError_t launch_green_poly(const double *d, double *out, int n, const DevReq &q, cudaStream_t st);
 cudaError_t launch_erfcx(const double *u, double *out, int n, bool fp64, cudaStream_t st);
-// rtab (optional): the real spectral tables; with it, normal incidence takes the fill's short form
+// g_p by the FP64 series or the general tabulated form
 cudaError_t launch_green(const double *d, double *out, int n, bool fp64, const float *stab, const float2 *ztab,
-                         const EwaldTables *ew, const EwaldF32 &ef, cudaStream_t st, const float4 *rtab = nullptr);
+                         const EwaldTables *ew, const EwaldF32 &ef, cudaStream_t st);
 cudaError_t launch_build_tables(const EwaldTables *ew, float *stab, float2 *ztab, int n_tab, cudaStream_t st,
                                 float4 *rtab = nullptr);
 
