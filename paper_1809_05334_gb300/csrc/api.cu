@@ -100,14 +100,16 @@ struct vie_ctx {
     DevBuf Z, b, x, r, u, w, V, h, y, Minv, MinvH, amax, tcpack, tcpack2, status, acc, J, rt, cout, xs;
     DevBuf Zh;     // 16-bit copy of Z read by the GMRES products (VIE_FP16 / VIE_BF16)
     size_t ld16 = 0;   // its row stride (column-interleaved layout, vie::ld16)
-    // the FP16 block inverses the preconditioner reads (interleaved): offsets and row strides
-    std::vector<size_t> moff16, mld16;
+    // the preconditioner's steps on the FP16 block factors: jobs (device), and per
+    // step the first job, the number of jobs and their work units
+    DevBuf pjobs, pvec;
+    struct PStage { int first, n; long long units; };
+    std::vector<PStage> pstages;
     DevBuf dens;   // per-tetrahedron absorbed fractions [2][nt] (request density_out)
     double zh_alpha = 1.0;   // 1 / (power-of-two scale of the FP16 copy)
     // set by the solve server when the request is cancelled: a solve checks it
     // between phases and at every GMRES iteration (the stream is idle there)
     const std::atomic<int> *cancel = nullptr;
-    std::vector<double> pinv;   // per domain block: 1 / (power-of-two scale of its FP16 inverse)
     // autotuner choices for this mesh (0: the defaults): the FP32 tables' Ewald
     // split multiplier per incidence class (0 normal, 1 oblique), and the row
     // ranges per resident CTA of the GMRES products; tuned[c]: class c was tuned
@@ -357,41 +359,25 @@ int fill(vie_ctx *ctx, const vie::DevMesh &m, const vie::DevReq &q, bool with_rh
     return VIE_OK;
 }
 
-// M^-1 applied block by block: out[blk] = Minv_d in[blk].  The largest block's
-// product runs on st, the smaller (latency-bound) ones beside it on the side
-// stream, joined before the application returns on st.
+// M^-1 applied: every stage of all domain blocks in one launch (the steps of a
+// block's forward and backward sweep, precond_step)
 template <typename TV>
-int precond_apply(vie_ctx *ctx, const HostReq &H, const std::vector<size_t> &moff, const std::vector<size_t> &mld,
-                  const TV *in, TV *out, cudaStream_t st) {
-    size_t kbig = 0;
-    for (size_t k = 1; k < H.blk_n.size(); ++k)
-        if (H.blk_n[k] > H.blk_n[kbig]) kbig = k;
-    const bool side = H.blk_n.size() > 1 && ctx->side_stream;
-    if (side) {
-        CK(cudaEventRecord(ctx->side_go, st));
-        CK(cudaStreamWaitEvent(ctx->side_stream, ctx->side_go, 0));
-    }
-    for (size_t k = 0; k < H.blk_off.size(); ++k) {
-        const __half *Mi = ctx->MinvH.as<__half>() + 2 * ctx->moff16[k];
-        CK((vie::matvec<__half, TV, TV>(Mi, ctx->mld16[k], H.blk_n[k], H.blk_n[k], in + 4 * (size_t)H.blk_off[k],
-                                         out + 4 * (size_t)H.blk_off[k], TV(ctx->pinv[k]), false,
-                                         side && k != kbig ? ctx->side_stream : st)));
-    }
-    if (side) {
-        CK(cudaEventRecord(ctx->side_done, ctx->side_stream));
-        CK(cudaStreamWaitEvent(st, ctx->side_done, 0));
-    }
+int precond_apply(vie_ctx *ctx, const TV *in, TV *out, cudaStream_t st) {
+    TV *y = ctx->pvec.as<TV>(), *z = y + 4 * (size_t)ctx->mesh->topo.N;
+    for (const auto &p : ctx->pstages)
+        CK(vie::precond_step<TV>(ctx->MinvH.as<__half>(), ctx->pjobs.as<vie::PrecondJob>() + p.first, p.n, p.units, in, out, y,
+                                 z, st));
     return VIE_OK;
 }
 
 // one application of M^-1 with CUDA events around it (options.timing); the
 // algorithmic bytes are one read of every FP16 block inverse plus the vectors
 template <typename TV>
-int timed_precond(vie_ctx *ctx, const HostReq &H, const std::vector<size_t> &moff, const std::vector<size_t> &mld,
-                  const TV *in, TV *out, cudaStream_t st, Timing &tm) {
+int timed_precond(vie_ctx *ctx, const HostReq &H, const std::vector<size_t> &mld, const TV *in, TV *out, cudaStream_t st,
+                  Timing &tm) {
     cudaEvent_t e0 = ctx->event(), e1 = ctx->event();
     if (e0) CK(cudaEventRecord(e0, st));
-    if (int e = precond_apply<TV>(ctx, H, moff, mld, in, out, st)) return e;
+    if (int e = precond_apply<TV>(ctx, in, out, st)) return e;
     if (e1) {
         CK(cudaEventRecord(e1, st));
         tm.pc.push_back({e0, e1});
@@ -418,8 +404,8 @@ constexpr double INNER_TOL_BF16 = 8e-3;
 // Z: at double length from FP32 arithmetic).  The sweep's products read Z
 // itself, or its 16-bit copy ctx->Zh for VIE_FP16 / VIE_BF16.
 template <typename TZ, typename TV>
-int gmres(vie_ctx *ctx, const HostReq &H, const std::vector<size_t> &moff, const std::vector<size_t> &mld,
-          vie_result *res, cudaStream_t st, Timing &tm) {
+int gmres(vie_ctx *ctx, const HostReq &H, const std::vector<size_t> &mld, vie_result *res, cudaStream_t st,
+          Timing &tm) {
     const int N = ctx->mesh->topo.N;
     const int m = std::max(2, ctx->opt.restart);
     const bool pre = ctx->opt.use_precond != 0;
@@ -438,6 +424,7 @@ int gmres(vie_ctx *ctx, const HostReq &H, const std::vector<size_t> &moff, const
     CK(ctx->V.ensure(sizeof(TV) * vs * (m + 1)));
     CK(ctx->h.ensure(sizeof(double) * 4 * (2 * m + 4)));
     CK(ctx->y.ensure(sizeof(double) * 4 * (m + 1)));
+    if (pre) CK(ctx->pvec.ensure(sizeof(TV) * 2 * vs));
     double *x = ctx->x.as<double>(), *r = ctx->r.as<double>(), *hd = ctx->h.as<double>();
     TV *u = ctx->u.as<TV>(), *w = ctx->w.as<TV>(), *V = ctx->V.as<TV>();
     const TZ *Z = ctx->Z.as<TZ>();
@@ -482,7 +469,7 @@ int gmres(vie_ctx *ctx, const HostReq &H, const std::vector<size_t> &moff, const
         if (!active[0]) s[0] = 0;
         if (!active[1]) s[2] = 0;
         CK((vie::scale<double, TV>(r, u, N, s, st)));
-        if (pre) { if (int e = timed_precond<TV>(ctx, H, moff, mld, u, w, st, tm)) return e; }
+        if (pre) { if (int e = timed_precond<TV>(ctx, H, mld, u, w, st, tm)) return e; }
         else CK(cudaMemcpyAsync(w, u, sizeof(TV) * vs, cudaMemcpyDeviceToDevice, st));
         CK(vie::dots<TV>(w, 0, 1, w, N, hd, st));
         ctx->d2h += sizeof(double) * 4;
@@ -527,7 +514,7 @@ int gmres(vie_ctx *ctx, const HostReq &H, const std::vector<size_t> &moff, const
                 CK((vie::matvec<TZ, TV, TV>(Z, ctx->ld, N, N, vk, pre ? u : vn, TV(1), false, st, mvg)));
             }
             if (e1) { CK(cudaEventRecord(e1, st)); tm.mv.push_back({e0, e1}); }
-            if (pre) { if (int e = timed_precond<TV>(ctx, H, moff, mld, u, vn, st, tm)) return e; }
+            if (pre) { if (int e = timed_precond<TV>(ctx, H, mld, u, vn, st, tm)) return e; }
             // classical Gram-Schmidt, twice; the projections of both passes and
             // the new norm stay on the device until one copy at the end
             const size_t nh = 4 * (size_t)(k + 1);
@@ -610,7 +597,11 @@ cudaEvent_t pool_event(void *c) { return static_cast<vie_ctx *>(c)->event(); }
 
 template <typename TZ>
 int factor(vie_ctx *ctx, const HostReq &H, std::vector<size_t> &moff, std::vector<size_t> &mld, cudaStream_t st,
-           vie::KernelTimer *kt) {
+           vie::KernelTimer *kt, bool full_inverse = false) {
+    const int pivot = ctx->opt.precond_pivot > 0 ? ctx->opt.precond_pivot : (ctx->tune_pivot > 0 ? ctx->tune_pivot : 512);
+    std::vector<int> grp(H.blk_n.size());   // columns per pivot group
+    for (size_t k = 0; k < H.blk_n.size(); ++k)
+        grp[k] = full_inverse ? H.blk_n[k] : vie::gj_group(H.blk_n[k], pivot);
     size_t tot = 0;
     moff.clear();
     mld.clear();
@@ -651,56 +642,85 @@ int factor(vie_ctx *ctx, const HostReq &H, std::vector<size_t> &moff, std::vecto
         float *B = ctx->Minv.as<float>() + 2 * moff[k];
         CK((vie::copy_block<TZ, float>(ctx->Z.as<TZ>(), ctx->ld, H.blk_off[k], H.blk_n[k], B, mld[k], sk)));
         CK(vie::gj_invert_tc(B, mld[k], H.blk_n[k], ctx->status.as<int>(), big ? ctx->tcpack.p : ctx->tcpack2.p, sk,
-                             big ? ctx->aux_stream : ctx->side_stream, kt,
-                             ctx->opt.precond_pivot > 0 ? ctx->opt.precond_pivot
-                                                        : (ctx->tune_pivot > 0 ? ctx->tune_pivot : 512)));
+                             big ? ctx->aux_stream : ctx->side_stream, kt, pivot, grp[k]));
     }
     if (side) {
         CK(cudaEventRecord(ctx->side_done, ctx->side_stream));
         CK(cudaStreamWaitEvent(st, ctx->side_done, 0));
     }
-    // the applications read FP16 copies of the inverses, each scaled by a power
-    // of two that brings its largest entry to [2^13, 2^14) (the scale is undone
-    // in the product): half the bytes of every GMRES preconditioner application
+    // the applications read FP16 copies of the factors: the inverted diagonal
+    // groups and the panels each scaled by a power of two that brings the largest
+    // entry to [2^13, 2^14) (the scales are undone in the products): half the bytes
+    // of every GMRES preconditioner application
     const size_t nblk = H.blk_n.size();
-    CK(ctx->amax.ensure(sizeof(unsigned) * std::max<size_t>(nblk, 1)));
-    CK(cudaMemsetAsync(ctx->amax.p, 0, sizeof(unsigned) * nblk, st));
+    CK(ctx->amax.ensure(sizeof(unsigned) * 2 * std::max<size_t>(nblk, 1)));
+    CK(cudaMemsetAsync(ctx->amax.p, 0, sizeof(unsigned) * 2 * nblk, st));
     for (size_t k = 0; k < nblk; ++k)
-        CK(vie::absmax(ctx->Minv.as<float>() + 2 * moff[k], 2 * mld[k] * (size_t)H.blk_n[k],
-                       ctx->amax.as<unsigned>() + k, st));
+        CK(vie::absmax_groups(ctx->Minv.as<float>() + 2 * moff[k], mld[k], H.blk_n[k], grp[k],
+                              ctx->amax.as<unsigned>() + 2 * k, st));
     int stat = 0;
-    std::vector<unsigned> am(nblk);
-    ctx->d2h += sizeof(int) + sizeof(unsigned) * nblk;
+    std::vector<unsigned> am(2 * nblk);
+    ctx->d2h += sizeof(int) + sizeof(unsigned) * 2 * nblk;
     CK(cudaMemcpyAsync(&stat, ctx->status.p, sizeof(int), cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(am.data(), ctx->amax.p, sizeof(unsigned) * nblk, cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(am.data(), ctx->amax.p, sizeof(unsigned) * 2 * nblk, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     if (stat & 2) return fail(ctx, VIE_DEVICE_TIMEOUT, "a bounded wait of the tensor-core block inversion ran out");
     if (stat) return fail(ctx, VIE_BREAKDOWN, "zero or non-finite pivot while inverting a domain block");
-    ctx->moff16.assign(nblk, 0);
-    ctx->mld16.assign(nblk, 0);
+    std::vector<size_t> moff16(nblk);
     size_t tot16 = 0;
     for (size_t k = 0; k < nblk; ++k) {
-        ctx->moff16[k] = tot16;
-        ctx->mld16[k] = vie::ld16(H.blk_n[k]);
-        tot16 += ctx->mld16[k] * (size_t)H.blk_n[k];
+        moff16[k] = tot16;
+        tot16 += vie::ld16(H.blk_n[k]) * (size_t)H.blk_n[k];
     }
     CK(ctx->MinvH.ensure(sizeof(__half) * 2 * std::max<size_t>(tot16, 1)));
-    ctx->pinv.assign(nblk, 1.0);
+    std::vector<std::vector<vie::PrecondJob>> stages;
     for (size_t k = 0; k < nblk; ++k) {
-        float mx;
-        std::memcpy(&mx, &am[k], sizeof(float));
-        double scale = 1.0;
-        if (mx > 0.f && std::isfinite(mx)) {
-            int ex = 0;
-            std::frexp((double)mx, &ex);   // mx in [2^(ex-1), 2^ex)
-            scale = std::ldexp(1.0, 14 - ex);
-        } else if (!(mx == 0.f)) {
-            return fail(ctx, VIE_BREAKDOWN, "non-finite entry in a domain block inverse");
+        double scale[2] = {1.0, 1.0};   // diagonal groups, panels
+        for (int c = 0; c < 2; ++c) {
+            float mx;
+            std::memcpy(&mx, &am[2 * k + c], sizeof(float));
+            if (mx > 0.f && std::isfinite(mx)) {
+                int ex = 0;
+                std::frexp((double)mx, &ex);   // mx in [2^(ex-1), 2^ex)
+                scale[c] = std::ldexp(1.0, 14 - ex);
+            } else if (!(mx == 0.f)) {
+                return fail(ctx, VIE_BREAKDOWN, "non-finite entry in a domain block inverse");
+            }
         }
-        ctx->pinv[k] = 1.0 / scale;
-        CK(vie::to_half_il(ctx->Minv.as<float>() + 2 * moff[k], mld[k], H.blk_n[k], H.blk_n[k], (float)scale,
-                           ctx->MinvH.as<__half>() + 2 * ctx->moff16[k], st));
+        const int n = H.blk_n[k], g = grp[k], p = (n + g - 1) / g, ld = (int)vie::ld16(n);
+        CK(vie::to_half_groups(ctx->Minv.as<float>() + 2 * moff[k], mld[k], n, g, (float)scale[0], (float)scale[1],
+                               ctx->MinvH.as<__half>() + 2 * moff16[k], st));
+        if (stages.size() < (size_t)(2 * p - 1)) stages.resize(2 * p - 1);
+        for (int s = 0; s < 2 * p - 1; ++s) {   // forward over groups 1 .. p-1, backward over p-1 .. 0
+            const bool bwd = s >= p - 1;
+            const int gi = bwd ? 2 * p - 2 - s : s + 1;
+            vie::PrecondJob j{};
+            j.ld16 = ld; j.voff = H.blk_off[k]; j.row0 = gi * g; j.rows = std::min(g, n - gi * g);
+            j.c0 = bwd ? gi * g : 0;
+            j.c1 = bwd ? n : gi * g;
+            j.split = std::min(n, bwd ? (gi + 1) * g : g);   // forward: the first group's y is the input itself
+            j.x1 = !bwd || gi == 0 ? 0 : 1;
+            j.x2 = bwd ? 2 : 1;
+            j.bwd = bwd;
+            j.alpha = 1.0 / (bwd ? scale[0] : scale[1]);
+            j.zscale = -scale[0] / scale[1];   // the panels' products take x of the later groups with their sign and scale
+            j.m = (long long)moff16[k] + (long long)j.row0 * ld + j.c0;
+            j.pre = 0;
+            stages[s].push_back(j);
+        }
     }
+    std::vector<vie::PrecondJob> jobs;
+    ctx->pstages.clear();
+    for (auto &v : stages) {
+        long long units = 0;
+        for (auto &j : v) { j.pre = units; units += vie::precond_units(j); }
+        ctx->pstages.push_back({(int)jobs.size(), (int)v.size(), units});
+        jobs.insert(jobs.end(), v.begin(), v.end());
+    }
+    CK(ctx->pjobs.ensure(sizeof(vie::PrecondJob) * std::max<size_t>(jobs.size(), 1)));
+    CK(cudaMemcpyAsync(ctx->pjobs.p, jobs.data(), sizeof(vie::PrecondJob) * jobs.size(), cudaMemcpyHostToDevice, st));
+    ctx->h2d += sizeof(vie::PrecondJob) * jobs.size();
+    CK(cudaStreamSynchronize(st));   // jobs is a temporary
     return VIE_OK;
 }
 
@@ -771,7 +791,7 @@ int solve_impl(vie_ctx *ctx, const vie_request *req, vie_result *res, cudaStream
     }
     auto t2 = clk::now();
     if (cancelled(ctx)) return fail(ctx, VIE_CANCELLED, "cancelled");
-    int stat = gmres<TZ, TV>(ctx, H, moff, mld, res, st, tm);
+    int stat = gmres<TZ, TV>(ctx, H, mld, res, st, tm);
     if (stat < 0) return stat;
     auto t3 = clk::now();
     // post-processing
@@ -879,7 +899,7 @@ int slot_footprint(vie_ctx *ctx, const vie_request *req, size_t *bytes) {
     minv += pk1 + pk2;
     const size_t m = (size_t)std::max(2, ctx->opt.restart);
     const size_t vs = 4 * N;
-    size_t b = 2 * sz * ld * N + minv + sz * vs * (m + 3) + 8 * vs * 4 + 64 * (size_t)ctx->mesh->nto[0];
+    size_t b = 2 * sz * ld * N + minv + sz * vs * (m + 5) + 8 * vs * 4 + 64 * (size_t)ctx->mesh->nto[0];
     if (ctx->opt.precision == VIE_FP16 || ctx->opt.precision == VIE_BF16) b += 2 * 2 * vie::ld16((int)N) * N;   // 16-bit copy of Z
     b += (size_t)ctx->mesh->topo.nt * 4 * 64 + (16u << 20);   // request arrays, tables, small buffers
     *bytes = b;
@@ -1476,10 +1496,10 @@ int vie_domain_block(vie_ctx *ctx, const vie_request *req, int32_t block, int32_
     const size_t ldz = ((size_t)ctx->mesh->topo.N + 3) / 4 * 4;
     if (ctx->opt.precision == VIE_FP64) {
         if ((e = fill<double>(ctx, m, q, false, st))) return e;
-        if ((e = factor<double>(ctx, H, moff, mld, st, nullptr))) return e;
+        if ((e = factor<double>(ctx, H, moff, mld, st, nullptr, true))) return e;
     } else {
         if ((e = fill<float>(ctx, m, q, false, st))) return e;
-        if ((e = factor<float>(ctx, H, moff, mld, st, nullptr))) return e;
+        if ((e = factor<float>(ctx, H, moff, mld, st, nullptr, true))) return e;
     }
     if (unknowns)
         for (int i = 0; i < ctx->mesh->topo.N; ++i)
@@ -1650,7 +1670,7 @@ void release_device_memory(vie_ctx *ctx) {
     ctx->mesh = std::make_shared<MeshState>();
     DevBuf *bufs[] = {&ctx->row, &ctx->coef, &ctx->wt, &ctx->kap, &ctx->ieps, &ctx->frow, &ctx->qs,
                       &ctx->perm, &ctx->pol, &ctx->orders, &ctx->stab, &ctx->ztab, &ctx->rtab, &ctx->ew,
-                      &ctx->fcoef, &ctx->frec,
+                      &ctx->fcoef, &ctx->frec, &ctx->pjobs, &ctx->pvec,
                       &ctx->Z, &ctx->b, &ctx->x, &ctx->r, &ctx->u, &ctx->w, &ctx->V, &ctx->h, &ctx->y,
                       &ctx->Minv, &ctx->MinvH, &ctx->amax, &ctx->tcpack, &ctx->tcpack2, &ctx->status, &ctx->acc,
                       &ctx->J, &ctx->xs, &ctx->Zh, &ctx->dens,

@@ -204,8 +204,6 @@ cudaError_t matvec(const TZ *A, size_t ld, int rows, int cols, const TX *x, TA *
 
 template cudaError_t matvec<float, float, float>(const float *, size_t, int, int, const float *, float *, float, bool, cudaStream_t, int);
 template cudaError_t matvec<__half, float, float>(const __half *, size_t, int, int, const float *, float *, float, bool, cudaStream_t, int);
-template cudaError_t matvec<__half, double, double>(const __half *, size_t, int, int, const double *, double *, double, bool,
-                                                    cudaStream_t, int);
 template cudaError_t matvec<__nv_bfloat16, float, float>(const __nv_bfloat16 *, size_t, int, int, const float *, float *,
                                                          float, bool, cudaStream_t, int);
 
@@ -240,6 +238,188 @@ __global__ void k_to16_il(const float *__restrict__ A, size_t lda, int rows, int
             B[2 * i + 1] = __float2bfloat16_rn(v.y);
         }
     }
+}
+
+// ---------------------------------------------------------------------------
+// Preconditioner steps (precond_step, linalg.h): the products of one stage of
+// all domain blocks in one launch.  HBM-bound: the grid is one wave and CTA b
+// takes the row groups whose first work unit lies in its share of the stage's
+// units (4 rows x 128 columns), so every CTA streams about the same bytes
+// whatever the blocks' sizes; inside a row group as k_matvec (the warps split the
+// columns, the next column step's loads in flight).
+// ---------------------------------------------------------------------------
+template <typename TV>
+__global__ void __launch_bounds__(MV_WARPS * 32, sizeof(TV) == 4 ? 3 : 2)
+k_precond(const __half *__restrict__ M, const PrecondJob *__restrict__ jobs, int njobs, long long total,
+          const TV *__restrict__ in, TV *__restrict__ out, TV *y, TV *z) {
+    __shared__ TV part[2][MV_WARPS][MV_ROWS * 4];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long lo = total * blockIdx.x / gridDim.x, hi = total * (blockIdx.x + 1) / gridDim.x;
+    int buf = 0;
+    for (int q = 0; q < njobs; ++q) {
+        const PrecondJob jb = jobs[q];
+        const int chunks = (jb.c1 - jb.c0 + 127) / 128, groups = (jb.rows + MV_ROWS - 1) / MV_ROWS;
+        const long long a = lo - jb.pre, b = hi - jb.pre;
+        if (b <= 0) break;
+        const int g0 = a <= 0 ? 0 : (int)min((long long)groups, (a + chunks - 1) / chunks);
+        const int g1 = (int)min((long long)groups, (b + chunks - 1) / chunks);
+        if (g0 >= g1) continue;
+        const TV *vec[3] = {in + 4 * (size_t)jb.voff, y + 4 * (size_t)jb.voff, z + 4 * (size_t)jb.voff};
+        const TV *xa = jb.x1 == 0 ? vec[0] : vec[1], *xb = jb.x2 == 1 ? vec[1] : vec[2];
+        const int v0 = (int)((long long)chunks * warp / MV_WARPS) * 32, v1 = (int)((long long)chunks * (warp + 1) / MV_WARPS) * 32;
+        for (int g = g0; g < g1; ++g, buf ^= 1) {
+            const int r0 = MV_ROWS * g;
+            const __half *A = M + 2 * (jb.m + (size_t)r0 * jb.ld16);
+            TV acc[MV_ROWS][4];
+#pragma unroll
+            for (int i = 0; i < MV_ROWS; ++i)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) acc[i][k] = TV(0);
+            auto zload = [&](int v, uint4 *w) {
+#pragma unroll
+                for (int i = 0; i < MV_ROWS; ++i)
+                    w[i] = r0 + i < jb.rows ? __ldcs(reinterpret_cast<const uint4 *>(A + 2 * (size_t)i * jb.ld16) + v)
+                                            : make_uint4(0u, 0u, 0u, 0u);
+            };
+            auto zuse = [&](int v, const uint4 *w) {
+                const int base = jb.c0 + (v >> 5) * 128;
+                const TV *x = base < jb.split ? xa : xb;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    TV xv[4] = {TV(0), TV(0), TV(0), TV(0)};
+                    const int cu = base + (v & 31) + 32 * u;   // the entry's column
+                    if (cu < jb.c1) {   // x may be written by this launch on other rows: no read-only path
+                        if constexpr (sizeof(TV) == 4) {
+                            const float4 f = *reinterpret_cast<const float4 *>(x + 4 * (size_t)cu);
+                            xv[0] = f.x; xv[1] = f.y; xv[2] = f.z; xv[3] = f.w;
+                        } else {
+                            const double2 f = *reinterpret_cast<const double2 *>(x + 4 * (size_t)cu);
+                            const double2 h = *reinterpret_cast<const double2 *>(x + 4 * (size_t)cu + 2);
+                            xv[0] = f.x; xv[1] = f.y; xv[2] = h.x; xv[3] = h.y;
+                        }
+                    }
+#pragma unroll
+                    for (int i = 0; i < MV_ROWS; ++i) {
+                        const uint32_t *wv = reinterpret_cast<const uint32_t *>(&w[i]);
+                        const float2 f = widen2<__half>(wv[u]);
+                        const TV zr = TV(f.x), zi = TV(f.y);
+                        acc[i][0] = fma(zr, xv[0], fma(-zi, xv[1], acc[i][0]));
+                        acc[i][1] = fma(zr, xv[1], fma(zi, xv[0], acc[i][1]));
+                        acc[i][2] = fma(zr, xv[2], fma(-zi, xv[3], acc[i][2]));
+                        acc[i][3] = fma(zr, xv[3], fma(zi, xv[2], acc[i][3]));
+                    }
+                }
+            };
+            uint4 zc[MV_ROWS], zn[MV_ROWS];
+            int v = v0 + lane;
+            if (v < v1) zload(v, zc);
+#pragma unroll 2
+            for (; v < v1; v += 32) {
+                if (v + 32 < v1) zload(v + 32, zn);
+                zuse(v, zc);
+#pragma unroll
+                for (int i = 0; i < MV_ROWS; ++i) zc[i] = zn[i];
+            }
+#pragma unroll
+            for (int i = 0; i < MV_ROWS; ++i)
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) acc[i][k] += __shfl_down_sync(0xffffffffu, acc[i][k], o);
+            if (lane == 0) {
+#pragma unroll
+                for (int i = 0; i < MV_ROWS; ++i)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) part[buf][warp][4 * i + k] = acc[i][k];
+            }
+            __syncthreads();
+            if (threadIdx.x < MV_ROWS * 4 && r0 + (int)threadIdx.x / 4 < jb.rows) {
+                TV s = TV(0);
+#pragma unroll
+                for (int w2 = 0; w2 < MV_WARPS; ++w2) s += part[buf][w2][threadIdx.x];
+                s *= TV(jb.alpha);
+                const size_t e = 4 * (size_t)(jb.voff + jb.row0 + r0) + threadIdx.x;
+                if (!jb.bwd) y[e] = in[e] + s;
+                else {
+                    out[e] = s;
+                    z[e] = TV(jb.zscale) * s;
+                }
+            }
+        }
+    }
+}
+
+template <typename TV>
+cudaError_t precond_step(const __half *M, const PrecondJob *jobs, int njobs, long long total, const TV *in, TV *out,
+                         TV *y, TV *z, cudaStream_t st) {
+    if (njobs <= 0) return cudaSuccess;
+    static int slots = 0;   // resident CTAs of the GPU (per instantiation; one device per process)
+    if (slots == 0) {
+        int dev = 0, sms = 0, per = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_precond<TV>, MV_WARPS * 32, 0);
+        if (e != cudaSuccess) return e;
+        slots = std::max(1, sms * per);
+    }
+    k_precond<TV><<<(unsigned)std::max(1ll, std::min((long long)slots, total)), MV_WARPS * 32, 0, st>>>(M, jobs, njobs, total, in,
+                                                                                                   out, y, z);
+    ++g_launches;
+    return cudaGetLastError();
+}
+template cudaError_t precond_step<float>(const __half *, const PrecondJob *, int, long long, const float *, float *, float *,
+                                         float *, cudaStream_t);
+template cudaError_t precond_step<double>(const __half *, const PrecondJob *, int, long long, const double *, double *,
+                                          double *, double *, cudaStream_t);
+
+__global__ void k_absmax_groups(const float *__restrict__ A, size_t ld, int n, int group, unsigned *out) {
+    float m[2] = {0.f, 0.f};
+    for (int r = blockIdx.x; r < n; r += gridDim.x) {
+        const int lo = r / group * group, hi = min(n, lo + group);
+        const float2 *row = reinterpret_cast<const float2 *>(A) + (size_t)r * ld;
+        for (int c = threadIdx.x; c < n; c += blockDim.x) {
+            const float2 v = row[c];
+            const float a = fmaxf(fabsf(v.x), fabsf(v.y));
+            if (c >= lo && c < hi) m[0] = fmaxf(m[0], a); else m[1] = fmaxf(m[1], a);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        for (int o = 16; o > 0; o >>= 1) m[k] = fmaxf(m[k], __shfl_down_sync(0xffffffffu, m[k], o));
+        if ((threadIdx.x & 31) == 0) atomicMax(out + k, __float_as_uint(m[k]));
+    }
+}
+cudaError_t absmax_groups(const float *A, size_t ld, int n, int group, unsigned *out, cudaStream_t st) {
+    k_absmax_groups<<<std::min(n, 1216), 256, 0, st>>>(A, ld, n, group, out); ++g_launches;
+    return cudaGetLastError();
+}
+
+__global__ void k_to16_groups(const float *__restrict__ A, size_t lda, int n, int group, float sd, float sw,
+                              __half *__restrict__ B) {
+    const int ldb = (n + 127) / 128 * 128;
+    for (int r = blockIdx.x; r < n; r += gridDim.x) {
+        const int lo = r / group * group, hi = lo + group;
+        const float2 *row = reinterpret_cast<const float2 *>(A) + (size_t)r * lda;
+        // one thread per 16-byte store: columns j, j + 32, j + 64, j + 96 of a chunk
+        for (int v = threadIdx.x; v < ldb / 4; v += blockDim.x) {
+            const int c0 = (v >> 5) * 128 + (v & 31);
+            uint4 o;
+            uint32_t *w = reinterpret_cast<uint32_t *>(&o);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int c = c0 + 32 * u;
+                const float s = c >= lo && c < hi ? sd : sw;
+                const float2 f = c < n ? row[c] : make_float2(0.f, 0.f);
+                const __half2 h = __floats2half2_rn(s * f.x, s * f.y);
+                w[u] = *reinterpret_cast<const uint32_t *>(&h);
+            }
+            reinterpret_cast<uint4 *>(B + 2 * (size_t)r * ldb)[v] = o;
+        }
+    }
+}
+cudaError_t to_half_groups(const float *A, size_t ld, int n, int group, float sd, float sw, __half *B, cudaStream_t st) {
+    k_to16_groups<<<std::min(n, 2432), 256, 0, st>>>(A, ld, n, group, sd, sw, B); ++g_launches;
+    return cudaGetLastError();
 }
 
 cudaError_t to_bf16_il(const float *A, size_t lda, int rows, int cols, __nv_bfloat16 *B, cudaStream_t st) {
@@ -474,53 +654,44 @@ cudaError_t wait_check(bool arrive, long long polls, int *status, cudaStream_t s
 // Gauss-Jordan with 512-wide outer pivot blocks and tensor-core products
 // (FP32 matrix; FP16 operands scaled by powers of two, FP32 accumulation).
 // ---------------------------------------------------------------------------
-constexpr int GJ_W = 128;     // pivot block width (the K of the tensor-core update)
+constexpr int GJ_T = 64;                // tile of the pivot-block inverse
+constexpr int GJ_DG = 4;                // row groups of its diagonal inverse (256 threads)
+constexpr int GJ_RQ = GJ_T / GJ_DG;     // rows per thread
+constexpr int GJ_THREADS = GJ_T * GJ_DG;
+constexpr int GJ_LDT = GJ_T + 2;        // row stride of the shared tiles (complex): conflict-free transposes
+constexpr size_t GJ_SMEM = 3 * (size_t)GJ_T * GJ_LDT * sizeof(float2);
 
-// In-place Gauss-Jordan inverse of the w x w (w <= GJ_W) pivot block, held in
-// registers, two pivots per step: 512 threads; warp v owns the columns
-// c = 32 (v / 4) + lane and the rows g + 4q (g = v % 4, q = 0..31), so the four
-// warps that own a column (the pivot columns' owners do the extra work of a
-// step) sit on the four schedulers; the block is padded with the identity up
-// to an even width.  Step (j, j+1) with the 2 x 2 pivot block P
-// and rows R = A[j:j+2, :] is one update of every entry,
+// In-place Gauss-Jordan inverse of a 64 x 64 block held in registers (thread
+// (c, g): column c, rows g + 4q), two pivots per step: warp v owns the columns
+// c = 32 (v / 4) + lane and the row group g = v % 4, so the warps that own a
+// column sit on the four schedulers.  Step (j, j+1) with the 2 x 2 pivot block
+// P and rows R = A[j:j+2, :] is one update of every entry,
 //   a_ic <- a_ic - f_i0 m_0c - f_i1 m_1c,
 // m_c = P^-1 R[:, c] off the pivot columns and the matching column of P^-1 on
 // them; f_i = (a_ij, a_i,j+1) off the pivot rows and the rows of P - I on them;
-// the owners of the pivot columns start from the unit vectors.  This gives
-// P^-1 R on the pivot rows, P^-1 on the pivot block, -F P^-1 on the pivot
-// columns and A - F P^-1 R elsewhere.  The pivot rows and the factors travel
-// through double-buffered shared memory; the owners of the next pair publish
-// them right after their update, so one barrier per two pivots suffices.
-constexpr int GJ_DG = 4;               // row groups of the pivot-block inverse (512 threads)
-constexpr int GJ_RQ = GJ_W / GJ_DG;    // rows per thread
-__global__ void __launch_bounds__(GJ_W * GJ_DG) k_gj_diag_w(float *A, size_t ld, int k0, int w, int *status) {
-    __shared__ float2 rowbuf[2][2][GJ_W];
+// the owners of the pivot columns start from the unit vectors.  The pivot rows
+// and the factors travel through double-buffered shared memory; the owners of
+// the next pair publish them right after their update, so one barrier per two
+// pivots suffices.  Returns false on a zero or non-finite pivot.
+__device__ __forceinline__ bool gj_diag(float2 (&a)[GJ_RQ], int c, int g) {
+    __shared__ float2 rowbuf[2][2][GJ_T];
     __shared__ __align__(16) float2 colbuf[2][GJ_DG][GJ_RQ][2];   // factors (f0, f1) of the pivot pair, row g + 4q
-    const int wv = threadIdx.x >> 5;
-    const int c = 32 * (wv >> 2) + (threadIdx.x & 31), g = wv & (GJ_DG - 1);
-    float2 a[GJ_RQ];
-#pragma unroll
-    for (int q = 0; q < GJ_RQ; ++q) {
-        const int i = g + GJ_DG * q;
-        a[q] = make_float2(i == c && (i >= w || c >= w) ? 1.f : 0.f, 0.f);   // identity on the padding
-        if (i < w && c < w) a[q] = *reinterpret_cast<const float2 *>(A + 2 * ((size_t)(k0 + i) * ld + k0 + c));
-    }
-    const int wr = (w + 1) & ~1;
-    // pair 0: rows 0, 1 (groups 0, 1, slot 0), columns 0, 1, the diagonal factors minus one
+    bool ok = true;
     if (g < 2) rowbuf[0][g][c] = a[0];
     if (c < 2) {
 #pragma unroll
         for (int q = 0; q < GJ_RQ; ++q) colbuf[0][g][q][c] = a[q];
         if (g == c) colbuf[0][g][0][c] = make_float2(a[0].x - 1.f, a[0].y);
     }
-    for (int j = 0; j < wr; j += 2) {
+#pragma unroll 1
+    for (int j = 0; j < GJ_T; j += 2) {
         const int b = (j >> 1) & 1, nb = b ^ 1, jn = j + 2;
         __syncthreads();
         const float2 p00 = rowbuf[b][0][j], p01 = rowbuf[b][0][j + 1], p10 = rowbuf[b][1][j], p11 = rowbuf[b][1][j + 1];
         const float dr = (p00.x * p11.x - p00.y * p11.y) - (p01.x * p10.x - p01.y * p10.y);
         const float di = (p00.x * p11.y + p00.y * p11.x) - (p01.x * p10.y + p01.y * p10.x);
         const float dd = dr * dr + di * di;
-        if (threadIdx.x == 0 && (!(dd > 0.f) || !isfinite(dd))) atomicOr(status, 1);
+        if (!(dd > 0.f) || !isfinite(dd)) ok = false;
         const float rd = __frcp_rn(dd);
         const float er = dr * rd, ei = -di * rd;   // 1 / det
         auto cm = [](float ar, float ai, float br, float bi) { return make_float2(ar * br - ai * bi, ar * bi + ai * br); };
@@ -545,22 +716,14 @@ __global__ void __launch_bounds__(GJ_W * GJ_DG) k_gj_diag_w(float *A, size_t ld,
             a[q].x = fmaf(-ff.x, m0.x, fmaf(ff.y, m0.y, fmaf(-ff.z, m1.x, fmaf(ff.w, m1.y, a[q].x))));
             a[q].y = fmaf(-ff.x, m0.y, fmaf(-ff.y, m0.x, fmaf(-ff.z, m1.y, fmaf(-ff.w, m1.x, a[q].y))));
         }
-        if (jn < wr) {
+        if (jn < GJ_T) {
             // rows jn, jn + 1: groups jn % 4 and jn % 4 + 1, slot jn / 4
             const int gj = jn & (GJ_DG - 1), qn = jn / GJ_DG;
             if (g == gj || g == gj + 1) {
-                float2 r = make_float2(0.f, 0.f);
-                switch (qn) {
-#define GJ_ROW_CASE(k) case k: r = a[k]; break;
-                    GJ_ROW_CASE(0) GJ_ROW_CASE(1) GJ_ROW_CASE(2) GJ_ROW_CASE(3) GJ_ROW_CASE(4) GJ_ROW_CASE(5)
-                    GJ_ROW_CASE(6) GJ_ROW_CASE(7) GJ_ROW_CASE(8) GJ_ROW_CASE(9) GJ_ROW_CASE(10) GJ_ROW_CASE(11)
-                    GJ_ROW_CASE(12) GJ_ROW_CASE(13) GJ_ROW_CASE(14) GJ_ROW_CASE(15) GJ_ROW_CASE(16) GJ_ROW_CASE(17)
-                    GJ_ROW_CASE(18) GJ_ROW_CASE(19) GJ_ROW_CASE(20) GJ_ROW_CASE(21) GJ_ROW_CASE(22) GJ_ROW_CASE(23)
-                    GJ_ROW_CASE(24) GJ_ROW_CASE(25) GJ_ROW_CASE(26) GJ_ROW_CASE(27) GJ_ROW_CASE(28) GJ_ROW_CASE(29)
-                    GJ_ROW_CASE(30) GJ_ROW_CASE(31)
-#undef GJ_ROW_CASE
-                    default: break;
-                }
+                float2 r = a[0];
+#pragma unroll
+                for (int q = 1; q < GJ_RQ; ++q)
+                    if (q == qn) r = a[q];
                 rowbuf[nb][g - gj][c] = r;
             }
             if (c == jn || c == jn + 1) {   // columns jn, jn + 1: the factors, diagonal ones minus one
@@ -574,13 +737,112 @@ __global__ void __launch_bounds__(GJ_W * GJ_DG) k_gj_diag_w(float *A, size_t ld,
             }
         }
     }
-    float *Ao;
-    asm volatile("mov.b64 %0, %1;" : "=l"(Ao) : "l"(A));
+    __syncthreads();
+    return ok;
+}
+
+// acc = L R for 64 x 64 complex tiles, L transposed in shared memory (Lt[k][row]),
+// R[k][col]: thread (ty, tx) of 16 x 16 owns rows 4 ty + i, columns tx + 16 j
+__device__ __forceinline__ void gj_tile_mul(const float2 *Lt, const float2 *R, float2 (&acc)[4][4], int ty, int tx) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+#pragma unroll 4
+    for (int k = 0; k < GJ_T; ++k) {
+        float2 l[4], r[4];
+        const float4 l01 = *reinterpret_cast<const float4 *>(Lt + k * GJ_LDT + 4 * ty);
+        const float4 l23 = *reinterpret_cast<const float4 *>(Lt + k * GJ_LDT + 4 * ty + 2);
+        l[0] = make_float2(l01.x, l01.y); l[1] = make_float2(l01.z, l01.w);
+        l[2] = make_float2(l23.x, l23.y); l[3] = make_float2(l23.z, l23.w);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) r[j] = R[k * GJ_LDT + tx + 16 * j];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                acc[i][j].x = fmaf(l[i].x, r[j].x, fmaf(-l[i].y, r[j].y, acc[i][j].x));
+                acc[i][j].y = fmaf(l[i].x, r[j].y, fmaf(l[i].y, r[j].x, acc[i][j].y));
+            }
+    }
+}
+
+// One 64-wide step of the Gauss-Jordan inverse of a w x w block in FP32, src ->
+// dst (different buffers unless there is a single tile): CTA (j, i) writes tile
+// (i, j), with D = src tile (s, s)^-1:
+//   (s, s): D      (s, j): D A_sj      (i, s): -A_is D      else: A_ij - (A_is D) A_sj.
+// Every CTA inverts the diagonal tile itself, so a step is one launch without
+// packing or a wait between CTAs.  The block is padded with the identity to
+// whole tiles (read so, not written).  Bound by the latency of the 32 pivot
+// pairs plus two 64^3 products on one SM (about 20 us a step); the 128-wide
+// register inverse with K = 128 tensor-core products in between took 104 us a
+// step for the inverse alone, and eleven launches.
+__global__ void __launch_bounds__(GJ_THREADS, 2)
+    k_gj_tile(const float *__restrict__ src, size_t lds, float *__restrict__ dst, size_t ldd, int w, int s, int *status) {
+    extern __shared__ __align__(16) float2 gj_smem[];
+    float2 *bD = gj_smem, *bL = bD + GJ_T * GJ_LDT, *bR = bL + GJ_T * GJ_LDT;
+    const int ti = blockIdx.y, tj = blockIdx.x;
+    const int wv = threadIdx.x >> 5;
+    const int c = 32 * (wv >> 2) + (threadIdx.x & 31), g = wv & (GJ_DG - 1);
+    auto load = [&](int r, int cc) {   // entry of the padded source
+        if (r < w && cc < w) return *reinterpret_cast<const float2 *>(src + 2 * ((size_t)r * lds + cc));
+        return make_float2(r == cc ? 1.f : 0.f, 0.f);
+    };
+    float2 a[GJ_RQ];
+#pragma unroll
+    for (int q = 0; q < GJ_RQ; ++q) a[q] = load(GJ_T * s + g + GJ_DG * q, GJ_T * s + c);
+    // the panel tiles meanwhile: A_is transposed, A_sj as it is
+    if (ti != s)
+#pragma unroll 4
+        for (int q = 0; q < GJ_RQ; ++q) bL[c * GJ_LDT + g + GJ_DG * q] = load(GJ_T * ti + g + GJ_DG * q, GJ_T * s + c);
+    if (tj != s)
+#pragma unroll 4
+        for (int q = 0; q < GJ_RQ; ++q) bR[(g + GJ_DG * q) * GJ_LDT + c] = load(GJ_T * s + g + GJ_DG * q, GJ_T * tj + c);
+    const bool ok = gj_diag(a, c, g);
+    if (!ok && ti == s && tj == s && threadIdx.x == 0) atomicOr(status, 1);
+    auto store = [&](int r, int cc, float2 v) {
+        if (r < w && cc < w) *reinterpret_cast<float2 *>(dst + 2 * ((size_t)r * ldd + cc)) = v;
+    };
+    if (ti == s && tj == s) {
+#pragma unroll
+        for (int q = 0; q < GJ_RQ; ++q) store(GJ_T * s + g + GJ_DG * q, GJ_T * s + c, a[q]);
+        return;
+    }
+    // D as the left operand (transposed) for the row panel, else as the right one
 #pragma unroll
     for (int q = 0; q < GJ_RQ; ++q) {
-        const int i = g + GJ_DG * q;
-        if (i < w && c < w) *reinterpret_cast<float2 *>(Ao + 2 * ((size_t)(k0 + i) * ld + k0 + c)) = a[q];
+        const int r = g + GJ_DG * q;
+        bD[ti == s ? c * GJ_LDT + r : r * GJ_LDT + c] = a[q];
     }
+    __syncthreads();
+    const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+    float2 acc[4][4];
+    if (ti == s) gj_tile_mul(bD, bR, acc, ty, tx);        // D A_sj
+    else gj_tile_mul(bL, bD, acc, ty, tx);                // A_is D
+    if (ti != s && tj != s) {
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) bL[(tx + 16 * j) * GJ_LDT + 4 * ty + i] = acc[i][j];
+        __syncthreads();
+        gj_tile_mul(bL, bR, acc, ty, tx);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int r = GJ_T * ti + 4 * ty + i, cc = GJ_T * tj + tx + 16 * j;
+            float2 v = acc[i][j];
+            if (ti != s) {
+                v = make_float2(-v.x, -v.y);
+                if (tj != s) {
+                    const float2 o = load(r, cc);
+                    v = make_float2(o.x + v.x, o.y + v.y);
+                }
+            }
+            store(r, cc, v);
+        }
 }
 
 namespace {
@@ -625,27 +887,32 @@ bool tensor_map(CUtensorMap *map, const void *base, uint64_t inner, uint64_t row
 constexpr int GJ_P = 512;
 constexpr int GJ_PMAX = 1024;
 // SMs the second part of each product (3) leaves free for the next pivot
-// block's inverse, at pivot width 512 and 1024 (measured on the 21k cell's
-// 16,790 block: at 1024, 8 / 12 / 16 / 24 / 32 / 48 SMs gave 47.0 / 46.0 /
-// 44.9 / 44.2 / 43.6 / 46.6 ms per inversion; at 512, 4 / 16 gave 48.1 / 47.1)
+// block's inverse, at pivot width 512 and 1024
 #ifndef VIE_GJ_RESERVE_WIDE
 #define VIE_GJ_RESERVE_WIDE 32
 #endif
 #ifndef VIE_GJ_RESERVE
-#define VIE_GJ_RESERVE 16
+#define VIE_GJ_RESERVE 32
+#endif
+#ifndef VIE_GROUPS4_MIN
+#define VIE_GROUPS4_MIN 6144
+#endif
+#ifndef VIE_GROUPS2_MIN
+#define VIE_GROUPS2_MIN 3072
 #endif
 static_assert(GJ_PMAX <= TC_KP, "the packed operands hold one outer pivot block");
-static_assert(GJ_RQ == 32, "the row-publish jump covers 32 slots");
-static_assert(GJ_W == 128 && GJ_P % GJ_W == 0 && GJ_PMAX % GJ_W == 0, "a pivot block is inverted in 128-wide steps");
+static_assert(GJ_P % GJ_T == 0 && GJ_PMAX % GJ_P == 0, "a pivot block is inverted in 64-wide steps, a wide one in two halves");
+static_assert(GJ_P % TC_TM == 0, "no product tile straddles a pivot block");
 
 constexpr int GJ_WORDS = 16;   // largest-entry words: 4 per set (products (a), (3)), 2 for the pivot blocks
+constexpr size_t GJ_PING = (size_t)GJ_P * GJ_P * 2 * sizeof(float);   // one buffer of the pivot-block inverse
 
 size_t gj_pack_bytes(int n) {
     // two sets (consecutive outer steps overlap) of Ap [mp] and Bp [2 mp] FP16
-    // rows, one set of 3 GJ_PMAX rows for the inversion of the pivot blocks, and
-    // the largest-entry words of the packed operands
+    // rows, one set of 3 GJ_PMAX rows for the two halves of a wide pivot block,
+    // the two buffers of the pivot-block inverse, and the largest-entry words
     const size_t mp = ((size_t)n + TC_TM - 1) / TC_TM * TC_TM;
-    return (2 * 3 * mp + 3 * (size_t)GJ_PMAX) * TC_PACK_ROW * sizeof(__half) + GJ_WORDS * sizeof(unsigned);
+    return (2 * 3 * mp + 3 * (size_t)GJ_PMAX) * TC_PACK_ROW * sizeof(__half) + 2 * GJ_PING + GJ_WORDS * sizeof(unsigned);
 }
 
 namespace {
@@ -653,8 +920,7 @@ int tiles(int r, int c) { return ((r + TC_TM - 1) / TC_TM) * ((c + TC_TN - 1) / 
 int kchunks(int w) { return (2 * w + TC_KCHUNK - 1) / TC_KCHUNK; }
 
 // Packs the operands of one product from A (row stride ld): panel pa into Ap
-// (mp rows, k_tc_pack_a) and panel pb, times sgn, into Bp (2 x 32 x bx rows,
-// k_tc_pack_b), each scaled by the power of two its largest entry (found first
+// (mp rows) and panel pb, times sgn, into Bp (2 x 32 x bx rows), each scaled by the power of two its largest entry (found first
 // into amax[0], amax[1]) selects.
 void tc_pack(cudaStream_t st, const float *A, size_t ld, const TcPanel &pa, int mp, const TcPanel &pb, float sgn,
              int bx, unsigned *amax, __half *Ap, __half *Bp) {
@@ -664,9 +930,8 @@ void tc_pack(cudaStream_t st, const float *A, size_t ld, const TcPanel &pa, int 
     k_tc_absmax<<<dim3(gx, 2), 256, 0, st>>>(A, ld, pa, pb, amax); ++g_launches;
     // only the K chunks the product reads: 32 complex K per chunk of 64 FP16
     const int kp = std::min(TC_KP, (std::max(pa.w, pb.w) + 31) / 32 * 32);
-    k_tc_pack_a<<<(unsigned)(((size_t)mp * kp + 255) / 256), 256, 0, st>>>(A, ld, pa.n1, pa.c0, pa.w, pa.at, pa.skip,
-                                                                          mp, kp, amax, Ap); ++g_launches;
-    k_tc_pack_b<<<dim3(bx, kp / 32), 256, 0, st>>>(A, ld, pb.n1, pb.c0, pb.w, pb.at, pb.skip, sgn, amax + 1, Bp);
+    const unsigned na = (unsigned)(((size_t)mp * kp / 2 + 255) / 256);
+    k_tc_pack<<<na + (unsigned)bx * (kp / 32), 256, 0, st>>>(A, ld, pa, pb, mp, kp, (int)na, bx, sgn, amax, Ap, Bp);
     ++g_launches;
 }
 
@@ -687,14 +952,28 @@ void tc_product(cudaStream_t s, const CUtensorMap &tA, const CUtensorMap &tB, co
     }
 }
 
+// In-place inverse of the w x w block at Ab (row stride ld, w <= GJ_P) by 64-wide
+// steps between the two buffers of `ping`
+cudaError_t invert_small(float *Ab, size_t ld, int w, int *status, float *ping, cudaStream_t st) {
+    const int S = (w + GJ_T - 1) / GJ_T;
+    float *buf[2] = {ping, ping + GJ_PING / sizeof(float)};
+    for (int s = 0; s < S; ++s) {
+        const float *src = s == 0 ? Ab : buf[(s - 1) & 1];
+        float *dst = s == S - 1 ? Ab : buf[s & 1];
+        k_gj_tile<<<dim3(S, S), GJ_THREADS, GJ_SMEM, st>>>(src, s == 0 ? ld : GJ_P, dst, s == S - 1 ? ld : GJ_P, w, s,
+                                                           status); ++g_launches;
+    }
+    return cudaGetLastError();
+}
+
 // In-place inverse of the w x w pivot block at Ab (row stride ld, w <= GJ_PMAX):
-// Gauss-Jordan with 128-wide pivots (register inverse of each 128 block, then
-// its column-panel and trailing/row-panel products, K = 128).  sub: packed
-// operand scratch of 3 GJ_PMAX rows; amax: two largest-entry words.
-cudaError_t invert_pivot_block(float *Ab, size_t ld, int w, int *status, __half *sub, unsigned *amax, int sms,
-                               cudaStream_t st) {
-    k_gj_diag_w<<<1, GJ_W * GJ_DG, 0, st>>>(Ab, ld, 0, std::min(w, GJ_W), status); ++g_launches;
-    if (w <= GJ_W) return cudaGetLastError();
+// a wide block by Gauss-Jordan with two 512-wide pivots, their products on the
+// tensor cores (K = 512).  sub: packed operand scratch of 3 GJ_PMAX rows; amax:
+// two largest-entry words.
+cudaError_t invert_pivot_block(float *Ab, size_t ld, int w, int *status, __half *sub, float *ping, unsigned *amax,
+                               int sms, cudaStream_t st) {
+    cudaError_t e = invert_small(Ab, ld, std::min(w, GJ_P), status, ping, st);
+    if (w <= GJ_P || e != cudaSuccess) return e;
     __half *Ap = sub, *Bp = sub + (size_t)GJ_PMAX * TC_PACK_ROW;
     const int wc = (w + 3) / 4 * 4;   // whole 16-byte column groups (padding columns stay zero)
     CUtensorMap tA, tB, tC, tCs;
@@ -704,15 +983,20 @@ cudaError_t invert_pivot_block(float *Ab, size_t ld, int w, int *status, __half 
         !tensor_map(&tCs, Ab, 2 * (uint64_t)wc, w, 8 * ld, 32, 32))
         return cudaErrorInvalidValue;
     const int wp = (w + TC_TM - 1) / TC_TM * TC_TM;
-    for (int k1 = 0; k1 < w; k1 += GJ_W) {
-        const int wi = std::min(GJ_W, w - k1), m1 = w - wi;
-        if (k1 > 0) { k_gj_diag_w<<<1, GJ_W * GJ_DG, 0, st>>>(Ab, ld, k1, wi, status); ++g_launches; }
+    for (int k1 = 0; k1 < w; k1 += GJ_P) {
+        const int wi = std::min(GJ_P, w - k1), m1 = w - wi;
+        if (k1 > 0) {
+            e = invert_small(Ab + 2 * ((size_t)k1 * ld + k1), ld, wi, status, ping, st);
+            if (e != cudaSuccess) return e;
+        }
         const int mp1 = (m1 + TC_TM - 1) / TC_TM * TC_TM;
-        tc_pack(st, Ab, ld, TcPanel{m1, k1, wi, k1, wi}, mp1, TcPanel{wi, k1, wi, 0, k1}, -1.f, TC_TN / 32, amax, Ap, Bp);
+        tc_pack(st, Ab, ld, TcPanel{m1, k1, wi, k1, wi}, mp1, TcPanel{wi, k1, wi, 0, k1}, -1.f,
+                (wi + TC_TN - 1) / TC_TN * TC_TN / 32, amax, Ap, Bp);
         tc_product(st, tA, tB, tC, tCs, TcMap{m1, wi, k1, wi, 0, k1, 0, 0, 1, 0, 0, 0, 0, kchunks(wi), amax},
                    std::min(tiles(m1, wi), sms), status, nullptr, 0, 0, 0);
         tc_pack(st, Ab, ld, TcPanel{w, k1, wi, w, 0}, wp, TcPanel{m1, k1, wi, k1, wi}, 1.f, mp1 / 32, amax, Ap, Bp);
-        tc_product(st, tA, tB, tC, tCs, TcMap{w, m1, w, 0, k1, wi, k1 / TC_TM, 1, 0, 0, 0, 0, 0, kchunks(wi), amax},
+        tc_product(st, tA, tB, tC, tCs,
+                   TcMap{w, m1, w, 0, k1, wi, k1 / TC_TM, (wi + TC_TM - 1) / TC_TM, 0, 0, 0, 0, 0, kchunks(wi), amax},
                    std::min(tiles(w, m1), sms), status, nullptr, 0, 0, 0);
     }
     return cudaGetLastError();
@@ -735,15 +1019,26 @@ cudaError_t invert_pivot_block(float *Ab, size_t ld, int w, int *status, __half 
 // step's pivot inverse and column-panel product need only the first part, so
 // they run on st while the rest of (3) streams through HBM; the next row-panel
 // packing waits for it.  Consecutive steps use alternate packing buffers.
+// Groups: the pivots are taken in groups of `group` columns (a multiple of the
+// pivot width).  The steps of a group leave the rows and columns of the groups
+// before it alone, so with M = [[A, B], [C, S]] (A the group) they turn the
+// remaining submatrix into [[A^-1, A^-1 B], [-C A^-1, S - C A^-1 B]]: the block
+// ends as a block-triangular factor with inverted diagonal blocks, row group k
+//   [ -C A^-1 of the groups before | A_k^-1 | A_k^-1 B of the groups after ],
+// applied by one forward and one backward sweep over the row groups with the
+// same n^2 entries (linalg.h, precond_step), for 8 n^3 (1 + 1/4 + ...) / p
+// flops instead of 8 n^3: 0.47 of them with four groups.  group >= n gives the
+// inverse itself.
 cudaError_t gj_invert_tc(float *A, size_t ld, int n, int *status, void *pack, cudaStream_t st, cudaStream_t aux,
-                         KernelTimer *kt, int pivot) {
+                         KernelTimer *kt, int pivot, int group) {
     const int P = (pivot == GJ_PMAX) ? GJ_PMAX : GJ_P;   // outer pivot width
     // SMs the rest of each product leaves to the next pivot block's inverse
-    // (its K = 128 products; a 1024-wide block has eight 128-wide steps)
     const int reserve = P > GJ_P ? VIE_GJ_RESERVE_WIDE : VIE_GJ_RESERVE;
     int dev = 0, sms = 0;
     {   // opt in to the large dynamic shared memory (per device, cheap to repeat)
         cudaError_t e = cudaFuncSetAttribute(k_tc_update, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_gj_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GJ_SMEM);
         if (e == cudaSuccess) e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
@@ -753,68 +1048,75 @@ cudaError_t gj_invert_tc(float *A, size_t ld, int n, int *status, void *pack, cu
     __half *const base = static_cast<__half *>(pack);
     __half *Ap[2], *Bp[2];
     __half *sub = base + 2 * set_halves;
-    unsigned *words = reinterpret_cast<unsigned *>(sub + 3 * (size_t)GJ_PMAX * TC_PACK_ROW);   // GJ_WORDS
+    float *ping = reinterpret_cast<float *>(sub + 3 * (size_t)GJ_PMAX * TC_PACK_ROW);
+    unsigned *words = reinterpret_cast<unsigned *>(ping + 2 * GJ_PING / sizeof(float));   // GJ_WORDS
     CUtensorMap tmA[2], tmB[2], tmC, tmCs;
     for (int b = 0; b < 2; ++b) {
         Ap[b] = base + b * set_halves;
         Bp[b] = Ap[b] + (size_t)mpmax * TC_PACK_ROW;
     }
-    if (n > P) {
+    if (n > P)
         for (int b = 0; b < 2; ++b)
             if (!tensor_map(&tmA[b], Ap[b], TC_PACK_ROW, mpmax, TC_PACK_ROW * 2, TC_KCHUNK, TC_TM, true) ||
                 !tensor_map(&tmB[b], Bp[b], TC_PACK_ROW, 2 * (uint64_t)mpmax, TC_PACK_ROW * 2, TC_KCHUNK, 2 * TC_TN,
                             true))
                 return cudaErrorInvalidValue;
-        if (!tensor_map(&tmC, A, 2 * (uint64_t)ld, n, 8 * ld, 32, TC_TM) ||
-            !tensor_map(&tmCs, A, 2 * (uint64_t)ld, n, 8 * ld, 32, 32))
-            return cudaErrorInvalidValue;
-    }
     cudaEvent_t evP = nullptr, evB = nullptr;
     cudaError_t e = cudaEventCreateWithFlags(&evP, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&evB, cudaEventDisableTiming);
     if (e != cudaSuccess) return e;
     bool pending = false;   // the second part of the previous product (3) is running on aux
-    e = invert_pivot_block(A, ld, std::min(n, P), status, sub, words + 8, sms, st);
-    for (int k0 = 0; k0 < n && e == cudaSuccess; k0 += P) {
-        const int w = std::min(P, n - k0);
-        const int m = n - w;
-        if (m <= 0) break;
-        const int cur = (k0 / P) & 1;
-        const int mp = (m + TC_TM - 1) / TC_TM * TC_TM;
-        const int kc = kchunks(w);
-        unsigned *wa = words + 4 * cur, *w3 = wa + 2;   // this set's largest-entry words
-        // (a) column panel: A[T, P] <- A[T, P] (-P^-1)
-        tc_pack(st, A, ld, TcPanel{m, k0, w, k0, w}, mp, TcPanel{w, k0, w, 0, k0}, -1.f,
-                (w + TC_TN - 1) / TC_TN * TC_TN / 32, wa, Ap[cur], Bp[cur]);
-        tc_product(st, tmA[cur], tmB[cur], tmC, tmCs, TcMap{m, w, k0, w, 0, k0, 0, 0, 1, 0, 0, 0, 0, kc, wa},
-                   std::min(tiles(m, w), sms), status, nullptr, 0, 0, 0);
-        // (3) reads this step's row panel, which the previous step's second part wrote
-        if (pending) { cudaStreamWaitEvent(st, evB, 0); pending = false; }
-        tc_pack(st, A, ld, TcPanel{n, k0, w, n, 0}, mpmax, TcPanel{m, k0, w, k0, w}, 1.f, mp / 32, w3, Ap[cur], Bp[cur]);
-        const int ntm = (n + TC_TM - 1) / TC_TM, nt = (m + TC_TN - 1) / TC_TN;
-        const int prow = k0 / TC_TM, nprow = (w + TC_TM - 1) / TC_TM;   // pivot tile rows: beta 0
-        const TcMap mb = {n, m, n, 0, k0, w, prow, nprow, 0, 0, 0, 0, 0, kc, w3};
-        const bool next = k0 + P < n;
-        const int tA = k0 / TC_TN, nA = std::min(P / TC_TN, nt - tA);   // tile columns of the next pivot block
-        if (next && nt > nA) {
-            TcMap ma = mb, mr = mb;
-            ma.only_lo = tA; ma.only_n = nA;
-            mr.skip_lo = tA; mr.skip_n = nA;
-            const int colsA = std::min(nA * TC_TN, m - k0);
-            tc_product(st, tmA[cur], tmB[cur], tmC, tmCs, ma, std::min(ntm * nA, sms), status, kt, n, colsA, w);
-            cudaEventRecord(evP, st);
-            cudaStreamWaitEvent(aux, evP, 0);
-            tc_product(aux, tmA[cur], tmB[cur], tmC, tmCs, mr, std::max(1, std::min(ntm * (nt - nA), sms - reserve)),
-                       status, kt, n, m - colsA, w);
-            cudaEventRecord(evB, aux);
-            pending = true;
-        } else {
-            tc_product(st, tmA[cur], tmB[cur], tmC, tmCs, mb, std::min(tiles(n, m), sms), status, kt, n, m, w);
+    e = invert_pivot_block(A, ld, std::min(n, P), status, sub, ping, words + 8, sms, st);
+    for (int g0 = 0; g0 < n && e == cudaSuccess; g0 += std::min(group, n - g0)) {
+        // the submatrix from the group's first pivot on: rows and columns before it are done
+        float *Ag = A + 2 * ((size_t)g0 * ld + g0);
+        const int ng = n - g0, bg = std::min(group, ng);
+        if (ng > std::min(P, bg) &&
+            (!tensor_map(&tmC, Ag, 2 * (uint64_t)(ld - g0), ng, 8 * ld, 32, TC_TM) ||
+             !tensor_map(&tmCs, Ag, 2 * (uint64_t)(ld - g0), ng, 8 * ld, 32, 32))) {
+            e = cudaErrorInvalidValue;
+            break;
         }
-        if (next) {
-            const int k1 = k0 + P;
-            e = invert_pivot_block(A + 2 * ((size_t)k1 * ld + k1), ld, std::min(n - k1, P), status, sub, words + 8,
-                                   sms, st);
+        for (int k0 = 0; k0 < bg && e == cudaSuccess; k0 += P) {
+            const int w = std::min(P, bg - k0);
+            const int m = ng - w;
+            if (m <= 0) break;
+            const int cur = ((g0 + k0) / P) & 1;
+            const int mp = (m + TC_TM - 1) / TC_TM * TC_TM, np = (ng + TC_TM - 1) / TC_TM * TC_TM;
+            const int kc = kchunks(w);
+            unsigned *wa = words + 4 * cur, *w3 = wa + 2;   // this set's largest-entry words
+            // (a) column panel: A[T, P] <- A[T, P] (-P^-1)
+            tc_pack(st, Ag, ld, TcPanel{m, k0, w, k0, w}, mp, TcPanel{w, k0, w, 0, k0}, -1.f,
+                    (w + TC_TN - 1) / TC_TN * TC_TN / 32, wa, Ap[cur], Bp[cur]);
+            tc_product(st, tmA[cur], tmB[cur], tmC, tmCs, TcMap{m, w, k0, w, 0, k0, 0, 0, 1, 0, 0, 0, 0, kc, wa},
+                       std::min(tiles(m, w), sms), status, nullptr, 0, 0, 0);
+            // (3) reads this step's row panel, which the previous step's second part wrote
+            if (pending) { cudaStreamWaitEvent(st, evB, 0); pending = false; }
+            tc_pack(st, Ag, ld, TcPanel{ng, k0, w, ng, 0}, np, TcPanel{m, k0, w, k0, w}, 1.f, mp / 32, w3, Ap[cur], Bp[cur]);
+            const int ntm = (ng + TC_TM - 1) / TC_TM, nt = (m + TC_TN - 1) / TC_TN;
+            const int prow = k0 / TC_TM, nprow = (w + TC_TM - 1) / TC_TM;   // pivot tile rows: beta 0
+            const TcMap mb = {ng, m, ng, 0, k0, w, prow, nprow, 0, 0, 0, 0, 0, kc, w3};
+            const int k1 = g0 + k0 + w;   // next pivot block (of this group or the next)
+            const bool next = k1 < n;
+            const int wn = next ? std::min(P, (k0 + w < bg ? bg - k0 - w : std::min(group, n - k1))) : 0;
+            const int tA = k0 / TC_TN, nA = std::min((wn + TC_TN - 1) / TC_TN, nt - tA);   // its tile columns
+            if (next && nt > nA) {
+                TcMap ma = mb, mr = mb;
+                ma.only_lo = tA; ma.only_n = nA;
+                mr.skip_lo = tA; mr.skip_n = nA;
+                const int colsA = std::min(nA * TC_TN, m - k0);
+                tc_product(st, tmA[cur], tmB[cur], tmC, tmCs, ma, std::min(ntm * nA, sms), status, kt, ng, colsA, w);
+                cudaEventRecord(evP, st);
+                cudaStreamWaitEvent(aux, evP, 0);
+                tc_product(aux, tmA[cur], tmB[cur], tmC, tmCs, mr,
+                           std::max(1, std::min(ntm * (nt - nA), sms - reserve)), status, kt, ng, m - colsA, w);
+                cudaEventRecord(evB, aux);
+                pending = true;
+            } else {
+                tc_product(st, tmA[cur], tmB[cur], tmC, tmCs, mb, std::min(tiles(ng, m), sms), status, kt, ng, m, w);
+            }
+            if (next)
+                e = invert_pivot_block(A + 2 * ((size_t)k1 * ld + k1), ld, wn, status, sub, ping, words + 8, sms, st);
         }
     }
     if (pending) cudaStreamWaitEvent(st, evB, 0);
@@ -822,6 +1124,13 @@ cudaError_t gj_invert_tc(float *A, size_t ld, int n, int *status, void *pack, cu
     cudaEventDestroy(evB);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
+}
+
+int gj_group(int n, int pivot) {
+    // groups trade flops of the factorisation (8 n^3 -> 0.63 / 0.47 of it with two /
+    // four) for steps of every application (3 / 7 launches instead of 1)
+    const int p = n >= VIE_GROUPS4_MIN ? 4 : (n >= VIE_GROUPS2_MIN ? 2 : 1);
+    return p == 1 ? n : ((n + p - 1) / p + pivot - 1) / pivot * pivot;
 }
 
 // copy a diagonal block Z[off:off+n, off:off+n] into B (ld_b), converting precision

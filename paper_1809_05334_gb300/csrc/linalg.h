@@ -35,19 +35,47 @@ struct KernelTimer {
         flops.push_back(f);
     }
 };
-// In-place inversion of an n x n complex FP32 block (no pivoting) by blocked
+// In-place factorisation of an n x n complex FP32 block (no pivoting) by blocked
 // Gauss-Jordan with 512-wide outer pivot blocks and the tcgen05 products
 // (FP16 operands with power-of-two scales, FP32 accumulation); *status gets
 // bit 0 for a zero or non-finite pivot and bit 1 for a bounded device wait
 // that ran out;
 // `pack` is device scratch of gj_pack_bytes(n) bytes (the packed operands and
 // their scale words), aux a second stream of the caller (look-ahead); the work
-// is complete on st when the last call returns on it
-size_t gj_pack_bytes(int n);
+// is complete on st when the last call returns on it.
 // pivot: width of the outer pivot blocks, 512 (default) or 1024 (half the
-// passes over the block, a longer chain of pivot-block inverses)
+// passes over the block).  group: columns per pivot group, a multiple of the
+// pivot width; group >= n leaves the inverse in A, a smaller one the
+// block-triangular factor that precond_step applies (linalg.cu)
+size_t gj_pack_bytes(int n);
 cudaError_t gj_invert_tc(float *A, size_t ld, int n, int *status, void *pack, cudaStream_t st, cudaStream_t aux,
-                         KernelTimer *kt = nullptr, int pivot = 512);
+                         KernelTimer *kt, int pivot, int group);
+// columns per pivot group that vie_solve takes for a block of n unknowns
+int gj_group(int n, int pivot);
+
+// One step of an application of the preconditioner: the row group `row0` of one
+// domain block times the columns [c0, c1) of its FP16 factor (column-interleaved
+// rows of ld16 entries; c0 a multiple of 128), two right-hand sides.
+//   forward (bwd 0):  y = in + alpha sum_c M x       backward (bwd 1): out = alpha sum_c M x,  z = zscale out
+// x is the vector x1 for columns below split (a multiple of 128 or c1) and x2 from
+// there on: 0 in, 1 y, 2 z.  All vector indices start at the block's offset voff.
+struct PrecondJob {
+    long long m;         // offset of entry (row0, c0) in the factor, complex entries
+    long long pre;       // work units (4-row groups x 128-column chunks) of the step's jobs before this one
+    int ld16, voff, row0, rows, c0, c1, split, x1, x2, bwd;
+    double alpha, zscale;
+};
+inline long long precond_units(const PrecondJob &j) { return (long long)((j.rows + 3) / 4) * ((j.c1 - j.c0 + 127) / 128); }
+// the njobs jobs (device array) of one step in one launch; total: their work units
+template <typename TV>
+cudaError_t precond_step(const __half *M, const PrecondJob *jobs, int njobs, long long total, const TV *in, TV *out,
+                         TV *y, TV *z, cudaStream_t st);
+// out[0], out[1] (zeroed by the caller) <- the largest |Re|, |Im| of an n x n
+// block inside and outside its diagonal groups, as float bits
+cudaError_t absmax_groups(const float *A, size_t ld, int n, int group, unsigned *out, cudaStream_t st);
+// FP16 copy of an n x n block (column-interleaved, rows of ld16(n)): entries
+// inside the diagonal groups times sd, the others times sw
+cudaError_t to_half_groups(const float *A, size_t ld, int n, int group, float sd, float sw, __half *B, cudaStream_t st);
 // one bounded mbarrier wait of at most `polls` polls on a barrier that gets its
 // arrival (arrive) or never does: bit 1 of *status (device) when it runs out
 cudaError_t wait_check(bool arrive, long long polls, int *status, cudaStream_t st);

@@ -128,9 +128,9 @@ __device__ __forceinline__ void mma_commit(uint64_t *mbar) {
                  ::"r"(smem_u32(mbar)) : "memory");
 }
 
-// One operand panel of a product, as the pack kernels read it: mode A (k_tc_pack_a)
+// One operand panel of a product, as the pack kernel reads it: mode A (Ap)
 // rows r < n1 at row(r) = r < at ? r : r + skip, columns c0 .. c0 + w; mode B
-// (k_tc_pack_b) rows c0 .. c0 + w, columns j < n1 at col(j) = j < at ? j : j + skip.
+// (Bp) rows c0 .. c0 + w, columns j < n1 at col(j) = j < at ? j : j + skip.
 struct TcPanel {
     int n1, c0, w, at, skip;
 };
@@ -159,47 +159,53 @@ __global__ void __launch_bounds__(256) k_tc_absmax(const float *__restrict__ A, 
     if ((threadIdx.x & 31) == 0) atomicMax(out + blockIdx.y, __float_as_uint(mx));
 }
 
-// Ap[r][2k..2k+1] = s A[row(r)][col0 + k] for r < rows, k < w, with
-// row(r) = r < at ? r : r + skip; zero elsewhere up to mp rows and kp columns
-// (the K chunks a product reads); s from *amax.
-__global__ void __launch_bounds__(256) k_tc_pack_a(const float *__restrict__ A, size_t ld, int rows, int col0, int w,
-                                                   int at, int skip, int mp, int kp, const unsigned *__restrict__ amax,
-                                                   __half *__restrict__ Ap) {
-    const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (size_t)mp * kp) return;
-    const int r = (int)(e / kp), k = (int)(e % kp);
-    float2 v = make_float2(0.f, 0.f);
-    if (r < rows && k < w) {
-        const int gr = r < at ? r : r + skip;
-        v = *reinterpret_cast<const float2 *>(A + 2 * ((size_t)gr * ld + col0 + k));
-    }
-    const float s = tc_pow2(tc_shift(*amax));
-    *reinterpret_cast<__half2 *>(Ap + (size_t)r * TC_PACK_ROW + 2 * k) = __floats2half2_rn(s * v.x, s * v.y);
-}
-
-// The sign- and power-of-two-scaled real expansion of B[k][j] = A[row0 + k][col(j)]
-// (k < w, j < cols, col(j) = j < at ? j : j + skip), K-major:
+// Both operands of one product.  CTAs below na write
+//   Ap[r][2k..2k+1] = s A[row(r)][c0 + k] for r < pa.n1, k < pa.w (zero elsewhere up
+// to mp rows and kp columns, the K chunks a product reads), two complex k per
+// thread; the others the sign- and power-of-two-scaled real expansion of
+// B[k][j] = A[pb.c0 + k][col(j)] (k < pb.w, j < pb.n1), K-major:
 //   Bp[2j][2k..] = sgn s (Re b, -Im b),  Bp[2j+1][2k..] = sgn s (Im b, Re b)
-// through a 32 x 32 shared-memory transpose (coalesced on both sides); rows up
-// to 2 * 32 * gridDim.x and K up to 32 * gridDim.y are written (zero beyond
-// cols and w).
-__global__ void __launch_bounds__(256) k_tc_pack_b(const float *__restrict__ A, size_t ld, int cols, int row0, int w,
-                                                   int at, int skip, float sgn, const unsigned *__restrict__ amax,
-                                                   __half *__restrict__ Bp) {
+// through a 32 x 32 shared-memory transpose (coalesced on both sides), bx tiles
+// of 32 rows by kp / 32 tiles of K (zero beyond n1 and w).  s from amax[0], amax[1].
+__global__ void __launch_bounds__(256) k_tc_pack(const float *__restrict__ A, size_t ld, TcPanel pa, TcPanel pb, int mp,
+                                                 int kp, int na, int bx, float sgn, const unsigned *__restrict__ amax,
+                                                 __half *__restrict__ Ap, __half *__restrict__ Bp) {
     __shared__ float2 t[32][33];
-    const int j0 = blockIdx.x * 32, kb = blockIdx.y * 32;
+    if ((int)blockIdx.x < na) {
+        const size_t e = 2 * ((size_t)blockIdx.x * blockDim.x + threadIdx.x);
+        if (e >= (size_t)mp * kp) return;
+        const int r = (int)(e / kp), k = (int)(e % kp);   // kp is even: both entries in one row
+        float2 v[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        if (r < pa.n1) {
+            const int gr = r < pa.at ? r : r + pa.skip;
+            const float *p = A + 2 * ((size_t)gr * ld + pa.c0 + k);   // c0, ld even: 16-byte aligned
+            if (k + 1 < pa.w) {
+                const float4 f = *reinterpret_cast<const float4 *>(p);
+                v[0] = make_float2(f.x, f.y);
+                v[1] = make_float2(f.z, f.w);
+            } else if (k < pa.w) {
+                v[0] = *reinterpret_cast<const float2 *>(p);
+            }
+        }
+        const float s = tc_pow2(tc_shift(amax[0]));
+        __half2 h[2] = {__floats2half2_rn(s * v[0].x, s * v[0].y), __floats2half2_rn(s * v[1].x, s * v[1].y)};
+        *reinterpret_cast<uint2 *>(Ap + (size_t)r * TC_PACK_ROW + 2 * k) = *reinterpret_cast<uint2 *>(h);
+        return;
+    }
+    const int tile = blockIdx.x - na;
+    const int j0 = (tile % bx) * 32, kb = (tile / bx) * 32;
     for (int idx = threadIdx.x; idx < 32 * 32; idx += blockDim.x) {
         const int kk = idx / 32, jj = idx % 32;
         const int j = j0 + jj, k = kb + kk;
         float2 v = make_float2(0.f, 0.f);
-        if (j < cols && k < w) {
-            const int gc = j < at ? j : j + skip;
-            v = *reinterpret_cast<const float2 *>(A + 2 * ((size_t)(row0 + k) * ld + gc));
+        if (j < pb.n1 && k < pb.w) {
+            const int gc = j < pb.at ? j : j + pb.skip;
+            v = *reinterpret_cast<const float2 *>(A + 2 * ((size_t)(pb.c0 + k) * ld + gc));
         }
         t[kk][jj] = v;
     }
     __syncthreads();
-    const float g = sgn * tc_pow2(tc_shift(*amax));
+    const float g = sgn * tc_pow2(tc_shift(amax[1]));
     for (int idx = threadIdx.x; idx < 32 * 32; idx += blockDim.x) {
         const int jj = idx / 32, kk = idx % 32;
         const float2 v = t[kk][jj];
