@@ -48,24 +48,53 @@ template <> __device__ __forceinline__ float2 widen2<__nv_bfloat16>(uint32_t w) 
 // flight while it multiplies the current ones (80 registers, three CTAs per
 // SM); FP32 and FP64 entries rely on the unrolled loop alone.
 // ---------------------------------------------------------------------------
-constexpr int MV_ROWS = 4;
+constexpr int MV_ROWS = 4;   // warp_sum16 reduces their 16 sums
 constexpr int MV_WARPS = 8;
 
-template <typename TX, typename TA> __device__ __forceinline__ void load_x(const TX *x, int c, TA out[4]);
-template <> __device__ __forceinline__ void load_x<float, float>(const float *x, int c, float out[4]) {
-    const float4 v = __ldg(reinterpret_cast<const float4 *>(x + 4 * (size_t)c));
+// not through the read-only path: the kernels below may be resident before the
+// launch that writes x has finished
+__device__ __forceinline__ void load_x(const float *x, int c, float out[4]) {
+    const float4 v = *reinterpret_cast<const float4 *>(x + 4 * (size_t)c);
     out[0] = v.x; out[1] = v.y; out[2] = v.z; out[3] = v.w;
 }
-template <> __device__ __forceinline__ void load_x<double, double>(const double *x, int c, double out[4]) {
-    const double2 a = __ldg(reinterpret_cast<const double2 *>(x + 4 * (size_t)c));
-    const double2 b = __ldg(reinterpret_cast<const double2 *>(x + 4 * (size_t)c + 2));
+__device__ __forceinline__ void load_x(const double *x, int c, double out[4]) {
+    const double2 a = *reinterpret_cast<const double2 *>(x + 4 * (size_t)c);
+    const double2 b = *reinterpret_cast<const double2 *>(x + 4 * (size_t)c + 2);
     out[0] = a.x; out[1] = a.y; out[2] = b.x; out[3] = b.y;
 }
+// Sums over the warp of 16 values per lane: halves the values a lane keeps with
+// every step (16 exchanges instead of 80); value lane / 2 ends in lane
+template <typename T> __device__ __forceinline__ T warp_sum16(const T (&acc)[MV_ROWS][4], int lane) {
+    T d[8];
+    {
+        const bool hi = lane & 16;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const T a = acc[q >> 2][q & 3], b = acc[2 + (q >> 2)][q & 3];
+            d[q] = (hi ? b : a) + __shfl_xor_sync(0xffffffffu, hi ? a : b, 16);
+        }
+    }
+#pragma unroll
+    for (int o = 8, k = 4; k >= 1; o >>= 1, k >>= 1) {
+        const bool hi = lane & o;
+#pragma unroll
+        for (int q = 0; q < k; ++q) {
+            const T a = d[q], b = d[q + k];
+            d[q] = (hi ? b : a) + __shfl_xor_sync(0xffffffffu, hi ? a : b, o);
+        }
+    }
+    return d[0] + __shfl_xor_sync(0xffffffffu, d[0], 1);
+}
+__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
-template <typename TZ, typename TX, typename TA, bool ACCUM>
-__global__ void __launch_bounds__(MV_WARPS * 32)
-k_matvec(const TZ *__restrict__ A, size_t ld, int rows, int cols, const TX *__restrict__ x,
-         TA *__restrict__ y, TA alpha) {
+// RINV: y[r] = alpha (sum_c A[r][c] x[c]) R with the upper triangular 2 x 2 R in
+// rinv (r11, r12.re, r12.im, r22): the columns of x normalised on the way out.
+// Launched in a stream of dependent kernels (launch_pdl): the matrix is prefetched
+// before the wait for the kernel that writes x.
+template <typename TZ, typename TX, typename TA, bool ACCUM, bool RINV = false>
+__global__ void __launch_bounds__(MV_WARPS * 32, sizeof(TZ) == 2 ? 3 : 2)
+k_matvec(const TZ *__restrict__ A, size_t ld, int rows, int cols, const TX *x, TA *y, TA alpha,
+         const float *rinv = nullptr) {
     __shared__ TA part[2][MV_WARPS][MV_ROWS * 4];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rb = (int)((long long)rows * blockIdx.x / gridDim.x);
@@ -80,30 +109,47 @@ k_matvec(const TZ *__restrict__ A, size_t ld, int rows, int cols, const TX *__re
         v0 &= ~31;
         v1 = warp + 1 == MV_WARPS ? nvec : (v1 & ~31);
     }
+    if (RINV) {
+#pragma unroll
+        for (int i = 0; i < MV_ROWS; ++i)
+            for (int v = v0 + lane; v < v1 && v < v0 + 4 * 32; v += 32)
+                if (rb + i < re && (lane & 7) == 0) prefetch_l2(A + 2 * ((size_t)(rb + i) * ld + (size_t)v * VEC));
+        cudaTriggerProgrammaticLaunchCompletion();
+        cudaGridDependencySynchronize();
+    }
+    auto zload = [&](int r0, int v, typename V2<TZ>::t *z) {
+        const int c = v * VEC;
+#pragma unroll
+        for (int i = 0; i < MV_ROWS; ++i) {
+            if (r0 + i < re)
+                z[i] = __ldcs(reinterpret_cast<const typename V2<TZ>::t *>(A + 2 * ((size_t)(r0 + i) * ld + c)));
+            else
+                z[i] = {};
+        }
+    };
+    typename V2<TZ>::t zc[MV_ROWS], zn[MV_ROWS];   // 16-bit entries: this column step and the next
+    if (VEC == 4 && rb < re && v0 + lane < v1) zload(rb, v0 + lane, zc);
     int buf = 0;
     for (int r0 = rb; r0 < re; r0 += MV_ROWS, buf ^= 1) {
+        if (VEC != 4) {   // the first lines of the next rows on the way to L2 during this row group
+#pragma unroll
+            for (int i = 0; i < MV_ROWS; ++i)
+                for (int v = v0 + lane; v < v1 && v < v0 + 8 * 32; v += 32)
+                    if (r0 + MV_ROWS + i < re && (lane & 7) == 0)
+                        prefetch_l2(A + 2 * ((size_t)(r0 + MV_ROWS + i) * ld + (size_t)v * VEC));
+        }
         TA acc[MV_ROWS][4];
 #pragma unroll
         for (int i = 0; i < MV_ROWS; ++i)
 #pragma unroll
             for (int k = 0; k < 4; ++k) acc[i][k] = TA(0);
-        auto zload = [&](int v, typename V2<TZ>::t *z) {
-            const int c = v * VEC;
-#pragma unroll
-            for (int i = 0; i < MV_ROWS; ++i) {
-                if (r0 + i < re)
-                    z[i] = __ldcs(reinterpret_cast<const typename V2<TZ>::t *>(A + 2 * ((size_t)(r0 + i) * ld + c)));
-                else
-                    z[i] = {};
-            }
-        };
         auto zuse = [&](int v, const typename V2<TZ>::t *z) {
             const int c = v * VEC;
 #pragma unroll
             for (int u = 0; u < VEC; ++u) {
                 TA xv[4] = {TA(0), TA(0), TA(0), TA(0)};
                 const int cu = VEC == 4 ? (v >> 5) * 128 + (v & 31) + 32 * u : c + u;   // the entry's column
-                if (cu < cols) load_x<TX, TA>(x, cu, xv);
+                if (cu < cols) load_x(x, cu, xv);
 #pragma unroll
                 for (int i = 0; i < MV_ROWS; ++i) {
                     TA zr, zi;
@@ -129,16 +175,10 @@ k_matvec(const TZ *__restrict__ A, size_t ld, int rows, int cols, const TX *__re
             }
         };
         if constexpr (VEC == 4) {   // 16-bit entries: the next column step's loads in flight during this one's products
-            typename V2<TZ>::t zc[MV_ROWS], zn[MV_ROWS];
-            int v = v0 + lane;
-            if (v < v1) zload(v, zc);
 #pragma unroll 2
-            for (; v < v1; v += 32) {
-                if (v + 32 < v1) zload(v + 32, zn);
-                else {
-#pragma unroll
-                    for (int i = 0; i < MV_ROWS; ++i) zn[i] = {};
-                }
+            for (int v = v0 + lane; v < v1; v += 32) {
+                if (v + 32 < v1) zload(r0, v + 32, zn);
+                else if (r0 + MV_ROWS < re) zload(r0 + MV_ROWS, v0 + lane, zn);   // the next rows' first step
                 zuse(v, zc);
 #pragma unroll
                 for (int i = 0; i < MV_ROWS; ++i) zc[i] = zn[i];
@@ -147,22 +187,12 @@ k_matvec(const TZ *__restrict__ A, size_t ld, int rows, int cols, const TX *__re
 #pragma unroll 8
             for (int v = v0 + lane; v < v1; v += 32) {
                 typename V2<TZ>::t z[MV_ROWS];
-                zload(v, z);
+                zload(r0, v, z);
                 zuse(v, z);
             }
         }
-#pragma unroll
-        for (int i = 0; i < MV_ROWS; ++i)
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) acc[i][k] += __shfl_down_sync(0xffffffffu, acc[i][k], o);
-        if (lane == 0) {
-#pragma unroll
-            for (int i = 0; i < MV_ROWS; ++i)
-#pragma unroll
-                for (int k = 0; k < 4; ++k) part[buf][warp][4 * i + k] = acc[i][k];
-        }
+        const TA sum = warp_sum16(acc, lane);
+        if (!(lane & 1)) part[buf][warp][lane >> 1] = sum;
         __syncthreads();
         if (threadIdx.x < MV_ROWS * 4) {
             const int i = threadIdx.x / 4, k = threadIdx.x % 4;
@@ -171,12 +201,43 @@ k_matvec(const TZ *__restrict__ A, size_t ld, int rows, int cols, const TX *__re
                 TA s = TA(0);
 #pragma unroll
                 for (int w2 = 0; w2 < MV_WARPS; ++w2) s += part[buf][w2][threadIdx.x];
+                if constexpr (RINV) {   // (c0, c1) R: lanes 4i .. 4i + 3 hold re, im of the two columns
+                    const unsigned m = __activemask();
+                    const int l0 = threadIdx.x & ~3;
+                    const TA a = __shfl_sync(m, s, l0), b = __shfl_sync(m, s, l0 + 1);
+                    if (k == 0) s = rinv[0] * s;
+                    else if (k == 1) s = rinv[0] * s;
+                    else if (k == 2) s = rinv[3] * s + rinv[1] * a - rinv[2] * b;
+                    else s = rinv[3] * s + rinv[1] * b + rinv[2] * a;
+                }
                 if (ACCUM) y[(size_t)r * 4 + k] += alpha * s;
                 else y[(size_t)r * 4 + k] = alpha * s;
             }
         }
     }
 }
+
+template <typename TZ>
+cudaError_t matvec_rinv(const TZ *A, size_t ld, int rows, int cols, const float *x, float *y, float alpha,
+                        const float *rinv, cudaStream_t st, int grid_mult) {
+    if (rows <= 0) return cudaSuccess;
+    static int slots = 0;   // resident CTAs of the GPU (per instantiation; one device per process)
+    if (slots == 0) {
+        int dev = 0, sms = 0, per = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_matvec<TZ, float, float, false, true>, MV_WARPS * 32, 0);
+        if (e != cudaSuccess) return e;
+        slots = std::max(1, sms * per);
+    }
+    const int grid = std::max(1, std::min(slots * std::max(1, grid_mult), (rows + MV_ROWS - 1) / MV_ROWS));
+    return launch_pdl(k_matvec<TZ, float, float, false, true>, grid, MV_WARPS * 32, st, A, ld, rows, cols, x, y, alpha, rinv);
+}
+template cudaError_t matvec_rinv<float>(const float *, size_t, int, int, const float *, float *, float, const float *, cudaStream_t, int);
+template cudaError_t matvec_rinv<__half>(const __half *, size_t, int, int, const float *, float *, float, const float *, cudaStream_t, int);
+template cudaError_t matvec_rinv<__nv_bfloat16>(const __nv_bfloat16 *, size_t, int, int, const float *, float *, float,
+                                                const float *, cudaStream_t, int);
 
 template <typename TZ, typename TX, typename TA>
 cudaError_t matvec(const TZ *A, size_t ld, int rows, int cols, const TX *x, TA *y, TA alpha, bool accumulate,
@@ -251,11 +312,12 @@ __global__ void k_to16_il(const float *__restrict__ A, size_t lda, int rows, int
 template <typename TV>
 __global__ void __launch_bounds__(MV_WARPS * 32, sizeof(TV) == 4 ? 3 : 2)
 k_precond(const __half *__restrict__ M, const PrecondJob *__restrict__ jobs, int njobs, long long total,
-          const TV *__restrict__ in, TV *__restrict__ out, TV *y, TV *z) {
+          const TV *in, TV *out, TV *y, TV *z) {
     __shared__ TV part[2][MV_WARPS][MV_ROWS * 4];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long lo = total * blockIdx.x / gridDim.x, hi = total * (blockIdx.x + 1) / gridDim.x;
     int buf = 0;
+    bool waited = false;   // for the launch before, which writes the vectors
     for (int q = 0; q < njobs; ++q) {
         const PrecondJob jb = jobs[q];
         const int chunks = (jb.c1 - jb.c0 + 127) / 128, groups = (jb.rows + MV_ROWS - 1) / MV_ROWS;
@@ -267,20 +329,31 @@ k_precond(const __half *__restrict__ M, const PrecondJob *__restrict__ jobs, int
         const TV *vec[3] = {in + 4 * (size_t)jb.voff, y + 4 * (size_t)jb.voff, z + 4 * (size_t)jb.voff};
         const TV *xa = jb.x1 == 0 ? vec[0] : vec[1], *xb = jb.x2 == 1 ? vec[1] : vec[2];
         const int v0 = (int)((long long)chunks * warp / MV_WARPS) * 32, v1 = (int)((long long)chunks * (warp + 1) / MV_WARPS) * 32;
+        if (!waited) {   // the factor is constant: its first rows on the way to L2 meanwhile
+            for (int i = 0; i < 2 * MV_ROWS; ++i)
+                for (int v = v0 + lane; v < v1 && v < v0 + 4 * 32; v += 32)
+                    if (MV_ROWS * g0 + i < jb.rows && (lane & 7) == 0)
+                        prefetch_l2(reinterpret_cast<const uint4 *>(M + 2 * (jb.m + (size_t)(MV_ROWS * g0 + i) * jb.ld16)) + v);
+            cudaTriggerProgrammaticLaunchCompletion();
+            cudaGridDependencySynchronize();
+            waited = true;
+        }
+        auto zload = [&](int r0, int v, uint4 *w) {
+            const __half *A = M + 2 * (jb.m + (size_t)r0 * jb.ld16);
+#pragma unroll
+            for (int i = 0; i < MV_ROWS; ++i)
+                w[i] = r0 + i < jb.rows ? __ldcs(reinterpret_cast<const uint4 *>(A + 2 * (size_t)i * jb.ld16) + v)
+                                        : make_uint4(0u, 0u, 0u, 0u);
+        };
+        uint4 zc[MV_ROWS], zn[MV_ROWS];
+        if (v0 + lane < v1) zload(MV_ROWS * g0, v0 + lane, zc);
         for (int g = g0; g < g1; ++g, buf ^= 1) {
             const int r0 = MV_ROWS * g;
-            const __half *A = M + 2 * (jb.m + (size_t)r0 * jb.ld16);
             TV acc[MV_ROWS][4];
 #pragma unroll
             for (int i = 0; i < MV_ROWS; ++i)
 #pragma unroll
                 for (int k = 0; k < 4; ++k) acc[i][k] = TV(0);
-            auto zload = [&](int v, uint4 *w) {
-#pragma unroll
-                for (int i = 0; i < MV_ROWS; ++i)
-                    w[i] = r0 + i < jb.rows ? __ldcs(reinterpret_cast<const uint4 *>(A + 2 * (size_t)i * jb.ld16) + v)
-                                            : make_uint4(0u, 0u, 0u, 0u);
-            };
             auto zuse = [&](int v, const uint4 *w) {
                 const int base = jb.c0 + (v >> 5) * 128;
                 const TV *x = base < jb.split ? xa : xb;
@@ -310,28 +383,16 @@ k_precond(const __half *__restrict__ M, const PrecondJob *__restrict__ jobs, int
                     }
                 }
             };
-            uint4 zc[MV_ROWS], zn[MV_ROWS];
-            int v = v0 + lane;
-            if (v < v1) zload(v, zc);
 #pragma unroll 2
-            for (; v < v1; v += 32) {
-                if (v + 32 < v1) zload(v + 32, zn);
+            for (int v = v0 + lane; v < v1; v += 32) {
+                if (v + 32 < v1) zload(r0, v + 32, zn);
                 zuse(v, zc);
 #pragma unroll
                 for (int i = 0; i < MV_ROWS; ++i) zc[i] = zn[i];
             }
-#pragma unroll
-            for (int i = 0; i < MV_ROWS; ++i)
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) acc[i][k] += __shfl_down_sync(0xffffffffu, acc[i][k], o);
-            if (lane == 0) {
-#pragma unroll
-                for (int i = 0; i < MV_ROWS; ++i)
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) part[buf][warp][4 * i + k] = acc[i][k];
-            }
+            if (g + 1 < g1 && v0 + lane < v1) zload(MV_ROWS * (g + 1), v0 + lane, zc);   // in flight during the sums
+            const TV sum = warp_sum16(acc, lane);
+            if (!(lane & 1)) part[buf][warp][lane >> 1] = sum;
             __syncthreads();
             if (threadIdx.x < MV_ROWS * 4 && r0 + (int)threadIdx.x / 4 < jb.rows) {
                 TV s = TV(0);
@@ -362,10 +423,8 @@ cudaError_t precond_step(const __half *M, const PrecondJob *jobs, int njobs, lon
         if (e != cudaSuccess) return e;
         slots = std::max(1, sms * per);
     }
-    k_precond<TV><<<(unsigned)std::max(1ll, std::min((long long)slots, total)), MV_WARPS * 32, 0, st>>>(M, jobs, njobs, total, in,
-                                                                                                   out, y, z);
-    ++g_launches;
-    return cudaGetLastError();
+    return launch_pdl(k_precond<TV>, (int)std::max(1ll, std::min((long long)slots, total)), MV_WARPS * 32, st, M, jobs, njobs,
+                      total, in, out, y, z);
 }
 template cudaError_t precond_step<float>(const __half *, const PrecondJob *, int, long long, const float *, float *, float *,
                                          float *, cudaStream_t);

@@ -21,6 +21,55 @@ cudaError_t matvec_ds(const float *A, size_t ld, int rows, int cols, const doubl
 template <typename TZ, typename TX, typename TA>
 cudaError_t matvec(const TZ *A, size_t ld, int rows, int cols, const TX *x, TA *y, TA alpha, bool accumulate,
                    cudaStream_t st, int grid_mult = 1);
+// Launch that may become resident before the kernel in front of it in the stream
+// has finished (programmatic dependent launch); every kernel launched so waits
+// (cudaGridDependencySynchronize) before it touches anything but constant data.
+// The gap between dependent launches, 2-4 us each, is most of a GMRES iteration on
+// small cells.
+template <typename... KA, typename... A>
+cudaError_t launch_pdl(void (*kernel)(KA...), dim3 grid, int block, cudaStream_t st, A... args) {
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    ++g_launches;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KA>(args)...);
+}
+// y <- alpha (A x) R, FP32 vectors, R the 2 x 2 upper triangular rinv (device: r11,
+// r12.re, r12.im, r22); launched with launch_pdl
+template <typename TZ>
+cudaError_t matvec_rinv(const TZ *A, size_t ld, int rows, int cols, const float *x, float *y, float alpha,
+                        const float *rinv, cudaStream_t st, int grid_mult);
+
+// ---- block GMRES over the two right-hand sides (krylov.cu), FP32 vectors ----
+// Basis block j is the pair of columns w_j stored as one [n][2] complex vector,
+// orthogonal to the blocks before it but not normalised: V_j = w_j R_j^-1 with
+// the Cholesky factor R_j of its Gram matrix.  `state`: device scratch of one solve,
+// dots of both passes, Grams, counters (zeroed before the first block), then the
+// coefficients, inverse Grams and inverse R
+size_t block_state_bytes(int m);
+// doubles of one message to the host (pinned): coefficients of both passes
+// [nv][8] each (as applied, FP32 values), Gram of pass 1 and of pass 2 [4] each,
+// then one 64-bit sequence word
+size_t block_message_doubles(int m);
+// C_j = (w_j^H w_j)^-1 w_j^H w for the nv blocks of V into pass `pass` of the state
+cudaError_t block_dots(const float *V, size_t vstride, int nv, const float *w, int n, int m, void *state, int pass,
+                       cudaStream_t st);
+// w -= sum_j w_j C_j; pass 0: then the Gram matrix of w; pass 1: also takes the part
+// along column 0 out of column 1 (by pass 0's Gram matrix), then forms the Gram
+// matrix of block nv, its R^-1 and inverse, sends the message with sequence number
+// seq and clears the state for the next block
+cudaError_t block_subtract(const float *V, size_t vstride, int nv, float *w, int n, int m, void *state, int pass,
+                           double *message, unsigned long long seq, cudaStream_t st);
+const float *block_rinv(void *state, int m, int j);   // device address of R_j^-1
+// x[i][p] += sum_j sum_a w_j[i][a] Y[j][a][p] (FP64; Y on the device, [nv][2][2] complex)
+cudaError_t block_combine(const float *V, size_t vstride, int nv, const double *Y, double *x, int n, cudaStream_t st);
+
 // CUDA-event timing of selected launches (optional)
 struct KernelTimer {
     cudaEvent_t (*alloc)(void *) = nullptr;   // returns the next event of the caller's pool
