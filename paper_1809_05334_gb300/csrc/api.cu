@@ -126,6 +126,7 @@ struct vie_ctx {
     DevBuf bstate;   // device state of the block GMRES iteration (krylov.cu)
     PinBuf pin;      // its messages
     unsigned long long seq = 0;
+    std::vector<vie::PrecondJob> hjobs;
     struct PStage { int first, n; long long units; };
     std::vector<PStage> pstages;
     DevBuf dens;   // per-tetrahedron absorbed fractions [2][nt] (request density_out)
@@ -386,10 +387,10 @@ int fill(vie_ctx *ctx, const vie::DevMesh &m, const vie::DevReq &q, bool with_rh
 // block's forward and backward sweep, precond_step)
 template <typename TV>
 int precond_apply(vie_ctx *ctx, const TV *in, TV *out, cudaStream_t st) {
-    TV *y = ctx->pvec.as<TV>(), *z = y + 4 * (size_t)ctx->mesh->topo.N;
+    TV *y = ctx->pvec.as<TV>(), *z = y + 4 * vie::pad_cols(ctx->mesh->topo.N);
     for (const auto &p : ctx->pstages)
-        CK(vie::precond_step<TV>(ctx->MinvH.as<__half>(), ctx->pjobs.as<vie::PrecondJob>() + p.first, p.n, p.units, in, out, y,
-                                 z, st));
+        CK(vie::precond_step<TV>(ctx->MinvH.as<__half>(), ctx->hjobs.data() + p.first,
+                                 ctx->pjobs.as<vie::PrecondJob>() + p.first, p.n, p.units, in, out, y, z, st));
     return VIE_OK;
 }
 
@@ -512,12 +513,13 @@ int gmres_block(vie_ctx *ctx, const std::vector<size_t> &mld, const HostReq &H, 
     const int zin = ctx->opt.precision == VIE_FP16 ? 1 : ctx->opt.precision == VIE_BF16 ? 2 : 0;
     const double inner_def = zin == 1 ? INNER_TOL_FP16 : zin == 2 ? INNER_TOL_BF16 : INNER_TOL_FP32;
     const double inner_tol = std::max(ctx->opt.inner_tol > 0 ? ctx->opt.inner_tol : inner_def, 1e-6);
-    const size_t vs = 4 * (size_t)N;     // stride of one basis block (two columns)
+    const size_t vs = 4 * vie::pad_cols(N);     // stride of one basis block (two columns, zero past N)
+    const size_t used = 4 * (size_t)N;
     const int mvg = ctx->tune_mv > 0 ? ctx->tune_mv : 1;   // launch shape of the Z products
     const size_t msg = vie::block_message_doubles(m);
     constexpr int RING = 4;
-    CK(ctx->x.ensure(sizeof(double) * vs));
-    CK(ctx->r.ensure(sizeof(double) * vs));
+    CK(ctx->x.ensure(sizeof(double) * used));
+    CK(ctx->r.ensure(sizeof(double) * used));
     CK(ctx->u.ensure(sizeof(float) * vs));
     CK(ctx->V.ensure(sizeof(float) * vs * (m + 1)));
     CK(ctx->h.ensure(sizeof(double) * 4));
@@ -525,12 +527,17 @@ int gmres_block(vie_ctx *ctx, const std::vector<size_t> &mld, const HostReq &H, 
     CK(ctx->xs.ensure(sizeof(float) * 8 * (size_t)N));
     CK(ctx->bstate.ensure(vie::block_state_bytes(m)));
     CK(ctx->pin.ensure(sizeof(double) * (8 + RING * msg)));
-    if (pre) CK(ctx->pvec.ensure(sizeof(float) * 2 * vs));
+    if (pre) {
+        CK(ctx->pvec.ensure(sizeof(float) * 2 * vs));
+        CK(cudaMemsetAsync(ctx->pvec.p, 0, sizeof(float) * 2 * vs, st));
+    }
+    CK(cudaMemsetAsync(ctx->u.p, 0, sizeof(float) * vs, st));
+    CK(cudaMemset2DAsync(ctx->V.as<float>() + used, sizeof(float) * vs, 0, sizeof(float) * (vs - used), m + 1, st));
     double *pin = static_cast<double *>(ctx->pin.p), *ring = pin + 8;
     double *x = ctx->x.as<double>();
     float *u = ctx->u.as<float>(), *V = ctx->V.as<float>();
     void *state = ctx->bstate.p;
-    CK(cudaMemsetAsync(x, 0, sizeof(double) * vs, st));
+    CK(cudaMemsetAsync(x, 0, sizeof(double) * used, st));
     double bn[2];
     {
         double *hd = ctx->h.as<double>();
@@ -754,12 +761,16 @@ int gmres(vie_ctx *ctx, const HostReq &H, const std::vector<size_t> &mld, vie_re
     const int mvg = ctx->tune_mv > 0 ? ctx->tune_mv : 1;   // launch shape of the Z products
     CK(ctx->x.ensure(sizeof(double) * vs));
     CK(ctx->r.ensure(sizeof(double) * vs));
-    CK(ctx->u.ensure(sizeof(TV) * vs));
+    CK(ctx->u.ensure(sizeof(TV) * 4 * vie::pad_cols(N)));   // zero past N (read by the preconditioner)
+    CK(cudaMemsetAsync(ctx->u.p, 0, sizeof(TV) * 4 * vie::pad_cols(N), st));
     CK(ctx->w.ensure(sizeof(TV) * vs));
     CK(ctx->V.ensure(sizeof(TV) * vs * (m + 1)));
     CK(ctx->h.ensure(sizeof(double) * 4 * (2 * m + 4)));
     CK(ctx->y.ensure(sizeof(double) * 4 * (m + 1)));
-    if (pre) CK(ctx->pvec.ensure(sizeof(TV) * 2 * vs));
+    if (pre) {
+        CK(ctx->pvec.ensure(sizeof(TV) * 8 * vie::pad_cols(N)));
+        CK(cudaMemsetAsync(ctx->pvec.p, 0, sizeof(TV) * 8 * vie::pad_cols(N), st));
+    }
     double *x = ctx->x.as<double>(), *r = ctx->r.as<double>(), *hd = ctx->h.as<double>();
     TV *u = ctx->u.as<TV>(), *w = ctx->w.as<TV>(), *V = ctx->V.as<TV>();
     const TZ *Z = ctx->Z.as<TZ>();
@@ -1035,7 +1046,7 @@ int factor(vie_ctx *ctx, const HostReq &H, std::vector<size_t> &moff, std::vecto
     CK(ctx->pjobs.ensure(sizeof(vie::PrecondJob) * std::max<size_t>(jobs.size(), 1)));
     CK(cudaMemcpyAsync(ctx->pjobs.p, jobs.data(), sizeof(vie::PrecondJob) * jobs.size(), cudaMemcpyHostToDevice, st));
     ctx->h2d += sizeof(vie::PrecondJob) * jobs.size();
-    CK(cudaStreamSynchronize(st));   // jobs is a temporary
+    ctx->hjobs = std::move(jobs);   // outlives the copy
     return VIE_OK;
 }
 
@@ -1216,7 +1227,7 @@ int slot_footprint(vie_ctx *ctx, const vie_request *req, size_t *bytes) {
     minv += pk1 + pk2;
     const size_t m = (size_t)std::max(2, ctx->opt.restart);
     const size_t vs = 4 * N;
-    size_t b = 2 * sz * ld * N + minv + sz * vs * (m + 5) + 8 * vs * 4 + 64 * (size_t)ctx->mesh->nto[0];
+    size_t b = 2 * sz * ld * N + minv + sz * 4 * vie::pad_cols((int)N) * (m + 5) + 8 * vs * 4 + 64 * (size_t)ctx->mesh->nto[0];
     if (ctx->opt.precision == VIE_FP16 || ctx->opt.precision == VIE_BF16) b += 2 * 2 * vie::ld16((int)N) * N;   // 16-bit copy of Z
     b += (size_t)ctx->mesh->topo.nt * 4 * 64 + (16u << 20);   // request arrays, tables, small buffers
     *bytes = b;
@@ -1339,17 +1350,15 @@ int tune_impl(vie_ctx *ctx, const vie_request *req, vie_tune_report *out, cudaSt
             if (int e = make_z16(ctx, st)) return e;
     }
     DevBuf xv, yv;
-    CK(xv.ensure(sizeof(TV) * 4 * (size_t)N));
+    CK(xv.ensure(sizeof(TV) * 4 * vie::pad_cols(N)));
     CK(yv.ensure(sizeof(TV) * 4 * (size_t)N));
-    CK(cudaMemsetAsync(xv.p, 0, sizeof(TV) * 4 * (size_t)N, st));
+    CK(cudaMemsetAsync(xv.p, 0, sizeof(TV) * 4 * vie::pad_cols(N), st));
     auto product = [&](int g) -> cudaError_t {
         if constexpr (std::is_same<TV, float>::value) {
             if (ctx->opt.precision == VIE_FP16)
-                return vie::matvec<__half, TV, TV>(ctx->Zh.as<__half>(), ctx->ld16, N, N, xv.as<TV>(), yv.as<TV>(),
-                                                   TV(ctx->zh_alpha), false, st, g);
+                return vie::matvec16(ctx->Zh.as<__half>(), ctx->ld16, N, xv.as<TV>(), yv.as<TV>(), TV(ctx->zh_alpha), st, g);
             if (ctx->opt.precision == VIE_BF16)
-                return vie::matvec<__nv_bfloat16, TV, TV>(ctx->Zh.as<__nv_bfloat16>(), ctx->ld16, N, N, xv.as<TV>(),
-                                                          yv.as<TV>(), TV(1), false, st, g);
+                return vie::matvec16(ctx->Zh.as<__nv_bfloat16>(), ctx->ld16, N, xv.as<TV>(), yv.as<TV>(), TV(1), st, g);
         }
         return vie::matvec<TZ, TV, TV>(ctx->Z.as<TZ>(), ctx->ld, N, N, xv.as<TV>(), yv.as<TV>(), TV(1), false, st, g);
     };

@@ -22,8 +22,6 @@ namespace vie {
 template <typename T> struct V2;
 template <> struct V2<float> { using t = float4; };
 template <> struct V2<double> { using t = double2; };
-template <> struct V2<__half> { using t = uint4; };   // four complex FP16 entries
-template <> struct V2<__nv_bfloat16> { using t = uint4; };   // four complex BF16 entries
 
 // one complex 16-bit entry (two halves of a 32-bit word) widened to FP32
 template <typename T> __device__ __forceinline__ float2 widen2(uint32_t w);
@@ -43,13 +41,13 @@ template <> __device__ __forceinline__ float2 widen2<__nv_bfloat16>(uint32_t w) 
 // (equal segments, 16-byte loads of A streamed with evict-first), reduce by
 // shuffles, and combine the warps' partial sums through shared memory (double
 // buffered: one barrier per row group).  x is read through L1/L2 (it is a few
-// hundred KB and every row group reuses it).  16-bit entries carry twice the
-// products per byte, so their loop keeps the next column step's loads in
-// flight while it multiplies the current ones (80 registers, three CTAs per
-// SM); FP32 and FP64 entries rely on the unrolled loop alone.
+// hundred KB and every row group reuses it).
 // ---------------------------------------------------------------------------
 constexpr int MV_ROWS = 4;   // warp_sum16 reduces their 16 sums
 constexpr int MV_WARPS = 8;
+// two CTAs per SM at 128 registers for all products: the unrolled FP32 loop holds 16
+// loads in flight (bench cell, GMRES phase: 61.5 ms; at 64 registers and four CTAs
+// 66); 16-bit entries 64.4 ms, three CTAs 67.0, four 68.1
 
 // not through the read-only path: the kernels below may be resident before the
 // launch that writes x has finished
@@ -87,28 +85,31 @@ template <typename T> __device__ __forceinline__ T warp_sum16(const T (&acc)[MV_
 }
 __device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
+// component k (re, im of column 0, of column 1) of the row (c0, c1) R, R upper
+// triangular (r11, r12.re, r12.im, r22); the row's components sit in four adjacent lanes
+template <typename T> __device__ __forceinline__ T times_r(T s, int k, const float *r) {
+    const unsigned m = __activemask();
+    const int l0 = threadIdx.x & ~3;
+    const T a = __shfl_sync(m, s, l0), b = __shfl_sync(m, s, l0 + 1);
+    if (k < 2) return r[0] * s;
+    return k == 2 ? r[3] * s + r[1] * a - r[2] * b : r[3] * s + r[1] * b + r[2] * a;
+}
+
 // RINV: y[r] = alpha (sum_c A[r][c] x[c]) R with the upper triangular 2 x 2 R in
 // rinv (r11, r12.re, r12.im, r22): the columns of x normalised on the way out.
 // Launched in a stream of dependent kernels (launch_pdl): the matrix is prefetched
 // before the wait for the kernel that writes x.
 template <typename TZ, typename TX, typename TA, bool ACCUM, bool RINV = false>
-__global__ void __launch_bounds__(MV_WARPS * 32, sizeof(TZ) == 2 ? 3 : 2)
+__global__ void __launch_bounds__(MV_WARPS * 32, 2)
 k_matvec(const TZ *__restrict__ A, size_t ld, int rows, int cols, const TX *x, TA *y, TA alpha,
          const float *rinv = nullptr) {
     __shared__ TA part[2][MV_WARPS][MV_ROWS * 4];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rb = (int)((long long)rows * blockIdx.x / gridDim.x);
     const int re = (int)((long long)rows * (blockIdx.x + 1) / gridDim.x);
-    constexpr int VEC = sizeof(TZ) == 4 ? 2 : (sizeof(TZ) == 8 ? 1 : 4);   // complex entries per 16-byte load
-    // 16-bit entries: the column-interleaved layout (ld16 columns per row, load
-    // v holds columns 128 (v / 32) + v % 32 + 32 u); warp segments start on a
-    // chunk, so a warp's x loads of one step are contiguous
-    const int nvec = VEC == 4 ? (cols + 127) / 128 * 32 : (cols + VEC - 1) / VEC;
-    int v0 = (int)((long long)nvec * warp / MV_WARPS), v1 = (int)((long long)nvec * (warp + 1) / MV_WARPS);
-    if (VEC == 4) {
-        v0 &= ~31;
-        v1 = warp + 1 == MV_WARPS ? nvec : (v1 & ~31);
-    }
+    constexpr int VEC = sizeof(TZ) == 4 ? 2 : 1;   // complex entries per 16-byte load
+    const int nvec = (cols + VEC - 1) / VEC;
+    const int v0 = (int)((long long)nvec * warp / MV_WARPS), v1 = (int)((long long)nvec * (warp + 1) / MV_WARPS);
     if (RINV) {
 #pragma unroll
         for (int i = 0; i < MV_ROWS; ++i)
@@ -127,17 +128,14 @@ k_matvec(const TZ *__restrict__ A, size_t ld, int rows, int cols, const TX *x, T
                 z[i] = {};
         }
     };
-    typename V2<TZ>::t zc[MV_ROWS], zn[MV_ROWS];   // 16-bit entries: this column step and the next
-    if (VEC == 4 && rb < re && v0 + lane < v1) zload(rb, v0 + lane, zc);
     int buf = 0;
     for (int r0 = rb; r0 < re; r0 += MV_ROWS, buf ^= 1) {
-        if (VEC != 4) {   // the first lines of the next rows on the way to L2 during this row group
+        // the first lines of the next rows on the way to L2 during this row group
 #pragma unroll
-            for (int i = 0; i < MV_ROWS; ++i)
-                for (int v = v0 + lane; v < v1 && v < v0 + 8 * 32; v += 32)
-                    if (r0 + MV_ROWS + i < re && (lane & 7) == 0)
-                        prefetch_l2(A + 2 * ((size_t)(r0 + MV_ROWS + i) * ld + (size_t)v * VEC));
-        }
+        for (int i = 0; i < MV_ROWS; ++i)
+            for (int v = v0 + lane; v < v1 && v < v0 + 8 * 32; v += 32)
+                if (r0 + MV_ROWS + i < re && (lane & 7) == 0)
+                    prefetch_l2(A + 2 * ((size_t)(r0 + MV_ROWS + i) * ld + (size_t)v * VEC));
         TA acc[MV_ROWS][4];
 #pragma unroll
         for (int i = 0; i < MV_ROWS; ++i)
@@ -148,17 +146,11 @@ k_matvec(const TZ *__restrict__ A, size_t ld, int rows, int cols, const TX *x, T
 #pragma unroll
             for (int u = 0; u < VEC; ++u) {
                 TA xv[4] = {TA(0), TA(0), TA(0), TA(0)};
-                const int cu = VEC == 4 ? (v >> 5) * 128 + (v & 31) + 32 * u : c + u;   // the entry's column
-                if (cu < cols) load_x(x, cu, xv);
+                if (c + u < cols) load_x(x, c + u, xv);
 #pragma unroll
                 for (int i = 0; i < MV_ROWS; ++i) {
                     TA zr, zi;
-                    if constexpr (VEC == 4) {
-                        const uint32_t *wv = reinterpret_cast<const uint32_t *>(&z[i]);
-                        const float2 f = widen2<TZ>(wv[u]);
-                        zr = TA(f.x);
-                        zi = TA(f.y);
-                    } else if constexpr (VEC == 2) {
+                    if constexpr (VEC == 2) {
                         const float4 f = *reinterpret_cast<const float4 *>(&z[i]);
                         zr = TA(u == 0 ? f.x : f.z);
                         zi = TA(u == 0 ? f.y : f.w);
@@ -174,22 +166,11 @@ k_matvec(const TZ *__restrict__ A, size_t ld, int rows, int cols, const TX *x, T
                 }
             }
         };
-        if constexpr (VEC == 4) {   // 16-bit entries: the next column step's loads in flight during this one's products
-#pragma unroll 2
-            for (int v = v0 + lane; v < v1; v += 32) {
-                if (v + 32 < v1) zload(r0, v + 32, zn);
-                else if (r0 + MV_ROWS < re) zload(r0 + MV_ROWS, v0 + lane, zn);   // the next rows' first step
-                zuse(v, zc);
-#pragma unroll
-                for (int i = 0; i < MV_ROWS; ++i) zc[i] = zn[i];
-            }
-        } else {
 #pragma unroll 8
-            for (int v = v0 + lane; v < v1; v += 32) {
-                typename V2<TZ>::t z[MV_ROWS];
-                zload(r0, v, z);
-                zuse(v, z);
-            }
+        for (int v = v0 + lane; v < v1; v += 32) {
+            typename V2<TZ>::t z[MV_ROWS];
+            zload(r0, v, z);
+            zuse(v, z);
         }
         const TA sum = warp_sum16(acc, lane);
         if (!(lane & 1)) part[buf][warp][lane >> 1] = sum;
@@ -201,15 +182,7 @@ k_matvec(const TZ *__restrict__ A, size_t ld, int rows, int cols, const TX *x, T
                 TA s = TA(0);
 #pragma unroll
                 for (int w2 = 0; w2 < MV_WARPS; ++w2) s += part[buf][w2][threadIdx.x];
-                if constexpr (RINV) {   // (c0, c1) R: lanes 4i .. 4i + 3 hold re, im of the two columns
-                    const unsigned m = __activemask();
-                    const int l0 = threadIdx.x & ~3;
-                    const TA a = __shfl_sync(m, s, l0), b = __shfl_sync(m, s, l0 + 1);
-                    if (k == 0) s = rinv[0] * s;
-                    else if (k == 1) s = rinv[0] * s;
-                    else if (k == 2) s = rinv[3] * s + rinv[1] * a - rinv[2] * b;
-                    else s = rinv[3] * s + rinv[1] * b + rinv[2] * a;
-                }
+                if constexpr (RINV) s = times_r(s, k, rinv);
                 if (ACCUM) y[(size_t)r * 4 + k] += alpha * s;
                 else y[(size_t)r * 4 + k] = alpha * s;
             }
@@ -217,10 +190,122 @@ k_matvec(const TZ *__restrict__ A, size_t ld, int rows, int cols, const TX *x, T
     }
 }
 
+// ---------------------------------------------------------------------------
+// The same product with 16-bit entries in the column-interleaved layout (linalg.h):
+// rows of 128-column chunks, a warp's 32 lanes load one chunk of a row as 32 x 16
+// bytes, entry u of lane l being column 32 u + l.  x is padded with zeros to whole
+// chunks, rows past the end read the last row: the inner loop has no bounds checks
+// (they, and the address arithmetic, were 135 of its 315 instructions per 2 KB of
+// matrix; at 62% of the issue slots the product ran at 4.7 TB/s).
+// ---------------------------------------------------------------------------
+template <typename TZ, typename TV>
+__device__ __forceinline__ void chunk_load(const char *const (&row)[MV_ROWS], unsigned off, uint4 (&z)[MV_ROWS]) {
+#pragma unroll
+    for (int i = 0; i < MV_ROWS; ++i) z[i] = __ldcs(reinterpret_cast<const uint4 *>(row[i] + off));
+}
+// x: the chunk's first column plus the lane
+template <typename TZ, typename TV>
+__device__ __forceinline__ void chunk_use(const uint4 (&z)[MV_ROWS], const TV *x, TV (&acc)[MV_ROWS][4]) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        TV xv[4];
+        load_x(x, 32 * u, xv);
+#pragma unroll
+        for (int i = 0; i < MV_ROWS; ++i) {
+            const uint32_t w = u == 0 ? z[i].x : (u == 1 ? z[i].y : (u == 2 ? z[i].z : z[i].w));
+            const float2 f = widen2<TZ>(w);
+            const TV zr = TV(f.x), zi = TV(f.y);
+            acc[i][0] = fma(zr, xv[0], fma(-zi, xv[1], acc[i][0]));
+            acc[i][1] = fma(zr, xv[1], fma(zi, xv[0], acc[i][1]));
+            acc[i][2] = fma(zr, xv[2], fma(-zi, xv[3], acc[i][2]));
+            acc[i][3] = fma(zr, xv[3], fma(zi, xv[2], acc[i][3]));
+        }
+    }
+}
+
+template <typename TZ, bool RINV>
+__global__ void __launch_bounds__(MV_WARPS * 32, 2)
+k_matvec16(const TZ *__restrict__ A, size_t ld, int rows, const float *x, float *y, float alpha, const float *rinv) {
+    __shared__ float part[2][MV_WARPS][MV_ROWS * 4];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rb = (int)((long long)rows * blockIdx.x / gridDim.x);
+    const int re = (int)((long long)rows * (blockIdx.x + 1) / gridDim.x);
+    const int chunks = (int)(ld / 128);
+    const int c0 = (int)((long long)chunks * warp / MV_WARPS), c1 = (int)((long long)chunks * (warp + 1) / MV_WARPS);
+    const char *row[MV_ROWS];
+    auto rows_at = [&](int r0) {
+#pragma unroll
+        for (int i = 0; i < MV_ROWS; ++i) row[i] = reinterpret_cast<const char *>(A + 2 * (size_t)min(r0 + i, rows - 1) * ld);
+    };
+    rows_at(rb);
+    const unsigned o0 = (unsigned)c0 * 512u + (unsigned)lane * 16u;
+    if (RINV) {
+#pragma unroll
+        for (int i = 0; i < MV_ROWS; ++i)
+            for (int c = c0; c < c1 && c < c0 + 4; ++c)
+                if ((lane & 7) == 0) prefetch_l2(row[i] + (o0 + 512u * (c - c0)));
+        cudaTriggerProgrammaticLaunchCompletion();
+        cudaGridDependencySynchronize();
+    }
+    uint4 zc[MV_ROWS], zn[MV_ROWS];
+    if (c0 < c1 && rb < re) chunk_load<TZ, float>(row, o0, zc);
+    int buf = 0;
+    for (int r0 = rb; r0 < re; r0 += MV_ROWS, buf ^= 1) {
+        float acc[MV_ROWS][4];
+#pragma unroll
+        for (int i = 0; i < MV_ROWS; ++i)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) acc[i][k] = 0.f;
+        const float *xp = x + 4 * (size_t)(128 * c0 + lane);
+        unsigned off = o0;
+#pragma unroll 2
+        for (int c = c0; c < c1; ++c, xp += 512) {   // the next step's loads in flight, across row groups too
+            if (c + 1 < c1) off += 512u;
+            else { off = o0; rows_at(min(r0 + MV_ROWS, re - 1)); }
+            chunk_load<TZ, float>(row, off, zn);
+            chunk_use<TZ, float>(zc, xp, acc);
+#pragma unroll
+            for (int i = 0; i < MV_ROWS; ++i) zc[i] = zn[i];
+        }
+        const float sum = warp_sum16(acc, lane);
+        if (!(lane & 1)) part[buf][warp][lane >> 1] = sum;
+        __syncthreads();
+        if (threadIdx.x < MV_ROWS * 4) {
+            const int k = threadIdx.x % 4, r = r0 + threadIdx.x / 4;
+            float s = 0.f;
+#pragma unroll
+            for (int w2 = 0; w2 < MV_WARPS; ++w2) s += part[buf][w2][threadIdx.x];
+            if constexpr (RINV) s = times_r(s, k, rinv);
+            if (r < re) y[(size_t)r * 4 + k] = alpha * s;
+        }
+    }
+}
+
+template <typename TZ, bool RINV>
+cudaError_t launch_matvec16(const TZ *A, size_t ld, int rows, const float *x, float *y, float alpha, const float *rinv,
+                            cudaStream_t st, int grid_mult) {
+    if (rows <= 0) return cudaSuccess;
+    static int slots = 0;   // resident CTAs of the GPU (per instantiation; one device per process)
+    if (slots == 0) {
+        int dev = 0, sms = 0, per = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_matvec16<TZ, RINV>, MV_WARPS * 32, 0);
+        if (e != cudaSuccess) return e;
+        slots = std::max(1, sms * per);
+    }
+    const int grid = std::max(1, std::min(slots * std::max(1, grid_mult), (rows + MV_ROWS - 1) / MV_ROWS));
+    if constexpr (RINV) return launch_pdl(k_matvec16<TZ, true>, grid, MV_WARPS * 32, st, A, ld, rows, x, y, alpha, rinv);
+    k_matvec16<TZ, false><<<grid, MV_WARPS * 32, 0, st>>>(A, ld, rows, x, y, alpha, nullptr); ++g_launches;
+    return cudaGetLastError();
+}
+
 template <typename TZ>
 cudaError_t matvec_rinv(const TZ *A, size_t ld, int rows, int cols, const float *x, float *y, float alpha,
                         const float *rinv, cudaStream_t st, int grid_mult) {
     if (rows <= 0) return cudaSuccess;
+    if constexpr (sizeof(TZ) == 2) return launch_matvec16<TZ, true>(A, ld, rows, x, y, alpha, rinv, st, grid_mult);
+    else {
     static int slots = 0;   // resident CTAs of the GPU (per instantiation; one device per process)
     if (slots == 0) {
         int dev = 0, sms = 0, per = 0;
@@ -233,6 +318,7 @@ cudaError_t matvec_rinv(const TZ *A, size_t ld, int rows, int cols, const float 
     }
     const int grid = std::max(1, std::min(slots * std::max(1, grid_mult), (rows + MV_ROWS - 1) / MV_ROWS));
     return launch_pdl(k_matvec<TZ, float, float, false, true>, grid, MV_WARPS * 32, st, A, ld, rows, cols, x, y, alpha, rinv);
+    }
 }
 template cudaError_t matvec_rinv<float>(const float *, size_t, int, int, const float *, float *, float, const float *, cudaStream_t, int);
 template cudaError_t matvec_rinv<__half>(const __half *, size_t, int, int, const float *, float *, float, const float *, cudaStream_t, int);
@@ -264,9 +350,13 @@ cudaError_t matvec(const TZ *A, size_t ld, int rows, int cols, const TX *x, TA *
 }
 
 template cudaError_t matvec<float, float, float>(const float *, size_t, int, int, const float *, float *, float, bool, cudaStream_t, int);
-template cudaError_t matvec<__half, float, float>(const __half *, size_t, int, int, const float *, float *, float, bool, cudaStream_t, int);
-template cudaError_t matvec<__nv_bfloat16, float, float>(const __nv_bfloat16 *, size_t, int, int, const float *, float *,
-                                                         float, bool, cudaStream_t, int);
+cudaError_t matvec16(const __half *A, size_t ld, int rows, const float *x, float *y, float alpha, cudaStream_t st, int grid_mult) {
+    return launch_matvec16<__half, false>(A, ld, rows, x, y, alpha, nullptr, st, grid_mult);
+}
+cudaError_t matvec16(const __nv_bfloat16 *A, size_t ld, int rows, const float *x, float *y, float alpha, cudaStream_t st,
+                     int grid_mult) {
+    return launch_matvec16<__nv_bfloat16, false>(A, ld, rows, x, y, alpha, nullptr, st, grid_mult);
+}
 
 // largest |Re|, |Im| of a block, as the bit pattern of a non-negative float
 // (for those the integer order is the float order, so atomicMax applies)
@@ -309,92 +399,71 @@ __global__ void k_to16_il(const float *__restrict__ A, size_t lda, int rows, int
 // whatever the blocks' sizes; inside a row group as k_matvec (the warps split the
 // columns, the next column step's loads in flight).
 // ---------------------------------------------------------------------------
+constexpr int PJ_INLINE = 8;   // jobs of one launch that travel as kernel parameters
+struct PrecondJobs {
+    PrecondJob j[PJ_INLINE];
+};
 template <typename TV>
-__global__ void __launch_bounds__(MV_WARPS * 32, sizeof(TV) == 4 ? 3 : 2)
-k_precond(const __half *__restrict__ M, const PrecondJob *__restrict__ jobs, int njobs, long long total,
-          const TV *in, TV *out, TV *y, TV *z) {
+__global__ void __launch_bounds__(MV_WARPS * 32, 2)
+k_precond(const __half *__restrict__ M, const __grid_constant__ PrecondJobs inl, const PrecondJob *__restrict__ jobs,
+          int njobs, long long total, const TV *in, TV *out, TV *y, TV *z) {
     __shared__ TV part[2][MV_WARPS][MV_ROWS * 4];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long lo = total * blockIdx.x / gridDim.x, hi = total * (blockIdx.x + 1) / gridDim.x;
     int buf = 0;
     bool waited = false;   // for the launch before, which writes the vectors
     for (int q = 0; q < njobs; ++q) {
-        const PrecondJob jb = jobs[q];
-        const int chunks = (jb.c1 - jb.c0 + 127) / 128, groups = (jb.rows + MV_ROWS - 1) / MV_ROWS;
+        const PrecondJob &jb = jobs ? jobs[q] : inl.j[q];
+        const int chunks = (jb.c1 - jb.c0 + 127) / 128, rows = jb.rows, groups = (rows + MV_ROWS - 1) / MV_ROWS;
         const long long a = lo - jb.pre, b = hi - jb.pre;
         if (b <= 0) break;
         const int g0 = a <= 0 ? 0 : (int)min((long long)groups, (a + chunks - 1) / chunks);
         const int g1 = (int)min((long long)groups, (b + chunks - 1) / chunks);
         if (g0 >= g1) continue;
-        const TV *vec[3] = {in + 4 * (size_t)jb.voff, y + 4 * (size_t)jb.voff, z + 4 * (size_t)jb.voff};
-        const TV *xa = jb.x1 == 0 ? vec[0] : vec[1], *xb = jb.x2 == 1 ? vec[1] : vec[2];
-        const int v0 = (int)((long long)chunks * warp / MV_WARPS) * 32, v1 = (int)((long long)chunks * (warp + 1) / MV_WARPS) * 32;
+        const TV *xa = (jb.x1 == 0 ? in : y) + 4 * (size_t)(jb.voff + jb.c0 + lane);
+        const TV *xb = (jb.x2 == 1 ? y : z) + 4 * (size_t)(jb.voff + jb.c0 + lane);
+        const int cs = (jb.split - jb.c0 + 127) / 128;   // chunks below it take xa (split is a chunk boundary or the end)
+        const int c0 = (int)((long long)chunks * warp / MV_WARPS), c1 = (int)((long long)chunks * (warp + 1) / MV_WARPS);
+        const unsigned o0 = (unsigned)c0 * 512u + (unsigned)lane * 16u;
+        const char *row[MV_ROWS];
+        auto rows_at = [&](int g) {
+#pragma unroll
+            for (int i = 0; i < MV_ROWS; ++i)
+                row[i] = reinterpret_cast<const char *>(M + 2 * (jb.m + (size_t)min(MV_ROWS * g + i, rows - 1) * jb.ld16));
+        };
+        rows_at(g0);
         if (!waited) {   // the factor is constant: its first rows on the way to L2 meanwhile
-            for (int i = 0; i < 2 * MV_ROWS; ++i)
-                for (int v = v0 + lane; v < v1 && v < v0 + 4 * 32; v += 32)
-                    if (MV_ROWS * g0 + i < jb.rows && (lane & 7) == 0)
-                        prefetch_l2(reinterpret_cast<const uint4 *>(M + 2 * (jb.m + (size_t)(MV_ROWS * g0 + i) * jb.ld16)) + v);
+#pragma unroll
+            for (int i = 0; i < MV_ROWS; ++i)
+                for (int c = c0; c < c1 && c < c0 + 4; ++c)
+                    if ((lane & 7) == 0) prefetch_l2(row[i] + (o0 + 512u * (c - c0)));
             cudaTriggerProgrammaticLaunchCompletion();
             cudaGridDependencySynchronize();
             waited = true;
         }
-        auto zload = [&](int r0, int v, uint4 *w) {
-            const __half *A = M + 2 * (jb.m + (size_t)r0 * jb.ld16);
-#pragma unroll
-            for (int i = 0; i < MV_ROWS; ++i)
-                w[i] = r0 + i < jb.rows ? __ldcs(reinterpret_cast<const uint4 *>(A + 2 * (size_t)i * jb.ld16) + v)
-                                        : make_uint4(0u, 0u, 0u, 0u);
-        };
         uint4 zc[MV_ROWS], zn[MV_ROWS];
-        if (v0 + lane < v1) zload(MV_ROWS * g0, v0 + lane, zc);
+        if (c0 < c1) chunk_load<__half, TV>(row, o0, zc);
         for (int g = g0; g < g1; ++g, buf ^= 1) {
-            const int r0 = MV_ROWS * g;
             TV acc[MV_ROWS][4];
 #pragma unroll
             for (int i = 0; i < MV_ROWS; ++i)
 #pragma unroll
                 for (int k = 0; k < 4; ++k) acc[i][k] = TV(0);
-            auto zuse = [&](int v, const uint4 *w) {
-                const int base = jb.c0 + (v >> 5) * 128;
-                const TV *x = base < jb.split ? xa : xb;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    TV xv[4] = {TV(0), TV(0), TV(0), TV(0)};
-                    const int cu = base + (v & 31) + 32 * u;   // the entry's column
-                    if (cu < jb.c1) {   // x may be written by this launch on other rows: no read-only path
-                        if constexpr (sizeof(TV) == 4) {
-                            const float4 f = *reinterpret_cast<const float4 *>(x + 4 * (size_t)cu);
-                            xv[0] = f.x; xv[1] = f.y; xv[2] = f.z; xv[3] = f.w;
-                        } else {
-                            const double2 f = *reinterpret_cast<const double2 *>(x + 4 * (size_t)cu);
-                            const double2 h = *reinterpret_cast<const double2 *>(x + 4 * (size_t)cu + 2);
-                            xv[0] = f.x; xv[1] = f.y; xv[2] = h.x; xv[3] = h.y;
-                        }
-                    }
-#pragma unroll
-                    for (int i = 0; i < MV_ROWS; ++i) {
-                        const uint32_t *wv = reinterpret_cast<const uint32_t *>(&w[i]);
-                        const float2 f = widen2<__half>(wv[u]);
-                        const TV zr = TV(f.x), zi = TV(f.y);
-                        acc[i][0] = fma(zr, xv[0], fma(-zi, xv[1], acc[i][0]));
-                        acc[i][1] = fma(zr, xv[1], fma(zi, xv[0], acc[i][1]));
-                        acc[i][2] = fma(zr, xv[2], fma(-zi, xv[3], acc[i][2]));
-                        acc[i][3] = fma(zr, xv[3], fma(zi, xv[2], acc[i][3]));
-                    }
-                }
-            };
+            unsigned off = o0;
 #pragma unroll 2
-            for (int v = v0 + lane; v < v1; v += 32) {
-                if (v + 32 < v1) zload(r0, v + 32, zn);
-                zuse(v, zc);
+            for (int c = c0; c < c1; ++c) {   // the next step's loads in flight, across row groups too
+                if (c + 1 < c1) off += 512u;
+                else { off = o0; rows_at(min(g + 1, g1 - 1)); }
+                chunk_load<__half, TV>(row, off, zn);
+                chunk_use<__half, TV>(zc, (c < cs ? xa : xb) + 512 * (size_t)c, acc);
 #pragma unroll
                 for (int i = 0; i < MV_ROWS; ++i) zc[i] = zn[i];
             }
-            if (g + 1 < g1 && v0 + lane < v1) zload(MV_ROWS * (g + 1), v0 + lane, zc);   // in flight during the sums
             const TV sum = warp_sum16(acc, lane);
             if (!(lane & 1)) part[buf][warp][lane >> 1] = sum;
             __syncthreads();
-            if (threadIdx.x < MV_ROWS * 4 && r0 + (int)threadIdx.x / 4 < jb.rows) {
+            const int r0 = MV_ROWS * g;
+            if (threadIdx.x < MV_ROWS * 4 && r0 + (int)threadIdx.x / 4 < rows) {
                 TV s = TV(0);
 #pragma unroll
                 for (int w2 = 0; w2 < MV_WARPS; ++w2) s += part[buf][w2][threadIdx.x];
@@ -411,9 +480,12 @@ k_precond(const __half *__restrict__ M, const PrecondJob *__restrict__ jobs, int
 }
 
 template <typename TV>
-cudaError_t precond_step(const __half *M, const PrecondJob *jobs, int njobs, long long total, const TV *in, TV *out,
-                         TV *y, TV *z, cudaStream_t st) {
+cudaError_t precond_step(const __half *M, const PrecondJob *host_jobs, const PrecondJob *jobs, int njobs, long long total,
+                         const TV *in, TV *out, TV *y, TV *z, cudaStream_t st) {
     if (njobs <= 0) return cudaSuccess;
+    PrecondJobs inl{};
+    if (njobs <= PJ_INLINE)
+        for (int q = 0; q < njobs; ++q) inl.j[q] = host_jobs[q];
     static int slots = 0;   // resident CTAs of the GPU (per instantiation; one device per process)
     if (slots == 0) {
         int dev = 0, sms = 0, per = 0;
@@ -423,12 +495,12 @@ cudaError_t precond_step(const __half *M, const PrecondJob *jobs, int njobs, lon
         if (e != cudaSuccess) return e;
         slots = std::max(1, sms * per);
     }
-    return launch_pdl(k_precond<TV>, (int)std::max(1ll, std::min((long long)slots, total)), MV_WARPS * 32, st, M, jobs, njobs,
-                      total, in, out, y, z);
+    return launch_pdl(k_precond<TV>, (int)std::max(1ll, std::min((long long)slots, total)), MV_WARPS * 32, st, M, inl,
+                      njobs <= PJ_INLINE ? (const PrecondJob *)nullptr : jobs, njobs, total, in, out, y, z);
 }
-template cudaError_t precond_step<float>(const __half *, const PrecondJob *, int, long long, const float *, float *, float *,
+template cudaError_t precond_step<float>(const __half *, const PrecondJob *, const PrecondJob *, int, long long, const float *, float *, float *,
                                          float *, cudaStream_t);
-template cudaError_t precond_step<double>(const __half *, const PrecondJob *, int, long long, const double *, double *,
+template cudaError_t precond_step<double>(const __half *, const PrecondJob *, const PrecondJob *, int, long long, const double *, double *,
                                           double *, double *, cudaStream_t);
 
 __global__ void k_absmax_groups(const float *__restrict__ A, size_t ld, int n, int group, unsigned *out) {
@@ -1226,10 +1298,6 @@ template cudaError_t copy_block<double, double>(const double *, size_t, int, int
 // of one basis vector with 16-byte loads, reduces in FP64 and adds 4 numbers.
 constexpr int DOT_CHUNK = 2048;
 
-__device__ __forceinline__ void load4(const float *p, double o[4]) {
-    const float4 v = *reinterpret_cast<const float4 *>(p);
-    o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
-}
 __device__ __forceinline__ void load4(const double *p, double o[4]) {
     const double2 a = *reinterpret_cast<const double2 *>(p), b = *reinterpret_cast<const double2 *>(p + 2);
     o[0] = a.x; o[1] = a.y; o[2] = b.x; o[3] = b.y;
@@ -1237,9 +1305,7 @@ __device__ __forceinline__ void load4(const double *p, double o[4]) {
 
 template <typename TV>
 __global__ void __launch_bounds__(256) k_dots(const TV *V, size_t vstride, int nv, const TV *w, int n, double *h) {
-    // FP32 vectors: FP32 products summed over a thread's 8 rows, FP64 from the
-    // warp reduction on (the FP64 pipe is narrow); FP64 vectors: FP64 throughout
-    using A = typename std::conditional<sizeof(TV) == 4, float, double>::type;
+    using A = TV;
     __shared__ double red[8][4];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int j = blockIdx.y;
@@ -1251,17 +1317,8 @@ __global__ void __launch_bounds__(256) k_dots(const TV *V, size_t vstride, int n
         const int i = base + u * 256 + threadIdx.x;
         if (i < n) {
             A x[4], y[4];
-            if constexpr (sizeof(TV) == 4) {
-                const float4 p = *reinterpret_cast<const float4 *>(v + 4 * (size_t)i);
-                const float4 q = *reinterpret_cast<const float4 *>(w + 4 * (size_t)i);
-                x[0] = p.x; x[1] = p.y; x[2] = p.z; x[3] = p.w;
-                y[0] = q.x; y[1] = q.y; y[2] = q.z; y[3] = q.w;
-            } else {
-                double xd[4], yd[4];
-                load4(v + 4 * (size_t)i, xd);
-                load4(w + 4 * (size_t)i, yd);
-                for (int c = 0; c < 4; ++c) { x[c] = xd[c]; y[c] = yd[c]; }
-            }
+            load4(v + 4 * (size_t)i, x);
+            load4(w + 4 * (size_t)i, y);
             a0 += x[0] * y[0] + x[1] * y[1];
             a1 += x[0] * y[1] - x[1] * y[0];
             a2 += x[2] * y[2] + x[3] * y[3];
@@ -1285,43 +1342,6 @@ __global__ void __launch_bounds__(256) k_dots(const TV *V, size_t vstride, int n
 }
 
 // w[i][r] -= sum_j V_j[i][r] h[j][r]   (h on the device, FP64)
-// FP32 vectors: a CTA owns 32 rows (one per lane) and its 8 warps split the
-// basis vectors; 16-byte loads, FP32 products and sums, the 8 partial sums
-// combined through shared memory.  FP64 vectors: one thread per row.
-__global__ void __launch_bounds__(256) k_subtract_f32(const float *V, size_t vstride, int nv, const double *h,
-                                                      float *w, int n) {
-    __shared__ float4 part[8][32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int i = blockIdx.x * 32 + lane;
-    float s0r = 0.f, s0i = 0.f, s1r = 0.f, s1i = 0.f;
-    if (i < n) {
-#pragma unroll 2
-        for (int j = warp; j < nv; j += 8) {
-            const float4 v = *reinterpret_cast<const float4 *>(V + (size_t)j * vstride + 4 * (size_t)i);
-            const double2 ha = __ldg(reinterpret_cast<const double2 *>(h + 4 * j));
-            const double2 hb = __ldg(reinterpret_cast<const double2 *>(h + 4 * j + 2));
-            const float h0 = (float)ha.x, h1 = (float)ha.y, h2 = (float)hb.x, h3 = (float)hb.y;
-            s0r = fmaf(v.x, h0, fmaf(-v.y, h1, s0r));
-            s0i = fmaf(v.x, h1, fmaf(v.y, h0, s0i));
-            s1r = fmaf(v.z, h2, fmaf(-v.w, h3, s1r));
-            s1i = fmaf(v.z, h3, fmaf(v.w, h2, s1i));
-        }
-    }
-    part[warp][lane] = make_float4(s0r, s0i, s1r, s1i);
-    __syncthreads();
-    if (warp == 0 && i < n) {
-        float4 t = part[0][lane];
-        for (int q = 1; q < 8; ++q) {
-            const float4 u = part[q][lane];
-            t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
-        }
-        float4 *o = reinterpret_cast<float4 *>(w + 4 * (size_t)i);
-        float4 c = *o;
-        c.x -= t.x; c.y -= t.y; c.z -= t.z; c.w -= t.w;
-        *o = c;
-    }
-}
-
 template <typename TV>
 __global__ void k_subtract(const TV *V, size_t vstride, int nv, const double *h, TV *w, int n) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1383,12 +1403,7 @@ cudaError_t dots(const TV *V, size_t vstride, int nv, const TV *w, int n, double
 }
 template <typename TV>
 cudaError_t subtract(const TV *V, size_t vstride, int nv, const double *h, TV *w, int n, cudaStream_t st) {
-    if constexpr (sizeof(TV) == 4) {
-        k_subtract_f32<<<(n + 31) / 32, 256, 0, st>>>(V, vstride, nv, h, w, n);
-    } else {
-        k_subtract<TV><<<(n + 255) / 256, 256, 0, st>>>(V, vstride, nv, h, w, n);
-    }
-    ++g_launches;
+    k_subtract<TV><<<(n + 255) / 256, 256, 0, st>>>(V, vstride, nv, h, w, n); ++g_launches;
     return cudaGetLastError();
 }
 template <typename TX, typename TY>
@@ -1401,14 +1416,10 @@ cudaError_t combine(const TV *V, size_t vstride, int nv, const double *y, double
     k_combine<TV><<<(n + 255) / 256, 256, 0, st>>>(V, vstride, nv, y, x, n); ++g_launches;
     return cudaGetLastError();
 }
-template cudaError_t dots<float>(const float *, size_t, int, const float *, int, double *, cudaStream_t);
 template cudaError_t dots<double>(const double *, size_t, int, const double *, int, double *, cudaStream_t);
-template cudaError_t subtract<float>(const float *, size_t, int, const double *, float *, int, cudaStream_t);
 template cudaError_t subtract<double>(const double *, size_t, int, const double *, double *, int, cudaStream_t);
 template cudaError_t scale<double, float>(const double *, float *, int, const double *, cudaStream_t);
-template cudaError_t scale<float, float>(const float *, float *, int, const double *, cudaStream_t);
 template cudaError_t scale<double, double>(const double *, double *, int, const double *, cudaStream_t);
-template cudaError_t combine<float>(const float *, size_t, int, const double *, double *, int, cudaStream_t);
 template cudaError_t combine<double>(const double *, size_t, int, const double *, double *, int, cudaStream_t);
 
 }  // namespace vie

@@ -40,7 +40,13 @@ cudaError_t launch_pdl(void (*kernel)(KA...), dim3 grid, int block, cudaStream_t
     ++g_launches;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KA>(args)...);
 }
-// y <- alpha (A x) R, FP32 vectors, R the 2 x 2 upper triangular rinv (device: r11,
+// y <- alpha A x for 16-bit A (column-interleaved rows of ld entries), FP32 vectors of
+// two right-hand sides, x zero up to pad_cols
+cudaError_t matvec16(const __half *A, size_t ld, int rows, const float *x, float *y, float alpha, cudaStream_t st,
+                     int grid_mult);
+cudaError_t matvec16(const __nv_bfloat16 *A, size_t ld, int rows, const float *x, float *y, float alpha, cudaStream_t st,
+                     int grid_mult);
+// y <- alpha (A x) R, FP32 vectors (16-bit A: x zero up to pad_cols), R the 2 x 2 upper triangular rinv (device: r11,
 // r12.re, r12.im, r22); launched with launch_pdl
 template <typename TZ>
 cudaError_t matvec_rinv(const TZ *A, size_t ld, int rows, int cols, const float *x, float *y, float alpha,
@@ -115,10 +121,14 @@ struct PrecondJob {
     double alpha, zscale;
 };
 inline long long precond_units(const PrecondJob &j) { return (long long)((j.rows + 3) / 4) * ((j.c1 - j.c0 + 127) / 128); }
-// the njobs jobs (device array) of one step in one launch; total: their work units
+// the njobs jobs of one step in one launch (on the host and as a device array: a few
+// travel as kernel parameters); total: their work units.  in, y, z are readable and
+// finite up to whole 128-column chunks of every block (pad_cols)
 template <typename TV>
-cudaError_t precond_step(const __half *M, const PrecondJob *jobs, int njobs, long long total, const TV *in, TV *out,
-                         TV *y, TV *z, cudaStream_t st);
+cudaError_t precond_step(const __half *M, const PrecondJob *host_jobs, const PrecondJob *jobs, int njobs, long long total,
+                         const TV *in, TV *out, TV *y, TV *z, cudaStream_t st);
+// columns of a vector that the 16-bit products read: whole 128-column chunks
+inline size_t pad_cols(int n) { return ((size_t)n + 127) / 128 * 128 + 128; }
 // out[0], out[1] (zeroed by the caller) <- the largest |Re|, |Im| of an n x n
 // block inside and outside its diagonal groups, as float bits
 cudaError_t absmax_groups(const float *A, size_t ld, int n, int group, unsigned *out, cudaStream_t st);

@@ -93,7 +93,7 @@ size_t mesh_footprint(const vie_mesh &m, const vie_options &opt) {
     if (opt.precision == VIE_FP16 || opt.precision == VIE_BF16) b += 2 * 2 * l16 * N;   // its 16-bit copy
     b += 8 * ld * N + 4 * l16 * N;                       // block inverses (FP32 and FP16), bounded by N^2
     b += 2 * vie::gj_pack_bytes((int)N);                 // packing scratch of the inversion (two blocks at once)
-    b += sz * 4 * N * (mres + 5) + 8 * 4 * N * 4;        // Krylov basis and vectors, x, r, b, coefficients
+    b += sz * 4 * (N + 256) * (mres + 5) + 8 * 4 * N * 4;        // Krylov basis and vectors, x, r, b, coefficients
     b += 2 * (nt * nt + nt * nf + nh * nt + nh * nf);    // near-image masks
     b += nt * 4096 + ((size_t)64 << 20);                 // per-element arrays, lists, tables, small buffers
     return b;
