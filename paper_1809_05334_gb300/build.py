@@ -21,7 +21,7 @@ CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "libvie.so")
 BUILD = os.path.join(HERE, "_build")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["api.cu", "fill.cu", "far.cu", "linalg.cu", "krylov.cu", "post.cu", "topology.cpp", "rules.cpp", "server.cpp",
+SOURCES = ["api.cu", "fill.cu", "far.cu", "linalg.cu", "krylov.cu", "mesh.cu", "post.cu", "topology.cpp", "rules.cpp", "server.cpp",
            "ewald_tables.cpp", "blocks.cpp"]
 
 

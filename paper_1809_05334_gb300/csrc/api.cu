@@ -17,12 +17,10 @@
 #include <cstdio>
 #include <cstring>
 #include <atomic>
-#include <map>
 #include <memory>
 #include <mutex>
 #include <thread>
 #include <new>
-#include <tuple>
 #include <type_traits>
 #include <string>
 #include <vector>
@@ -32,6 +30,7 @@
 #include "device_math.cuh"
 #include "fill.h"
 #include "linalg.h"
+#include "mesh.h"
 #include "post.h"
 #include "vie_internal.h"
 
@@ -105,7 +104,7 @@ struct MeshState {
     DevBuf tv, cen, vol, q5, far32, far64, fv, f5, farea, ffar32, ffar64, hf, n32, n64, fn32, fn64, fcen;
     DevBuf mk[4], pr[4], to[4], tdom, tpart;
     DevBuf thalf, tsc[4];   // static integrals of the touching near images (per mesh)
-    int npr[4] = {0, 0, 0, 0}, nto[4] = {0, 0, 0, 0};
+    int npr[4] = {0, 0, 0, 0}, nto[4] = {0, 0, 0, 0}, n_near_tt = 0;
 };
 
 struct vie_ctx {
@@ -1174,7 +1173,7 @@ int solve_impl(vie_ctx *ctx, const vie_request *req, vie_result *res, cudaStream
     res->t_solve_ms = ms(t2, t3);
     res->t_post_ms = ms(t3, t4);
     res->n_unknowns = ctx->mesh->topo.N;
-    res->n_near_pairs = (int32_t)ctx->mesh->topo.near_tt.size();
+    res->n_near_pairs = ctx->mesh->n_near_tt;
     res->h2d_bytes = ctx->h2d;
     res->d2h_bytes = ctx->d2h;
     res->far_pair_evals = 16 * (int64_t)ctx->mesh->topo.nt * ctx->mesh->topo.nt;
@@ -1468,7 +1467,7 @@ int vie_set_mesh(vie_ctx *ctx, const double *verts, int32_t n_verts, const int32
     ctx->tune_pivot = 0;
     ctx->tuned[0] = ctx->tuned[1] = false;
     std::string e = vie::build_topology(verts, n_verts, tets, n_tets, tet_domain, n_domains, period_a, period_b,
-                                        active_domain, ctx->mesh->topo);
+                                        active_domain, ctx->mesh->topo, false);
     if (!e.empty()) return fail(ctx, e.find("range") != std::string::npos ? VIE_EINVAL : VIE_BAD_MESH, e);
     const vie::Topology &T = ctx->mesh->topo;
     cudaStream_t st = 0;
@@ -1546,19 +1545,6 @@ int vie_set_mesh(vie_ctx *ctx, const double *verts, int32_t n_verts, const int32
     }
     std::vector<float> fn32(fn64.begin(), fn64.end());
     const int nh = (int)T.hf.size();
-    // dense near-image masks and the (pair, image) entry lists
-    auto masks = [](const std::vector<vie::NearPair> &L, size_t nx, size_t ny) {
-        std::vector<uint16_t> mk(std::max<size_t>(nx * ny, 1), 0);
-        for (auto &p : L) mk[(size_t)p.x * ny + p.y] = p.mask;
-        return mk;
-    };
-    auto entries = [](const std::vector<vie::NearPair> &L, bool touching) {
-        std::vector<vie::NearEntry> out;
-        for (auto &p : L)
-            for (int k = 0; k < 9; ++k)
-                if (((p.mask >> k) & 1u) && (((p.touch >> k) & 1u) != 0) == touching) out.push_back({p.x, p.y, k, 0});
-        return out;
-    };
     std::vector<int32_t> hf = T.hf;
     if (hf.empty()) hf.push_back(0);
     std::vector<double> fv = T.fv;
@@ -1581,29 +1567,61 @@ int vie_set_mesh(vie_ctx *ctx, const double *verts, int32_t n_verts, const int32
     CK(upload(ctx->mesh->fn32, fn32, st));
     CK(upload(ctx->mesh->fcen, fcen, st));
     CK(upload(ctx->mesh->tdom, T.dom, st));
-    const std::vector<vie::NearPair> *lists[4] = {&T.near_tt, &T.near_tf, &T.near_ft, &T.near_ff};
-    const size_t dims[4][2] = {{(size_t)T.nt, (size_t)T.nt}, {(size_t)T.nt, (size_t)nf}, {(size_t)nh, (size_t)T.nt},
-                               {(size_t)nh, (size_t)nf}};
-    for (int i = 0; i < 4; ++i) {
-        CK(upload(ctx->mesh->mk[i], masks(*lists[i], dims[i][0], dims[i][1]), st));
-        auto p = entries(*lists[i], false), q = entries(*lists[i], true);
-        ctx->mesh->npr[i] = (int)p.size();
-        ctx->mesh->nto[i] = (int)q.size();
-        if (p.empty()) p.push_back({0, 0, 0, 0});
-        if (q.empty()) q.push_back({0, 0, 0, 0});
-        CK(upload(ctx->mesh->pr[i], p, st));
-        CK(upload(ctx->mesh->to[i], q, st));
-        if (i == 0) {   // partner (y, x, 8-k) of every touching tetrahedron entry
-            std::map<std::tuple<int, int, int>, int> idx;
-            for (int e = 0; e < ctx->mesh->nto[0]; ++e) idx[std::make_tuple(q[e].x, q[e].y, q[e].k)] = e;
-            std::vector<int32_t> part(std::max(ctx->mesh->nto[0], 1), 0);
-            for (int e = 0; e < ctx->mesh->nto[0]; ++e) {
-                auto it = idx.find(std::make_tuple(q[e].y, q[e].x, 8 - q[e].k));
-                if (it == idx.end()) return fail(ctx, VIE_BAD_MESH, "near-pair lists are not symmetric");
-                part[e] = it->second;
-            }
-            CK(upload(ctx->mesh->tpart, part, st));
+    // near-image masks and the (pair, image) entry lists, on the device
+    {
+        double reach = 0;
+        for (int v = 0; v < 3 * n_verts; ++v) reach = std::max(reach, std::fabs(verts[v]));
+        std::vector<double> hcen(3 * (size_t)std::max(nh, 1)), hrad(std::max(nh, 1)), hv(9 * (size_t)std::max(nh, 1));
+        for (int h = 0; h < nh; ++h) {
+            const int f = T.hf[h];
+            std::copy_n(&T.fcen[3 * (size_t)f], 3, &hcen[3 * (size_t)h]);
+            std::copy_n(&T.fv[9 * (size_t)f], 9, &hv[9 * (size_t)h]);
+            hrad[h] = T.frad[f];
         }
+        DevBuf rad, frad, dhcen, dhrad, dhv, work, bad;
+        std::vector<double> fr = T.frad;
+        if (fr.empty()) fr.assign(1, 0.0);
+        CK(upload(rad, T.rad, st));
+        CK(upload(frad, fr, st));
+        CK(upload(dhcen, hcen, st));
+        CK(upload(dhrad, hrad, st));
+        CK(upload(dhv, hv, st));
+        CK(bad.ensure(sizeof(int)));
+        CK(cudaMemsetAsync(bad.p, 0, sizeof(int), st));
+        const vie::ElementSet tet{ctx->mesh->cen.as<double>(), rad.as<double>(), ctx->mesh->tv.as<double>(), T.nt, 4};
+        const vie::ElementSet face{ctx->mesh->fcen.as<double>(), frad.as<double>(), ctx->mesh->fv.as<double>(), nf, 3};
+        const vie::ElementSet half{dhcen.as<double>(), dhrad.as<double>(), dhv.as<double>(), nh, 3};
+        const vie::ElementSet sx[4] = {tet, tet, half, half}, sy[4] = {tet, face, tet, face};
+        const size_t wmax = vie::near_work_words(std::max(T.nt, nh));
+        CK(work.ensure(sizeof(unsigned) * 4 * wmax));
+        unsigned totals[4][3] = {};
+        for (int i = 0; i < 4; ++i) {
+            const vie::ElementSet &x = sx[i], &y = sy[i];
+            CK(ctx->mesh->mk[i].ensure(sizeof(uint16_t) * std::max<size_t>((size_t)x.n * y.n, 1)));
+            if (!x.n || !y.n) continue;
+            unsigned *w = work.as<unsigned>() + wmax * i;
+            CK(vie::near_count(x, y, T.a, T.b, reach, ctx->mesh->mk[i].as<uint16_t>(), w, st));
+            CK(cudaMemcpyAsync(totals[i], w + 6 * (size_t)x.n, sizeof(totals[i]), cudaMemcpyDeviceToHost, st));
+        }
+        CK(cudaStreamSynchronize(st));
+        ctx->mesh->n_near_tt = (int)totals[0][2];
+        for (int i = 0; i < 4; ++i) {
+            const vie::ElementSet &x = sx[i], &y = sy[i];
+            ctx->mesh->npr[i] = (int)totals[i][0];
+            ctx->mesh->nto[i] = (int)totals[i][1];
+            CK(ctx->mesh->pr[i].ensure(sizeof(vie::NearEntry) * std::max<size_t>(totals[i][0], 1)));
+            CK(ctx->mesh->to[i].ensure(sizeof(vie::NearEntry) * std::max<size_t>(totals[i][1], 1)));
+            if (!x.n || !y.n) continue;
+            CK(vie::near_emit(x, y, T.a, T.b, reach, ctx->mesh->mk[i].as<uint16_t>(), work.as<unsigned>() + wmax * i,
+                              ctx->mesh->pr[i].as<vie::NearEntry>(), ctx->mesh->to[i].as<vie::NearEntry>(), st));
+        }
+        CK(ctx->mesh->tpart.ensure(sizeof(int32_t) * std::max(ctx->mesh->nto[0], 1)));
+        CK(vie::near_partner(ctx->mesh->to[0].as<vie::NearEntry>(), ctx->mesh->nto[0], T.nt, work.as<unsigned>(),
+                             ctx->mesh->tpart.as<int32_t>(), bad.as<int>(), st));
+        int is_bad = 0;
+        CK(cudaMemcpyAsync(&is_bad, bad.p, sizeof(int), cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+        if (is_bad) return fail(ctx, VIE_BAD_MESH, "near-pair lists are not symmetric");
     }
     // static integrals of the touching near images: geometry only, once per mesh
     CK(ctx->mesh->thalf.ensure(sizeof(double) * 8 * std::max(ctx->mesh->nto[0], 1)));
@@ -1614,7 +1632,9 @@ int vie_set_mesh(vie_ctx *ctx, const double *verts, int32_t n_verts, const int32
     }
     {
         const vie::DevMesh dm = dev_mesh(ctx);
-        CK(vie::launch_static_cache(dm, ctx->mesh->thalf.as<double>(), tsc, st));
+        DevBuf geom;
+        CK(geom.ensure(vie::static_geom_bytes((size_t)T.nt, (size_t)nf)));
+        CK(vie::launch_static_cache(dm, ctx->mesh->thalf.as<double>(), tsc, geom.p, st));
         CK(cudaStreamSynchronize(st));
     }
     ctx->mesh->have_mesh = true;

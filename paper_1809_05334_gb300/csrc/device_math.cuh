@@ -379,174 +379,163 @@ __device__ __forceinline__ cx<float> green_tab(float dx, float dy, float dz, uns
 }
 
 // ---------------------------------------------------------------------------
-// Closed forms (divergence theorem, polygonal / polyhedral sources):
-//  triangle: int 1/R = sum_i t_i ln[(R+_i + s+_i)/(R-_i + s-_i)]
-//                      - |h| sum_i [atan(t s+/(R0^2+|h|R+)) - atan(t s-/(R0^2+|h|R-))]
+// Closed forms (divergence theorem, polygonal / polyhedral sources), observer at
+// the origin:
+//  triangle: int 1/R = sum_i t_i ln[(R+_i + s+_i)/(R-_i + s-_i)] - |h| Omega
 //            int R   = ( h^2 int 1/R + 1/2 sum_i t_i (s+R+ - s-R- + R0^2 ln(..)) ) / 3
 //  tetrahedron: int 1/R = 1/2 sum_f d_f int_f 1/R,  int (r'-r)/R = sum_f n_f int_f R
-template <typename T>
-__host__ __device__ __forceinline__ T log_rs(T R, T s, T R0sq) {
-    // ln(R + s) without cancellation for s < 0: R + s = R0^2 / (R - s)
-    return (s >= T(0)) ? log(R + s) : log(R0sq) - log(R - s);
+// t_i: signed in-plane distance to edge i, R0^2 = t^2 + h^2, Omega the solid angle
+// of the triangle, from its vertices (van Oosterom and Strackee, IEEE Trans.
+// Biomed. Eng. 30, 1983): tan(Omega/2) = |a.(b x c)| / (abc + (a.b)c + (a.c)b + (b.c)a).
+// What depends on the source alone (edge directions, normals) is a record built
+// once per element.
+struct TriGeom {
+    double lh[3][3], len[3];   // edge directions (vertex q to q + 1) and lengths
+    double n[3], a2;           // unit normal, twice the area
+    double u[3][3];            // in-plane outward normals of the edges
+    double tiny;
+};
+struct TetGeom {
+    double lh[6][3], len[6];   // edges (0,1) (0,2) (0,3) (1,2) (1,3) (2,3)
+    double n[4][3], a2[4];     // outward unit normal and twice the area of the face opposite each vertex
+    double u[4][3][3];         // in-plane outward normals of its edges
+    double tiny;
+};
+__host__ __device__ __forceinline__ double dot3(const double *a, const double *b) { return a[0] * b[0] + a[1] * b[1] + a[2] * b[2]; }
+__host__ __device__ __forceinline__ void cross3(const double *a, const double *b, double *c) {
+    c[0] = a[1] * b[2] - a[2] * b[1];
+    c[1] = a[2] * b[0] - a[0] * b[2];
+    c[2] = a[0] * b[1] - a[1] * b[0];
 }
-
-template <typename T>
-__host__ __device__ void tri_integrals(const T r[3], const T *v, T &inv, T &rint, bool want_r) {
-    T e1[3] = {v[3] - v[0], v[4] - v[1], v[5] - v[2]};
-    T e2[3] = {v[6] - v[0], v[7] - v[1], v[8] - v[2]};
-    T n[3] = {e1[1] * e2[2] - e1[2] * e2[1], e1[2] * e2[0] - e1[0] * e2[2], e1[0] * e2[1] - e1[1] * e2[0]};
-    T nn = sqrt(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
-    n[0] /= nn; n[1] /= nn; n[2] /= nn;
-    T h = n[0] * (r[0] - v[0]) + n[1] * (r[1] - v[1]) + n[2] * (r[2] - v[2]);
-    T ah = fabs(h);
-    T scale = fmax(sqrt(e1[0] * e1[0] + e1[1] * e1[1] + e1[2] * e1[2]),
-                   sqrt(e2[0] * e2[0] + e2[1] * e2[1] + e2[2] * e2[2]));
-    T tiny = (sizeof(T) == 8 ? T(1e-13) : T(1e-6)) * scale;
-    T slog = 0, satan = 0, sr = 0;
-    T Rv[3];
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        T d0 = r[0] - v[3 * j], d1 = r[1] - v[3 * j + 1], d2 = r[2] - v[3 * j + 2];
-        Rv[j] = sqrt(d0 * d0 + d1 * d1 + d2 * d2);
-    }
-#pragma unroll
-    for (int e = 0; e < 3; ++e) {
-        const int ja = e, jb = (e + 1) % 3;
-        const T *pa = v + 3 * ja, *pb = v + 3 * jb;
-        T L[3] = {pb[0] - pa[0], pb[1] - pa[1], pb[2] - pa[2]};
-        T ll = sqrt(L[0] * L[0] + L[1] * L[1] + L[2] * L[2]);
-        L[0] /= ll; L[1] /= ll; L[2] /= ll;
-        // in-plane outward normal u = l x n
-        T u[3] = {L[1] * n[2] - L[2] * n[1], L[2] * n[0] - L[0] * n[2], L[0] * n[1] - L[1] * n[0]};
-        T t = u[0] * (pa[0] - r[0]) + u[1] * (pa[1] - r[1]) + u[2] * (pa[2] - r[2]);
-        T sm = L[0] * (pa[0] - r[0]) + L[1] * (pa[1] - r[1]) + L[2] * (pa[2] - r[2]);
-        T sp = sm + ll;
-        T Rm = Rv[ja], Rp = Rv[jb];
-        T R0sq = t * t + h * h;
-        if (fabs(t) > tiny) {
-            T lr = log_rs(Rp, sp, R0sq) - log_rs(Rm, sm, R0sq);
-            slog += t * lr;
-            if (want_r) sr += t * (sp * Rp - sm * Rm + R0sq * lr);
-            if (ah > tiny) satan += atan2(t * sp, R0sq + ah * Rp) - atan2(t * sm, R0sq + ah * Rm);
-        }
-    }
-    inv = slog - ah * satan;
-    rint = want_r ? (h * h * inv + T(0.5) * sr) / T(3) : T(0);
-}
-
-template <typename T>
-__host__ __device__ void tet_integrals(const T r[3], const T *tv, T &inv, T vec[3], bool want_vec) {
-    inv = 0;
-    vec[0] = vec[1] = vec[2] = 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        T f[9];
-        int k = 0;
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (j != i) {
-                f[3 * k] = tv[3 * j]; f[3 * k + 1] = tv[3 * j + 1]; f[3 * k + 2] = tv[3 * j + 2];
-                ++k;
-            }
-        T e1[3] = {f[3] - f[0], f[4] - f[1], f[5] - f[2]};
-        T e2[3] = {f[6] - f[0], f[7] - f[1], f[8] - f[2]};
-        T n[3] = {e1[1] * e2[2] - e1[2] * e2[1], e1[2] * e2[0] - e1[0] * e2[2], e1[0] * e2[1] - e1[1] * e2[0]};
-        T nn = sqrt(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
-        T o = n[0] * (f[0] - tv[3 * i]) + n[1] * (f[1] - tv[3 * i + 1]) + n[2] * (f[2] - tv[3 * i + 2]);
-        T sg = (o >= T(0)) ? T(1) / nn : T(-1) / nn;   // outward unit normal
-        n[0] *= sg; n[1] *= sg; n[2] *= sg;
-        T d = n[0] * (f[0] - r[0]) + n[1] * (f[1] - r[1]) + n[2] * (f[2] - r[2]);
-        T fi, fr;
-        tri_integrals<T>(r, f, fi, fr, want_vec);
-        inv += T(0.5) * d * fi;
-        if (want_vec) {
-            vec[0] += n[0] * fr; vec[1] += n[1] * fr; vec[2] += n[2] * fr;
-        }
-    }
-}
-
-// The same tetrahedron closed forms with the per-edge quantities shared by the
-// two faces of each edge: 4 vertex distances, 6 edge logarithms
-// ln[(R_b + s_b)/(R_a + s_a)] (orientation independent) and one combined
-// arctangent per (face, edge): atan2(t s_b, R0^2+|h|R_b) - atan2(t s_a, R0^2+|h|R_a)
-// = atan2(y_b x_a - x_b y_a, x_a x_b + y_a y_b) (both angles lie in (-pi/2, pi/2)).
-// tv holds the vertices relative to the observer (the observer is the origin).
-__host__ __device__ inline void tet_integrals_shared(const double *tv, double &inv, double vec[3]) {
-    constexpr int EA[6] = {0, 0, 0, 1, 1, 2}, EB[6] = {1, 2, 3, 2, 3, 3};
-    // edges of face f (opposite vertex f) in the face's vertex order, and the face's third vertex per edge
+// edges of the face opposite vertex f and the face's third vertex per edge
+__host__ __device__ __forceinline__ constexpr int tet_fe(int f, int q) {
     constexpr int FE[4][3] = {{3, 5, 4}, {1, 5, 2}, {0, 4, 2}, {0, 3, 1}};
+    return FE[f][q];
+}
+__host__ __device__ __forceinline__ constexpr int tet_fc(int f, int q) {
     constexpr int FC[4][3] = {{3, 1, 2}, {3, 0, 2}, {3, 0, 1}, {2, 0, 1}};
-    double Rv[4];
-#pragma unroll
-    for (int v = 0; v < 4; ++v) Rv[v] = sqrt(tv[3 * v] * tv[3 * v] + tv[3 * v + 1] * tv[3 * v + 1] + tv[3 * v + 2] * tv[3 * v + 2]);
+    return FC[f][q];
+}
+__host__ __device__ __forceinline__ constexpr int tet_ea(int e) { return e < 3 ? 0 : (e < 5 ? 1 : 2); }
+__host__ __device__ __forceinline__ constexpr int tet_eb(int e) { return e < 3 ? e + 1 : (e < 5 ? e - 1 : 3); }
+
+__host__ __device__ inline void tri_geom(const double *v, TriGeom &g) {   // v: vertices [3][3]
+    double e1[3], e2[3];
+    for (int d = 0; d < 3; ++d) { e1[d] = v[3 + d] - v[d]; e2[d] = v[6 + d] - v[d]; }
+    cross3(e1, e2, g.n);
+    g.a2 = sqrt(dot3(g.n, g.n));
+    for (int d = 0; d < 3; ++d) g.n[d] /= g.a2;
     double scale = 0;
-    double L[6], lh[6][3], sa[6], sb[6], sR[6];
+    for (int q = 0; q < 3; ++q) {
+        const double *pa = v + 3 * q, *pb = v + 3 * ((q + 1) % 3);
+        double d[3] = {pb[0] - pa[0], pb[1] - pa[1], pb[2] - pa[2]};
+        g.len[q] = sqrt(dot3(d, d));
+        scale = fmax(scale, g.len[q]);
+        for (int k = 0; k < 3; ++k) g.lh[q][k] = d[k] / g.len[q];
+        cross3(g.lh[q], g.n, g.u[q]);
+    }
+    g.tiny = 1e-13 * scale;
+}
+__host__ __device__ inline void tet_geom(const double *v, TetGeom &g) {   // v: vertices [4][3]
+    double scale = 0;
+    for (int e = 0; e < 6; ++e) {
+        const double *pa = v + 3 * tet_ea(e), *pb = v + 3 * tet_eb(e);
+        double d[3] = {pb[0] - pa[0], pb[1] - pa[1], pb[2] - pa[2]};
+        g.len[e] = sqrt(dot3(d, d));
+        scale = fmax(scale, g.len[e]);
+        for (int k = 0; k < 3; ++k) g.lh[e][k] = d[k] / g.len[e];
+    }
+    g.tiny = 1e-13 * scale;
+    for (int f = 0; f < 4; ++f) {
+        const int fv[3] = {f == 0 ? 1 : 0, f <= 1 ? 2 : 1, f <= 2 ? 3 : 2};
+        const double *p0 = v + 3 * fv[0], *p1 = v + 3 * fv[1], *p2 = v + 3 * fv[2];
+        double e1[3], e2[3], o[3];
+        for (int d = 0; d < 3; ++d) { e1[d] = p1[d] - p0[d]; e2[d] = p2[d] - p0[d]; o[d] = p0[d] - v[3 * f + d]; }
+        cross3(e1, e2, g.n[f]);
+        g.a2[f] = sqrt(dot3(g.n[f], g.n[f]));
+        const double sg = dot3(g.n[f], o) >= 0 ? 1.0 / g.a2[f] : -1.0 / g.a2[f];
+        for (int d = 0; d < 3; ++d) g.n[f][d] *= sg;
+        for (int q = 0; q < 3; ++q) {   // outward: away from the face's third vertex
+            const int e = tet_fe(f, q);
+            cross3(g.lh[e], g.n[f], g.u[f][q]);
+            const double *pa = v + 3 * tet_ea(e), *pc = v + 3 * tet_fc(f, q);
+            const double w[3] = {pa[0] - pc[0], pa[1] - pc[1], pa[2] - pc[2]};
+            if (dot3(g.u[f][q], w) < 0)
+                for (int d = 0; d < 3; ++d) g.u[f][q][d] = -g.u[f][q][d];
+        }
+    }
+}
+// ln[(Rb + sb)/(Ra + sa)] along an edge, with R + s = d2/(R - s) for s < 0 (d2: squared
+// distance to the edge line)
+__host__ __device__ __forceinline__ double edge_log(const double *pa, const double *lh, double sa, double sb, double Ra,
+                                                    double Rb) {
+    if (sa >= 0) return log((Rb + sb) / (Ra + sa));
+    if (sb <= 0) return log((Ra - sa) / (Rb - sb));
+    double c[3];
+    cross3(pa, lh, c);
+    const double d2 = dot3(c, c);
+    return d2 > 0 ? log((Rb + sb) * (Ra - sa) / d2) : 0.0;
+}
+// int 1/R over a triangle; v: its vertices relative to the observer
+__host__ __device__ inline double tri_inv(const TriGeom &g, const double *v) {
+    const double R[3] = {sqrt(dot3(v, v)), sqrt(dot3(v + 3, v + 3)), sqrt(dot3(v + 6, v + 6))};
+    const double ah = fabs(dot3(g.n, v));
+    double slog = 0;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const double *pa = v + 3 * q;
+        const double t = dot3(g.u[q], pa);
+        if (fabs(t) <= g.tiny) continue;
+        const double sa = dot3(g.lh[q], pa);
+        slog += t * edge_log(pa, g.lh[q], sa, sa + g.len[q], R[q], R[(q + 1) % 3]);
+    }
+    if (ah > g.tiny) {
+        const double den = R[0] * R[1] * R[2] + dot3(v, v + 3) * R[2] + dot3(v, v + 6) * R[1] + dot3(v + 3, v + 6) * R[0];
+        slog -= ah * 2.0 * atan2(g.a2 * ah, den);
+    }
+    return slog;
+}
+// int 1/R and (VEC) int (r' - r)/R over a tetrahedron; v: its vertices relative to the observer
+template <bool VEC>
+__host__ __device__ inline void tet_integrals(const TetGeom &g, const double *v, double &inv, double *vec) {
+    double R[4], L[6], sR[6], dt[6];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) R[k] = sqrt(dot3(v + 3 * k, v + 3 * k));
 #pragma unroll
     for (int e = 0; e < 6; ++e) {
-        const double *pa = tv + 3 * EA[e], *pb = tv + 3 * EB[e];
-        double d[3] = {pb[0] - pa[0], pb[1] - pa[1], pb[2] - pa[2]};
-        const double len = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-        scale = fmax(scale, len);
-        for (int q = 0; q < 3; ++q) lh[e][q] = d[q] / len;
-        sa[e] = lh[e][0] * pa[0] + lh[e][1] * pa[1] + lh[e][2] * pa[2];   // along the edge, observer at 0
-        sb[e] = sa[e] + len;
-        const double c0 = pa[1] * lh[e][2] - pa[2] * lh[e][1], c1 = pa[2] * lh[e][0] - pa[0] * lh[e][2],
-                     c2 = pa[0] * lh[e][1] - pa[1] * lh[e][0];
-        const double d2 = c0 * c0 + c1 * c1 + c2 * c2;   // squared distance to the edge line
-        const double Ra = Rv[EA[e]], Rb = Rv[EB[e]];
-        // ln[(Rb + sb)/(Ra + sa)] with R + s = d2/(R - s) for s < 0
-        double lv;
-        if (sa[e] >= 0) lv = log((Rb + sb[e]) / (Ra + sa[e]));
-        else if (sb[e] <= 0) lv = log((Ra - sa[e]) / (Rb - sb[e]));
-        else lv = (d2 > 0) ? log((Rb + sb[e]) * (Ra - sa[e]) / d2) : 0.0;
-        L[e] = lv;
-        sR[e] = sb[e] * Rb - sa[e] * Ra;
+        const double *pa = v + 3 * tet_ea(e), *pb = v + 3 * tet_eb(e);
+        const double sa = dot3(g.lh[e], pa), sb = sa + g.len[e], Ra = R[tet_ea(e)], Rb = R[tet_eb(e)];
+        L[e] = edge_log(pa, g.lh[e], sa, sb, Ra, Rb);
+        if (VEC) sR[e] = sb * Rb - sa * Ra;
+        dt[e] = dot3(pa, pb);
     }
-    const double tiny = 1e-13 * scale;
     inv = 0;
-    vec[0] = vec[1] = vec[2] = 0;
+    if (VEC) vec[0] = vec[1] = vec[2] = 0;
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
-        // face opposite vertex f; outward normal
-        const int fv[3] = {f == 0 ? 1 : 0, f <= 1 ? 2 : 1, f <= 2 ? 3 : 2};
-        const double *p0 = tv + 3 * fv[0], *p1 = tv + 3 * fv[1], *p2 = tv + 3 * fv[2];
-        const double e1[3] = {p1[0] - p0[0], p1[1] - p0[1], p1[2] - p0[2]};
-        const double e2[3] = {p2[0] - p0[0], p2[1] - p0[1], p2[2] - p0[2]};
-        double n[3] = {e1[1] * e2[2] - e1[2] * e2[1], e1[2] * e2[0] - e1[0] * e2[2], e1[0] * e2[1] - e1[1] * e2[0]};
-        const double nn = sqrt(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
-        const double o = n[0] * (p0[0] - tv[3 * f]) + n[1] * (p0[1] - tv[3 * f + 1]) + n[2] * (p0[2] - tv[3 * f + 2]);
-        const double sg = (o >= 0) ? 1.0 / nn : -1.0 / nn;
-        n[0] *= sg; n[1] *= sg; n[2] *= sg;
-        const double dfc = n[0] * p0[0] + n[1] * p0[1] + n[2] * p0[2];   // n.(p0 - r): signed distance
-        const double h = -dfc, ah = fabs(h);
-        double slog = 0, satan = 0, sr = 0;
+        const double d = dot3(g.n[f], v + 3 * (f == 0 ? 1 : 0));   // signed distance of the face
+        const double ah = fabs(d);
+        double slog = 0, sr = 0;
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            const int e = FE[f][q];
-            // in-plane outward normal of the edge: u = l x n, its sign fixed by
-            // pointing away from the face's third vertex
-            const double *pc = tv + 3 * FC[f][q];
-            double u[3] = {lh[e][1] * n[2] - lh[e][2] * n[1], lh[e][2] * n[0] - lh[e][0] * n[2],
-                           lh[e][0] * n[1] - lh[e][1] * n[0]};
-            const double *pa = tv + 3 * EA[e];
-            if (u[0] * (pa[0] - pc[0]) + u[1] * (pa[1] - pc[1]) + u[2] * (pa[2] - pc[2]) < 0) {
-                u[0] = -u[0]; u[1] = -u[1]; u[2] = -u[2];
-            }
-            const double t = u[0] * pa[0] + u[1] * pa[1] + u[2] * pa[2];
-            if (fabs(t) <= tiny) continue;
-            const double R0sq = t * t + h * h;
+            const int e = tet_fe(f, q);
+            const double t = dot3(g.u[f][q], v + 3 * tet_ea(e));
+            if (fabs(t) <= g.tiny) continue;
             slog += t * L[e];
-            sr += t * (sR[e] + R0sq * L[e]);
-            if (ah > tiny) {
-                const double xa = R0sq + ah * Rv[EA[e]], ya = t * sa[e];
-                const double xb = R0sq + ah * Rv[EB[e]], yb = t * sb[e];
-                satan += atan2(yb * xa - xb * ya, xa * xb + ya * yb);
-            }
+            if (VEC) sr += t * (sR[e] + (t * t + d * d) * L[e]);
         }
-        const double fi = slog - ah * satan;
-        const double fr = (h * h * fi + 0.5 * sr) / 3.0;
-        inv += 0.5 * dfc * fi;
-        vec[0] += n[0] * fr; vec[1] += n[1] * fr; vec[2] += n[2] * fr;
+        if (ah > g.tiny) {
+            const int i = f == 0 ? 1 : 0, j = f <= 1 ? 2 : 1, k = f <= 2 ? 3 : 2;
+            double den = R[i] * R[j] * R[k];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) den += dt[tet_fe(f, q)] * R[tet_fc(f, q)];
+            slog -= ah * 2.0 * atan2(g.a2[f] * ah, den);
+        }
+        inv += 0.5 * d * slog;
+        if (VEC) {
+            const double fr = (d * d * slog + 0.5 * sr) / 3.0;
+            for (int q = 0; q < 3; ++q) vec[q] += g.n[f][q] * fr;
+        }
     }
 }
 

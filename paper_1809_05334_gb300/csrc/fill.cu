@@ -349,46 +349,6 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 8 : 6)
 // ---------------------------------------------------------------------------
 // near tetrahedron pairs: one warp per pair
 // ---------------------------------------------------------------------------
-template <typename U>
-__device__ void static_tt_term(const double *r5, double w, const double *tv_other, const double *R,
-                               double sgnR, const double *c_self, const double *c_other, bool order_i,
-                               cx<double> ph, Mom<double> &acc) {
-    // outer point r (double), closed form over the other tetrahedron shifted by
-    // sgnR*R; coordinates relative to r are formed in FP64 before narrowing to U
-    U r[3] = {U(0), U(0), U(0)};
-    U tv[12];
-    for (int j = 0; j < 4; ++j)
-        for (int d = 0; d < 3; ++d) tv[3 * j + d] = U((tv_other[3 * j + d] + sgnR * R[d]) - r5[d]);
-    U inv, vec[3];
-    tet_integrals<U>(r, tv, inv, vec, true);
-    double I = double(inv);
-    double f[3], rho[3];
-    for (int d = 0; d < 3; ++d) {
-        // int (r' - c_other_shifted)/R dV' and the outer point relative to its centroid
-        f[d] = double(vec[d]) + (r5[d] - (c_other[d] + sgnR * R[d])) * I;
-        rho[d] = r5[d] - c_self[d];
-    }
-    cx<double> pw = {ph.re * w, ph.im * w};
-    acc.S = acc.S + I * pw;
-    if (order_i) {   // outer on test: A gets rho*I, B gets f
-        for (int d = 0; d < 3; ++d) {
-            acc.A[d] = acc.A[d] + (rho[d] * I) * pw;
-            acc.B[d] = acc.B[d] + f[d] * pw;
-        }
-    } else {          // outer on source: B gets rho'*I, A gets f
-        for (int d = 0; d < 3; ++d) {
-            acc.B[d] = acc.B[d] + (rho[d] * I) * pw;
-            acc.A[d] = acc.A[d] + f[d] * pw;
-        }
-    }
-    acc.C = acc.C + (rho[0] * f[0] + rho[1] * f[1] + rho[2] * f[2]) * pw;
-}
-
-__device__ __forceinline__ double warp_sum(double v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
-
 __device__ __forceinline__ float inv_sqrt(float x) { return rsqrt_ftz(x); }
 __device__ __forceinline__ double inv_sqrt(double x) { return rsqrt(x); }
 
@@ -445,54 +405,23 @@ __global__ void __launch_bounds__(128) k_pr_tt(DevMesh m, const __grid_constant_
     scatter_tt<T>(m, q, Z, N, t, s, mo);
 }
 
-// near image of a pair whose elements touch: closed form over one element at
-// the degree-5 points of the other, both orders averaged, in FP64; one warp per
-// (pair, image), lanes 0..13 order (i), 14..27 order (ii)
-template <typename T>
-__global__ void __launch_bounds__(128) k_touch_tt(DevMesh m, const __grid_constant__ DevReq q, T *Z, size_t N, const NearEntry *list,
-                                                  int n) {
-    const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (wid >= n) return;
-    const NearEntry en = list[wid];
-    const int t = en.x, s = en.y, k = en.k;
-    Mom<double> acc;
-    acc.zero();
-    if (lane < 28) {
-        const double R[3] = {(k / 3 - 1) * m.a, (k % 3 - 1) * m.b, 0.0};
-        const cx<double> hph = {0.5 * q.img_ph[2 * k], 0.5 * q.img_ph[2 * k + 1]};
-        const bool oi = lane < 14;
-        const int qi = oi ? lane : lane - 14;
-        const int self = oi ? t : s, other = oi ? s : t;
-        const double *r5 = m.q5 + (size_t)self * 42 + 3 * qi;
-        const double w = m.vol[self] * c_w5tet[qi];
-        static_tt_term<double>(r5, w, m.tv + 12 * (size_t)other, R, oi ? -1.0 : 1.0, m.cen + 3 * self,
-                               m.cen + 3 * other, oi, hph, acc);
-    }
-    double v[16] = {acc.S.re, acc.S.im, acc.C.re, acc.C.im, acc.A[0].re, acc.A[0].im, acc.A[1].re, acc.A[1].im,
-                    acc.A[2].re, acc.A[2].im, acc.B[0].re, acc.B[0].im, acc.B[1].re, acc.B[1].im, acc.B[2].re,
-                    acc.B[2].im};
-    for (int i = 0; i < 16; ++i) v[i] = warp_sum(v[i]);
-    if (lane == 0) {
-        Mom<T> mo;
-        mo.S = {T(v[0]), T(v[1])};
-        mo.C = {T(v[2]), T(v[3])};
-        for (int d = 0; d < 3; ++d) {
-            mo.A[d] = {T(v[4 + 2 * d]), T(v[5 + 2 * d])};
-            mo.B[d] = {T(v[10 + 2 * d]), T(v[11 + 2 * d])};
-        }
-        scatter_tt<T>(m, q, Z, N, t, s, mo);
-    }
-}
-
 // Touching images, exploiting the symmetry of the two integration orders:
 // order (ii) of the entry (t, s, k) is order (i) of its partner (s, t, 8-k)
 // with the test and source polynomial moments exchanged.  k_touch_half
 // computes order (i) of every entry once (phase-free real moments, FP64;
 // half a warp per entry, lane q = degree-5 point q of the test element);
 // k_touch_combine averages each entry with its partner and scatters.
-__global__ void __launch_bounds__(128) k_touch_half(DevMesh m, const NearEntry *list, int n, double *out) {
-    const int e = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 2 + ((threadIdx.x >> 4) & 1);
+// Bound by the FP64 pipe: the source's geometry comes from its record, the
+// arctangents of a face are one solid angle (6 logarithms, 4 arctangents and 4
+// square roots per point; 12 arctangents, 10 square roots and 25 divisions before).
+__global__ void k_geom(DevMesh m, TetGeom *tet, TriGeom *tri) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < m.nt) tet_geom(m.tv + 12 * (size_t)e, tet[e]);
+    else if (e - m.nt < m.nf) tri_geom(m.fv + 9 * (size_t)(e - m.nt), tri[e - m.nt]);
+}
+
+__global__ void __launch_bounds__(128) k_touch_half(DevMesh m, const TetGeom *geom, const NearEntry *list, int n, double *out) {
+    const int e = (blockIdx.x * blockDim.x + threadIdx.x) >> 4;
     const int hl = threadIdx.x & 15;
     double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     if (e < n && hl < 14) {
@@ -507,7 +436,7 @@ __global__ void __launch_bounds__(128) k_touch_half(DevMesh m, const NearEntry *
         for (int j = 0; j < 4; ++j)
             for (int d = 0; d < 3; ++d) rel[3 * j + d] = (src[3 * j + d] - R[d]) - r5[d];
         double I, vec[3];
-        tet_integrals_shared(rel, I, vec);
+        tet_integrals<true>(geom[s], rel, I, vec);
         double f[3], rho[3];
         for (int d = 0; d < 3; ++d) {
             f[d] = vec[d] + (r5[d] - (cs[d] - R[d])) * I;   // int (r' - c_s)/R over the image source
@@ -646,25 +575,6 @@ __global__ void __launch_bounds__(128) k_far_scalar(DevMesh m, const __grid_cons
     scatter_scalar<T, PK>(m, q, Z, N, x, y, S);
 }
 
-template <typename U>
-__device__ double static_scalar(const double *r5, bool other_tet, const double *verts_other, const double *R,
-                                double sgnR) {
-    U r[3] = {U(0), U(0), U(0)};   // coordinates relative to the outer point (formed in FP64)
-    U inv;
-    if (other_tet) {
-        U tv[12], vec[3];
-        for (int j = 0; j < 4; ++j)
-            for (int d = 0; d < 3; ++d) tv[3 * j + d] = U((verts_other[3 * j + d] + sgnR * R[d]) - r5[d]);
-        tet_integrals<U>(r, tv, inv, vec, false);
-    } else {
-        U fv[9], rr;
-        for (int j = 0; j < 3; ++j)
-            for (int d = 0; d < 3; ++d) fv[3 * j + d] = U((verts_other[3 * j + d] + sgnR * R[d]) - r5[d]);
-        tri_integrals<U>(r, fv, inv, rr, false);
-    }
-    return double(inv);
-}
-
 template <typename T, int PK>
 __global__ void __launch_bounds__(128) k_pr_scalar(DevMesh m, const __grid_constant__ DevReq q, T *Z, size_t N, const NearEntry *list,
                                                    int n) {
@@ -695,40 +605,39 @@ __global__ void __launch_bounds__(128) k_pr_scalar(DevMesh m, const __grid_const
     scatter_scalar<T, PK>(m, q, Z, N, x, y, s0 * cx<T>{T(q.img_ph[2 * k]), T(q.img_ph[2 * k + 1])});
 }
 
-// Touching face entries: the static integral, both integration orders
-// averaged, summed over the degree-5 points (phase-free, FP64; one warp per
-// entry, lanes = the points of the two elements).  Request independent.
-template <int PK>
-__global__ void __launch_bounds__(128) k_touch_scalar(DevMesh m, const NearEntry *list, int n, double *out) {
-    const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (wid >= n) return;
+// Touching face entries: the static integral, both integration orders averaged,
+// summed over the degree-5 points (phase-free, FP64, request independent).  One
+// launch per order, so that the lanes of a warp integrate over the same kind of
+// element: OX: the outer points are those of x, else of y (then added to the
+// first order's sum); 16 lanes per entry for a tetrahedron's 14 points, 8 for a
+// face's 7.
+template <int PK, bool OX>
+__global__ void __launch_bounds__(128) k_touch_scalar(DevMesh m, const TetGeom *tet, const TriGeom *tri,
+                                                      const NearEntry *list, int n, double *out) {
     constexpr bool XT = PKTraits<PK>::xtet, YT = PKTraits<PK>::ytet;
-    const NearEntry en = list[wid];
-    const int x = en.x, y = en.y, k = en.k;
-    const int xf = XT ? x : m.hf[x];
-    const int yf = y;
-    constexpr int nqx = XT ? 14 : 7, nqy = YT ? 14 : 7;
-    const double *x5 = XT ? m.q5 + (size_t)xf * 42 : m.f5 + (size_t)xf * 21;
-    const double *y5 = YT ? m.q5 + (size_t)yf * 42 : m.f5 + (size_t)yf * 21;
-    const double mx = XT ? m.vol[xf] : m.farea[xf];
-    const double my = YT ? m.vol[yf] : m.farea[yf];
+    constexpr bool OT = OX ? XT : YT, ST = OX ? YT : XT;   // outer and source element are tetrahedra
+    constexpr int G = OT ? 16 : 8, NP = OT ? 14 : 7;
+    const int e = (blockIdx.x * blockDim.x + threadIdx.x) / G, q = threadIdx.x % G;
     double acc = 0;
-    if (lane < nqx + nqy) {
-        const double R[3] = {(k / 3 - 1) * m.a, (k % 3 - 1) * m.b, 0.0};
-        const bool oi = lane < nqx;
-        const int qi = oi ? lane : lane - nqx;
-        const bool self_tet = oi ? XT : YT;
-        const bool other_tet = oi ? YT : XT;
-        const int other = oi ? yf : xf;
-        const double *r5 = (oi ? x5 : y5) + 3 * qi;
-        const double w = (oi ? mx : my) * (self_tet ? c_w5tet[qi] : c_w5tri[qi]);
-        const double *vo = other_tet ? m.tv + 12 * (size_t)other : m.fv + 9 * (size_t)other;
-        const double I = static_scalar<double>(r5, other_tet, vo, R, oi ? -1.0 : 1.0);
+    if (e < n && q < NP) {
+        const NearEntry en = list[e];
+        const int xf = XT ? en.x : m.hf[en.x], yf = en.y, k = en.k;
+        const int o = OX ? xf : yf, s = OX ? yf : xf;
+        const double sg = OX ? -1.0 : 1.0;   // the source's image as the outer element sees it
+        const double R[3] = {sg * (k / 3 - 1) * m.a, sg * (k % 3 - 1) * m.b, 0.0};
+        const double *r5 = (OT ? m.q5 + (size_t)o * 42 : m.f5 + (size_t)o * 21) + 3 * q;
+        const double w = OT ? m.vol[o] * c_w5tet[q] : m.farea[o] * c_w5tri[q];
+        const double *v = ST ? m.tv + 12 * (size_t)s : m.fv + 9 * (size_t)s;
+        double rel[ST ? 12 : 9];
+        for (int j = 0; j < (ST ? 4 : 3); ++j)
+            for (int d = 0; d < 3; ++d) rel[3 * j + d] = (v[3 * j + d] + R[d]) - r5[d];
+        double I;
+        if constexpr (ST) tet_integrals<false>(tet[s], rel, I, nullptr);
+        else I = tri_inv(tri[s], rel);
         acc = 0.5 * w * I;
     }
-    const double sum = warp_sum(acc);
-    if (lane == 0) out[wid] = sum;
+    for (int h = G / 2; h > 0; h >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, h, G);
+    if (e < n && q == 0) out[e] = OX ? acc : out[e] + acc;
 }
 
 // scatter the cached static integral of every touching face entry with the
@@ -893,16 +802,28 @@ cudaError_t launch_fill(const DevMesh &m, const DevReq &q, T *Z, size_t ld, doub
     return cudaGetLastError();
 }
 
-cudaError_t launch_static_cache(const DevMesh &m, double *touch_half, double *const touch_sc[4], cudaStream_t st) {
+size_t static_geom_bytes(size_t nt, size_t nf) { return sizeof(TetGeom) * nt + sizeof(TriGeom) * (nf + 1); }
+
+cudaError_t launch_static_cache(const DevMesh &m, double *touch_half, double *const touch_sc[4], void *geom,
+                                cudaStream_t st) {
+    TetGeom *tet = static_cast<TetGeom *>(geom);
+    TriGeom *tri = reinterpret_cast<TriGeom *>(tet + m.nt);
     const dim3 blk(128);
-    auto gridw = [](int n) { return (unsigned)(((size_t)n * 32 + 127) / 128); };
-    if (m.nto[0]) {
-        k_touch_half<<<(unsigned)(((size_t)(m.nto[0] + 1) / 2 * 32 + 127) / 128), blk, 0, st>>>(m, m.to[0], m.nto[0],
-                                                                                              touch_half); ++g_launches;
+    auto grid = [](int n, int lanes) { return (unsigned)(((size_t)n * lanes + 127) / 128); };
+    k_geom<<<(m.nt + m.nf + 127) / 128, blk, 0, st>>>(m, tet, tri); ++g_launches;
+    if (m.nto[0]) { k_touch_half<<<grid(m.nto[0], 16), blk, 0, st>>>(m, tet, m.to[0], m.nto[0], touch_half); ++g_launches; }
+    if (m.nto[1]) {
+        k_touch_scalar<PK_TF, true><<<grid(m.nto[1], 16), blk, 0, st>>>(m, tet, tri, m.to[1], m.nto[1], touch_sc[1]); ++g_launches;
+        k_touch_scalar<PK_TF, false><<<grid(m.nto[1], 8), blk, 0, st>>>(m, tet, tri, m.to[1], m.nto[1], touch_sc[1]); ++g_launches;
     }
-    if (m.nto[1]) { k_touch_scalar<PK_TF><<<gridw(m.nto[1]), blk, 0, st>>>(m, m.to[1], m.nto[1], touch_sc[1]); ++g_launches; }
-    if (m.nto[2]) { k_touch_scalar<PK_FT><<<gridw(m.nto[2]), blk, 0, st>>>(m, m.to[2], m.nto[2], touch_sc[2]); ++g_launches; }
-    if (m.nto[3]) { k_touch_scalar<PK_FF><<<gridw(m.nto[3]), blk, 0, st>>>(m, m.to[3], m.nto[3], touch_sc[3]); ++g_launches; }
+    if (m.nto[2]) {
+        k_touch_scalar<PK_FT, true><<<grid(m.nto[2], 8), blk, 0, st>>>(m, tet, tri, m.to[2], m.nto[2], touch_sc[2]); ++g_launches;
+        k_touch_scalar<PK_FT, false><<<grid(m.nto[2], 16), blk, 0, st>>>(m, tet, tri, m.to[2], m.nto[2], touch_sc[2]); ++g_launches;
+    }
+    if (m.nto[3]) {
+        k_touch_scalar<PK_FF, true><<<grid(m.nto[3], 8), blk, 0, st>>>(m, tet, tri, m.to[3], m.nto[3], touch_sc[3]); ++g_launches;
+        k_touch_scalar<PK_FF, false><<<grid(m.nto[3], 8), blk, 0, st>>>(m, tet, tri, m.to[3], m.nto[3], touch_sc[3]); ++g_launches;
+    }
     return cudaGetLastError();
 }
 

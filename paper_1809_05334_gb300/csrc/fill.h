@@ -107,7 +107,10 @@ cudaError_t launch_fill(const DevMesh &m, const DevReq &q, T *Z, size_t ld, doub
                         cudaEvent_t far0 = nullptr, cudaEvent_t far1 = nullptr);
 // the request-independent static integrals of the touching near images:
 // touch_half [nto[0]][8] and touch_sc[i] [nto[i]] (i = 1..3)
-cudaError_t launch_static_cache(const DevMesh &m, double *touch_half, double *const touch_sc[4], cudaStream_t st);
+// (geom: device scratch of static_geom_bytes)
+size_t static_geom_bytes(size_t nt, size_t nf);
+cudaError_t launch_static_cache(const DevMesh &m, double *touch_half, double *const touch_sc[4], void *geom,
+                                cudaStream_t st);
 // Builds the element records of a request and runs the far pairs in the
 // polynomial form (q.fp.mode != FAR_NONE): tetrahedron pairs, and pairs with
 // charge faces (pk: 0 tetrahedron-face, 1 half face-tetrahedron, 2 half face-face)

@@ -10,15 +10,12 @@
 #include <cmath>
 #include <cstdio>
 #include <map>
-#include <tuple>
 
 #include "vie_internal.h"
 
 namespace vie {
 
 namespace {
-
-using Key = std::array<int32_t, 3>;
 
 inline void face_local(int i, int out[3]) {
     int k = 0;
@@ -52,7 +49,7 @@ double norm3(const double *v) { return std::sqrt(v[0] * v[0] + v[1] * v[1] + v[2
 
 std::string build_topology(const double *verts, int nv, const int32_t *tets, int nt,
                            const int32_t *tet_domain, int n_dom, double a, double b,
-                           int active, Topology &T) {
+                           int active, Topology &T, bool near_lists) {
     T = Topology();
     T.nt = nt;
     T.nv = nv;
@@ -109,23 +106,46 @@ std::string build_topology(const double *verts, int nv, const int32_t *tets, int
         }
     }
 
-    // faces and owners
-    std::map<Key, std::vector<std::pair<int, int>>> owners;
+    // faces (local face i of tetrahedron t is 4 t + i) sorted by their vertices: the two
+    // owners of an interior face are neighbours
+    struct Face {
+        int32_t v[3], e;
+        bool same(const Face &o) const { return v[0] == o.v[0] && v[1] == o.v[1] && v[2] == o.v[2]; }
+    };
+    std::vector<Face> faces(4 * (size_t)nt);
     for (int t = 0; t < nt; ++t)
         for (int i = 0; i < 4; ++i) {
             int l[3];
             face_local(i, l);
-            Key k = {tets[4 * t + l[0]], tets[4 * t + l[1]], tets[4 * t + l[2]]};
-            std::sort(k.begin(), k.end());
-            owners[k].push_back({t, i});
+            Face &f = faces[4 * (size_t)t + i];
+            for (int j = 0; j < 3; ++j) f.v[j] = tets[4 * t + l[j]];
+            std::sort(f.v, f.v + 3);
+            f.e = 4 * t + i;
         }
-    for (auto &kv : owners)
-        if (kv.second.size() > 2) return "a face is shared by more than two tetrahedra";
+    std::sort(faces.begin(), faces.end(), [](const Face &p, const Face &q) {
+        for (int j = 0; j < 3; ++j)
+            if (p.v[j] != q.v[j]) return p.v[j] < q.v[j];
+        return p.e < q.e;
+    });
+    std::vector<int32_t> mate(4 * (size_t)nt, -1);   // the other owner of an interior face
+    std::vector<const Face *> boundary;
+    for (size_t f = 0; f < faces.size();) {
+        size_t g = f + 1;
+        while (g < faces.size() && faces[g].same(faces[f])) ++g;
+        if (g - f > 2) return "a face is shared by more than two tetrahedra";
+        if (g - f == 2) {
+            mate[faces[f].e] = faces[f + 1].e;
+            mate[faces[f + 1].e] = faces[f].e;
+        } else {
+            boundary.push_back(&faces[f]);
+        }
+        f = g;
+    }
 
-    auto wall = [&](const Key &k) -> int {  // 0 x0, 1 xa, 2 y0, 3 yb, -1 none
+    auto wall = [&](const Face &k) -> int {  // 0 x0, 1 xa, 2 y0, 3 yb, -1 none
         bool all[4] = {true, true, true, true};
         for (int j = 0; j < 3; ++j) {
-            const double *p = verts + 3 * k[j];
+            const double *p = verts + 3 * k.v[j];
             all[0] &= std::fabs(p[0]) < tol;
             all[1] &= std::fabs(p[0] - a) < tol;
             all[2] &= std::fabs(p[1]) < tol;
@@ -136,64 +156,54 @@ std::string build_topology(const double *verts, int nv, const int32_t *tets, int
         return -1;
     };
     // periodic pairing: face on the low wall <-> face on the high wall
-    std::map<Key, std::pair<Key, int>> partner;  // key -> (other key, axis 1=x 2=y)
-    std::map<Key, bool> is_high;
+    std::vector<int32_t> partner(4 * (size_t)nt, -1);   // the paired face
+    std::vector<int8_t> axis_of(4 * (size_t)nt, 0), is_high(4 * (size_t)nt, 0);
     for (int axis = 0; axis < 2; ++axis) {
-        std::map<GeoKey, Key> lo, hi;
-        for (auto &kv : owners) {
-            if (kv.second.size() != 1) continue;
-            int w = wall(kv.first);
-            const double *p0 = verts + 3 * kv.first[0], *p1 = verts + 3 * kv.first[1], *p2 = verts + 3 * kv.first[2];
-            if (w == 2 * axis) lo[geo_key(p0, p1, p2, 0, 0)] = kv.first;
-            if (w == 2 * axis + 1) hi[geo_key(p0, p1, p2, axis == 0 ? a : 0, axis == 1 ? b : 0)] = kv.first;
+        std::map<GeoKey, int32_t> lo, hi;
+        for (const Face *f : boundary) {
+            const int w = wall(*f);
+            const double *p0 = verts + 3 * f->v[0], *p1 = verts + 3 * f->v[1], *p2 = verts + 3 * f->v[2];
+            if (w == 2 * axis) lo[geo_key(p0, p1, p2, 0, 0)] = f->e;
+            if (w == 2 * axis + 1) hi[geo_key(p0, p1, p2, axis == 0 ? a : 0, axis == 1 ? b : 0)] = f->e;
         }
         if (lo.size() != hi.size()) return "periodic walls do not match";
         for (auto &kv : lo) {
             auto it = hi.find(kv.first);
             if (it == hi.end()) return "periodic walls do not match";
-            partner[kv.second] = {it->second, axis + 1};
-            partner[it->second] = {kv.second, axis + 1};
-            is_high[it->second] = true;
+            partner[kv.second] = it->second;
+            partner[it->second] = kv.second;
+            axis_of[kv.second] = axis_of[it->second] = (int8_t)(axis + 1);
+            is_high[it->second] = 1;
         }
     }
 
     T.basis.assign(4 * (size_t)nt, -1);
     T.sgn.assign(4 * (size_t)nt, 0);
     T.shift.assign(4 * (size_t)nt, 0);
-    for (int t = 0; t < nt; ++t)
-        for (int i = 0; i < 4; ++i) {
-            if (T.basis[4 * t + i] >= 0) continue;
-            int l[3];
-            face_local(i, l);
-            Key k = {tets[4 * t + l[0]], tets[4 * t + l[1]], tets[4 * t + l[2]]};
-            std::sort(k.begin(), k.end());
-            auto &own = owners[k];
-            int n = (int)T.kind.size();
-            if (own.size() == 2) {
-                auto p = std::min(own[0], own[1]), m = std::max(own[0], own[1]);
-                T.kind.push_back(KIND_INTERIOR);
-                T.tp.push_back(p.first); T.ip.push_back(p.second);
-                T.tm.push_back(m.first); T.im.push_back(m.second);
-                T.basis[4 * p.first + p.second] = n; T.sgn[4 * p.first + p.second] = 1;
-                T.basis[4 * m.first + m.second] = n; T.sgn[4 * m.first + m.second] = -1;
-            } else if (partner.count(k)) {
-                auto pr = partner[k];
-                Key klo = is_high.count(k) ? pr.first : k;
-                Key khi = is_high.count(k) ? k : pr.first;
-                auto p = owners[klo][0], m = owners[khi][0];
-                T.kind.push_back(KIND_PERIODIC);
-                T.tp.push_back(p.first); T.ip.push_back(p.second);
-                T.tm.push_back(m.first); T.im.push_back(m.second);
-                T.basis[4 * p.first + p.second] = n; T.sgn[4 * p.first + p.second] = 1;
-                T.basis[4 * m.first + m.second] = n; T.sgn[4 * m.first + m.second] = -1;
-                T.shift[4 * m.first + m.second] = (int8_t)pr.second;
-            } else {
-                T.kind.push_back(KIND_HALF);
-                T.tp.push_back(t); T.ip.push_back(i);
-                T.tm.push_back(-1); T.im.push_back(-1);
-                T.basis[4 * t + i] = n; T.sgn[4 * t + i] = 1;
-            }
+    auto full = [&](int kind, int p, int m) {   // a function on the two faces p (T+) and m (T-)
+        const int n = (int)T.kind.size();
+        T.kind.push_back(kind);
+        T.tp.push_back(p / 4); T.ip.push_back(p % 4);
+        T.tm.push_back(m / 4); T.im.push_back(m % 4);
+        T.basis[p] = n; T.sgn[p] = 1;
+        T.basis[m] = n; T.sgn[m] = -1;
+    };
+    for (int e = 0; e < 4 * nt; ++e) {
+        if (T.basis[e] >= 0) continue;
+        if (mate[e] >= 0) {
+            full(KIND_INTERIOR, std::min(e, (int)mate[e]), std::max(e, (int)mate[e]));
+        } else if (partner[e] >= 0) {
+            const int plo = is_high[e] ? partner[e] : e, phi = is_high[e] ? e : partner[e];
+            full(KIND_PERIODIC, plo, phi);
+            T.shift[phi] = axis_of[e];
+        } else {
+            T.basis[e] = (int)T.kind.size();
+            T.sgn[e] = 1;
+            T.kind.push_back(KIND_HALF);
+            T.tp.push_back(e / 4); T.ip.push_back(e % 4);
+            T.tm.push_back(-1); T.im.push_back(-1);
         }
+    }
     T.N = (int)T.kind.size();
 
     // charge-carrying faces: half functions and faces between two domains
@@ -221,6 +231,7 @@ std::string build_topology(const double *verts, int nv, const int32_t *tets, int
         T.frad.push_back(r);
     }
 
+    if (!near_lists) return "";
     // near-pair lists: for every x and image R_k, the y whose centroid lies
     // within NEAR_FACTOR (rho_x + rho_y) of c_x + R_k, found through a uniform
     // bucket grid over the y centroids (cell size NEAR_FACTOR * 2 max rho_y)

@@ -62,9 +62,10 @@ struct Topology {
     std::vector<NearPair> near_tt, near_tf, near_ft, near_ff;
 };
 
-// Builds the topology; returns an empty string or an error message.
+// Builds the topology; returns an empty string or an error message.  near_lists:
+// the near-pair lists too (vie_set_mesh builds them on the device, mesh.cu).
 std::string build_topology(const double *verts, int nv, const int32_t *tets, int nt,
                            const int32_t *tet_domain, int n_dom, double a, double b,
-                           int active, Topology &out);
+                           int active, Topology &out, bool near_lists = true);
 
 }  // namespace vie
