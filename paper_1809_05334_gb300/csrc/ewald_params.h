@@ -22,6 +22,7 @@ struct EwaldTables {
     int near_img[9];        // image-table index of (m,n) = (k/3-1, k%3-1)
     double E, bb, a, b, xcut64;
     float xcut32;
+    double xs_h;             // spatial table interval in x = R E
     double reg0_re;          // limit R->0 of (image term - static term), without the phase
     // tabulated FP32 evaluation (see green_tab): spatial kernel F(x) on [0, xs_max],
     // spectral G_g(z) per distinct gamma on [0, z_max], piecewise cubic Hermite
@@ -66,7 +67,7 @@ struct EwaldF32 {
     int near_img[9];
     int n_img, p0, np, q0, nq, sym;
     float xs_max, xs_inv_h, z_inv_h, e_mb2, Ef, kx, ky, step_x, step_y;
-    float Eih;                            // E * xs_inv_h: table intervals per unit distance (a power of two)
+    float Eih;                            // E * xs_inv_h: table intervals per unit distance (far kernels: a power of two)
     int sq_pq;                            // max(P, Q) >= 1 of the short form; 0 where it does not apply
     int sq_off[SQ_MAX + 1][SQ_MAX + 1];   // order (p, q): offset of its real table in rtab (float4 units)
     int sq_im;                            // offset of the (0, 0) order's imaginary table in rtab
@@ -133,7 +134,8 @@ inline bool mode_rect(double kx, double ky, double a, double b, double kmax, int
     return np * nq <= MAX_MODE;
 }
 
-inline EwaldF32 make_ewald_f32(const EwaldTables &t) {
+// pow2: as build_ewald_tables had it
+inline EwaldF32 make_ewald_f32(const EwaldTables &t, bool pow2 = true) {
     EwaldF32 f{};
     for (int i = 0; i < MAX_IMG; ++i)
         for (int k = 0; k < 4; ++k) f.img[i][k] = t.img32[i][k];
@@ -142,7 +144,7 @@ inline EwaldF32 make_ewald_f32(const EwaldTables &t) {
     f.n_img = t.n_img; f.p0 = t.p0; f.np = t.np; f.q0 = t.q0; f.nq = t.nq; f.sym = t.sym;
     f.xs_max = t.xs_max; f.xs_inv_h = t.xs_inv_h; f.z_inv_h = t.z_inv_h; f.e_mb2 = t.e_mb2; f.Ef = t.Ef;
     f.kx = t.kx; f.ky = t.ky; f.step_x = t.step_x; f.step_y = t.step_y;
-    f.Eih = (float)std::exp2(std::round(std::log2((double)t.Ef * t.xs_inv_h)));   // a power of two (ewald_tables.cpp)
+    f.Eih = pow2 ? (float)std::exp2(std::round(std::log2((double)t.Ef * t.xs_inv_h))) : t.Ef * t.xs_inv_h;
     f.sq_pq = 0;
     const int zero = t.n_tab * NZTAB;   // the zero table
     for (int p = 0; p <= SQ_MAX; ++p)

@@ -24,7 +24,7 @@ namespace vie {
 // Returns VIE_OK, VIE_RAYLEIGH_ANOMALY (a Floquet order at grazing) or
 // VIE_EINVAL (a table would overflow), with *why set.
 int build_ewald_tables(double a, double b, double k0, double kx, double ky, double z_extent, bool fp64,
-                       EwaldTables &E, std::vector<double> *orders, const char **why, double split_mult) {
+                       EwaldTables &E, std::vector<double> *orders, const char **why, double split_mult, bool pow2) {
     std::memset(&E, 0, sizeof(E));
     if (orders) orders->clear();
     E.E = ewald_split(a, b, k0, !fp64, kx == 0.0 && ky == 0.0, split_mult);
@@ -88,7 +88,10 @@ int build_ewald_tables(double a, double b, double k0, double kx, double ky, doub
     // intervals per unit of x: such that E xs_inv_h, the table intervals per unit of
     // distance, is a power of two (distances scaled to table units stay exact) and
     // the cut falls in the table's upper half
-    E.xs_inv_h = (float)(std::exp2(std::floor(std::log2(NSPAT * E.E / (xc32 + 0.5)))) / E.E);
+    E.xs_inv_h = (float)(pow2 ? std::exp2(std::floor(std::log2(NSPAT * E.E / (xc32 + 0.5)))) / E.E : NSPAT / (xc32 + 0.5));
+    // the interval itself in FP64: the kernels index with the exact power of two, and an
+    // interval off by FP32 rounding would give the images another E than the orders have
+    E.xs_h = pow2 ? E.E / std::exp2(std::floor(std::log2(NSPAT * E.E / (xc32 + 0.5)))) : (double)E.xs_max / NSPAT;
     E.z_max = (float)zr;
     E.z_inv_h = (float)(NZTAB / zr);
     E.e_mb2 = (float)std::exp(-E.bb * E.bb);

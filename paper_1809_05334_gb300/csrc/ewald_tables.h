@@ -7,10 +7,12 @@
 namespace vie {
 
 // Ewald parameters and tables of one incidence; status as vie_status;
-// split_mult > 0: the FP32 tables' Ewald split multiplier (else the default)
+// split_mult > 0: the FP32 tables' Ewald split multiplier (else the default);
+// pow2: the spatial table's spacing for the far kernels (a power of two of the
+// distance), else as fine as its size allows
 int build_ewald_tables(double a, double b, double k0, double kx, double ky, double z_extent, bool fp64,
                        EwaldTables &E, std::vector<double> *orders, const char **why,
-                       double split_mult = 0.0);
+                       double split_mult = 0.0, bool pow2 = true);
 
 // Polynomials of the spectral series for the far kernels (FarPoly) from the
 // order map of make_ewald_f32: fp.mode = FAR_NONE where no short form applies,

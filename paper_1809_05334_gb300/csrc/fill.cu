@@ -118,7 +118,7 @@ __global__ void k_build_tables(const EwaldTables *__restrict__ ew, float *stab, 
                                float4 *rtab) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < NSPAT) {
-        const double h = 1.0 / double(ew->xs_inv_h);
+        const double h = ew->xs_h;
         double F0, D0, F1, D1, c[4];
         spatial_node(ew, i * h, F0, D0);
         spatial_node(ew, (i + 1) * h, F1, D1);
@@ -917,7 +917,7 @@ extern "C" int vie_green_noalloc(double lambda_nm, double theta, double phi, dou
     const char *why = "";
     const int rc = build_ewald_tables(period_a, period_b, k0, k0 * std::sin(theta) * std::cos(phi),
                                       k0 * std::sin(theta) * std::sin(phi), z_extent, precision == VIE_FP64, tabs,
-                                      nullptr, &why);
+                                      nullptr, &why, 0.0, false);   // results leave in FP64: the finest spacing
     if (rc != VIE_OK) return rc;
     if (precision == VIE_FP32 && tabs.n_tab > NOALLOC_MAX_TAB) return VIE_EINVAL;   // scratch too small
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -926,7 +926,7 @@ extern "C" int vie_green_noalloc(double lambda_nm, double theta, double phi, dou
     float *stab = reinterpret_cast<float *>(base + NOALLOC_EW_FLOAT2);
     float2 *ztab = base + NOALLOC_EW_FLOAT2 + 2 * NSPAT;
     if (precision == VIE_FP32 && launch_build_tables(ewd, stab, ztab, tabs.n_tab, st) != cudaSuccess) return VIE_ECUDA;
-    if (launch_green(d_dev, out_dev, n, precision == VIE_FP64, stab, ztab, ewd, make_ewald_f32(tabs), st) !=
+    if (launch_green(d_dev, out_dev, n, precision == VIE_FP64, stab, ztab, ewd, make_ewald_f32(tabs, false), st) !=
         cudaSuccess)
         return VIE_ECUDA;
     return VIE_OK;
