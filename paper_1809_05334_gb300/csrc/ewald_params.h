@@ -94,6 +94,10 @@ struct FarPoly {
     int mode, nq, rows, n_coef;
     int off[FP_ROWS], deg[FP_ROWS], im_off[FP_ROWS], im_deg[FP_ROWS];   // im_deg -1: no imaginary part
     float t_scale;   // t = t_scale (z Eih)^2 - 1
+    // FAR_NORMAL: G_00(0), which the kernels leave out of g_p in the charge term (else 0).  At
+    // normal incidence every test function carries no net charge, so a constant in g_p
+    // cancels there exactly; in FP32 the cancellation left a coherent rounding of this near-constant.
+    float k_re, k_im;
 };
 // Ewald splitting parameter: sqrt(pi / ab) balances the spatial and spectral
 // series, bounded below by k0/6 (b = k0 / 2E <= 3 keeps exp(b^2) moderate).  The

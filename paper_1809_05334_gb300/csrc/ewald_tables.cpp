@@ -294,6 +294,19 @@ void build_far_poly(const EwaldTables &t, const EwaldF32 &f, FarPoly &fp, std::v
     fp.n_coef = (int)coef.size();
     const double zs = zm * f.Eih;
     fp.t_scale = (float)(2.0 / (zs * zs));
+    if (mode == FAR_NORMAL) {
+        auto at_zero = [](const std::vector<double> &c) {   // t = -1
+            double s = 0;
+            for (int n = 0; n < (int)c.size(); ++n) s += n & 1 ? -c[n] : c[n];
+            return s;
+        };
+        bool prop;
+        const int tb = entry(0, 0, prop);
+        if (tb >= 0) {
+            fp.k_re = (float)at_zero(re[tb]);
+            fp.k_im = prop ? (float)at_zero(im[tb]) : 0.f;
+        }
+    }
     fp.mode = mode;
 }
 

@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(FAR_THREADS, MODE == FAR_FULL ? VIE_FAR_MINB_F
     const int t = blockIdx.y;
     if ((int)(blockIdx.x * blockDim.x + blockDim.x) <= t) return;   // the whole block is below the diagonal
     const EwaldF32 &ef = q.ef;
-    far_stage<MODE>(q, S, s_coef);
+    far_stage<MODE, NQ>(q, S, s_coef);
     far_stage_points<MODE, 4>(q.ptet, m.nt, t, S);
     const int s0 = blockIdx.x * blockDim.x + threadIdx.x;
     const bool live = s0 < m.nt && s0 >= t;   // lanes off the pair range stay until the warp's masks are formed
@@ -175,7 +175,8 @@ __global__ void __launch_bounds__(FAR_THREADS, MODE == FAR_FULL ? VIE_FAR_MINB_F
         mo.C = wgt * mo.C;
 #pragma unroll
         for (int d = 0; d < 3; ++d) { mo.A[d] = wgt * mo.A[d]; mo.B[d] = wgt * mo.B[d]; }
-        scatter_rec<true>(Z, N, k2, rt, rs, mo, s != t);
+        const float w16 = 16.f * wgt;
+        scatter_rec<true>(Z, N, k2, rt, rs, mo, {fmaf(w16, q.fp.k_re, mo.S.re), fmaf(w16, q.fp.k_im, mo.S.im)}, s != t);
     } else {
         // g_p(-d) = conj(g_p(d)) + 2 j conj(T): the reversed pair's moments, A and B exchanged
         auto rev = [&](cx<float> g, cx<float> c) { return cx<float>{wgt * fmaf(2.f, c.im, g.re), wgt * fmaf(2.f, c.re, -g.im)}; };
@@ -188,8 +189,8 @@ __global__ void __launch_bounds__(FAR_THREADS, MODE == FAR_FULL ? VIE_FAR_MINB_F
         mo.C = wgt * mo.C;
 #pragma unroll
         for (int d = 0; d < 3; ++d) { mo.A[d] = wgt * mo.A[d]; mo.B[d] = wgt * mo.B[d]; }
-        scatter_rec<false>(Z, N, k2, rt, rs, mo, false);
-        if (s != t) scatter_rec<false>(Z, N, k2, rs, rt, mr, false);
+        scatter_rec<false>(Z, N, k2, rt, rs, mo, mo.S, false);
+        if (s != t) scatter_rec<false>(Z, N, k2, rs, rt, mr, mr.S, false);
     }
 }
 
@@ -209,7 +210,7 @@ __global__ void __launch_bounds__(FAR_THREADS) k_far_scalar_p(DevMesh m, const _
     const EwaldF32 &ef = q.ef;
     const int x = blockIdx.y;
     const int xe = XT ? x : m.hf[x];   // a test face is addressed by its half-function index
-    far_stage<MODE>(q, S, s_coef);
+    far_stage<MODE, NQ>(q, S, s_coef);
     far_stage_points<MODE, qx>(XT ? q.ptet : q.pface, XT ? m.nt : m.nf, xe, S);
     const int y0 = blockIdx.x * blockDim.x + threadIdx.x;
     const bool live = y0 < ny;
@@ -285,7 +286,7 @@ __global__ void __launch_bounds__(FAR_THREADS) k_green_p(const double *d, double
     __shared__ FarShared S;
     extern __shared__ __align__(16) p2 s_coef[];
     const EwaldF32 &ef = q.ef;
-    far_stage<MODE>(q, S, s_coef);
+    far_stage<MODE, NQ>(q, S, s_coef);
     if (threadIdx.x < 2 * 14) (&S.pt[0][0])[threadIdx.x] = 0ull;
     __syncthreads();
     if (threadIdx.x < 2) {   // test points at the origin: unit phases
@@ -312,8 +313,8 @@ __global__ void __launch_bounds__(FAR_THREADS) k_green_p(const double *d, double
     p2 gre[1], gim[1], tre[1], tim[1];
     far_eval<MODE, NQ, 1>(S, s_coef, q, 0, rec[FPT_POS], rec[FPT_PH0], MODE == FAR_NORMAL ? rec[FPT_PH0] : rec[FPT_PH1],
                           n_list, 0ull, 0ull, gre, gim, tre, tim);
-    out[2 * i] = double(upk(gre[0]).x);
-    out[2 * i + 1] = double(upk(gim[0]).x);
+    out[2 * i] = double(upk(gre[0]).x + q.fp.k_re);
+    out[2 * i + 1] = double(upk(gim[0]).x + q.fp.k_im);
 }
 
 // ---------------------------------------------------------------------------

@@ -230,7 +230,7 @@ template <typename T>
 __device__ void scatter_tt(const DevMesh &m, const DevReq &q, T *Z, size_t N, int t, int s,
                            const Mom<T> &mo) {
     if constexpr (sizeof(T) == 4) {
-        scatter_rec<false>(Z, N, float(q.k0 * q.k0), load_tet_rec(q.etet, m.nt, t), load_tet_rec(q.etet, m.nt, s), mo,
+        scatter_rec<false>(Z, N, float(q.k0 * q.k0), load_tet_rec(q.etet, m.nt, t), load_tet_rec(q.etet, m.nt, s), mo, mo.S,
                            false);
         return;
     }
