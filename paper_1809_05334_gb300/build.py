@@ -7,7 +7,7 @@ VIE_NVCC_DEFINES (optional, space-separated -D flags) overrides the schedule
 constants that have a compile-time default, for sweeps, e.g.
     VIE_NVCC_DEFINES="-DVIE_GJ_RESERVE_WIDE=24" python -m paper_1809_05334_gb300.build --force
 (VIE_SPLIT_NORMAL, VIE_SPLIT_OBLIQUE, VIE_FAR_MINB, VIE_FAR_MINB_FULL,
-VIE_GJ_RESERVE, VIE_GJ_RESERVE_WIDE).  The defines are part of the staleness
+VIE_GJ_RESERVE, VIE_GJ_RESERVE_WIDE, VIE_GROUPS4_MIN, VIE_GROUPS2_MIN).  The defines are part of the staleness
 check: a build with other defines rebuilds.
 """
 import concurrent.futures
@@ -21,7 +21,7 @@ CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "libvie.so")
 BUILD = os.path.join(HERE, "_build")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["api.cu", "fill.cu", "far.cu", "linalg.cu", "krylov.cu", "mesh.cu", "post.cu", "topology.cpp", "rules.cpp", "server.cpp",
+SOURCES = ["api.cu", "fill.cu", "far.cu", "far64.cu", "linalg.cu", "krylov.cu", "mesh.cu", "post.cu", "topology.cpp", "rules.cpp", "server.cpp",
            "ewald_tables.cpp", "blocks.cpp"]
 
 

@@ -113,7 +113,7 @@ struct vie_ctx {
     std::string err;
     std::shared_ptr<MeshState> mesh = std::make_shared<MeshState>();
     // request (device)
-    DevBuf row, coef, wt, kap, ieps, frow, qs, perm, pol, orders, stab, ztab, rtab, ew, fcoef, frec;
+    DevBuf row, coef, wt, kap, ieps, frow, qs, perm, pol, orders, stab, ztab, rtab, ew, fcoef, frec, blob64, ph64;
     double z_extent = 0;
     // solve buffers
     DevBuf Z, b, x, r, u, w, V, h, y, Minv, MinvH, amax, tcpack, tcpack2, status, acc, J, rt, cout, xs;
@@ -203,6 +203,7 @@ struct HostReq {
     vie::EwaldTables ew;
     std::vector<double> orders;          // [n][4]: k_tx, k_ty, k_z, is (0,0)
     double pol[6], kinc[3];
+    bool fp64 = false;                   // tables of the FP64 series
 };
 
 int prepare(vie_ctx *ctx, const vie_request *req, HostReq &H) {
@@ -232,7 +233,7 @@ int prepare(vie_ctx *ctx, const vie_request *req, HostReq &H) {
     vie::domain_blocks(T, eps_abs, ctx->opt.precond_block_max, H.perm, H.blk_off, H.blk_n);
     // Ewald parameters and tables (Sec. 2.2) and the propagating Floquet orders
     const char *why = "";
-    const bool fp64 = ctx->opt.precision == VIE_FP64;
+    const bool fp64 = H.fp64 = ctx->opt.precision == VIE_FP64;
     const double split = ctx->tune_split[(H.kx == 0.0 && H.ky == 0.0) ? 0 : 1];
     if (int rc = vie::build_ewald_tables(T.a, T.b, H.k0, H.kx, H.ky, ctx->z_extent, fp64, H.ew, &H.orders, &why,
                                          split))
@@ -315,6 +316,16 @@ int upload_request(vie_ctx *ctx, const HostReq &H, vie::DevReq &q, cudaStream_t 
     q.etet = q.ptet + 16 * nt;
     q.pface = q.etet + 9 * nt;
     q.eface = q.pface + 12 * ((size_t)nf + 1);
+    if (H.fp64) {   // the far kernels' FP64 form
+        std::vector<double> blob;
+        vie::build_far64(H.ew, H.k0, H.kx, H.ky, q.f64, blob);
+        if (q.f64.n_blob > 0) {
+            CK(upload(ctx->blob64, blob, st));
+            CK(ctx->ph64.ensure(sizeof(double) * 8 * (4 * nt + 3 * (size_t)nf)));
+            q.blob64 = ctx->blob64.as<double>();
+            q.ph64 = ctx->ph64.as<double>();
+        }
+    }
     q.k0 = H.k0; q.kx = H.kx; q.ky = H.ky;
     for (int k = 0; k < 9; ++k) {
         const double phs = H.kx * (k / 3 - 1) * ctx->mesh->topo.a + H.ky * (k % 3 - 1) * ctx->mesh->topo.b;
@@ -2016,7 +2027,7 @@ void release_device_memory(vie_ctx *ctx) {
     ctx->mesh = std::make_shared<MeshState>();
     DevBuf *bufs[] = {&ctx->row, &ctx->coef, &ctx->wt, &ctx->kap, &ctx->ieps, &ctx->frow, &ctx->qs,
                       &ctx->perm, &ctx->pol, &ctx->orders, &ctx->stab, &ctx->ztab, &ctx->rtab, &ctx->ew,
-                      &ctx->fcoef, &ctx->frec, &ctx->pjobs, &ctx->pvec, &ctx->bstate,
+                      &ctx->fcoef, &ctx->frec, &ctx->blob64, &ctx->ph64, &ctx->pjobs, &ctx->pvec, &ctx->bstate,
                       &ctx->Z, &ctx->b, &ctx->x, &ctx->r, &ctx->u, &ctx->w, &ctx->V, &ctx->h, &ctx->y,
                       &ctx->Minv, &ctx->MinvH, &ctx->amax, &ctx->tcpack, &ctx->tcpack2, &ctx->status, &ctx->acc,
                       &ctx->J, &ctx->xs, &ctx->Zh, &ctx->dens,

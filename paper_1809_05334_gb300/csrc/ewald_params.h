@@ -99,6 +99,25 @@ struct FarPoly {
     // cancels there exactly; in FP32 the cancellation left a coherent rounding of this near-constant.
     float k_re, k_im;
 };
+// The FP64 series of the far kernels (far64.cu): the same orders, images and cut as
+// green_p, each order as a polynomial in t = t_scale z^2 - 1 and F(x) = exp(-x^2) Re
+// erfcx(x + j b) by F64_SPAT polynomials of degree F64_DEG.  The blob (doubles):
+//   at 0         spatial table [F64_SPAT + 1][F64_DEG + 1] (constant term first; the last entry zero)
+//   at img       images [n_img][4]: m a, n b, Re, Im of the phase exp(b^2) / (4 pi) exp(j k_par.R)
+//   at dir       per order (i, j), two doubles holding four ints: offset and degree of the
+//                real part's coefficients (highest power first), of the imaginary part's
+//                (degree -1: none); rows x cols
+// sym: normal incidence, the quadrant p, q >= 0 of orders with weights 1, 2 cos.
+constexpr int F64_SPAT = 128;
+constexpr int F64_DEG = 8;
+struct Far64 {
+    int n_blob;               // doubles; 0: not available (the series itself is summed)
+    int sym, rows, cols, n_img, img, dir;
+    int i0, j0;               // row and column of order (0, 0)
+    int near_img[9];
+    double t_scale, kx, ky, sx, sy, xs, e_mb2;   // xs: table intervals per unit distance
+    double E, bb, reg0;   // reg0: (F(RE) - F(0)) / R at R = 0
+};
 // Ewald splitting parameter: sqrt(pi / ab) balances the spatial and spectral
 // series, bounded below by k0/6 (b = k0 / 2E <= 3 keeps exp(b^2) moderate).  The
 // tabulated FP32 path makes the spectral terms cheaper than the images (table

@@ -4,6 +4,7 @@
 // FP32 tables.  Host code only (the library and the host-logic tests compile
 // it).
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <complex>
 #include <cstring>
@@ -308,6 +309,176 @@ void build_far_poly(const EwaldTables &t, const EwaldF32 &f, FarPoly &fp, std::v
         }
     }
     fp.mode = mode;
+}
+
+// ---------------------------------------------------------------------------
+// The FP64 form
+// ---------------------------------------------------------------------------
+namespace {
+
+// Chebyshev coefficients of f on [-1, 1] from M nodes
+using ld = long double;
+using cld = std::complex<long double>;
+const ld PI_L = 3.14159265358979323846264338327950288L;
+// as erfcx_host, with 64 terms in extended precision
+cld erfcx_ld(cld u) {
+    constexpr int NT = 64;
+    static const ld L = std::sqrt((ld)NT / std::sqrt((ld)2));
+    static const std::vector<ld> a = [] {
+        std::vector<ld> c(NT + 1, 0);
+        const int M = 16 * NT;
+        for (int k = 0; k < M; ++k) {
+            const ld th = -PI_L + (k + 0.5L) * 2 * PI_L / M, t = L * std::tan(th / 2), F = std::exp(-t * t) * (L * L + t * t);
+            for (int n = 0; n <= NT; ++n) c[n] += F * std::cos(n * th) / M;
+        }
+        return c;
+    }();
+    const cld inv = (ld)1 / (L + u), z = (L - u) * inv;
+    cld p = a[NT];
+    for (int n = NT - 1; n >= 1; --n) p = cld(p.real() * z.real() - p.imag() * z.imag() + a[n], p.real() * z.imag() + p.imag() * z.real());
+    return inv * ((ld)2 * p * inv + (ld)1 / std::sqrt(PI_L));
+}
+template <typename F> std::vector<ld> cheb_fit(int M, F &&f) {
+    std::vector<ld> v(M), c(M, 0);
+    for (int k = 0; k < M; ++k) {
+        const ld x = std::cos(PI_L * (k + 0.5L) / M), y = f(x);
+        ld t0 = 1, t1 = x;
+        for (int n = 0; n < M; ++n) {
+            c[n] += (n ? 2 : 1) * y * t0 / M;
+            const ld t2 = 2 * x * t1 - t0;
+            t0 = t1;
+            t1 = t2;
+        }
+    }
+    return c;
+}
+// the series up to degree d as a polynomial, constant term first
+std::vector<ld> cheb_poly(const std::vector<ld> &c, int d) {
+    std::vector<ld> out(d + 1, 0), a(d + 1, 0), b(d + 1, 0), n(d + 1);
+    a[0] = 1;
+    out[0] += c[0];
+    if (d >= 1) { b[1] = 1; out[1] += c[1]; }
+    for (int k = 2; k <= d; ++k) {
+        for (int q = 0; q <= d; ++q) n[q] = (q ? 2 * b[q - 1] : 0) - a[q];
+        for (int q = 0; q <= k; ++q) out[q] += c[k] * n[q];
+        a.swap(b);
+        b.swap(n);
+    }
+    return out;
+}
+
+}  // namespace
+
+void build_far64(const EwaldTables &t, double k0, double kx, double ky, Far64 &f, std::vector<double> &blob) {
+    f = Far64{};
+    blob.clear();
+    const double a = t.a, b = t.b, E = t.E, bb = t.bb, xc = FP64_XCUT, kmax = 2.0 * E * xc + k0;
+    const double zm = t.z_max, Ez = E * zm, ts = 2.0 / (zm * zm);
+    if (!(Ez < 6.0)) return;
+    int p0, np, q0, nq;
+    if (!mode_rect(kx, ky, a, b, kmax, p0, np, q0, nq) || np == 0) return;
+    const bool sym = kx == 0.0 && ky == 0.0 && 2 * p0 + np == 1 && 2 * q0 + nq == 1;
+    if (p0 > 0 || q0 > 0 || p0 + np <= 0 || q0 + nq <= 0) return;   // (0, 0) is always inside the cut
+    if (sym) { p0 = q0 = 0; np = (np + 1) / 2; nq = (nq + 1) / 2; }
+    // spatial kernel: F on [i h, (i + 1) h] in v = x / h - i
+    const double h = (xc + 0.5) / F64_SPAT;   // as the series: images up to the cut + 0.5
+    for (int i = 0; i < F64_SPAT; ++i) {
+        const std::vector<ld> c = cheb_fit(F64_DEG + 5, [&](ld u) {
+            const ld x = (i + (u + 1) / 2) * (ld)h;
+            return std::exp(-x * x) * erfcx_ld(cld(x, bb)).real();
+        });
+        // polynomial in u = 2 v - 1, shifted to v
+        const std::vector<ld> pu = cheb_poly(c, F64_DEG);
+        std::vector<ld> pv(F64_DEG + 1, 0);
+        for (int n = F64_DEG; n >= 0; --n) {   // Horner in (2 v - 1)
+            for (int q = F64_DEG; q >= 0; --q) pv[q] = (q ? 2 * pv[q - 1] : 0) - pv[q];
+            pv[0] += pu[n];
+        }
+        blob.insert(blob.end(), pv.begin(), pv.end());
+    }
+    blob.resize((size_t)(F64_SPAT + 1) * (F64_DEG + 1), 0.0);
+    f.img = (int)blob.size();
+    for (int i = 0; i < t.n_img; ++i) blob.insert(blob.end(), t.img64[i], t.img64[i] + 4);
+    f.dir = (int)blob.size();
+    blob.resize(blob.size() + 2 * (size_t)np * nq, 0.0);
+    const int M = std::min(64, (int)std::ceil(24 + 7 * Ez));
+    double g00 = 0;   // the size of the sum: the largest order at z = 0
+    struct Fit { double g2; std::vector<ld> re, im; };
+    std::vector<Fit> fits;   // per distinct decay constant
+    std::vector<int> which((size_t)np * nq, -1);
+    for (int i = 0; i < np; ++i)
+        for (int j = 0; j < nq; ++j) {
+            const double ktx = kx + 2 * M_PI * (p0 + i) / a, kty = ky + 2 * M_PI * (q0 + j) / b, kt2 = ktx * ktx + kty * kty;
+            if (std::sqrt(kt2) > kmax) continue;
+            const double g2 = kt2 - k0 * k0;
+            int k = 0;
+            while (k < (int)fits.size() && std::fabs(fits[k].g2 - g2) > 1e-12 * std::max(1e-6, std::fabs(g2))) ++k;
+            which[(size_t)i * nq + j] = k;
+            if (k < (int)fits.size()) continue;
+            const ld kx_ = (ld)kx + 2 * PI_L * (p0 + i) / a, ky_ = (ld)ky + 2 * PI_L * (q0 + j) / b, g2l = kx_ * kx_ + ky_ * ky_ - (ld)k0 * k0;
+            const ld gr = g2l >= 0 ? std::sqrt(g2l) : 0, gi = g2l >= 0 ? 0 : std::sqrt(-g2l), El = E;
+            const ld pre0 = std::exp(-g2l / (4 * El * El)), zs = std::sqrt((ld)2 / (ld)ts);
+            auto value = [&](ld u) {
+                const ld z = zs * std::sqrt(std::max((ld)0, (u + 1) / 2));
+                if (gi == 0) {
+                    const ld w = gr / (2 * El);
+                    return cld((std::exp(gr * z) * std::erfc(w + z * El) + std::exp(-gr * z) * std::erfc(w - z * El)) / (4 * (ld)a * b * gr), 0);
+                }
+                const cld e1 = erfcx_ld(cld(z * El, gi / (2 * El)));
+                const ld pre = pre0 * std::exp(-(z * El) * (z * El));
+                return cld(2 * std::cos(gi * z), 2 * pre * e1.imag() - 2 * std::sin(gi * z)) / cld(0, 4 * (ld)a * b * gi);
+            };
+            Fit fit{g2, cheb_fit(M, [&](ld u) { return value(u).real(); }), {}};
+            if (gi > 0) fit.im = cheb_fit(M, [&](ld u) { return value(u).imag(); });
+            g00 = std::max(g00, (double)std::abs(value(-1)));
+            fits.push_back(std::move(fit));
+        }
+    if (!(g00 > 0) || !std::isfinite(g00)) { blob.clear(); return; }
+    // up to the last term that stands out of the rounding of the fit (the level of its
+    // last terms); M if it has not converged to 1e-13 of the largest order
+    auto degree = [&](const std::vector<ld> &c) {
+        ld rest = 0;
+        int d = M - 1;
+        while (d > 0 && rest + std::fabs(c[d]) <= 2e-17L * g00) rest += std::fabs(c[d--]);
+        return d >= M - 1 ? M : d;
+    };
+    std::vector<std::array<int, 4>> at(fits.size());
+    for (size_t k = 0; k < fits.size(); ++k) {
+        at[k] = {0, -1, 0, -1};
+        for (int part = 0; part < 2; ++part) {
+            const std::vector<ld> &c = part ? fits[k].im : fits[k].re;
+            if (c.empty()) continue;
+            const int d = degree(c);
+            if (d >= M) { blob.clear(); return; }
+            const std::vector<ld> q = cheb_poly(c, d);
+            at[k][2 * part] = (int)blob.size();
+            at[k][2 * part + 1] = d;
+            blob.insert(blob.end(), q.rbegin(), q.rend());
+        }
+    }
+    for (size_t e = 0; e < which.size(); ++e) {
+        const std::array<int, 4> v = which[e] >= 0 ? at[which[e]] : std::array<int, 4>{0, -1, 0, -1};
+        std::memcpy(&blob[f.dir + 2 * e], v.data(), sizeof(v));
+    }
+    if (blob.size() > 4096) { blob.clear(); return; }   // 32 KB of shared memory
+    f.sym = sym;
+    f.rows = np;
+    f.cols = nq;
+    f.n_img = t.n_img;
+    for (int k = 0; k < 9; ++k) f.near_img[k] = t.near_img[k];
+    f.t_scale = ts;
+    f.sx = 2 * M_PI / a;
+    f.sy = 2 * M_PI / b;
+    f.i0 = -p0;
+    f.j0 = -q0;
+    f.kx = kx;
+    f.ky = ky;
+    f.xs = E / h;
+    f.e_mb2 = std::exp(-bb * bb);
+    f.E = E;
+    f.bb = bb;
+    f.reg0 = 4.0 * M_PI * f.e_mb2 * t.reg0_re;
+    f.n_blob = (int)blob.size();
 }
 
 }  // namespace vie

@@ -20,5 +20,8 @@ int build_ewald_tables(double a, double b, double k0, double kx, double ky, doub
 // thick); then the general tabulated form is used.  coef receives fp.n_coef
 // floats.
 void build_far_poly(const EwaldTables &t, const EwaldF32 &f, FarPoly &fp, std::vector<float> &coef);
+// The FP64 form of a request whose tables were built with fp64 = true; f.n_blob = 0
+// where it does not apply (an order of too high a degree, or too large a blob).
+void build_far64(const EwaldTables &t, double k0, double kx, double ky, Far64 &f, std::vector<double> &blob);
 
 }  // namespace vie

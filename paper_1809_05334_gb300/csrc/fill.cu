@@ -58,6 +58,8 @@ cudaError_t upload_constants() {
     for (int n = 0; n <= NW32; ++n) w.a32[n] = (float)a[n];
     cudaError_t e = cudaMemcpyToSymbol(c_weid, &w, sizeof(w));
     if (e != cudaSuccess) return e;
+    e = upload_far64_constants(&w);   // far64.cu's own copy of c_weid
+    if (e != cudaSuccess) return e;
     double w5t[14], w5f[7];
     tet_rule5(nullptr, w5t);
     tri_rule5(nullptr, w5f);
@@ -747,6 +749,10 @@ void far_scalar(bool sym, dim3 grid, size_t sm, cudaStream_t st, const DevMesh &
         if (sym) k_far_scalar<T, PK, true><<<grid, 128, sm, st>>>(m, q, Z, N, nx, ny, mk);
         else k_far_scalar<T, PK, false><<<grid, 128, sm, st>>>(m, q, Z, N, nx, ny, mk);
     } else {
+        if (q.f64.n_blob > 0) {
+            launch_far64_scalar(PK, m, q, Z, N, st);
+            return;
+        }
         k_far_scalar<T, PK, false><<<grid, 128, sm, st>>>(m, q, Z, N, nx, ny, mk);
     }
     ++g_launches;
@@ -763,6 +769,7 @@ cudaError_t launch_fill(const DevMesh &m, const DevReq &q, T *Z, size_t ld, doub
     k_gram<T><<<(m.nt + 127) / 128, blk, 0, st>>>(m, q, Z, N); ++g_launches;
     if (b) { k_rhs<<<(m.nt + 127) / 128, blk, 0, st>>>(m, q, b); ++g_launches; }
     if (sizeof(T) == 4) launch_far_prep(m, q, st);   // element records of the FP32 kernels
+    else if (q.f64.n_blob > 0) launch_far64_prep(m, q, st);
     const size_t sm = stab_bytes<T>();
     if (far0) cudaEventRecord(far0, st);
     const bool sym = sizeof(T) == 4 && q.ef.sym;   // normal incidence: the symmetric tabulated path
@@ -775,6 +782,8 @@ cudaError_t launch_fill(const DevMesh &m, const DevReq &q, T *Z, size_t ld, doub
             else k_far_tt<T, false><<<gtt, blk, sm, st>>>(m, q, Z, N);
             ++g_launches;
         }
+    } else if (q.f64.n_blob > 0) {
+        launch_far64_tt(m, q, Z, N, st);
     } else {
         k_far_tt<T, false><<<dim3((m.nt + 127) / 128, m.nt), blk, sm, st>>>(m, q, Z, N);
         ++g_launches;

@@ -86,6 +86,9 @@ struct DevReq {
     // element records of the FP32 kernels, built per request (k_far_prep): points
     // [4 FPT][nt] and [3 FPT][nf], elements [FEL_TET][nt] and [FEL_FACE][nf]
     float4 *ptet, *pface, *etet, *eface;
+    Far64 f64;             // the FP64 series as polynomials (f64.n_blob 0: summed term by term)
+    const double *blob64;
+    double *ph64;          // phases of the points, [8] per point: tetrahedra [nt][4], faces [nf][3]
 };
 
 // degree-5 rules: barycentric points [14][4] / [7][3] (may be null) and weights
@@ -117,6 +120,11 @@ cudaError_t launch_static_cache(const DevMesh &m, double *touch_half, double *co
 cudaError_t launch_far_prep(const DevMesh &m, const DevReq &q, cudaStream_t st);
 cudaError_t launch_far_tt(const DevMesh &m, const DevReq &q, float *Z, size_t N, cudaStream_t st);
 cudaError_t launch_far_scalar(int pk, const DevMesh &m, const DevReq &q, float *Z, size_t N, cudaStream_t st);
+// the same in FP64 (q.f64.n_blob > 0): phases of the points, tetrahedron pairs, pairs with faces
+cudaError_t upload_far64_constants(const void *weideman);
+cudaError_t launch_far64_prep(const DevMesh &m, const DevReq &q, cudaStream_t st);
+cudaError_t launch_far64_tt(const DevMesh &m, const DevReq &q, double *Z, size_t N, cudaStream_t st);
+cudaError_t launch_far64_scalar(int pk, const DevMesh &m, const DevReq &q, double *Z, size_t N, cudaStream_t st);
 // g_p at single displacements in the polynomial form
 cudaError_t launch_green_poly(const double *d, double *out, int n, const DevReq &q, cudaStream_t st);
 cudaError_t launch_erfcx(const double *u, double *out, int n, bool fp64, cudaStream_t st);

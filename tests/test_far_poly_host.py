@@ -145,3 +145,103 @@ def test_too_thick_a_cell_is_left_to_the_tabulated_form(harness):
     out = subprocess.run([harness, "40", "40", "500", "0", "0", "300"], check=True, capture_output=True, text=True).stdout
     t = json.loads(out)
     assert t["mode"] == 0 and t["n"] == 0
+
+
+HARNESS64 = r"""
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include "ewald_tables.h"
+using namespace vie;
+int main(int argc, char **argv) {
+    const double a = atof(argv[1]), b = atof(argv[2]), lam = atof(argv[3]), th = atof(argv[4]), ph = atof(argv[5]);
+    const double z = atof(argv[6]), k0 = 6.283185307179586 / lam, kx = k0 * sin(th) * cos(ph), ky = k0 * sin(th) * sin(ph);
+    static EwaldTables E;
+    const char *why = "";
+    if (build_ewald_tables(a, b, k0, kx, ky, z, true, E, nullptr, &why)) return 1;
+    Far64 f;
+    std::vector<double> c;
+    build_far64(E, k0, kx, ky, f, c);
+    printf("{\"n\": %d, \"sym\": %d, \"rows\": %d, \"cols\": %d, \"n_img\": %d, \"ts\": %.17g, \"kx0\": %.17g, \"ky0\": %.17g, "
+           "\"xs\": %.17g, \"E\": %.17g, \"k0\": %.17g, \"bb\": %.17g, \"kx\": %.17g, \"ky\": %.17g, \"n_mode\": %d, \"dir\": [",
+           f.n_blob, f.sym, f.rows, f.cols, f.n_img, f.t_scale, kx - f.i0 * f.sx, ky - f.j0 * f.sy, f.xs, E.E, k0, E.bb, kx, ky, E.n_mode);
+    for (int i = 0; i < f.rows * f.cols; ++i) {
+        int v[4];
+        memcpy(v, &c[f.dir + 2 * i], sizeof(v));
+        printf("%s[%d,%d,%d,%d]", i ? "," : "", v[0], v[1], v[2], v[3]);
+    }
+    printf("], \"c\": [");
+    for (int i = 0; i < 2 * f.rows * f.cols; ++i) c[f.dir + i] = 0;   // ints, printed above
+    for (int i = 0; i < f.n_blob; ++i) printf("%s%.17g", i ? "," : "", c[i]);
+    printf("]}\n");
+    return 0;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def harness64(tmp_path_factory):
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if cxx is None:
+        pytest.skip("no C++ compiler")
+    d = tmp_path_factory.mktemp("far64")
+    (d / "h.cpp").write_text(HARNESS64)
+    exe = d / "h"
+    subprocess.run([cxx, "-O1", "-std=c++17", "-I", CSRC, str(d / "h.cpp"), os.path.join(CSRC, "ewald_tables.cpp"),
+                    "-o", str(exe)], check=True)
+    return str(exe)
+
+
+@pytest.mark.parametrize("case", [(200.0, 200.0, 500.0, 0.0, 0.0, 140.0), (150.0, 120.0, 430.0, 0.0, 0.0, 90.0),
+                                  (40.0, 40.0, 400.0, 0.0, 0.0, 80.0), (200.0, 200.0, 500.0, 0.5, 0.0, 0.5),
+                                  (180.0, 150.0, 430.0, 0.6, 0.3, 100.0), (400.0, 400.0, 650.0, 0.9, 1.1, 160.0)])
+def test_fp64_form_reproduces_the_series(harness64, case):
+    """The FP64 orders and spatial kernel against their closed forms: 2e-13 of the
+    summed orders (the 40-term Faddeeva expansion behind the propagating orders and
+    F carries 3e-14, Horner and the dropped terms a few 1e-16 each)."""
+    out = subprocess.run([harness64] + ["%r" % v for v in case], check=True, capture_output=True, text=True).stdout
+    t = json.loads(out)
+    a, b, _, _, _, zmax = case
+    assert t["n"] > 0 and t["sym"] == (case[3] == 0.0)
+    c = np.array(t["c"])
+    rng = np.random.default_rng(5)
+    for z in [0.0, zmax] + list(rng.uniform(0, zmax, 4)):
+        dx, dy = rng.uniform(-1, 1, 2) * np.array([a, b])
+        tt = t["ts"] * z * z - 1.0
+        g = ref = 0j
+        size = 0.0
+        for i in range(t["rows"]):
+            for j in range(t["cols"]):
+                ro, rd, io, idg = t["dir"][i * t["cols"] + j]
+                G = 0j
+                if rd >= 0:
+                    G += np.polyval(c[ro:ro + rd + 1], tt)
+                if idg >= 0:
+                    G += 1j * np.polyval(c[io:io + idg + 1], tt)
+                if t["sym"]:
+                    w = (1 if i == 0 else 2 * np.cos(2 * np.pi * i / a * dx)) * (1 if j == 0 else 2 * np.cos(2 * np.pi * j / b * dy))
+                    p, q = i, j
+                else:
+                    w = np.exp(-1j * ((t["kx0"] + 2 * np.pi * i / a) * dx + (t["ky0"] + 2 * np.pi * j / b) * dy))
+                    p = i + int(round((t["kx0"] - t["kx"]) * a / (2 * np.pi)))
+                    q = j + int(round((t["ky0"] - t["ky"]) * b / (2 * np.pi)))
+                g += w * G
+                if rd >= 0:
+                    R = _order(t, a, b, p, q, z)[0]
+                    ref += w * R
+                    size += abs(w) * abs(_order(t, a, b, p, q, 0.0)[0])
+        assert abs(g - ref) <= 2e-13 * size, (case, z, abs(g - ref) / size)
+    # every order inside the cut is there
+    kmax = 2.0 * t["E"] * 6.0 + t["k0"]
+    n = sum(1 for p in range(-40, 41) for q in range(-40, 41)
+            if np.hypot(t["kx"] + 2 * np.pi * p / a, t["ky"] + 2 * np.pi * q / b) <= kmax)
+    have = sum((4 if i and j else 2 if i or j else 1) if t["sym"] else 1
+               for i in range(t["rows"]) for j in range(t["cols"]) if t["dir"][i * t["cols"] + j][1] >= 0)
+    assert have == n
+    # spatial kernel F(x) = exp(-x^2) Re erfcx(x + j b)
+    x = rng.uniform(0, 6.49, 400)
+    u = x * t["xs"] / t["E"]
+    i = u.astype(int)
+    F = np.array([np.polyval(c[9 * k:9 * k + 9][::-1], v - k) for k, v in zip(i, u)])
+    ref = np.exp(-x * x) * wofz(1j * (x + 1j * t["bb"])).real
+    assert np.max(np.abs(F - ref)) <= 2e-13
