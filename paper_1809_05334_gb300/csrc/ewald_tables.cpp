@@ -383,10 +383,38 @@ void build_far64(const EwaldTables &t, double k0, double kx, double ky, Far64 &f
     // spatial kernel: F on [i h, (i + 1) h] in v = x / h - i
     const double h = (xc + 0.5) / F64_SPAT;   // as the series: images up to the cut + 0.5
     for (int i = 0; i < F64_SPAT; ++i) {
-        const std::vector<ld> c = cheb_fit(F64_DEG + 5, [&](ld u) {
-            const ld x = (i + (u + 1) / 2) * (ld)h;
-            return std::exp(-x * x) * erfcx_ld(cld(x, bb)).real();
-        });
+        // F = Re y with y' = 2 j b y - (2 / sqrt pi) exp(-x^2): one value of y at the middle of
+        // the interval and its Taylor terms by recurrence, then the Chebyshev terms of that
+        // (13 values of y per interval, on a host whose extended precision is in software,
+        // were 16 ms a request)
+        constexpr int NT = 14;   // (h / 2)^15 < 1e-23
+        const ld x = (i + 0.5L) * (ld)h, hh = (ld)h / 2, r = 2 / std::sqrt(PI_L);
+        cld y = std::exp(-x * x) * erfcx_ld(cld(x, bb));
+        ld g0 = 0, g1 = std::exp(-x * x);   // terms of exp(-x^2), n - 1 and n
+        std::vector<ld> tay(NT + 1), c(NT + 1, 0);
+        ld p = 1;
+        for (int n = 0; n <= NT; ++n) {
+            tay[n] = y.real() * p;   // in u: x = centre + u h / 2
+            p *= hh;
+            y = (cld(-2 * (ld)bb * y.imag(), 2 * (ld)bb * y.real()) - r * g1) / (ld)(n + 1);
+            const ld g2 = -2 * (x * g1 + g0) / (n + 1);
+            g0 = g1;
+            g1 = g2;
+        }
+        // Chebyshev series by Horner in u: u T_k = (T_{k+1} + T_{k-1}) / 2
+        std::vector<ld> w(NT + 2);
+        for (int n = NT; n >= 0; --n) {
+            std::fill(w.begin(), w.end(), (ld)0);
+            for (int k = 0; k < NT - n; ++k) {   // degree so far
+                if (k == 0) w[1] += c[0];
+                else {
+                    w[k + 1] += c[k] / 2;
+                    w[k - 1] += c[k] / 2;
+                }
+            }
+            w[0] += tay[n];
+            c.assign(w.begin(), w.begin() + NT + 1);
+        }
         // polynomial in u = 2 v - 1, shifted to v
         const std::vector<ld> pu = cheb_poly(c, F64_DEG);
         std::vector<ld> pv(F64_DEG + 1, 0);

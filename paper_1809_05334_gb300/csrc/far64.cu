@@ -2,7 +2,7 @@
 // as polynomials and the spatial kernel from a table of polynomials (Far64,
 // ewald_params.h), both fitted on the host in extended precision: against 32-digit
 // values of g_p at six cells its rms error is 0.29 to 0.67 of the series' own (fitted in
-// FP64: up to 3.6).  6 x 6 x 2 slab, FP64: 273 -> 39 ms a solve.  Bound by the
+// FP64: up to 3.6).  6 x 6 x 2 slab, FP64: 273 -> 27 ms a solve.  Bound by the
 // FP64 pipe (1/64 of the FP32 rate): what counts is FP64 instructions per
 // evaluation.  Summed term by term (green_p) each Floquet order takes two
 // 40-term Faddeeva expansions, an exponential and a sincos, each image one complex
