@@ -544,11 +544,12 @@ def run_ours(args):
 # (4860 tets), lambda = 500 nm, at the default Ewald split (the series has the
 # same terms per value for every cell of this period, wavelength and incidence
 # class): executed warp instructions and FP32 operations (2 FFMA + FADD + FMUL,
-# thread level).  Normal incidence: k_far_tt_n (split 1.5); oblique incidence
-# at theta = 0.3 rad, phi = 0: k_far_tt_o, the k_y = 0 fold (split 1.0).  With
+# thread level; as the counters report them, which count a packed two-lane
+# instruction at most once, so the FP32 rate is a lower bound).  k_far_tt_p: normal
+# incidence (split 1.5), and the k_y = 0 fold at theta = 0.3 rad (split 1.0).  With
 # another split (the autotuner's choice) the counts do not apply and the
 # issue-rate figures are left out.
-FAR_COUNTS = {"normal": (13.61, 279.2, 1.5), "oblique": (34.09, 512.2, 1.0)}
+FAR_COUNTS = {"normal": (8.76, 98.5, 1.5), "oblique": (12.25, 136.9, 1.0)}
 FAR_SPLIT_CHOSEN = None   # set by the main leg from its autotune report
 SMS, FP32_LANES, SCHEDULERS = 152, 128, 4
 MATVEC_Z_TRAFFIC = 3.5527e9   # DRAM read + write per FP32 Z product, 21,024 unknowns (ncu)
@@ -560,7 +561,8 @@ Z_BYTES = {0: 16, 1: 8, 2: 4, 3: 4}   # bytes per complex entry of the Z the GMR
 def roofline(last, n, peaks, prec, n_tets):
     """Roofline of the dominant kernel (largest device time in the solve), plus the others.
 
-    k_far_tt (far tetrahedron pairs of the fill): instruction-issue bound ("alu");
+    k_far_tt (far tetrahedron pairs of the fill): against the instruction-issue rate ("alu";
+    the shared-memory table reads bind first, L1 at 83% busy);
     achieved = warp instructions per value (FAR_COUNTS) x 16 n_tets^2 values / event time, against
     152 SMs x 4 schedulers x 1 warp instruction per clock x the maximum SM
     clock; the FP32 rate (FAR_COUNTS) is reported beside it.

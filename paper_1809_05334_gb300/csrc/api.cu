@@ -2,8 +2,9 @@
 //
 // vie_solve runs, on the caller's stream:
 //   fill   Eq. (2) with the Ewald-summed periodic Green's function (Sec. 2.2)
-//   factor the inverse of every domain block A_dd of Eq. (5)-(6)
-//   solve  GMRES on diag(A_dd^-1) Z x = diag(A_dd^-1) b, restarted; every restart
+//   factor the inverse of every domain block A_dd of Eq. (5)-(6), large blocks as a
+//          block-triangular factor with inverted diagonal groups
+//   solve  block GMRES over TE and TM on diag(A_dd^-1) Z x = diag(A_dd^-1) b, restarted; every restart
 //          recomputes the FP64 residual b - Z x (iterative refinement)
 //   post   absorbed fraction per domain (Eq. (7)), reflectance, transmittance
 #include <cuda_bf16.h>

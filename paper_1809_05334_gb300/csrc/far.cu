@@ -7,11 +7,11 @@
 
 namespace vie {
 
-// CTAs per SM of the tetrahedron-pair kernels (bench cell, 21,024 unknowns): at
-// normal incidence and in the fold 128 registers and four CTAs (18.4 / 24.9 ms;
-// three 18.5 / 26.8, five 18.5 / 27.1, spilling); the full rectangle keeps the
-// complex columns of four test points in 168 registers (31.9 ms; two points at a
-// time in 128: 34.2)
+// CTAs per SM of the tetrahedron-pair kernels (bench cell, 21,024 unknowns; compared
+// before the image cut and the scatter took their present form): at normal incidence
+// and in the fold 128 registers and four CTAs (18.4 / 24.9 ms; three 18.5 / 26.8,
+// five 18.5 / 27.1, spilling); the full rectangle keeps the complex columns of four
+// test points in 168 registers (31.9 ms; two points at a time in 128: 34.2)
 #ifndef VIE_FAR_MINB
 #define VIE_FAR_MINB 4
 #endif
@@ -85,11 +85,11 @@ __global__ void __launch_bounds__(128) k_far_prep(DevMesh m, const __grid_consta
 // blocks from the same 16 evaluations.  Four test points against one source
 // point per step: they share the coefficient and image loads, and the moments
 // factor (sums over the test points first).  Bound by L1: the gathers of the
-// spatial table (5.7-way conflicts, 55% of the wavefronts) at 77% busy, 56% of
-// the issue slots.  Measured (ms, far tetrahedron pairs; per-lane spectral table
-// entries, single points and scalar atomics before): 21,024 unknowns 37.3 ->
-// 18.2 at normal incidence, 59.3 -> 24.9 in the fold, 82.6 -> 31.9 full
-// rectangle; 48,678 unknowns 223 -> 90.
+// spatial table, 83% busy, 56% of the issue slots (9,882 unknowns, normal incidence).
+// Measured (ms, far tetrahedron pairs; per-lane spectral table entries, single
+// points and scalar atomics before): 21,024 unknowns 37.3 -> 19.8 at normal
+// incidence, 59.3 -> 26.6 in the fold, 82.6 -> 33.7 full rectangle; 48,678
+// unknowns 223 -> 98.
 // ---------------------------------------------------------------------------
 template <int MODE, int NQ>
 __global__ void __launch_bounds__(FAR_THREADS, MODE == FAR_FULL ? VIE_FAR_MINB_FULL : VIE_FAR_MINB)
