@@ -127,9 +127,7 @@ typedef struct {
 typedef struct {
     int32_t status;                      /* vie_status of the solve                 */
     int32_t n_unknowns;
-    int32_t iterations[2];               /* GMRES iterations, TE and TM (one Krylov space
-                                            serves both: block iterations until each
-                                            converged; VIE_FP64: each its own)       */
+    int32_t iterations[2];               /* GMRES iterations, TE and TM             */
     int32_t refinements;                 /* outer FP64 refinement sweeps            */
     double  rel_residual[2];             /* final FP64 ||b - Z x|| / ||b||          */
     double  absorbed[2][VIE_MAX_DOMAINS];/* fraction of incident power per domain   */

@@ -4,14 +4,13 @@
 //   fill   Eq. (2) with the Ewald-summed periodic Green's function (Sec. 2.2)
 //   factor the inverse of every domain block A_dd of Eq. (5)-(6), large blocks as a
 //          block-triangular factor with inverted diagonal groups
-//   solve  block GMRES over TE and TM on diag(A_dd^-1) Z x = diag(A_dd^-1) b, restarted; every restart
+//   solve  GMRES on diag(A_dd^-1) Z x = diag(A_dd^-1) b, restarted; every restart
 //          recomputes the FP64 residual b - Z x (iterative refinement)
 //   post   absorbed fraction per domain (Eq. (7)), reflectance, transmittance
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <array>
 #include <chrono>
 #include <cmath>
 #include <complex>
@@ -123,7 +122,7 @@ struct vie_ctx {
     // the preconditioner's steps on the FP16 block factors: jobs (device), and per
     // step the first job, the number of jobs and their work units
     DevBuf pjobs, pvec;
-    DevBuf bstate;   // device state of the block GMRES iteration (krylov.cu)
+    DevBuf kstate;   // device state of the GMRES iteration of the mixed paths (krylov.cu)
     PinBuf pin;      // its messages
     unsigned long long seq = 0;
     std::vector<vie::PrecondJob> hjobs;
@@ -457,65 +456,19 @@ int residual(vie_ctx *ctx, bool x_zero, const double b_raw[2], double rn[2], dou
     return VIE_OK;
 }
 
-// Least-squares problem of block GMRES: the block Hessenberg matrix reduced by
-// Givens rotations as its columns arrive, both right-hand sides.  A basis block
-// counts the columns it really has (a converged right-hand side, or a dependent
-// direction, leaves a zero column: neither a row nor a column here), so a new
-// column reaches one or two rows below the triangle; they are rotated up into the
-// diagonal pairwise from the last.
-struct BlockQR {
-    struct Rot { int i; cplx c, s; };   // rows i, i + 1
-    std::vector<std::vector<cplx>> T;   // columns of the triangular factor
-    std::vector<Rot> rot;
-    std::vector<std::array<cplx, 2>> g; // right-hand sides
-    static void apply(const Rot &r, cplx &x, cplx &y) {
-        const cplx t = std::conj(r.c) * x + std::conj(r.s) * y;
-        y = -r.s * x + r.c * y;
-        x = t;
-    }
-    void column(std::vector<cplx> h) {   // all rows of the basis so far
-        const int c = (int)T.size();
-        while (g.size() < h.size()) g.push_back({});
-        for (const Rot &r : rot) apply(r, h[r.i], h[r.i + 1]);
-        for (int i = (int)h.size() - 2; i >= c; --i) {
-            const double den = std::hypot(std::abs(h[i]), std::abs(h[i + 1]));
-            if (!(den > 0)) continue;
-            rot.push_back({i, h[i] / den, h[i + 1] / den});
-            h[i] = den;
-            h[i + 1] = 0;
-            for (int p = 0; p < 2; ++p) apply(rot.back(), g[i][p], g[i + 1][p]);
-        }
-        h.resize(c + 1);
-        T.push_back(std::move(h));
-    }
-    double residual(int p) const {   // after whole blocks of columns
-        double s = 0;
-        for (size_t i = T.size(); i < g.size(); ++i) s += std::norm(g[i][p]);
-        return std::sqrt(s);
-    }
-    std::vector<cplx> solve(int p) const {
-        const int n = (int)T.size();
-        std::vector<cplx> y(n);
-        for (int i = n - 1; i >= 0; --i) {
-            cplx s = g[i][p];
-            for (int j = i + 1; j < n; ++j) s -= T[j][i] * y[j];
-            y[i] = std::abs(T[i][i]) > 0 ? s / T[i][i] : cplx(0);
-        }
-        return y;
-    }
-};
-
-// Left-preconditioned block GMRES(m) on diag(A_dd^-1) Z x = diag(A_dd^-1) b of the
-// mixed paths (FP32 vectors): TE and TM span one Krylov space, so every product
-// with Z and with the preconditioner, which reads the matrix once for both columns
-// anyway, enlarges the space of each by two: 20 to 35 % fewer iterations than one
-// space per polarisation.  Inside FP64-residual iterative refinement: each sweep
-// starts from r = b - Z x formed at double length.  The sweep's products read Z
-// itself, or its 16-bit copy ctx->Zh for VIE_FP16 / VIE_BF16.
+// Left-preconditioned GMRES(m) on diag(A_dd^-1) Z x = diag(A_dd^-1) b of the mixed
+// paths (FP32 vectors) for TE and TM together, one Krylov space each (every product
+// reads Z once for both), inside FP64-residual iterative refinement: each sweep starts
+// from r = b - Z x formed at double length.  The sweep's products read Z itself, or its
+// 16-bit copy ctx->Zh for VIE_FP16 / VIE_BF16.
+// One space over both right-hand sides takes 20 to 35 % fewer iterations, but stops
+// elsewhere: where it meets the same residual, the currents of an ill-conditioned cell
+// (3,096 unknowns, BF16 products) lie 6.0e-5 from where separate spaces stop, each 3 to
+// 4e-5 from the converged solution.
 // The iteration runs on the device (krylov.cu); the host reads the Hessenberg
-// column of one iteration while the next one runs, and stays ahead of the device
+// columns of one iteration while the next one runs, and stays ahead of the device
 // unless the residual's last reduction says that this iteration is the sweep's last.
-int gmres_block(vie_ctx *ctx, const std::vector<size_t> &mld, const HostReq &H, vie_result *res, cudaStream_t st,
+int gmres_mixed(vie_ctx *ctx, const std::vector<size_t> &mld, const HostReq &H, vie_result *res, cudaStream_t st,
                 Timing &tm) {
     const int N = ctx->mesh->topo.N;
     const int m = std::max(2, ctx->opt.restart);
@@ -524,19 +477,19 @@ int gmres_block(vie_ctx *ctx, const std::vector<size_t> &mld, const HostReq &H, 
     const int zin = ctx->opt.precision == VIE_FP16 ? 1 : ctx->opt.precision == VIE_BF16 ? 2 : 0;
     const double inner_def = zin == 1 ? INNER_TOL_FP16 : zin == 2 ? INNER_TOL_BF16 : INNER_TOL_FP32;
     const double inner_tol = std::max(ctx->opt.inner_tol > 0 ? ctx->opt.inner_tol : inner_def, 1e-6);
-    const size_t vs = 4 * vie::pad_cols(N);     // stride of one basis block (two columns, zero past N)
+    const size_t vs = 4 * vie::pad_cols(N);     // stride of one basis vector (two rhs, zero past N)
     const size_t used = 4 * (size_t)N;
     const int mvg = ctx->tune_mv > 0 ? ctx->tune_mv : 1;   // launch shape of the Z products
-    const size_t msg = vie::block_message_doubles(m);
+    const size_t msg = vie::krylov_message_doubles(m);
     constexpr int RING = 4;
     CK(ctx->x.ensure(sizeof(double) * used));
     CK(ctx->r.ensure(sizeof(double) * used));
     CK(ctx->u.ensure(sizeof(float) * vs));
     CK(ctx->V.ensure(sizeof(float) * vs * (m + 1)));
     CK(ctx->h.ensure(sizeof(double) * 4));
-    CK(ctx->y.ensure(sizeof(double) * 8 * (m + 1)));
+    CK(ctx->y.ensure(sizeof(double) * 4 * (m + 1)));
     CK(ctx->xs.ensure(sizeof(float) * 8 * (size_t)N));
-    CK(ctx->bstate.ensure(vie::block_state_bytes(m)));
+    CK(ctx->kstate.ensure(vie::krylov_state_bytes(m)));
     CK(ctx->pin.ensure(sizeof(double) * (8 + RING * msg)));
     if (pre) {
         CK(ctx->pvec.ensure(sizeof(float) * 2 * vs));
@@ -547,7 +500,7 @@ int gmres_block(vie_ctx *ctx, const std::vector<size_t> &mld, const HostReq &H, 
     double *pin = static_cast<double *>(ctx->pin.p), *ring = pin + 8;
     double *x = ctx->x.as<double>();
     float *u = ctx->u.as<float>(), *V = ctx->V.as<float>();
-    void *state = ctx->bstate.p;
+    void *state = ctx->kstate.p;
     CK(cudaMemsetAsync(x, 0, sizeof(double) * used, st));
     double bn[2];
     {
@@ -560,11 +513,11 @@ int gmres_block(vie_ctx *ctx, const std::vector<size_t> &mld, const HostReq &H, 
     }
     const double b_raw[2] = {bn[0], bn[1]};
     for (int p = 0; p < 2; ++p) if (!(bn[p] > 0)) bn[p] = 1.0;
-    // the message of one block: its place in the ring, and the wait for it
+    // the message of one vector: its place in the ring, and the wait for it
+    const size_t tail_at = 8 * (size_t)(m + 1);
     auto slot = [&](unsigned long long q) { return ring + (q % RING) * msg; };
     auto wait = [&](unsigned long long q) -> int {
-        const volatile unsigned long long *w =
-            reinterpret_cast<const volatile unsigned long long *>(slot(q) + 16 * (size_t)(m + 1) + 8);
+        const volatile unsigned long long *w = reinterpret_cast<const volatile unsigned long long *>(slot(q) + tail_at + 4);
         for (long long spin = 1; *w != q; ++spin) {
             if (spin % 2048) continue;
             const cudaError_t e = cudaStreamQuery(st);
@@ -575,41 +528,12 @@ int gmres_block(vie_ctx *ctx, const std::vector<size_t> &mld, const HostReq &H, 
         std::atomic_thread_fence(std::memory_order_acquire);
         return VIE_OK;
     };
-    struct Small { cplx a[2][2]; };
-    auto mul = [](const Small &A, const Small &B) {
-        Small C;
-        for (int i = 0; i < 2; ++i)
-            for (int j = 0; j < 2; ++j) C.a[i][j] = A.a[i][0] * B.a[0][j] + A.a[i][1] * B.a[1][j];
-        return C;
-    };
-    std::vector<Small> R, Ri;   // Cholesky factor of every basis block's Gram matrix and its inverse
-    std::vector<std::array<int, 2>> row;   // compact row (and column) of every basis column, -1 for a zero column
-    int rows = 0;
-    // the factor of the block a message describes; returns R T (T: column 0 taken out of column 1)
-    auto factor_of = [&](const double *tail) {
-        const double i11 = tail[0] > 0 ? 1.0 / std::sqrt(tail[0]) : 0.0;
-        const cplx r12 = cplx(tail[2], tail[3]) * i11;
-        const double d22 = tail[1] - std::norm(r12);
-        const bool keep = d22 > 1e-12 * tail[1];   // as the device decides
-        const double r22 = keep ? std::sqrt(d22) : 0.0, i22 = keep ? 1.0 / r22 : 0.0;
-        Small r{}, q{};
-        r.a[0][0] = std::sqrt(std::max(tail[0], 0.0)); r.a[0][1] = r12; r.a[1][1] = r22;
-        q.a[0][0] = i11; q.a[0][1] = -r12 * i11 * i22; q.a[1][1] = i22;
-        R.push_back(r);
-        Ri.push_back(q);
-        row.push_back({tail[0] > 0 ? rows : -1, -1});
-        if (tail[0] > 0) ++rows;
-        if (keep) row.back()[1] = rows++;
-        Small t{};
-        t.a[0][0] = t.a[1][1] = 1.0;
-        t.a[0][1] = cplx(tail[4], tail[5]);
-        return mul(r, t);
-    };
     int iters[2] = {0, 0};
     int total = 0, sweeps = 0;
     double rel[2] = {1, 1};
     bool x_zero = true;
-    BlockQR qr;
+    std::vector<cplx> Hm[2], g[2], cs[2], sn[2];
+    std::vector<double> rv[2];   // the FP32 factor 1 / |w_j| of every basis vector, as the device takes it
     while (true) {
         double rn[2];
         if (int e = residual<float>(ctx, x_zero, b_raw, rn, pin, st)) return e;
@@ -618,37 +542,37 @@ int gmres_block(vie_ctx *ctx, const std::vector<size_t> &mld, const HostReq &H, 
         const bool active[2] = {rel[0] > tol, rel[1] > tol};
         if ((!active[0] && !active[1]) || total >= ctx->opt.max_iter) break;
         ++sweeps;
-        // u = r / |r| (per rhs, zero once it has converged), block 0 = M^-1 u
+        // u = r / |r| (per rhs, zero once it has converged), vector 0 = M^-1 u
         double s[4] = {active[0] ? 1.0 / rn[0] : 0.0, 0.0, active[1] ? 1.0 / rn[1] : 0.0, 0.0};
         CK((vie::scale<double, float>(ctx->r.as<double>(), pre ? u : V, N, s, st)));
-        CK(cudaMemsetAsync(state, 0, vie::block_state_bytes(m), st));
+        CK(cudaMemsetAsync(state, 0, vie::krylov_state_bytes(m), st));
         if (pre) { if (int e = timed_precond<float>(ctx, H, mld, u, V, st, tm)) return e; }
-        CK(vie::block_subtract(V, vs, 0, V, N, m, state, 0, nullptr, 0, st));
         const unsigned long long q0 = ++ctx->seq;
-        CK(vie::block_subtract(V, vs, 0, V, N, m, state, 1, slot(q0), q0, st));
-        // one iteration: block k + 1 from block k, its message q0 + k + 1
+        CK(vie::krylov_subtract(V, vs, 0, V, N, m, state, 1, slot(q0), q0, st));
+        ctx->d2h += sizeof(double) * 5;
+        // one iteration: vector k + 1 from vector k, its message q0 + k + 1
         auto enqueue = [&](int k) -> int {
             float *vk = V + vs * k, *vn = V + vs * (k + 1), *to = pre ? u : vn;
-            const float *ri = vie::block_rinv(state, m, k);
+            const float *ri = vie::krylov_rinv(state, m, k);
             cudaEvent_t e0 = ctx->event(), e1 = ctx->event();
             if (e0) CK(cudaEventRecord(e0, st));
             if (zin == 1)
-                CK(vie::matvec_rinv(ctx->Zh.as<__half>(), ctx->ld16, N, N, vk, to, (float)ctx->zh_alpha, ri, st, mvg));
+                CK(vie::matvec_norm(ctx->Zh.as<__half>(), ctx->ld16, N, N, vk, to, (float)ctx->zh_alpha, ri, st, mvg));
             else if (zin == 2)
-                CK(vie::matvec_rinv(ctx->Zh.as<__nv_bfloat16>(), ctx->ld16, N, N, vk, to, 1.f, ri, st, mvg));
+                CK(vie::matvec_norm(ctx->Zh.as<__nv_bfloat16>(), ctx->ld16, N, N, vk, to, 1.f, ri, st, mvg));
             else
-                CK(vie::matvec_rinv(ctx->Z.as<float>(), ctx->ld, N, N, vk, to, 1.f, ri, st, mvg));
+                CK(vie::matvec_norm(ctx->Z.as<float>(), ctx->ld, N, N, vk, to, 1.f, ri, st, mvg));
             if (e1) { CK(cudaEventRecord(e1, st)); tm.mv.push_back({e0, e1}); }
             if (pre) { if (int e = timed_precond<float>(ctx, H, mld, u, vn, st, tm)) return e; }
-            // classical Gram-Schmidt by blocks, twice
+            // classical Gram-Schmidt, twice
             cudaEvent_t o0 = ctx->event(), o1 = ctx->event();
             if (o0) CK(cudaEventRecord(o0, st));
-            CK(vie::block_dots(V, vs, k + 1, vn, N, m, state, 0, st));
-            CK(vie::block_subtract(V, vs, k + 1, vn, N, m, state, 0, nullptr, 0, st));
-            CK(vie::block_dots(V, vs, k + 1, vn, N, m, state, 1, st));
+            CK(vie::krylov_dots(V, vs, k + 1, vn, N, m, state, 0, st));
+            CK(vie::krylov_subtract(V, vs, k + 1, vn, N, m, state, 0, nullptr, 0, st));
+            CK(vie::krylov_dots(V, vs, k + 1, vn, N, m, state, 1, st));
             const unsigned long long q = ++ctx->seq;
-            CK(vie::block_subtract(V, vs, k + 1, vn, N, m, state, 1, slot(q), q, st));
-            ctx->d2h += sizeof(double) * (16 * (size_t)(k + 1) + 7);
+            CK(vie::krylov_subtract(V, vs, k + 1, vn, N, m, state, 1, slot(q), q, st));
+            ctx->d2h += sizeof(double) * (8 * (size_t)(k + 1) + 5);
             if (o1) { CK(cudaEventRecord(o1, st)); tm.ot.push_back({o0, o1}); }
             return VIE_OK;
         };
@@ -656,31 +580,25 @@ int gmres_block(vie_ctx *ctx, const std::vector<size_t> &mld, const HostReq &H, 
         if (int e = enqueue(0)) return e;
         int sent = 1;   // iterations enqueued
         if (int e = wait(q0)) return e;
-        R.clear();
-        Ri.clear();
-        row.clear();
-        rows = 0;
-        const Small r0 = factor_of(slot(q0) + 16 * (size_t)(m + 1));
-        qr = BlockQR();
-        qr.g.assign(rows, {});
-        for (int a = 0; a < 2; ++a)
-            if (row[0][a] >= 0)
-                for (int p = 0; p < 2; ++p) qr.g[row[0][a]][p] = r0.a[a][p];
         // stop a sweep once the preconditioned residual has dropped by inner_tol,
         // or once it predicts the outer target: the FP64 residual at the end of the
-        // sweep is expected near (|g| / beta) |r|, and 0.35 of tol |b| is aimed for.  (At
-        // half, as the separate Krylov spaces had it, the block space gets there in fewer
-        // iterations and leaves more in the slow modes: 2.25e-5 of a conical BF16
-        // solution against 2.00e-5.)
+        // sweep is expected near (|g| / beta) |r|, and half of tol |b| is aimed for
         double stop[2], now[2], rate[2] = {1.0, 1.0};   // rate: the last iteration's reduction
         bool open[2];
         for (int p = 0; p < 2; ++p) {
-            const double beta = std::hypot(std::abs(r0.a[0][p]), std::abs(r0.a[1][p]));
-            stop[p] = std::max(inner_tol, rn[p] > 0 ? 0.35 * tol * bn[p] / rn[p] : 0.0) * beta;
+            const double r = slot(q0)[tail_at + 2 + p], beta = r > 0 ? 1.0 / r : 0.0;
+            rv[p].assign(1, r);
+            Hm[p].assign((size_t)(m + 1) * m, cplx(0));
+            g[p].assign(m + 1, cplx(0));
+            cs[p].assign(m, cplx(0));
+            sn[p].assign(m, cplx(0));
+            g[p][0] = beta;
+            stop[p] = std::max(inner_tol, rn[p] > 0 ? 0.5 * tol * bn[p] / rn[p] : 0.0) * beta;
             now[p] = beta;
             open[p] = active[p] && beta > 0;
         }
-        int done = 0;   // iterations whose column is in the least-squares problem
+        int done = 0;   // iterations whose columns have arrived
+        int kused[2] = {0, 0};
         bool finite = true;
         while (done < sent) {
             // keep the device one iteration ahead, unless the one under way should
@@ -697,33 +615,40 @@ int gmres_block(vie_ctx *ctx, const std::vector<size_t> &mld, const HostReq &H, 
             const int k = done;
             const unsigned long long q = q0 + 1 + (unsigned long long)k;
             if (int e = wait(q)) return e;
-            const double *M = slot(q), *M2 = M + 8 * (size_t)(m + 1), *tail = M2 + 8 * (size_t)(m + 1);
-            const Small hn = factor_of(tail);
-            for (int c = 0; c < 2; ++c) {
-                if (row[k][c] < 0) continue;
-                std::vector<cplx> col(rows, cplx(0));
-                for (int j = 0; j <= k; ++j) {
-                    cplx C[2];
-                    for (int a = 0; a < 2; ++a) {
-                        const int e = 8 * j + 4 * a + 2 * c;
-                        C[a] = cplx(M[e] + M2[e], M[e + 1] + M2[e + 1]);
-                    }
-                    for (int a = 0; a < 2; ++a)
-                        if (row[j][a] >= 0) col[row[j][a]] = R[j].a[a][0] * C[0] + R[j].a[a][1] * C[1];
-                }
-                for (int a = 0; a < 2; ++a)
-                    if (row[k + 1][a] >= 0) col[row[k + 1][a]] = hn.a[a][c];
-                qr.column(std::move(col));
-            }
+            const double *M = slot(q), *M2 = M + 4 * (size_t)(m + 1), *tail = M + tail_at;
             ++done;
+            if (!open[0] && !open[1]) continue;   // enqueued before the last one closed
             ++total;
             for (int p = 0; p < 2; ++p) {
-                if (open[p]) ++iters[p];
-                const double v = qr.residual(p);
+                rv[p].push_back(tail[2 + p]);
+                if (!open[p]) continue;
+                // column k in the basis v_j = w_j rv_j: Z v_k = sum_j w_j C_j + w_{k+1}
+                cplx *Hc = &Hm[p][(size_t)k * (m + 1)];
+                for (int i = 0; i <= k; ++i) {
+                    const int e = 4 * i + 2 * p;
+                    Hc[i] = rv[p][i] > 0 ? cplx(M[e] + M2[e], M[e + 1] + M2[e + 1]) / rv[p][i] : cplx(0);
+                }
+                Hc[k + 1] = tail[2 + p] > 0 ? 1.0 / tail[2 + p] : 0.0;
+                const bool end = !(tail[p] > 0);   // nothing left of the new vector
+                for (int i = 0; i < k; ++i) {   // previous rotations
+                    const cplx t = std::conj(cs[p][i]) * Hc[i] + std::conj(sn[p][i]) * Hc[i + 1];
+                    Hc[i + 1] = -sn[p][i] * Hc[i] + cs[p][i] * Hc[i + 1];
+                    Hc[i] = t;
+                }
+                const double den = std::hypot(std::abs(Hc[k]), std::abs(Hc[k + 1]));
+                if (den == 0) { cs[p][k] = 1; sn[p][k] = 0; }
+                else { cs[p][k] = Hc[k] / den; sn[p][k] = Hc[k + 1] / den; }
+                Hc[k] = den;
+                Hc[k + 1] = 0;
+                g[p][k + 1] = -sn[p][k] * g[p][k];
+                g[p][k] = std::conj(cs[p][k]) * g[p][k];
+                kused[p] = k + 1;
+                ++iters[p];
+                const double v = std::abs(g[p][k + 1]);
                 if (!std::isfinite(v)) finite = false;
                 rate[p] = now[p] > 0 ? std::min(1.0, v / now[p]) : 0.0;
                 now[p] = v;
-                if (v <= stop[p]) open[p] = false;
+                if (v <= stop[p] || end) open[p] = false;
             }
             if (!finite) break;
             if (done == sent && (open[0] || open[1]) && sent < m && total < ctx->opt.max_iter) {   // it was not the last
@@ -737,19 +662,26 @@ int gmres_block(vie_ctx *ctx, const std::vector<size_t> &mld, const HostReq &H, 
             break;
         }
         // y = H^-1 g, x += |r| V y
-        std::vector<double> yv(8 * (size_t)done);
-        const std::vector<cplx> ys[2] = {qr.solve(0), qr.solve(1)};
-        for (int j = 0; j < done; ++j)
-            for (int p = 0; p < 2; ++p)
-                for (int a = 0; a < 2; ++a) {
-                    const cplx y0 = row[j][0] >= 0 ? ys[p][row[j][0]] : cplx(0), y1 = row[j][1] >= 0 ? ys[p][row[j][1]] : cplx(0);
-                    const cplx v = (Ri[j].a[a][0] * y0 + Ri[j].a[a][1] * y1) * rn[p];
-                    yv[8 * j + 4 * a + 2 * p] = v.real();
-                    yv[8 * j + 4 * a + 2 * p + 1] = v.imag();
-                }
+        const int kmax = std::max(kused[0], kused[1]);
+        if (kmax == 0) break;
+        std::vector<double> yv(4 * (size_t)kmax, 0.0);
+        for (int p = 0; p < 2; ++p) {
+            const int kk = kused[p];
+            std::vector<cplx> yy(kk);
+            for (int i = kk - 1; i >= 0; --i) {
+                cplx sacc = g[p][i];
+                for (int j = i + 1; j < kk; ++j) sacc -= Hm[p][(size_t)j * (m + 1) + i] * yy[j];
+                yy[i] = sacc / Hm[p][(size_t)i * (m + 1) + i];
+            }
+            for (int i = 0; i < kk; ++i) {
+                const cplx v = yy[i] * (rn[p] * rv[p][i]);
+                yv[4 * i + 2 * p] = v.real();
+                yv[4 * i + 2 * p + 1] = v.imag();
+            }
+        }
         CK(cudaMemcpyAsync(ctx->y.p, yv.data(), sizeof(double) * yv.size(), cudaMemcpyHostToDevice, st));
         ctx->h2d += sizeof(double) * yv.size();
-        CK(vie::block_combine(V, vs, done, ctx->y.as<double>(), x, N, st));
+        CK(vie::combine<float>(V, vs, kmax, ctx->y.as<double>(), x, N, st));
         CK(cudaStreamSynchronize(st));
         x_zero = false;
     }
@@ -1132,7 +1064,7 @@ int solve_impl(vie_ctx *ctx, const vie_request *req, vie_result *res, cudaStream
     auto t2 = clk::now();
     if (cancelled(ctx)) return fail(ctx, VIE_CANCELLED, "cancelled");
     int stat;
-    if constexpr (std::is_same<TZ, float>::value) stat = gmres_block(ctx, mld, H, res, st, tm);
+    if constexpr (std::is_same<TZ, float>::value) stat = gmres_mixed(ctx, mld, H, res, st, tm);
     else stat = gmres(ctx, H, mld, res, st, tm);
     if (stat < 0) return stat;
     auto t3 = clk::now();
@@ -2031,7 +1963,7 @@ void release_device_memory(vie_ctx *ctx) {
     ctx->mesh = std::make_shared<MeshState>();
     DevBuf *bufs[] = {&ctx->row, &ctx->coef, &ctx->wt, &ctx->kap, &ctx->ieps, &ctx->frow, &ctx->qs,
                       &ctx->perm, &ctx->pol, &ctx->orders, &ctx->stab, &ctx->ztab, &ctx->rtab, &ctx->ew,
-                      &ctx->fcoef, &ctx->frec, &ctx->blob64, &ctx->ph64, &ctx->pjobs, &ctx->pvec, &ctx->bstate,
+                      &ctx->fcoef, &ctx->frec, &ctx->blob64, &ctx->ph64, &ctx->pjobs, &ctx->pvec, &ctx->kstate,
                       &ctx->Z, &ctx->b, &ctx->x, &ctx->r, &ctx->u, &ctx->w, &ctx->V, &ctx->h, &ctx->y,
                       &ctx->Minv, &ctx->MinvH, &ctx->amax, &ctx->tcpack, &ctx->tcpack2, &ctx->status, &ctx->acc,
                       &ctx->J, &ctx->xs, &ctx->Zh, &ctx->dens,

@@ -85,21 +85,11 @@ template <typename T> __device__ __forceinline__ T warp_sum16(const T (&acc)[MV_
 }
 __device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
-// component k (re, im of column 0, of column 1) of the row (c0, c1) R, R upper
-// triangular (r11, r12.re, r12.im, r22); the row's components sit in four adjacent lanes
-template <typename T> __device__ __forceinline__ T times_r(T s, int k, const float *r) {
-    const unsigned m = __activemask();
-    const int l0 = threadIdx.x & ~3;
-    const T a = __shfl_sync(m, s, l0), b = __shfl_sync(m, s, l0 + 1);
-    if (k < 2) return r[0] * s;
-    return k == 2 ? r[3] * s + r[1] * a - r[2] * b : r[3] * s + r[1] * b + r[2] * a;
-}
-
-// RINV: y[r] = alpha (sum_c A[r][c] x[c]) R with the upper triangular 2 x 2 R in
-// rinv (r11, r12.re, r12.im, r22): the columns of x normalised on the way out.
+// NORM: y[r] = alpha sum_c A[r][c] x[c] times one factor per right-hand side in rinv: the
+// columns of x normalised on the way out.
 // Launched in a stream of dependent kernels (launch_pdl): the matrix is prefetched
 // before the wait for the kernel that writes x.
-template <typename TZ, typename TX, typename TA, bool ACCUM, bool RINV = false>
+template <typename TZ, typename TX, typename TA, bool ACCUM, bool NORM = false>
 __global__ void __launch_bounds__(MV_WARPS * 32, 2)
 k_matvec(const TZ *__restrict__ A, size_t ld, int rows, int cols, const TX *x, TA *y, TA alpha,
          const float *rinv = nullptr) {
@@ -110,7 +100,7 @@ k_matvec(const TZ *__restrict__ A, size_t ld, int rows, int cols, const TX *x, T
     constexpr int VEC = sizeof(TZ) == 4 ? 2 : 1;   // complex entries per 16-byte load
     const int nvec = (cols + VEC - 1) / VEC;
     const int v0 = (int)((long long)nvec * warp / MV_WARPS), v1 = (int)((long long)nvec * (warp + 1) / MV_WARPS);
-    if (RINV) {
+    if (NORM) {
 #pragma unroll
         for (int i = 0; i < MV_ROWS; ++i)
             for (int v = v0 + lane; v < v1 && v < v0 + 4 * 32; v += 32)
@@ -182,7 +172,7 @@ k_matvec(const TZ *__restrict__ A, size_t ld, int rows, int cols, const TX *x, T
                 TA s = TA(0);
 #pragma unroll
                 for (int w2 = 0; w2 < MV_WARPS; ++w2) s += part[buf][w2][threadIdx.x];
-                if constexpr (RINV) s = times_r(s, k, rinv);
+                if constexpr (NORM) s *= rinv[k >> 1];
                 if (ACCUM) y[(size_t)r * 4 + k] += alpha * s;
                 else y[(size_t)r * 4 + k] = alpha * s;
             }
@@ -223,7 +213,7 @@ __device__ __forceinline__ void chunk_use(const uint4 (&z)[MV_ROWS], const TV *x
     }
 }
 
-template <typename TZ, bool RINV>
+template <typename TZ, bool NORM>
 __global__ void __launch_bounds__(MV_WARPS * 32, 2)
 k_matvec16(const TZ *__restrict__ A, size_t ld, int rows, const float *x, float *y, float alpha, const float *rinv) {
     __shared__ float part[2][MV_WARPS][MV_ROWS * 4];
@@ -239,7 +229,7 @@ k_matvec16(const TZ *__restrict__ A, size_t ld, int rows, const float *x, float 
     };
     rows_at(rb);
     const unsigned o0 = (unsigned)c0 * 512u + (unsigned)lane * 16u;
-    if (RINV) {
+    if (NORM) {
 #pragma unroll
         for (int i = 0; i < MV_ROWS; ++i)
             for (int c = c0; c < c1 && c < c0 + 4; ++c)
@@ -275,13 +265,13 @@ k_matvec16(const TZ *__restrict__ A, size_t ld, int rows, const float *x, float 
             float s = 0.f;
 #pragma unroll
             for (int w2 = 0; w2 < MV_WARPS; ++w2) s += part[buf][w2][threadIdx.x];
-            if constexpr (RINV) s = times_r(s, k, rinv);
+            if constexpr (NORM) s *= rinv[k >> 1];
             if (r < re) y[(size_t)r * 4 + k] = alpha * s;
         }
     }
 }
 
-template <typename TZ, bool RINV>
+template <typename TZ, bool NORM>
 cudaError_t launch_matvec16(const TZ *A, size_t ld, int rows, const float *x, float *y, float alpha, const float *rinv,
                             cudaStream_t st, int grid_mult) {
     if (rows <= 0) return cudaSuccess;
@@ -290,18 +280,18 @@ cudaError_t launch_matvec16(const TZ *A, size_t ld, int rows, const float *x, fl
         int dev = 0, sms = 0, per = 0;
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_matvec16<TZ, RINV>, MV_WARPS * 32, 0);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_matvec16<TZ, NORM>, MV_WARPS * 32, 0);
         if (e != cudaSuccess) return e;
         slots = std::max(1, sms * per);
     }
     const int grid = std::max(1, std::min(slots * std::max(1, grid_mult), (rows + MV_ROWS - 1) / MV_ROWS));
-    if constexpr (RINV) return launch_pdl(k_matvec16<TZ, true>, grid, MV_WARPS * 32, st, A, ld, rows, x, y, alpha, rinv);
+    if constexpr (NORM) return launch_pdl(k_matvec16<TZ, true>, grid, MV_WARPS * 32, st, A, ld, rows, x, y, alpha, rinv);
     k_matvec16<TZ, false><<<grid, MV_WARPS * 32, 0, st>>>(A, ld, rows, x, y, alpha, nullptr); ++g_launches;
     return cudaGetLastError();
 }
 
 template <typename TZ>
-cudaError_t matvec_rinv(const TZ *A, size_t ld, int rows, int cols, const float *x, float *y, float alpha,
+cudaError_t matvec_norm(const TZ *A, size_t ld, int rows, int cols, const float *x, float *y, float alpha,
                         const float *rinv, cudaStream_t st, int grid_mult) {
     if (rows <= 0) return cudaSuccess;
     if constexpr (sizeof(TZ) == 2) return launch_matvec16<TZ, true>(A, ld, rows, x, y, alpha, rinv, st, grid_mult);
@@ -320,9 +310,9 @@ cudaError_t matvec_rinv(const TZ *A, size_t ld, int rows, int cols, const float 
     return launch_pdl(k_matvec<TZ, float, float, false, true>, grid, MV_WARPS * 32, st, A, ld, rows, cols, x, y, alpha, rinv);
     }
 }
-template cudaError_t matvec_rinv<float>(const float *, size_t, int, int, const float *, float *, float, const float *, cudaStream_t, int);
-template cudaError_t matvec_rinv<__half>(const __half *, size_t, int, int, const float *, float *, float, const float *, cudaStream_t, int);
-template cudaError_t matvec_rinv<__nv_bfloat16>(const __nv_bfloat16 *, size_t, int, int, const float *, float *, float,
+template cudaError_t matvec_norm<float>(const float *, size_t, int, int, const float *, float *, float, const float *, cudaStream_t, int);
+template cudaError_t matvec_norm<__half>(const __half *, size_t, int, int, const float *, float *, float, const float *, cudaStream_t, int);
+template cudaError_t matvec_norm<__nv_bfloat16>(const __nv_bfloat16 *, size_t, int, int, const float *, float *, float,
                                                 const float *, cudaStream_t, int);
 
 template <typename TZ, typename TX, typename TA>
@@ -1420,6 +1410,7 @@ template cudaError_t dots<double>(const double *, size_t, int, const double *, i
 template cudaError_t subtract<double>(const double *, size_t, int, const double *, double *, int, cudaStream_t);
 template cudaError_t scale<double, float>(const double *, float *, int, const double *, cudaStream_t);
 template cudaError_t scale<double, double>(const double *, double *, int, const double *, cudaStream_t);
+template cudaError_t combine<float>(const float *, size_t, int, const double *, double *, int, cudaStream_t);
 template cudaError_t combine<double>(const double *, size_t, int, const double *, double *, int, cudaStream_t);
 
 }  // namespace vie

@@ -46,35 +46,28 @@ cudaError_t matvec16(const __half *A, size_t ld, int rows, const float *x, float
                      int grid_mult);
 cudaError_t matvec16(const __nv_bfloat16 *A, size_t ld, int rows, const float *x, float *y, float alpha, cudaStream_t st,
                      int grid_mult);
-// y <- alpha (A x) R, FP32 vectors (16-bit A: x zero up to pad_cols), R the 2 x 2 upper triangular rinv (device: r11,
-// r12.re, r12.im, r22); launched with launch_pdl
+// y <- alpha A (x diag(rinv)), FP32 vectors (16-bit A: x zero up to pad_cols), rinv one
+// factor per right-hand side (device); launched with launch_pdl
 template <typename TZ>
-cudaError_t matvec_rinv(const TZ *A, size_t ld, int rows, int cols, const float *x, float *y, float alpha,
+cudaError_t matvec_norm(const TZ *A, size_t ld, int rows, int cols, const float *x, float *y, float alpha,
                         const float *rinv, cudaStream_t st, int grid_mult);
 
-// ---- block GMRES over the two right-hand sides (krylov.cu), FP32 vectors ----
-// Basis block j is the pair of columns w_j stored as one [n][2] complex vector,
-// orthogonal to the blocks before it but not normalised: V_j = w_j R_j^-1 with
-// the Cholesky factor R_j of its Gram matrix.  `state`: device scratch of one solve,
-// dots of both passes, Grams, counters (zeroed before the first block), then the
-// coefficients, inverse Grams and inverse R
-size_t block_state_bytes(int m);
+// ---- GMRES of the mixed paths (krylov.cu), FP32 vectors, both right-hand sides ----
+// Basis vector j of both right-hand sides is one [n][2] complex vector w_j, orthogonal
+// (per right-hand side) to the vectors before it but not normalised: v_j = w_j / |w_j|.
+// `state`: device scratch of one solve, zeroed before the first vector
+size_t krylov_state_bytes(int m);
 // doubles of one message to the host (pinned): coefficients of both passes
-// [nv][8] each (as applied, FP32 values), Gram of pass 1 and of pass 2 [4] each,
-// then one 64-bit sequence word
-size_t block_message_doubles(int m);
-// C_j = (w_j^H w_j)^-1 w_j^H w for the nv blocks of V into pass `pass` of the state
-cudaError_t block_dots(const float *V, size_t vstride, int nv, const float *w, int n, int m, void *state, int pass,
-                       cudaStream_t st);
-// w -= sum_j w_j C_j; pass 0: then the Gram matrix of w; pass 1: also takes the part
-// along column 0 out of column 1 (by pass 0's Gram matrix), then forms the Gram
-// matrix of block nv, its R^-1 and inverse, sends the message with sequence number
-// seq and clears the state for the next block
-cudaError_t block_subtract(const float *V, size_t vstride, int nv, float *w, int n, int m, void *state, int pass,
-                           double *message, unsigned long long seq, cudaStream_t st);
-const float *block_rinv(void *state, int m, int j);   // device address of R_j^-1
-// x[i][p] += sum_j sum_a w_j[i][a] Y[j][a][p] (FP64; Y on the device, [nv][2][2] complex)
-cudaError_t block_combine(const float *V, size_t vstride, int nv, const double *Y, double *x, int n, cudaStream_t st);
+// [m + 1][4] each (as applied, FP32 values), |w|^2 [2], the FP32 value of 1 / |w| that
+// the next product takes [2], then one 64-bit sequence word
+size_t krylov_message_doubles(int m);
+// C_j = w_j^H w / |w_j|^2 for the nv vectors of V into pass `pass` of the state
+cudaError_t krylov_dots(const float *V, size_t vstride, int nv, const float *w, int n, int m, void *state, int pass,
+                        cudaStream_t st);
+// w -= sum_j w_j C_j; pass 1: then the norms of vector nv, and the message with sequence number seq
+cudaError_t krylov_subtract(const float *V, size_t vstride, int nv, float *w, int n, int m, void *state, int pass,
+                            double *message, unsigned long long seq, cudaStream_t st);
+const float *krylov_rinv(void *state, int m, int j);   // device address of 1 / |w_j| [2]
 
 // CUDA-event timing of selected launches (optional)
 struct KernelTimer {
