@@ -104,7 +104,7 @@ struct FarPoly {
 // erfcx(x + j b) by F64_SPAT polynomials of degree F64_DEG.  The blob (doubles):
 //   at 0         spatial table [F64_SPAT + 1][F64_DEG + 1] (constant term first; the last entry zero)
 //   at img       images [n_img][4]: m a, n b, Re, Im of the phase exp(b^2) / (4 pi) exp(j k_par.R)
-//   at dir       per order (i, j), two doubles holding four ints: offset and degree of the
+//   at dir       (even: int4 loads) per order (i, j), two doubles holding four ints: offset and degree of the
 //                real part's coefficients (highest power first), of the imaginary part's
 //                (degree -1: none); rows x cols
 // sym: normal incidence, the quadrant p, q >= 0 of orders with weights 1, 2 cos.

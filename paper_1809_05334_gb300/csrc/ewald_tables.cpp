@@ -427,6 +427,7 @@ void build_far64(const EwaldTables &t, double k0, double kx, double ky, Far64 &f
     blob.resize((size_t)(F64_SPAT + 1) * (F64_DEG + 1), 0.0);
     f.img = (int)blob.size();
     for (int i = 0; i < t.n_img; ++i) blob.insert(blob.end(), t.img64[i], t.img64[i] + 4);
+    if (blob.size() & 1) blob.push_back(0.0);   // the directory's entries are read as int4: 16-byte boundaries
     f.dir = (int)blob.size();
     blob.resize(blob.size() + 2 * (size_t)np * nq, 0.0);
     const int M = std::min(64, (int)std::ceil(24 + 7 * Ez));
