@@ -28,11 +28,11 @@ struct NearArgs {
     float slack;       // bound on the FP32 rounding of a coordinate difference
 };
 
-// bits of the near images of (i, j), bit k of *touch where they share a vertex
-__device__ __forceinline__ unsigned near_mask(const NearArgs &g, int i, int j, unsigned *touch) {
+// Bits of the near images of (i, j).
+__device__ __forceinline__ unsigned near_mask(const NearArgs &g, int i, int j) {
     const double *cx = g.x.cen + 3 * (size_t)i, *cy = g.y.cen + 3 * (size_t)j;
     const float rf = (float)(g.x.rad[i] + g.y.rad[j]);
-    const float limf = 1.5f * rf * 1.0001f + 2.f * g.slack;
+    const float limf = (float)NEAR_FACTOR * rf * 1.0001f + 2.f * g.slack;
     const float fx = (float)cx[0] - (float)cy[0], fy = (float)cx[1] - (float)cy[1], fz = (float)cx[2] - (float)cy[2];
     const float af = (float)g.a, bf = (float)g.b;
     unsigned cand = 0u;
@@ -47,27 +47,45 @@ __device__ __forceinline__ unsigned near_mask(const NearArgs &g, int i, int j, u
     unsigned mask = 0u;
     for (unsigned c = cand; c; c &= c - 1u) {
         const int k = __ffs((int)c) - 1;
-        const double R0 = (k / 3 - 1) * g.a, R1 = (k % 3 - 1) * g.b;
-        const double e0 = d0 + R0, e1 = d1 + R1;
-        const double dist = sqrt(e0 * e0 + e1 * e1 + d2 * d2);
-        if (!(dist < lim)) continue;
-        mask |= 1u << k;
-        if (!touch) continue;
-        if ((float)dist > rf * 1.0001f + 2.f * g.slack) continue;   // too far apart to share a vertex
+        const double e0 = d0 + (k / 3 - 1) * g.a, e1 = d1 + (k % 3 - 1) * g.b;
+        if (sqrt(e0 * e0 + e1 * e1 + d2 * d2) < lim) mask |= 1u << k;
+    }
+    return mask;
+}
+
+// Of the near images `mask` of (i, j), those in which the elements share a vertex.  Both
+// passes call it with the stored mask, the first to count the entries of a list, the
+// second to write them, so the same bits have to come out: every operation is rounded by
+// itself (nothing that the compiler may contract in one kernel and not in the other).
+__device__ __forceinline__ unsigned touch_mask(const NearArgs &g, int i, int j, unsigned mask) {
+    const double tol2 = __dmul_rn(g.tol, g.tol);
+    // centroids further apart than both radii (FP32, with a margin for its rounding): no shared vertex
+    const double *cx = g.x.cen + 3 * (size_t)i, *cy = g.y.cen + 3 * (size_t)j;
+    const float rf = __fadd_rn((float)g.x.rad[i], (float)g.y.rad[j]);
+    const float lim = __fadd_rn(__fmul_rn(rf, 1.0001f), __fmul_rn(2.f, g.slack)), lim2 = __fmul_rn(lim, lim);
+    const float fx = __fsub_rn((float)cx[0], (float)cy[0]), fy = __fsub_rn((float)cx[1], (float)cy[1]),
+                fz = __fsub_rn((float)cx[2], (float)cy[2]);
+    unsigned touch = 0u;
+    for (unsigned c = mask; c; c &= c - 1u) {
+        const int k = __ffs((int)c) - 1;
+        const float dx = __fadd_rn(fx, __fmul_rn((float)(k / 3 - 1), (float)g.a)),
+                    dy = __fadd_rn(fy, __fmul_rn((float)(k % 3 - 1), (float)g.b));
+        if (__fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(fz, fz)) > lim2) continue;
+        const double R0 = __dmul_rn((double)(k / 3 - 1), g.a), R1 = __dmul_rn((double)(k % 3 - 1), g.b);
         bool t = false;
         for (int p = 0; p < g.x.kv && !t; ++p) {
             const double *u = g.x.verts + 3 * ((size_t)g.x.kv * i + p);
             for (int q = 0; q < g.y.kv; ++q) {
                 const double *v = g.y.verts + 3 * ((size_t)g.y.kv * j + q);
-                const double x = u[0] - (v[0] - R0);
+                const double x = __dsub_rn(u[0], __dsub_rn(v[0], R0));
                 if (fabs(x) >= g.tol) continue;
-                const double y = u[1] - (v[1] - R1), z = u[2] - v[2];
-                if (sqrt(x * x + y * y + z * z) < g.tol) { t = true; break; }
+                const double y = __dsub_rn(u[1], __dsub_rn(v[1], R1)), z = __dsub_rn(u[2], v[2]);
+                if (__dadd_rn(__dadd_rn(__dmul_rn(x, x), __dmul_rn(y, y)), __dmul_rn(z, z)) < tol2) { t = true; break; }
             }
         }
-        if (t) *touch |= 1u << k;
+        if (t) touch |= 1u << k;
     }
-    return mask;
+    return touch;
 }
 
 // exclusive ordered scan over the 256 threads of a CTA of two counts packed in one
@@ -104,7 +122,8 @@ __global__ void __launch_bounds__(256) k_near(NearArgs g, uint16_t *mk, unsigned
     for (int j0 = 0; j0 < ny; j0 += 256) {
         const int j = j0 + threadIdx.x;
         unsigned mask = 0u, touch = 0u;
-        if (j < ny && (!EMIT || mk[(size_t)i * ny + j])) mask = near_mask(g, i, j, &touch);
+        if (j < ny) mask = EMIT ? (unsigned)mk[(size_t)i * ny + j] : near_mask(g, i, j);
+        if (mask) touch = touch_mask(g, i, j, mask);
         if (!EMIT) {
             if (j < ny) mk[(size_t)i * ny + j] = (uint16_t)mask;
             n_pr += __popc(mask & ~touch);
