@@ -739,23 +739,18 @@ __global__ void k_green(const double *d, double *out, int n, const float *stab, 
 // launchers
 // ---------------------------------------------------------------------------
 template <typename T, int PK>
-void far_scalar(bool sym, dim3 grid, size_t sm, cudaStream_t st, const DevMesh &m, const DevReq &q, T *Z, size_t N,
-                int nx, int ny, const uint16_t *mk) {
+cudaError_t far_scalar(bool sym, dim3 grid, size_t sm, cudaStream_t st, const DevMesh &m, const DevReq &q, T *Z, size_t N,
+                       int nx, int ny, const uint16_t *mk) {
     if constexpr (sizeof(T) == 4) {
-        if (q.fp.mode != FAR_NONE) {
-            launch_far_scalar(PK, m, q, Z, N, st);
-            return;
-        }
+        if (q.fp.mode != FAR_NONE) return launch_far_scalar(PK, m, q, Z, N, st);
         if (sym) k_far_scalar<T, PK, true><<<grid, 128, sm, st>>>(m, q, Z, N, nx, ny, mk);
         else k_far_scalar<T, PK, false><<<grid, 128, sm, st>>>(m, q, Z, N, nx, ny, mk);
     } else {
-        if (q.f64.n_blob > 0) {
-            launch_far64_scalar(PK, m, q, Z, N, st);
-            return;
-        }
+        if (q.f64.n_blob > 0) return launch_far64_scalar(PK, m, q, Z, N, st);
         k_far_scalar<T, PK, false><<<grid, 128, sm, st>>>(m, q, Z, N, nx, ny, mk);
     }
     ++g_launches;
+    return cudaGetLastError();
 }
 
 template <typename T>
@@ -763,31 +758,36 @@ cudaError_t launch_fill(const DevMesh &m, const DevReq &q, T *Z, size_t ld, doub
                         cudaEvent_t far0, cudaEvent_t far1) {
     // Z: N rows of ld complex entries (row stride ld >= N), domain-blocked order
     const size_t N = ld;
-    cudaMemsetAsync(Z, 0, sizeof(T) * 2 * ld * (size_t)m.N, st);
-    if (b) cudaMemsetAsync(b, 0, sizeof(double) * 4 * (size_t)m.N, st);
+    // the first error of any part (the launchers take theirs from the runtime and return it)
+    cudaError_t err = cudaSuccess;
+    auto part = [&](cudaError_t e) { if (err == cudaSuccess) err = e; };
+    part(cudaMemsetAsync(Z, 0, sizeof(T) * 2 * ld * (size_t)m.N, st));
+    if (b) part(cudaMemsetAsync(b, 0, sizeof(double) * 4 * (size_t)m.N, st));
     dim3 blk(128);
     k_gram<T><<<(m.nt + 127) / 128, blk, 0, st>>>(m, q, Z, N); ++g_launches;
     if (b) { k_rhs<<<(m.nt + 127) / 128, blk, 0, st>>>(m, q, b); ++g_launches; }
-    if (sizeof(T) == 4) launch_far_prep(m, q, st);   // element records of the FP32 kernels
-    else if (q.f64.n_blob > 0) launch_far64_prep(m, q, st);
+    part(cudaGetLastError());
+    if (sizeof(T) == 4) part(launch_far_prep(m, q, st));   // element records of the FP32 kernels
+    else if (q.f64.n_blob > 0) part(launch_far64_prep(m, q, st));
     const size_t sm = stab_bytes<T>();
     if (far0) cudaEventRecord(far0, st);
     const bool sym = sizeof(T) == 4 && q.ef.sym;   // normal incidence: the symmetric tabulated path
     if constexpr (sizeof(T) == 4) {
         const dim3 gtt((m.nt + 127) / 128, m.nt);
         if (q.fp.mode != FAR_NONE) {
-            launch_far_tt(m, q, Z, N, st);
+            part(launch_far_tt(m, q, Z, N, st));
         } else {
             if (sym) k_far_tt<T, true><<<gtt, blk, sm, st>>>(m, q, Z, N);
             else k_far_tt<T, false><<<gtt, blk, sm, st>>>(m, q, Z, N);
             ++g_launches;
         }
     } else if (q.f64.n_blob > 0) {
-        launch_far64_tt(m, q, Z, N, st);
+        part(launch_far64_tt(m, q, Z, N, st));
     } else {
         k_far_tt<T, false><<<dim3((m.nt + 127) / 128, m.nt), blk, sm, st>>>(m, q, Z, N);
         ++g_launches;
     }
+    part(cudaGetLastError());
     if (far1) cudaEventRecord(far1, st);
     auto grid1 = [](int n) { return (unsigned)((n + 127) / 128); };
     if (m.npr[0]) { k_pr_tt<T><<<grid1(m.npr[0]), blk, 0, st>>>(m, q, Z, N, m.pr[0], m.npr[0]); ++g_launches; }
@@ -796,19 +796,20 @@ cudaError_t launch_fill(const DevMesh &m, const DevReq &q, T *Z, size_t ld, doub
                                                             m.nto[0]); ++g_launches;
     }
     if (m.nf) {
-        far_scalar<T, PK_TF>(sym, dim3((m.nf + 127) / 128, m.nt), sm, st, m, q, Z, N, m.nt, m.nf, m.mk_tf);
+        part(far_scalar<T, PK_TF>(sym, dim3((m.nf + 127) / 128, m.nt), sm, st, m, q, Z, N, m.nt, m.nf, m.mk_tf));
         if (m.npr[1]) { k_pr_scalar<T, PK_TF><<<grid1(m.npr[1]), blk, 0, st>>>(m, q, Z, N, m.pr[1], m.npr[1]); ++g_launches; }
         if (m.nto[1]) { k_touch_apply<T, PK_TF><<<grid1(m.nto[1]), blk, 0, st>>>(m, q, Z, N, m.to[1], m.touch_sc[1], m.nto[1]); ++g_launches; }
     }
     if (m.nh) {
-        far_scalar<T, PK_FT>(sym, dim3((m.nt + 127) / 128, m.nh), sm, st, m, q, Z, N, m.nh, m.nt, m.mk_ft);
+        part(far_scalar<T, PK_FT>(sym, dim3((m.nt + 127) / 128, m.nh), sm, st, m, q, Z, N, m.nh, m.nt, m.mk_ft));
         if (m.npr[2]) { k_pr_scalar<T, PK_FT><<<grid1(m.npr[2]), blk, 0, st>>>(m, q, Z, N, m.pr[2], m.npr[2]); ++g_launches; }
         if (m.nto[2]) { k_touch_apply<T, PK_FT><<<grid1(m.nto[2]), blk, 0, st>>>(m, q, Z, N, m.to[2], m.touch_sc[2], m.nto[2]); ++g_launches; }
-        far_scalar<T, PK_FF>(sym, dim3((m.nf + 127) / 128, m.nh), sm, st, m, q, Z, N, m.nh, m.nf, m.mk_ff);
+        part(far_scalar<T, PK_FF>(sym, dim3((m.nf + 127) / 128, m.nh), sm, st, m, q, Z, N, m.nh, m.nf, m.mk_ff));
         if (m.npr[3]) { k_pr_scalar<T, PK_FF><<<grid1(m.npr[3]), blk, 0, st>>>(m, q, Z, N, m.pr[3], m.npr[3]); ++g_launches; }
         if (m.nto[3]) { k_touch_apply<T, PK_FF><<<grid1(m.nto[3]), blk, 0, st>>>(m, q, Z, N, m.to[3], m.touch_sc[3], m.nto[3]); ++g_launches; }
     }
-    return cudaGetLastError();
+    part(cudaGetLastError());
+    return err;
 }
 
 size_t static_geom_bytes(size_t nt, size_t nf) { return sizeof(TetGeom) * nt + sizeof(TriGeom) * (nf + 1); }
