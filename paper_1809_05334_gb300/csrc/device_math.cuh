@@ -162,13 +162,14 @@ __device__ cx<T> green_p(T dx, T dy, T dz, unsigned sub, const EwaldTables *__re
         T x = dx + im[0], y = dy + im[1];
         T R2 = x * x + y * y + dz * dz;
         T R = sqrt(R2);
-        if (R * E > xc) continue;
         bool regular = false;
         if (sub) {
 #pragma unroll
             for (int k = 0; k < 9; ++k)
                 if (((sub >> k) & 1u) && ew->near_img[k] == i) regular = true;
         }
+        const bool beyond = R * E > xc;   // nothing of the image term itself left
+        if (beyond && !regular) continue;
         if (regular && R * E < T(1e-6)) {
             // continuous limit at R = 0 of (image term - static term):
             // reg0 = (E/4pi)[2 b erfi(b) - (2/sqrt pi) exp(b^2)]; the table
@@ -178,7 +179,7 @@ __device__ cx<T> green_p(T dx, T dy, T dz, unsigned sub, const EwaldTables *__re
             acc = acc + unscale * ph;
             continue;
         }
-        T val = exp(-R2 * E * E) * erfcx_c(cx<T>{R * E, bb}).re / R;
+        T val = beyond ? T(0) : exp(-R2 * E * E) * erfcx_c(cx<T>{R * E, bb}).re / R;
         if (regular) val -= exp(-bb * bb) / R;   // static part phase/(4 pi R) in table units
         cx<T> ph = {im[2], im[3]};
         acc = acc + val * ph;
@@ -310,23 +311,26 @@ __device__ __forceinline__ void green_tab_impl(float dx, float dy, float dz, uns
         const float *im = ew.img[i];
         const float x = dx + im[0], y = dy + im[1];
         const float R2 = x * x + y * y + dz * dz;
-        if (R2 > r2max) return;            // outside the cut: skip before the square root
-        const float rinv = R2 > 0.f ? rsqrtf(R2) : 0.f;   // R = 0 only on a regularised image (no 1/R)
-        const float R = R2 * rinv;
-        const float xr = R * E;
-        if (xr > xmax) return;
         bool regular = false;
         if (sub) {
 #pragma unroll
             for (int k = 0; k < 9; ++k)
                 if (((sub >> k) & 1u) && ew.near_img[k] == i) regular = true;
         }
+        if (R2 > r2max && !regular) return;   // outside the cut: skip before the square root
+        const float rinv = R2 > 0.f ? rsqrtf(R2) : 0.f;   // R = 0 only on a regularised image (no 1/R)
+        const float R = R2 * rinv;
+        const float xr = R * E;
+        const bool beyond = xr > xmax;
+        if (beyond && !regular) return;
         const float xu = xr * ih;
         const int ix = min((int)xu, NSPAT - 1);
         const float v = xu - ix;
         const float4 cs = *reinterpret_cast<const float4 *>(stab + 4 * ix);   // one 16-byte load
         float val;
-        if (regular) {
+        if (beyond) {   // F is zero there: what is left is the static part removed
+            val = -ew.e_mb2 * rinv;
+        } else if (regular) {
             if (ix == 0)   // (F(x) - F(0))/R = E (c1 + v (c2 + v c3)) / h
                 val = E * ih * fmaf(v, fmaf(v, cs.w, cs.z), cs.y);
             else
@@ -346,7 +350,10 @@ __device__ __forceinline__ void green_tab_impl(float dx, float dy, float dz, uns
         }
     };
     // images 0..63 as the caller's mask selects them (it leaves out only images
-    // beyond the cut), the rest one by one
+    // beyond the cut) and those whose static part is removed, the rest one by one
+    if (sub)
+        for (int k = 0; k < 9; ++k)
+            if (((sub >> k) & 1u) && ew.near_img[k] < 64) imask |= 1ull << ew.near_img[k];
     if (ew.n_img < 64) imask &= (1ull << ew.n_img) - 1ull;
     for (unsigned long long mk = imask; mk; mk &= mk - 1ull) image(__ffsll((long long)mk) - 1);
     for (int i = 64; i < ew.n_img; ++i) image(i);
