@@ -1300,18 +1300,23 @@ int tune_impl(vie_ctx *ctx, const vie_request *req, vie_tune_report *out, cudaSt
         if (ctx->opt.precision == VIE_FP16 || ctx->opt.precision == VIE_BF16)
             if (int e = make_z16(ctx, st)) return e;
     }
-    DevBuf xv, yv;
+    // the kernels of the iteration itself (mixed paths: matvec_norm, here with factors of one)
+    DevBuf xv, yv, ones;
     CK(xv.ensure(sizeof(TV) * 4 * vie::pad_cols(N)));
     CK(yv.ensure(sizeof(TV) * 4 * (size_t)N));
     CK(cudaMemsetAsync(xv.p, 0, sizeof(TV) * 4 * vie::pad_cols(N), st));
+    CK(upload(ones, std::vector<float>{1.f, 1.f}, st));
     auto product = [&](int g) -> cudaError_t {
         if constexpr (std::is_same<TV, float>::value) {
+            const float *one = ones.as<float>();
             if (ctx->opt.precision == VIE_FP16)
-                return vie::matvec16(ctx->Zh.as<__half>(), ctx->ld16, N, xv.as<TV>(), yv.as<TV>(), TV(ctx->zh_alpha), st, g);
+                return vie::matvec_norm(ctx->Zh.as<__half>(), ctx->ld16, N, N, xv.as<TV>(), yv.as<TV>(), TV(ctx->zh_alpha), one, st, g);
             if (ctx->opt.precision == VIE_BF16)
-                return vie::matvec16(ctx->Zh.as<__nv_bfloat16>(), ctx->ld16, N, xv.as<TV>(), yv.as<TV>(), TV(1), st, g);
+                return vie::matvec_norm(ctx->Zh.as<__nv_bfloat16>(), ctx->ld16, N, N, xv.as<TV>(), yv.as<TV>(), TV(1), one, st, g);
+            return vie::matvec_norm(ctx->Z.as<TZ>(), ctx->ld, N, N, xv.as<TV>(), yv.as<TV>(), TV(1), one, st, g);
+        } else {
+            return vie::matvec<TZ, TV, TV>(ctx->Z.as<TZ>(), ctx->ld, N, N, xv.as<TV>(), yv.as<TV>(), TV(1), false, st, g);
         }
-        return vie::matvec<TZ, TV, TV>(ctx->Z.as<TZ>(), ctx->ld, N, N, xv.as<TV>(), yv.as<TV>(), TV(1), false, st, g);
     };
     double bmv = 1e300;
     int bg = 1;

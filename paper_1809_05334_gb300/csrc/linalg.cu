@@ -213,7 +213,7 @@ __device__ __forceinline__ void chunk_use(const uint4 (&z)[MV_ROWS], const TV *x
     }
 }
 
-template <typename TZ, bool NORM>
+template <typename TZ>
 __global__ void __launch_bounds__(MV_WARPS * 32, 2)
 k_matvec16(const TZ *__restrict__ A, size_t ld, int rows, const float *x, float *y, float alpha, const float *rinv) {
     __shared__ float part[2][MV_WARPS][MV_ROWS * 4];
@@ -229,14 +229,12 @@ k_matvec16(const TZ *__restrict__ A, size_t ld, int rows, const float *x, float 
     };
     rows_at(rb);
     const unsigned o0 = (unsigned)c0 * 512u + (unsigned)lane * 16u;
-    if (NORM) {
 #pragma unroll
-        for (int i = 0; i < MV_ROWS; ++i)
-            for (int c = c0; c < c1 && c < c0 + 4; ++c)
-                if ((lane & 7) == 0) prefetch_l2(row[i] + (o0 + 512u * (c - c0)));
-        cudaTriggerProgrammaticLaunchCompletion();
-        cudaGridDependencySynchronize();
-    }
+    for (int i = 0; i < MV_ROWS; ++i)
+        for (int c = c0; c < c1 && c < c0 + 4; ++c)
+            if ((lane & 7) == 0) prefetch_l2(row[i] + (o0 + 512u * (c - c0)));
+    cudaTriggerProgrammaticLaunchCompletion();
+    cudaGridDependencySynchronize();
     uint4 zc[MV_ROWS], zn[MV_ROWS];
     if (c0 < c1 && rb < re) chunk_load<TZ, float>(row, o0, zc);
     int buf = 0;
@@ -265,36 +263,33 @@ k_matvec16(const TZ *__restrict__ A, size_t ld, int rows, const float *x, float 
             float s = 0.f;
 #pragma unroll
             for (int w2 = 0; w2 < MV_WARPS; ++w2) s += part[buf][w2][threadIdx.x];
-            if constexpr (NORM) s *= rinv[k >> 1];
+            s *= rinv[k >> 1];
             if (r < re) y[(size_t)r * 4 + k] = alpha * s;
         }
     }
 }
 
-template <typename TZ, bool NORM>
+template <typename TZ>
 cudaError_t launch_matvec16(const TZ *A, size_t ld, int rows, const float *x, float *y, float alpha, const float *rinv,
                             cudaStream_t st, int grid_mult) {
-    if (rows <= 0) return cudaSuccess;
     static int slots = 0;   // resident CTAs of the GPU (per instantiation; one device per process)
     if (slots == 0) {
         int dev = 0, sms = 0, per = 0;
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_matvec16<TZ, NORM>, MV_WARPS * 32, 0);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_matvec16<TZ>, MV_WARPS * 32, 0);
         if (e != cudaSuccess) return e;
         slots = std::max(1, sms * per);
     }
     const int grid = std::max(1, std::min(slots * std::max(1, grid_mult), (rows + MV_ROWS - 1) / MV_ROWS));
-    if constexpr (NORM) return launch_pdl(k_matvec16<TZ, true>, grid, MV_WARPS * 32, st, A, ld, rows, x, y, alpha, rinv);
-    k_matvec16<TZ, false><<<grid, MV_WARPS * 32, 0, st>>>(A, ld, rows, x, y, alpha, nullptr); ++g_launches;
-    return cudaGetLastError();
+    return launch_pdl(k_matvec16<TZ>, grid, MV_WARPS * 32, st, A, ld, rows, x, y, alpha, rinv);
 }
 
 template <typename TZ>
 cudaError_t matvec_norm(const TZ *A, size_t ld, int rows, int cols, const float *x, float *y, float alpha,
                         const float *rinv, cudaStream_t st, int grid_mult) {
     if (rows <= 0) return cudaSuccess;
-    if constexpr (sizeof(TZ) == 2) return launch_matvec16<TZ, true>(A, ld, rows, x, y, alpha, rinv, st, grid_mult);
+    if constexpr (sizeof(TZ) == 2) return launch_matvec16(A, ld, rows, x, y, alpha, rinv, st, grid_mult);
     else {
     static int slots = 0;   // resident CTAs of the GPU (per instantiation; one device per process)
     if (slots == 0) {
@@ -337,15 +332,6 @@ cudaError_t matvec(const TZ *A, size_t ld, int rows, int cols, const TX *x, TA *
         k_matvec<TZ, TX, TA, false><<<grid, MV_WARPS * 32, 0, st>>>(A, ld, rows, cols, x, y, alpha);
     ++g_launches;
     return cudaGetLastError();
-}
-
-template cudaError_t matvec<float, float, float>(const float *, size_t, int, int, const float *, float *, float, bool, cudaStream_t, int);
-cudaError_t matvec16(const __half *A, size_t ld, int rows, const float *x, float *y, float alpha, cudaStream_t st, int grid_mult) {
-    return launch_matvec16<__half, false>(A, ld, rows, x, y, alpha, nullptr, st, grid_mult);
-}
-cudaError_t matvec16(const __nv_bfloat16 *A, size_t ld, int rows, const float *x, float *y, float alpha, cudaStream_t st,
-                     int grid_mult) {
-    return launch_matvec16<__nv_bfloat16, false>(A, ld, rows, x, y, alpha, nullptr, st, grid_mult);
 }
 
 // largest |Re|, |Im| of a block, as the bit pattern of a non-negative float

@@ -40,13 +40,8 @@ cudaError_t launch_pdl(void (*kernel)(KA...), dim3 grid, int block, cudaStream_t
     ++g_launches;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KA>(args)...);
 }
-// y <- alpha A x for 16-bit A (column-interleaved rows of ld entries), FP32 vectors of
-// two right-hand sides, x zero up to pad_cols
-cudaError_t matvec16(const __half *A, size_t ld, int rows, const float *x, float *y, float alpha, cudaStream_t st,
-                     int grid_mult);
-cudaError_t matvec16(const __nv_bfloat16 *A, size_t ld, int rows, const float *x, float *y, float alpha, cudaStream_t st,
-                     int grid_mult);
-// y <- alpha A (x diag(rinv)), FP32 vectors (16-bit A: x zero up to pad_cols), rinv one
+// y <- alpha A (x diag(rinv)), FP32 vectors (16-bit A: column-interleaved rows of ld
+// entries, x zero up to pad_cols), rinv one
 // factor per right-hand side (device); launched with launch_pdl
 template <typename TZ>
 cudaError_t matvec_norm(const TZ *A, size_t ld, int rows, int cols, const float *x, float *y, float alpha,
