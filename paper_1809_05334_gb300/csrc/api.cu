@@ -242,17 +242,12 @@ int prepare(vie_ctx *ctx, const vie_request *req, HostReq &H) {
 }
 
 // the spectral polynomials of the far kernels and their coefficients on the device
-int far_poly(vie_ctx *ctx, const HostReq &H, vie::DevReq &q, cudaStream_t st) {
-    const vie::EwaldTables &ew = H.ew;
+int far_poly(vie_ctx *ctx, const vie::EwaldTables &ew, vie::DevReq &q, cudaStream_t st) {
     std::vector<float> coef;
     vie::build_far_poly(ew, q.ef, q.fp, coef);
     if (coef.empty()) coef.assign(1, 0.f);
     CK(upload(ctx->fcoef, coef, st));
     q.fcoef = ctx->fcoef.as<float>();
-    q.ph[0] = H.kx / M_PI + 2.0 * ew.p0 / ew.a;
-    q.ph[1] = H.ky / M_PI + 2.0 * ew.q0 / ew.b;
-    q.ph[2] = 2.0 / ew.a;
-    q.ph[3] = 2.0 / ew.b;
     return VIE_OK;
 }
 
@@ -314,7 +309,7 @@ int upload_request(vie_ctx *ctx, const HostReq &H, vie::DevReq &q, cudaStream_t 
     q.rtab = ctx->rtab.as<float4>();
     q.ew = ctx->ew.as<vie::EwaldTables>();
     q.ef = vie::make_ewald_f32(H.ew);
-    if (int e = far_poly(ctx, H, q, st)) return e;
+    if (int e = far_poly(ctx, H.ew, q, st)) return e;
     const size_t nt = (size_t)T.nt;
     CK(ctx->frec.ensure(sizeof(float4) * vie::far_record_count(nt, (size_t)nf)));
     q.ptet = ctx->frec.as<float4>();
@@ -1920,7 +1915,7 @@ int vie_green(vie_ctx *ctx, const vie_request *req, const double *d, double *out
     q.ef = vie::make_ewald_f32(H.ew);
     q.stab = ctx->stab.as<float>();
     if (precision != VIE_FP64)
-        if (int pe = far_poly(ctx, H, q, st)) return pe;
+        if (int pe = far_poly(ctx, H.ew, q, st)) return pe;
     if (q.fp.mode != vie::FAR_NONE)
         CK(vie::launch_green_poly(dd.as<double>(), dout.as<double>(), n, q, st));
     else

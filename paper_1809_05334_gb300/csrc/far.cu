@@ -22,40 +22,33 @@ namespace vie {
 // ---------------------------------------------------------------------------
 // element records of one request
 // ---------------------------------------------------------------------------
-// The phases are formed in FP64 and rounded once: a rounding of their argument is the same
-// for every partner of the point, so it does not average out over the pairs (as 2 x / a in
-// FP32 it shifted the orders, but not the images, by up to 1e-7 of a period).
-__device__ __forceinline__ void point_record(const DevReq &q, float4 *p, size_t n, const float *x, const float *c,
+__device__ __forceinline__ void point_record(const EwaldF32 &ef, float4 *p, size_t n, const float *x, const float *c,
                                              float w) {
-    const EwaldF32 &ef = q.ef;
     p[(size_t)FPT_POS * n] = make_float4(ef.Eih * x[0], ef.Eih * x[1], ef.Eih * x[2], w);
     p[(size_t)FPT_REL * n] = make_float4(x[0] - c[0], x[1] - c[1], x[2] - c[2], 0.f);
-    double s0, c0, s1, c1, s2, c2, s3, c3;
-    sincospi(q.ph[2] * x[0], &s2, &c2);
-    sincospi(q.ph[3] * x[1], &s3, &c3);
+    const float ip = 0.31830988618f;
+    float s0, c0, s1, c1, s2, c2, s3, c3;
+    sincospif(ef.step_x * ip * x[0], &s2, &c2);
+    sincospif(ef.step_y * ip * x[1], &s3, &c3);
     if (ef.sym) {
-        p[(size_t)FPT_PH0 * n] = make_float4((float)c2, (float)c3, (float)s2, (float)s3);
+        p[(size_t)FPT_PH0 * n] = make_float4(c2, c3, s2, s3);
         return;
     }
-    sincospi(q.ph[0] * x[0], &s0, &c0);
-    sincospi(q.ph[1] * x[1], &s1, &c1);
-    p[(size_t)FPT_PH0 * n] = make_float4((float)c0, (float)s0, (float)c1, (float)s1);
-    p[(size_t)FPT_PH1 * n] = make_float4((float)c2, (float)s2, (float)c3, (float)s3);
+    sincospif(ef.ob_kx0 * ip * x[0], &s0, &c0);
+    sincospif(ef.ob_ky0 * ip * x[1], &s1, &c1);
+    p[(size_t)FPT_PH0 * n] = make_float4(c0, s0, c1, s1);
+    p[(size_t)FPT_PH1 * n] = make_float4(c2, s2, c3, s3);
 }
 
-// four threads per element: each the record of one point (its phases are a few microseconds
-// of FP64 latency), the first also the element's
 __global__ void __launch_bounds__(128) k_far_prep(DevMesh m, const __grid_constant__ DevReq q) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int e = i >> 2, a = i & 3;
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
     const EwaldF32 &ef = q.ef;
     if (e < m.nt) {
         const float *f = m.far<float>(e);
-        point_record(q, q.ptet + (size_t)a * FPT * m.nt + e, m.nt, f + 3 * a, f + 12, f[27]);
-        if (a != 0) return;
         float rad = 0.f;
-        for (int p = 0; p < 4; ++p) {
-            const float u[3] = {f[3 * p] - f[12], f[3 * p + 1] - f[13], f[3 * p + 2] - f[14]};
+        for (int a = 0; a < 4; ++a) {
+            point_record(ef, q.ptet + (size_t)a * FPT * m.nt + e, m.nt, f + 3 * a, f + 12, f[27]);
+            const float u[3] = {f[3 * a] - f[12], f[3 * a + 1] - f[13], f[3 * a + 2] - f[14]};
             rad = fmaxf(rad, sqrtf(u[0] * u[0] + u[1] * u[1] + u[2] * u[2]));
         }
         float4 *o = q.etet + e;
@@ -71,17 +64,15 @@ __global__ void __launch_bounds__(128) k_far_prep(DevMesh m, const __grid_consta
         o[FEL_VY * n] = make_float4(f[16], f[19], f[22], f[25]);
         o[FEL_VZ * n] = make_float4(f[17], f[20], f[23], f[26]);
         o[FEL_ROW * n] = make_float4(__int_as_float(r[0]), __int_as_float(r[1]), __int_as_float(r[2]), __int_as_float(r[3]));
-        return;
     }
     const int fi = e - m.nt;
-    if (fi < m.nf && a < 3) {
+    if (fi >= 0 && fi < m.nf) {
         const float *f = m.ffar<float>(fi);
         float c[3], rad = 0.f;
         for (int d = 0; d < 3; ++d) c[d] = (f[d] + f[3 + d] + f[6 + d]) / 3.f;
-        point_record(q, q.pface + (size_t)a * FPT * m.nf + fi, m.nf, f + 3 * a, c, f[9]);
-        if (a != 0) return;
-        for (int p = 0; p < 3; ++p) {
-            const float u[3] = {f[3 * p] - c[0], f[3 * p + 1] - c[1], f[3 * p + 2] - c[2]};
+        for (int a = 0; a < 3; ++a) {
+            point_record(ef, q.pface + (size_t)a * FPT * m.nf + fi, m.nf, f + 3 * a, c, f[9]);
+            const float u[3] = {f[3 * a] - c[0], f[3 * a + 1] - c[1], f[3 * a + 2] - c[2]};
             rad = fmaxf(rad, sqrtf(u[0] * u[0] + u[1] * u[1] + u[2] * u[2]));
         }
         q.eface[fi] = make_float4(ef.Eih * c[0], ef.Eih * c[1], ef.Eih * c[2], ef.Eih * rad);
@@ -318,7 +309,7 @@ __global__ void __launch_bounds__(FAR_THREADS) k_green_p(const double *d, double
     const float x[3] = {-float(d[3 * i]), -float(d[3 * i + 1]), -float(d[3 * i + 2])};
     float4 rec[FPT];
     const float zero[3] = {0.f, 0.f, 0.f};
-    point_record(q, rec, 1, x, zero, 1.f);
+    point_record(ef, rec, 1, x, zero, 1.f);
     p2 gre[1], gim[1], tre[1], tim[1];
     far_eval<MODE, NQ, 1>(S, s_coef, q, 0, rec[FPT_POS], rec[FPT_PH0], MODE == FAR_NORMAL ? rec[FPT_PH0] : rec[FPT_PH1],
                           n_list, 0ull, 0ull, gre, gim, tre, tim);
@@ -342,7 +333,7 @@ static cudaError_t far_dispatch(const FarPoly &fp, F &&f) {
 }
 
 cudaError_t launch_far_prep(const DevMesh &m, const DevReq &q, cudaStream_t st) {
-    k_far_prep<<<(4 * (m.nt + m.nf) + 127) / 128, 128, 0, st>>>(m, q); ++g_launches;
+    k_far_prep<<<(m.nt + m.nf + 127) / 128, 128, 0, st>>>(m, q); ++g_launches;
     return cudaGetLastError();
 }
 

@@ -81,7 +81,6 @@ struct DevReq {
     const float4 *rtab;    // real parts of ztab (16 bytes per interval), read for the real tables
     const EwaldTables *ew; // Ewald parameters of the request (device memory)
     EwaldF32 ef;           // FP32 inner-loop parameters (kernel parameter space)
-    double ph[4];          // 1/pi times the wave numbers of the point records' phases: first order, step (x, y each)
     FarPoly fp;            // the spectral series as polynomials (fp.mode FAR_NONE: the tabulated form)
     const float *fcoef;    // their coefficients [fp.n_coef]
     // element records of the FP32 kernels, built per request (k_far_prep): points
