@@ -119,6 +119,8 @@ __global__ void __launch_bounds__(FAR_THREADS, MODE == FAR_FULL ? VIE_FAR_MINB_F
     constexpr int NP = 2;   // both pairs of test points at once
     const size_t nt = m.nt;
     float ws = 0.f;
+    // oblique incidence: S and T as 16 times their first value plus the sum of the differences
+    float ref[4] = {0.f, 0.f, 0.f, 0.f}, dif[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
     for (int b = 0; b < 4; ++b) {
         const float4 *p = q.ptet + (size_t)b * FPT * nt + s;
@@ -152,7 +154,18 @@ __global__ void __launch_bounds__(FAR_THREADS, MODE == FAR_FULL ? VIE_FAR_MINB_F
                 }
             };
             sums(gre, gim, s0c, sA);
-            if constexpr (MODE != FAR_NORMAL) sums(tre, tim, t0, tA);
+            if constexpr (MODE != FAR_NORMAL) {
+                sums(tre, tim, t0, tA);
+                auto differences = [&](const p2 (&v)[NP], float &r, float &d) {
+                    if (b == 0) r = upk(v[0]).x;
+                    const p2 nr = dup(-r);
+                    d += hsum(add2(add2(v[0], nr), add2(v[1], nr)));
+                };
+                differences(gre, ref[0], dif[0]);
+                differences(gim, ref[1], dif[1]);
+                differences(tre, ref[2], dif[2]);
+                differences(tim, ref[3], dif[3]);
+            }
         }
         const float r[3] = {rb.x, rb.y, rb.z};
         auto add = [&](Mom<float> &M, cx<float> z0, const cx<float> (&zA)[3]) {
@@ -167,7 +180,7 @@ __global__ void __launch_bounds__(FAR_THREADS, MODE == FAR_FULL ? VIE_FAR_MINB_F
         add(mo, s0c, sA);
         if constexpr (MODE != FAR_NORMAL) add(mc, t0, tA);
     }
-    const float wgt = q.ptet[(size_t)FPT_POS * nt + t].w * ws;
+    const float wt = q.ptet[(size_t)FPT_POS * nt + t].w, wgt = wt * ws;
     const TetRec rt = load_tet_rec(q.etet, m.nt, t), rs = load_tet_rec(q.etet, m.nt, s);
     const float k2 = float(q.k0 * q.k0);
     if constexpr (MODE == FAR_NORMAL) {
@@ -189,8 +202,10 @@ __global__ void __launch_bounds__(FAR_THREADS, MODE == FAR_FULL ? VIE_FAR_MINB_F
         mo.C = wgt * mo.C;
 #pragma unroll
         for (int d = 0; d < 3; ++d) { mo.A[d] = wgt * mo.A[d]; mo.B[d] = wgt * mo.B[d]; }
-        scatter_rec<false>(Z, N, k2, rt, rs, mo, mo.S, false);
-        if (s != t) scatter_rec<false>(Z, N, k2, rs, rt, mr, mr.S, false);
+        const W2 sr = {16.f * ref[0], dif[0]}, si = {16.f * ref[1], dif[1]}, tr = {32.f * ref[2], 2.f * dif[2]},
+                 ti = {32.f * ref[3], 2.f * dif[3]};   // T twice
+        scatter_w2(Z, N, k2, rt, rs, mo, charge_base({sr, si}, rs.kap, wt, ws, 9.f));
+        if (s != t) scatter_w2(Z, N, k2, rs, rt, mr, charge_base({w2_add(sr, ti), w2_add(tr, {-si.h, -si.l})}, rt.kap, wt, ws, 9.f));
     }
 }
 
@@ -229,7 +244,7 @@ __global__ void __launch_bounds__(FAR_THREADS) k_far_scalar_p(DevMesh m, const _
     const size_t n = YT ? m.nt : m.nf;
     const float4 *py = (YT ? q.ptet : q.pface) + y;
     cx<float> Sm = {0.f, 0.f};
-    float wy = 0.f;
+    float wy = 0.f, ref[2] = {0.f, 0.f}, dif[2] = {0.f, 0.f};   // oblique incidence: as k_far_tt_p
 #pragma unroll 1
     for (int b = 0; b < qy; ++b) {
         const float4 *p = py + (size_t)b * FPT * n;
@@ -244,37 +259,55 @@ __global__ void __launch_bounds__(FAR_THREADS) k_far_scalar_p(DevMesh m, const _
             for (int h = 0; h < NP; ++h) {
                 const float2 re = upk(gre[h]), im = upk(gim[h]);
                 const bool both = qx == 4 || h0 + h == 0;   // a face has no fourth point
-                Sm.re += both ? re.x + re.y : re.x;
-                Sm.im += both ? im.x + im.y : im.x;
+                if (MODE == FAR_NORMAL) {
+                    Sm.re += both ? re.x + re.y : re.x;
+                    Sm.im += both ? im.x + im.y : im.x;
+                } else {
+                    if (b == 0 && h == 0) { ref[0] = re.x; ref[1] = im.x; }
+                    dif[0] += both ? (re.x - ref[0]) + (re.y - ref[0]) : re.x - ref[0];
+                    dif[1] += both ? (im.x - ref[1]) + (im.y - ref[1]) : im.x - ref[1];
+                }
             }
         }
     }
     const float wx = (XT ? q.ptet : q.pface)[(XT ? (size_t)FPT_POS * m.nt : (size_t)FPT_POS * m.nf) + xe].w;
-    Sm = (wx * wy) * Sm;
+    // S times the weights and c: at normal incidence Sm, else both parts of the value
+    const float c = PK == 0 ? 3.f : (PK == 1 ? -3.f : -1.f);
+    const float np = float(qx * qy);   // 9, 12: np ref is rounded, the rest of it goes with the differences
+    auto two = [&](int k) { const float h = np * ref[k]; return W2{h, fmaf(np, ref[k], -h) + dif[k]}; };
+    auto base = [&](cx<float> f) -> CW2 {
+        if (MODE == FAR_NORMAL) {
+            const cx<float> v = f * ((wx * wy) * Sm);
+            return {{c * v.re, 0.f}, {c * v.im, 0.f}};
+        }
+        return charge_base({two(0), two(1)}, f, wx, wy, c);
+    };
+    auto times = [](CW2 v, float f) { return CW2{w2_mul(v.re, f), w2_mul(v.im, f)}; };
+    const cx<float> none = {0.f, 0.f};
     if constexpr (PK == 0) {
         const float4 fr = q.eface[(size_t)m.nf + y];
         const TetRec r = load_tet_rec(q.etet, m.nt, x);
-        const cx<float> qS = cx<float>{fr.x, fr.y} * Sm;
+        const CW2 qS = base({fr.x, fr.y});
         const size_t col = (size_t)__float_as_int(fr.z);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const cx<float> v = (3.f * r.coef[i]) * (r.w[i] * qS);
+            const cx<float> v = charge_value(times(qS, r.coef[i]), r.w[i], none);
             red_c(Z, (size_t)r.row[i] * N + col, v.re, v.im);
         }
     } else if constexpr (PK == 1) {
         const size_t row = (size_t)__float_as_int(q.eface[(size_t)m.nf + xe].z);
         const TetRec r = load_tet_rec(q.etet, m.nt, y);
-        const cx<float> kS = r.kap * Sm;
+        const CW2 kS = base(r.kap);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const cx<float> v = (-3.f * r.coef[j]) * (cconj(r.w[j]) * kS);
+            const cx<float> v = charge_value(times(kS, r.coef[j]), cconj(r.w[j]), none);
             red_c(Z, row * N + (size_t)r.row[j], v.re, v.im);
         }
     } else {
         const size_t row = (size_t)__float_as_int(q.eface[(size_t)m.nf + xe].z);
         const float4 fr = q.eface[(size_t)m.nf + y];
-        const cx<float> v = cx<float>{fr.x, fr.y} * Sm;
-        red_c(Z, row * N + (size_t)__float_as_int(fr.z), -v.re, -v.im);
+        const cx<float> v = charge_value(base({fr.x, fr.y}), {1.f, 0.f}, none);
+        red_c(Z, row * N + (size_t)__float_as_int(fr.z), v.re, v.im);
     }
 }
 
