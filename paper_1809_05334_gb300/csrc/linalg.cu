@@ -765,6 +765,11 @@ constexpr int GJ_T = 64;                // tile of the pivot-block inverse
 constexpr int GJ_DG = 4;                // row groups of its diagonal inverse (256 threads)
 constexpr int GJ_RQ = GJ_T / GJ_DG;     // rows per thread
 constexpr int GJ_THREADS = GJ_T * GJ_DG;
+// max|A_ss| max|D| from which the inverse D of a diagonal tile is refined.  Measured at 64 / 256 /
+// 1024 / 4096 with one step: 135 / 132 / 140 / 143 GMRES iterations at 20,618 unknowns with blocks
+// of condition 6e3 (131 before the tiles), 11.4 / 10.4 / 10.3 / 9.9 ms of factorisation at 9,882
+// unknowns (9.4 without it; 11.1 at 256 with the second step, 14.6 before the tiles)
+constexpr float GJ_REFINE = 256.f;
 constexpr int GJ_LDT = GJ_T + 2;        // row stride of the shared tiles (complex): conflict-free transposes
 constexpr size_t GJ_SMEM = 3 * (size_t)GJ_T * GJ_LDT * sizeof(float2);
 
@@ -879,7 +884,11 @@ __device__ __forceinline__ void gj_tile_mul(const float2 *Lt, const float2 *R, f
 // (i, j), with D = src tile (s, s)^-1:
 //   (s, s): D      (s, j): D A_sj      (i, s): -A_is D      else: A_ij - (A_is D) A_sj.
 // Every CTA inverts the diagonal tile itself, so a step is one launch without
-// packing or a wait between CTAs.  The block is padded with the identity to
+// packing or a wait between CTAs.  D is refined (Newton, one step or two): used as an explicit
+// inverse in both panels, its error, u cond(A_ss), would come back in every entry of
+// the block; without it blocks of condition 5e5 to 3e7 took 5 to 80 % more GMRES
+// iterations than with 128-wide inverses by elimination (15,840 unknowns 483 against 259,
+// with it 171; |M A - I| of a 4,320 block 0.63 -> 0.060, 0.45 by elimination).  The block is padded with the identity to
 // whole tiles (read so, not written).  Bound by the latency of the 32 pivot
 // pairs plus two 64^3 products on one SM (about 20 us a step); the 128-wide
 // register inverse with K = 128 tensor-core products in between took 104 us a
@@ -895,18 +904,78 @@ __global__ void __launch_bounds__(GJ_THREADS, 2)
         if (r < w && cc < w) return *reinterpret_cast<const float2 *>(src + 2 * ((size_t)r * lds + cc));
         return make_float2(r == cc ? 1.f : 0.f, 0.f);
     };
-    float2 a[GJ_RQ];
+    const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+    float2 a[GJ_RQ], acc[4][4];
+    auto largest = [&](unsigned *word) {   // into *word, the largest |Re|, |Im| of the tile
+        float v = 0.f;
+#pragma unroll
+        for (int q = 0; q < GJ_RQ; ++q) v = fmaxf(v, fmaxf(fabsf(a[q].x), fabsf(a[q].y)));
+        const unsigned u = __reduce_max_sync(0xffffffffu, __float_as_uint(v));
+        if ((threadIdx.x & 31) == 0) atomicMax(word, u);
+    };
+    // the panel tiles, A_is transposed and A_sj as it is
+    auto panels = [&] {
+        if (ti != s)
+#pragma unroll 4
+            for (int q = 0; q < GJ_RQ; ++q) bL[c * GJ_LDT + g + GJ_DG * q] = load(GJ_T * ti + g + GJ_DG * q, GJ_T * s + c);
+        if (tj != s)
+#pragma unroll 4
+            for (int q = 0; q < GJ_RQ; ++q) bR[(g + GJ_DG * q) * GJ_LDT + c] = load(GJ_T * s + g + GJ_DG * q, GJ_T * tj + c);
+    };
+    __shared__ unsigned size[2];   // the largest entries of A_ss and of D
+    if (threadIdx.x < 2) size[threadIdx.x] = 0u;
 #pragma unroll
     for (int q = 0; q < GJ_RQ; ++q) a[q] = load(GJ_T * s + g + GJ_DG * q, GJ_T * s + c);
-    // the panel tiles meanwhile: A_is transposed, A_sj as it is
-    if (ti != s)
-#pragma unroll 4
-        for (int q = 0; q < GJ_RQ; ++q) bL[c * GJ_LDT + g + GJ_DG * q] = load(GJ_T * ti + g + GJ_DG * q, GJ_T * s + c);
-    if (tj != s)
-#pragma unroll 4
-        for (int q = 0; q < GJ_RQ; ++q) bR[(g + GJ_DG * q) * GJ_LDT + c] = load(GJ_T * s + g + GJ_DG * q, GJ_T * tj + c);
+    __syncthreads();
+    largest(&size[0]);
+    panels();   // meanwhile
     const bool ok = gj_diag(a, c, g);
     if (!ok && ti == s && tj == s && threadIdx.x == 0) atomicOr(status, 1);
+    largest(&size[1]);
+    __syncthreads();
+    if (__uint_as_float(size[0]) * __uint_as_float(size[1]) > GJ_REFINE) {
+        // D + D (I - A_ss D); once more where the square of the residual would show
+        bool again = true;
+        for (int step = 0; again && step < 2; ++step) {
+#pragma unroll
+            for (int q = 0; q < GJ_RQ; ++q) {
+                const int r = g + GJ_DG * q;
+                bL[c * GJ_LDT + r] = load(GJ_T * s + r, GJ_T * s + c);
+                bR[r * GJ_LDT + c] = a[q];
+                bD[c * GJ_LDT + r] = a[q];
+            }
+            __syncthreads();
+            gj_tile_mul(bL, bR, acc, ty, tx);
+            __syncthreads();
+            float big = 0.f;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int r = 4 * ty + i, cc = tx + 16 * j;
+                    const float2 v = make_float2((r == cc ? 1.f : 0.f) - acc[i][j].x, -acc[i][j].y);
+                    big = fmaxf(big, fmaxf(fabsf(v.x), fabsf(v.y)));
+                    bR[r * GJ_LDT + cc] = v;
+                }
+            const bool gains = __syncthreads_and(big < 1.f);   // else the step would not converge
+            again = gains && __syncthreads_or(big > 1.f / 256.f);
+            if (gains) {
+                gj_tile_mul(bD, bR, acc, ty, tx);
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) bL[(4 * ty + i) * GJ_LDT + tx + 16 * j] = acc[i][j];
+                __syncthreads();
+#pragma unroll
+                for (int q = 0; q < GJ_RQ; ++q) {
+                    const float2 d = bL[(g + GJ_DG * q) * GJ_LDT + c];
+                    a[q] = make_float2(a[q].x + d.x, a[q].y + d.y);
+                }
+            }
+            __syncthreads();
+        }
+        panels();
+    }
     auto store = [&](int r, int cc, float2 v) {
         if (r < w && cc < w) *reinterpret_cast<float2 *>(dst + 2 * ((size_t)r * ldd + cc)) = v;
     };
@@ -922,8 +991,6 @@ __global__ void __launch_bounds__(GJ_THREADS, 2)
         bD[ti == s ? c * GJ_LDT + r : r * GJ_LDT + c] = a[q];
     }
     __syncthreads();
-    const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
-    float2 acc[4][4];
     if (ti == s) gj_tile_mul(bD, bR, acc, ty, tx);        // D A_sj
     else gj_tile_mul(bL, bD, acc, ty, tx);                // A_is D
     if (ti != s && tj != s) {
