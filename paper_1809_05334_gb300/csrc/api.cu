@@ -870,10 +870,13 @@ cudaEvent_t pool_event(void *c) { return static_cast<vie_ctx *>(c)->event(); }
 template <typename TZ>
 int factor(vie_ctx *ctx, const HostReq &H, std::vector<size_t> &moff, std::vector<size_t> &mld, cudaStream_t st,
            vie::KernelTimer *kt, bool full_inverse = false) {
+    // the FP64 path's stopped solutions hold the roundings of its preconditioner: the whole
+    // inverse, pivot blocks in registers (gj_invert_tc)
+    constexpr bool fp64 = std::is_same<TZ, double>::value;
     const int pivot = ctx->opt.precond_pivot > 0 ? ctx->opt.precond_pivot : (ctx->tune_pivot > 0 ? ctx->tune_pivot : 512);
     std::vector<int> grp(H.blk_n.size());   // columns per pivot group
     for (size_t k = 0; k < H.blk_n.size(); ++k)
-        grp[k] = full_inverse ? H.blk_n[k] : vie::gj_group(H.blk_n[k], pivot);
+        grp[k] = full_inverse || fp64 ? H.blk_n[k] : vie::gj_group(H.blk_n[k], pivot);
     size_t tot = 0;
     moff.clear();
     mld.clear();
@@ -914,7 +917,7 @@ int factor(vie_ctx *ctx, const HostReq &H, std::vector<size_t> &moff, std::vecto
         float *B = ctx->Minv.as<float>() + 2 * moff[k];
         CK((vie::copy_block<TZ, float>(ctx->Z.as<TZ>(), ctx->ld, H.blk_off[k], H.blk_n[k], B, mld[k], sk)));
         CK(vie::gj_invert_tc(B, mld[k], H.blk_n[k], ctx->status.as<int>(), big ? ctx->tcpack.p : ctx->tcpack2.p, sk,
-                             big ? ctx->aux_stream : ctx->side_stream, kt, pivot, grp[k]));
+                             big ? ctx->aux_stream : ctx->side_stream, kt, pivot, grp[k], fp64));
     }
     if (side) {
         CK(cudaEventRecord(ctx->side_done, ctx->side_stream));

@@ -773,8 +773,9 @@ constexpr float GJ_REFINE = 256.f;
 constexpr int GJ_LDT = GJ_T + 2;        // row stride of the shared tiles (complex): conflict-free transposes
 constexpr size_t GJ_SMEM = 3 * (size_t)GJ_T * GJ_LDT * sizeof(float2);
 
-// In-place Gauss-Jordan inverse of a 64 x 64 block held in registers (thread
-// (c, g): column c, rows g + 4q), two pivots per step: warp v owns the columns
+// In-place Gauss-Jordan inverse of a W x W block held in registers (thread
+// (c, g): column c, rows g + 4q), two pivots per step, `pivots` of them (even;
+// the block is the identity from there on): warp v owns the columns
 // c = 32 (v / 4) + lane and the row group g = v % 4, so the warps that own a
 // column sit on the four schedulers.  Step (j, j+1) with the 2 x 2 pivot block
 // P and rows R = A[j:j+2, :] is one update of every entry,
@@ -785,18 +786,20 @@ constexpr size_t GJ_SMEM = 3 * (size_t)GJ_T * GJ_LDT * sizeof(float2);
 // and the factors travel through double-buffered shared memory; the owners of
 // the next pair publish them right after their update, so one barrier per two
 // pivots suffices.  Returns false on a zero or non-finite pivot.
-__device__ __forceinline__ bool gj_diag(float2 (&a)[GJ_RQ], int c, int g) {
-    __shared__ float2 rowbuf[2][2][GJ_T];
-    __shared__ __align__(16) float2 colbuf[2][GJ_DG][GJ_RQ][2];   // factors (f0, f1) of the pivot pair, row g + 4q
+template <int W>
+__device__ __forceinline__ bool gj_diag(float2 (&a)[W / GJ_DG], int c, int g, int pivots) {
+    constexpr int RQ = W / GJ_DG;
+    __shared__ float2 rowbuf[2][2][W];
+    __shared__ __align__(16) float2 colbuf[2][GJ_DG][RQ][2];   // factors (f0, f1) of the pivot pair, row g + 4q
     bool ok = true;
     if (g < 2) rowbuf[0][g][c] = a[0];
     if (c < 2) {
 #pragma unroll
-        for (int q = 0; q < GJ_RQ; ++q) colbuf[0][g][q][c] = a[q];
+        for (int q = 0; q < RQ; ++q) colbuf[0][g][q][c] = a[q];
         if (g == c) colbuf[0][g][0][c] = make_float2(a[0].x - 1.f, a[0].y);
     }
 #pragma unroll 1
-    for (int j = 0; j < GJ_T; j += 2) {
+    for (int j = 0; j < pivots; j += 2) {
         const int b = (j >> 1) & 1, nb = b ^ 1, jn = j + 2;
         __syncthreads();
         const float2 p00 = rowbuf[b][0][j], p01 = rowbuf[b][0][j + 1], p10 = rowbuf[b][1][j], p11 = rowbuf[b][1][j + 1];
@@ -814,7 +817,7 @@ __device__ __forceinline__ bool gj_diag(float2 (&a)[GJ_RQ], int c, int g) {
             m0 = c == j ? q00 : q01;
             m1 = c == j ? q10 : q11;
 #pragma unroll
-            for (int q = 0; q < GJ_RQ; ++q) a[q] = make_float2(g + GJ_DG * q == c ? 1.f : 0.f, 0.f);
+            for (int q = 0; q < RQ; ++q) a[q] = make_float2(g + GJ_DG * q == c ? 1.f : 0.f, 0.f);
         } else {
             const float2 r0 = rowbuf[b][0][c], r1 = rowbuf[b][1][c];
             m0 = make_float2(q00.x * r0.x - q00.y * r0.y + q01.x * r1.x - q01.y * r1.y,
@@ -823,25 +826,25 @@ __device__ __forceinline__ bool gj_diag(float2 (&a)[GJ_RQ], int c, int g) {
                              q10.x * r0.y + q10.y * r0.x + q11.x * r1.y + q11.y * r1.x);
         }
 #pragma unroll
-        for (int q = 0; q < GJ_RQ; ++q) {
+        for (int q = 0; q < RQ; ++q) {
             const float4 ff = *reinterpret_cast<const float4 *>(&colbuf[b][g][q][0]);
             a[q].x = fmaf(-ff.x, m0.x, fmaf(ff.y, m0.y, fmaf(-ff.z, m1.x, fmaf(ff.w, m1.y, a[q].x))));
             a[q].y = fmaf(-ff.x, m0.y, fmaf(-ff.y, m0.x, fmaf(-ff.z, m1.y, fmaf(-ff.w, m1.x, a[q].y))));
         }
-        if (jn < GJ_T) {
+        if (jn < pivots) {
             // rows jn, jn + 1: groups jn % 4 and jn % 4 + 1, slot jn / 4
             const int gj = jn & (GJ_DG - 1), qn = jn / GJ_DG;
             if (g == gj || g == gj + 1) {
                 float2 r = a[0];
 #pragma unroll
-                for (int q = 1; q < GJ_RQ; ++q)
+                for (int q = 1; q < RQ; ++q)
                     if (q == qn) r = a[q];
                 rowbuf[nb][g - gj][c] = r;
             }
             if (c == jn || c == jn + 1) {   // columns jn, jn + 1: the factors, diagonal ones minus one
                 const int h = c - jn;
 #pragma unroll
-                for (int q = 0; q < GJ_RQ; ++q) colbuf[nb][g][q][h] = a[q];
+                for (int q = 0; q < RQ; ++q) colbuf[nb][g][q][h] = a[q];
                 if (g == gj + h) {
                     const float2 dj = rowbuf[nb][h][c];
                     colbuf[nb][g][qn][h] = make_float2(dj.x - 1.f, dj.y);
@@ -851,6 +854,29 @@ __device__ __forceinline__ bool gj_diag(float2 (&a)[GJ_RQ], int c, int g) {
     }
     __syncthreads();
     return ok;
+}
+
+// In-place inverse of the w x w block (w <= GJ_W) at A in the registers of one CTA, for
+// the preconditioner of the FP64 path (gj_invert_tc, regs).  Latency, one barrier per two
+// pivots on one SM: slower than the tiles above a block of 64.
+constexpr int GJ_W = 128;
+__global__ void __launch_bounds__(GJ_W * GJ_DG) k_gj_regs(float *A, size_t ld, int w, int *status) {
+    const int wv = threadIdx.x >> 5;
+    const int c = 32 * (wv >> 2) + (threadIdx.x & 31), g = wv & (GJ_DG - 1);
+    float2 a[GJ_W / GJ_DG];
+#pragma unroll
+    for (int q = 0; q < GJ_W / GJ_DG; ++q) {
+        const int i = g + GJ_DG * q;
+        a[q] = make_float2(i == c && (i >= w || c >= w) ? 1.f : 0.f, 0.f);   // identity on the padding
+        if (i < w && c < w) a[q] = *reinterpret_cast<const float2 *>(A + 2 * ((size_t)i * ld + c));
+    }
+    const bool ok = gj_diag<GJ_W>(a, c, g, (w + 1) & ~1);
+    if (!ok && threadIdx.x == 0) atomicOr(status, 1);
+#pragma unroll
+    for (int q = 0; q < GJ_W / GJ_DG; ++q) {
+        const int i = g + GJ_DG * q;
+        if (i < w && c < w) *reinterpret_cast<float2 *>(A + 2 * ((size_t)i * ld + c)) = a[q];
+    }
 }
 
 // acc = L R for 64 x 64 complex tiles, L transposed in shared memory (Lt[k][row]),
@@ -929,7 +955,7 @@ __global__ void __launch_bounds__(GJ_THREADS, 2)
     __syncthreads();
     largest(&size[0]);
     panels();   // meanwhile
-    const bool ok = gj_diag(a, c, g);
+    const bool ok = gj_diag<GJ_T>(a, c, g, GJ_T);
     if (!ok && ti == s && tj == s && threadIdx.x == 0) atomicOr(status, 1);
     largest(&size[1]);
     __syncthreads();
@@ -1075,7 +1101,7 @@ constexpr int GJ_PMAX = 1024;
 #define VIE_GROUPS2_MIN 3072
 #endif
 static_assert(GJ_PMAX <= TC_KP, "the packed operands hold one outer pivot block");
-static_assert(GJ_P % GJ_T == 0 && GJ_PMAX % GJ_P == 0, "a pivot block is inverted in 64-wide steps, a wide one in two halves");
+static_assert(GJ_P % GJ_W == 0 && GJ_P % GJ_T == 0 && GJ_PMAX % GJ_P == 0, "a pivot block is inverted in 64- or 128-wide steps, a wide one in two halves");
 static_assert(GJ_P % TC_TM == 0, "no product tile straddles a pivot block");
 
 constexpr int GJ_WORDS = 16;   // largest-entry words: 4 per set (products (a), (3)), 2 for the pivot blocks
@@ -1140,14 +1166,20 @@ cudaError_t invert_small(float *Ab, size_t ld, int w, int *status, float *ping, 
     return cudaGetLastError();
 }
 
-// In-place inverse of the w x w pivot block at Ab (row stride ld, w <= GJ_PMAX):
-// a wide block by Gauss-Jordan with two 512-wide pivots, their products on the
-// tensor cores (K = 512).  sub: packed operand scratch of 3 GJ_PMAX rows; amax:
-// two largest-entry words.
+// In-place inverse of the w x w pivot block at Ab (row stride ld, w <= GJ_PMAX): by
+// Gauss-Jordan with 512-wide pivots (a wide block has two), or with 128-wide ones
+// inverted in registers (regs), their products on the tensor cores (K = the pivots'
+// width).  sub: packed operand scratch of 3 GJ_PMAX rows; amax: two largest-entry words.
 cudaError_t invert_pivot_block(float *Ab, size_t ld, int w, int *status, __half *sub, float *ping, unsigned *amax,
-                               int sms, cudaStream_t st) {
-    cudaError_t e = invert_small(Ab, ld, std::min(w, GJ_P), status, ping, st);
-    if (w <= GJ_P || e != cudaSuccess) return e;
+                               int sms, bool regs, cudaStream_t st) {
+    const int W = regs ? GJ_W : GJ_P;
+    auto invert = [&](float *A, int wi) -> cudaError_t {
+        if (!regs) return invert_small(A, ld, wi, status, ping, st);
+        k_gj_regs<<<1, GJ_W * GJ_DG, 0, st>>>(A, ld, wi, status); ++g_launches;
+        return cudaGetLastError();
+    };
+    cudaError_t e = invert(Ab, std::min(w, W));
+    if (w <= W || e != cudaSuccess) return e;
     __half *Ap = sub, *Bp = sub + (size_t)GJ_PMAX * TC_PACK_ROW;
     const int wc = (w + 3) / 4 * 4;   // whole 16-byte column groups (padding columns stay zero)
     CUtensorMap tA, tB, tC, tCs;
@@ -1157,10 +1189,10 @@ cudaError_t invert_pivot_block(float *Ab, size_t ld, int w, int *status, __half 
         !tensor_map(&tCs, Ab, 2 * (uint64_t)wc, w, 8 * ld, 32, 32))
         return cudaErrorInvalidValue;
     const int wp = (w + TC_TM - 1) / TC_TM * TC_TM;
-    for (int k1 = 0; k1 < w; k1 += GJ_P) {
-        const int wi = std::min(GJ_P, w - k1), m1 = w - wi;
+    for (int k1 = 0; k1 < w; k1 += W) {
+        const int wi = std::min(W, w - k1), m1 = w - wi;
         if (k1 > 0) {
-            e = invert_small(Ab + 2 * ((size_t)k1 * ld + k1), ld, wi, status, ping, st);
+            e = invert(Ab + 2 * ((size_t)k1 * ld + k1), wi);
             if (e != cudaSuccess) return e;
         }
         const int mp1 = (m1 + TC_TM - 1) / TC_TM * TC_TM;
@@ -1203,8 +1235,16 @@ cudaError_t invert_pivot_block(float *Ab, size_t ld, int w, int *status, __half 
 // same n^2 entries (linalg.h, precond_step), for 8 n^3 (1 + 1/4 + ...) / p
 // flops instead of 8 n^3: 0.47 of them with four groups.  group >= n gives the
 // inverse itself.
+// regs: pivot blocks by 128-wide steps in registers, for the FP64 path.  Its iteration
+// stops three or four steps in, at a residual that is a power of the inverse's rounding
+// error, so the stopped solution holds the roundings of this very inverse: with the tiles
+// it moved by up to 4e-9 in 36 slab solutions (tolerance 1e-8; converged ones agree to 5e-14),
+// more than double-precision results may move; with these steps 33 of them repeat to 1e-14
+// (one FP32 rounding of the matrix falls the other way in the rest, 3.4e-10 at most).  The
+// factor takes 1.41 ms at 936 unknowns.  The FP32 and 16-bit paths, refined to 1e-6, take
+// the tiles.
 cudaError_t gj_invert_tc(float *A, size_t ld, int n, int *status, void *pack, cudaStream_t st, cudaStream_t aux,
-                         KernelTimer *kt, int pivot, int group) {
+                         KernelTimer *kt, int pivot, int group, bool regs) {
     const int P = (pivot == GJ_PMAX) ? GJ_PMAX : GJ_P;   // outer pivot width
     // SMs the rest of each product leaves to the next pivot block's inverse
     const int reserve = P > GJ_P ? VIE_GJ_RESERVE_WIDE : VIE_GJ_RESERVE;
@@ -1240,7 +1280,7 @@ cudaError_t gj_invert_tc(float *A, size_t ld, int n, int *status, void *pack, cu
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&evB, cudaEventDisableTiming);
     if (e != cudaSuccess) return e;
     bool pending = false;   // the second part of the previous product (3) is running on aux
-    e = invert_pivot_block(A, ld, std::min(n, P), status, sub, ping, words + 8, sms, st);
+    e = invert_pivot_block(A, ld, std::min(n, P), status, sub, ping, words + 8, sms, regs, st);
     for (int g0 = 0; g0 < n && e == cudaSuccess; g0 += std::min(group, n - g0)) {
         // the submatrix from the group's first pivot on: rows and columns before it are done
         float *Ag = A + 2 * ((size_t)g0 * ld + g0);
@@ -1290,7 +1330,7 @@ cudaError_t gj_invert_tc(float *A, size_t ld, int n, int *status, void *pack, cu
                 tc_product(st, tmA[cur], tmB[cur], tmC, tmCs, mb, std::min(tiles(ng, m), sms), status, kt, ng, m, w);
             }
             if (next)
-                e = invert_pivot_block(A + 2 * ((size_t)k1 * ld + k1), ld, wn, status, sub, ping, words + 8, sms, st);
+                e = invert_pivot_block(A + 2 * ((size_t)k1 * ld + k1), ld, wn, status, sub, ping, words + 8, sms, regs, st);
         }
     }
     if (pending) cudaStreamWaitEvent(st, evB, 0);

@@ -89,10 +89,11 @@ struct KernelTimer {
 // pivot: width of the outer pivot blocks, 512 (default) or 1024 (half the
 // passes over the block).  group: columns per pivot group, a multiple of the
 // pivot width; group >= n leaves the inverse in A, a smaller one the
-// block-triangular factor that precond_step applies (linalg.cu)
+// block-triangular factor that precond_step applies (linalg.cu).  regs: pivot blocks
+// by 128-wide steps in registers (the FP64 path)
 size_t gj_pack_bytes(int n);
 cudaError_t gj_invert_tc(float *A, size_t ld, int n, int *status, void *pack, cudaStream_t st, cudaStream_t aux,
-                         KernelTimer *kt, int pivot, int group);
+                         KernelTimer *kt, int pivot, int group, bool regs = false);
 // columns per pivot group that vie_solve takes for a block of n unknowns
 int gj_group(int n, int pivot);
 
