@@ -131,7 +131,8 @@ struct vie_ctx {
     DevBuf dens;   // per-tetrahedron absorbed fractions [2][nt] (request density_out)
     double zh_alpha = 1.0;   // 1 / (power-of-two scale of the FP16 copy)
     // set by the solve server when the request is cancelled: a solve checks it
-    // between phases and at every GMRES iteration (the stream is idle there)
+    // between phases and before every GMRES iteration, and waits for its stream
+    // before it returns
     const std::atomic<int> *cancel = nullptr;
     // autotuner choices for this mesh (0: the defaults): the FP32 tables' Ewald
     // split multiplier per incidence class (0 normal, 1 oblique), and the row

@@ -88,7 +88,8 @@ __global__ void __launch_bounds__(128) k_far_prep(DevMesh m, const __grid_consta
 // spatial table, 83% busy, 56% of the issue slots (9,882 unknowns, normal incidence).
 // Measured (ms, far tetrahedron pairs; per-lane spectral table entries, single
 // points and scalar atomics before): 21,024 unknowns 37.3 -> 19.8 at normal
-// incidence, 59.3 -> 26.6 in the fold, 82.6 -> 33.7 full rectangle; 48,678
+// incidence, 59.3 -> 28.7 in the fold, 82.6 -> 35.1 full rectangle (26.6 and 33.7 with
+// the charge term in single roundings, far_poly.cuh); 48,678
 // unknowns 223 -> 98.
 // ---------------------------------------------------------------------------
 template <int MODE, int NQ>
